@@ -383,9 +383,8 @@ jagp_status_t jagp_walker_status(jagp_handle_t h, const void *d_state, int W, in
 /* Tile autotuner (no counterpart in the paper: a property of this GPU code).
  * Times the candidate tilings of the per-walker products (proposed rows and
  * columns: one output per thread, 32x32 or 64x64 register-blocked tiles; the
- * refresh product G~ = Phi_up Bt^T likewise) and, in the mixed path, the
- * output-tile width (32..128 columns) and pipeline depth of the tensor-core
- * lambda products, on
+ * refresh product G~ = Phi_up Bt^T likewise) and, with tensor-core lambda
+ * products, their output-tile width and K chunk width, on
  * this handle's operands and the caller's state buffer of W walkers; keeps the
  * fastest in the handle for every later call.  The choices change only the
  * tiling of outputs, never the order of a sum: results are identical with or
@@ -396,13 +395,13 @@ typedef struct {
   int tile_proposals;  /* 0: one output per thread; 32 / 64: blocked tiles; 16 (refresh, mixed,
                           N_up <= 16): four walkers per CTA, 2x2 outputs per thread */
   int tile_refresh;
-  int umma_bn_left;    /* mixed path: tensor-core tile width, A_up = phi^T lambda (0 in FP64) */
-  int umma_bn_right;   /* mixed path: tensor-core tile width, Bt = lambda phi */
+  int umma_bn_left;    /* tensor-core tile width at most, A_up = phi^T lambda (0 in plain FP64; 64: as
+                          wide as tensor memory holds the accumulators of, by the shape) */
+  int umma_bn_right;   /* the same, Bt = lambda phi */
   float ms[4];
-  int umma_stages_left;   /* pipeline stages of those products (0: as many as fit in 200 KB;
-                             -1, -2, -3: chunk-major, two to four stages each holding every
-                             slice of one K chunk of 64, 32 or 16 elements, so that a slice
-                             is read once for all its pairs) */
+  int umma_stages_left;   /* K chunk of a stage of those products: -1, -2, -3: 64, 32 or 16 elements;
+                             0 and any other value: by the shape (every stage holds every slice of its
+                             K chunk, and as many stages are kept as fit in shared memory) */
   int umma_stages_right;
 } jagp_tuning_t;
 jagp_status_t jagp_autotune(jagp_handle_t h, void *d_state, int W, jagp_tuning_t *out, void *stream);

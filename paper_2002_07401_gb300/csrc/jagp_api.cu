@@ -178,7 +178,8 @@ jagp_status_t lambda_products(jagp_ctx *h, const double *P, const float *, doubl
            launch_umma_gemm(pack, max_rows, count, h->tc_slices, left ? h->split_lamT : h->split_lam, h->ds.L,
                             h->tc_slices, h->kp, np, pa, pb, nullptr, h->ds.L, rows, h->d_err, st, exps,
                             left ? h->exp_lamT : h->exp_lam, nullptr, left ? h->tune_bn_left : h->tune_bn_right, out,
-                            h->tc_bits, 0, 0, left ? h->tune_st_left : h->tune_st_right));
+                            h->tc_bits, 0, 0, left ? h->tune_st_left : h->tune_st_right, 0, 0, 0, 0,
+                            left ? h->range_lamT : h->range_lam, h->ds.L));
     return JAGP_OK;
   }
   LAUNCH(JAGP_KERNEL_LAMBDA_ROWS, 1,
@@ -204,7 +205,8 @@ jagp_status_t lambda_products(jagp_ctx *h, const float *P, const float *P_lo, fl
                           kFixedSlices, h->kp, kFixedPairs, kPairA, kPairB, out, h->ds.L,
                           rows, h->d_err, st, exps, left ? h->exp_lamT : h->exp_lam, out_lo,
                           left ? h->tune_bn_left : h->tune_bn_right, nullptr, 8, 0, 0,
-                          left ? h->tune_st_left : h->tune_st_right));
+                          left ? h->tune_st_left : h->tune_st_right, 0, 0, 0, 0,
+                          left ? h->range_lamT : h->range_lam, h->ds.L));
   return JAGP_OK;
 }
 
@@ -265,7 +267,7 @@ jagp_status_t run_kinetic_mixed(jagp_ctx *h, const double *r, void *state, int W
                           pb, eb, nullptr, 0, 0, st));
   LAUNCH(JAGP_KERNEL_ENERGY, 1,
          launch_umma_gemm(pb, W * Lb, nullptr, kFixedSlices, pa, n, kFixedSlices, kpn, kFixedPairs, kPairA, kPairB, mb,
-                          0, nullptr, h->d_err, st, eb, ea, ml, 0, nullptr, 8, Lb, W, 0, n, NL, 1, Lb));
+                          0, nullptr, h->d_err, st, eb, ea, ml, 0, nullptr, 8, Lb, W, 0, n, NL, 1, Lb, nullptr, n));
   if (nd > 0) {
     // down electrons: A = columns of A_up, B = rows j < N_dn of G~^{-1}
     LAUNCH(0, 1,
@@ -276,7 +278,7 @@ jagp_status_t run_kinetic_mixed(jagp_ctx *h, const double *r, void *state, int W
     LAUNCH(JAGP_KERNEL_ENERGY, 1,
            launch_umma_gemm(pb, W * Lb, nullptr, kFixedSlices, pa, nd, kFixedSlices, kpn, kFixedPairs, kPairA, kPairB,
                             mb + (size_t)n * Lb, 0, nullptr, h->d_err, st, eb, ea, ml + (size_t)n * Lb, 0, nullptr, 8,
-                            Lb, W, 0, nd, NL, 1, Lb));
+                            Lb, W, 0, nd, NL, 1, Lb, nullptr, n));
   }
   LAUNCH(JAGP_KERNEL_ENERGY, 1, launch_kinetic_m2(d, r, mb, ml, at<double>(state, L.kin), W, st));
   return JAGP_OK;
@@ -331,7 +333,8 @@ jagp_status_t run_refresh(jagp_ctx *h, const double *r, void *state, int W, int 
     group_subkey(1);
     LAUNCH(JAGP_KERNEL_GEMM_ROWS, 1,
            launch_umma_gemm(pa, W * n, nullptr, kFixedSlices, pb, n, kFixedSlices, h->kp, kFixedPairs, kPairA, kPairB,
-                            nullptr, n, nullptr, h->d_err, st, ea, eb, nullptr, 0, gm, 8, n, W));
+                            nullptr, n, nullptr, h->d_err, st, ea, eb, nullptr, 0, gm, 8, n, W, 0, 0, 0, 0, 0,
+                            nullptr, Lb));
   } else {
     group_subkey(1);
     LAUNCH(JAGP_KERNEL_GEMM_ROWS, 1,
@@ -657,7 +660,7 @@ static jagp_status_t jagp_grad_impl(jagp_handle_t h, const double *d_r, void *d_
     LAUNCH(JAGP_KERNEL_LAMBDA_ROWS, 1,
            launch_umma_gemm(pu, G.nseg * Lb, nullptr, kLamBarSlices, pv, Lb, kLamBarSlices, G.kpseg, np, pa, pb,
                             nullptr, 0, nullptr, h->d_err, st, eu, ev, nullptr, 0, wp(G.tc_part), kLamBarBits, Lb,
-                            G.nseg, 0, Lb, (long long)Lb * Lb, Lb, 1));
+                            G.nseg, 0, Lb, (long long)Lb * Lb, Lb, 1, nullptr, G.seg_w * n));
     LAUNCH(0, 1, launch_adj_lambda_sum(wp(G.tc_part), G.nseg, Lb, d_dlambda, st));
   } else if (d_dlambda) {
     LAUNCH(0, 1,
@@ -817,12 +820,26 @@ jagp_status_t jagp_create(jagp_handle_t *out, const jagp_system_t *sys, const ja
   const size_t split_bytes = tc ? (size_t)L * nterms * kp * 2 : 0;
   const size_t exp_bytes = tc ? (size_t)L * 4 : 0;
   const size_t oSA = take(split_bytes), oSB = take(split_bytes), oXA = take(exp_bytes), oXB = take(exp_bytes);
+  const size_t oGA = take((tc ? (L + 15) / 16 : 0) * sizeof(int2)), oGB = take((tc ? (L + 15) / 16 : 0) * sizeof(int2));
   const size_t oE = take(16);
   const size_t oJG = take((size_t)jgeo.size() * sizeof(double4)), oJI = take(jinfo.size() * sizeof(int));
   const size_t oJP = take((size_t)LJ * LJ * 8), oJA = take((size_t)LJ * LJ * 8);
   std::vector<uint16_t> sA(split_bytes / 2, 0), sB(split_bytes / 2, 0);
   std::vector<int> xA(tc ? L : 0), xB(tc ? L : 0);
+  // rows of the sliced operands in blocks of 16: the range of K in which any of
+  // them is non-zero (a banded lambda's products skip the rest)
+  const int nblk = tc ? (L + 15) / 16 : 0;
+  std::vector<int2> gA(nblk, make_int2(L, 0)), gB(nblk, make_int2(L, 0));
   if (tc) {
+    for (int i = 0; i < L; ++i)
+      for (int j = 0; j < L; ++j)
+        if (sys->lambda[(size_t)i * L + j] != 0.0) {
+          int2 &a = gA[j / 16], &b = gB[i / 16];
+          a.x = std::min(a.x, i);
+          a.y = std::max(a.y, i + 1);
+          b.x = std::min(b.x, j);
+          b.y = std::max(b.y, j + 1);
+        }
     for (int nn = 0; nn < L; ++nn) {
       // column nn, then row nn
       uint16_t *ra = &sA[(size_t)nn * nterms * kp], *rb = &sB[(size_t)nn * nterms * kp];
@@ -855,7 +872,9 @@ jagp_status_t jagp_create(jagp_handle_t *out, const jagp_system_t *sys, const ja
             (!tc || (cudaMemcpy(b + oSA, sA.data(), split_bytes, cudaMemcpyHostToDevice) == cudaSuccess &&
                         cudaMemcpy(b + oSB, sB.data(), split_bytes, cudaMemcpyHostToDevice) == cudaSuccess &&
                         cudaMemcpy(b + oXA, xA.data(), exp_bytes, cudaMemcpyHostToDevice) == cudaSuccess &&
-                        cudaMemcpy(b + oXB, xB.data(), exp_bytes, cudaMemcpyHostToDevice) == cudaSuccess)) &&
+                        cudaMemcpy(b + oXB, xB.data(), exp_bytes, cudaMemcpyHostToDevice) == cudaSuccess &&
+                        cudaMemcpy(b + oGA, gA.data(), nblk * sizeof(int2), cudaMemcpyHostToDevice) == cudaSuccess &&
+                        cudaMemcpy(b + oGB, gB.data(), nblk * sizeof(int2), cudaMemcpyHostToDevice) == cudaSuccess)) &&
             cudaMemset(b + oE, 0, 16) == cudaSuccess &&
             (LJ == 0 ||
              (cudaMemcpy(b + oJG, jgeo.data(), jgeo.size() * sizeof(double4), cudaMemcpyHostToDevice) == cudaSuccess &&
@@ -911,6 +930,8 @@ jagp_status_t jagp_create(jagp_handle_t *out, const jagp_system_t *sys, const ja
   h->split_lam = tc ? reinterpret_cast<const uint16_t *>(b + oSB) : nullptr;
   h->exp_lamT = tc ? reinterpret_cast<const int *>(b + oXA) : nullptr;
   h->exp_lam = tc ? reinterpret_cast<const int *>(b + oXB) : nullptr;
+  h->range_lamT = tc ? reinterpret_cast<const int2 *>(b + oGA) : nullptr;
+  h->range_lam = tc ? reinterpret_cast<const int2 *>(b + oGB) : nullptr;
   h->tc_lambda = tc;
   h->tc_slices = nsl;
   h->tc_bits = bits;
@@ -1027,20 +1048,17 @@ jagp_status_t tune_products(jagp_ctx *h, void *state, int W, cudaStream_t st, ja
   const int np64 = slice_pairs(h->tc_slices, pa64, pb64);
   for (int side = 0; side < 2; ++side) {
     const bool left = side == 0;
-    // tile widths; 16 lets several CTAs share an SM's tensor memory (6 x 16 columns each)
-    const int cands[7] = {16, 32, 48, 64, 80, 96, 128};
-    // stages: as many as fit (one CTA per SM), three or two (several CTAs per SM),
-    // or chunk-major (every slice of a K chunk of 64, 32 or 16 per stage, each
-    // loaded once for all pairs; two to four stages, where they fit)
-    const int stages[6] = {0, 3, 2, -1, -2, -3};
+    // tile widths (64: the widest that fits, by the shape rule) and K chunk widths
+    // (0: the rule; -1, -2, -3: 64, 32, 16 where two stages of every slice fit)
+    const int cands[4] = {64, 48, 32, 16};
+    const int stages[4] = {0, -1, -2, -3};
     const int npairs = f64 ? np64 : kFixedPairs;
     const int *tpa = f64 ? pa64 : kPairA, *tpb = f64 ? pb64 : kPairB;
-    const int limit = 64;  // six or more accumulators of bn columns in tensor memory
+    const int2 *range = left ? h->range_lamT : h->range_lam;
     float bs = 0.0f;
     int bbn = 0, bst = 0;
-    for (int c = 0; c < 7; ++c)
-      for (int q = 0; q < 6; ++q) {
-        if (cands[c] > limit) continue;
+    for (int c = 0; c < 4; ++c)
+      for (int q = 0; q < 4; ++q) {
         if (stages[q] < 0 && !umma_chunk_fits(npairs, tpa, tpb, cands[c], stages[q])) continue;
         float ms = 0.0f;
         JAGP_CU(time_calls(
@@ -1050,12 +1068,12 @@ jagp_status_t tune_products(jagp_ctx *h, void *state, int W, cudaStream_t st, ja
                 return launch_umma_gemm(pack, rows, nullptr, h->tc_slices, left ? h->split_lamT : h->split_lam, Lb,
                                         h->tc_slices, h->kp, np64, pa64, pb64, nullptr, Lb, nullptr, h->d_err, st,
                                         exps, left ? h->exp_lamT : h->exp_lam, nullptr, cands[c],
-                                        reinterpret_cast<double *>(dst), h->tc_bits, 0, 0, stages[q]);
+                                        reinterpret_cast<double *>(dst), h->tc_bits, 0, 0, stages[q], 0, 0, 0, 0, range, Lb);
               return launch_umma_gemm(pack, rows, nullptr, kFixedSlices, left ? h->split_lamT : h->split_lam, Lb,
                                       kFixedSlices, h->kp, kFixedPairs, kPairA, kPairB,
                                       reinterpret_cast<float *>(dst), Lb, nullptr, h->d_err, st, exps,
                                       left ? h->exp_lamT : h->exp_lam, at<float>(state, left ? L.a_up_lo : L.bt_lo),
-                                      cands[c], nullptr, 8, 0, 0, stages[q]);
+                                      cands[c], nullptr, 8, 0, 0, stages[q], 0, 0, 0, 0, range, Lb);
             },
             st, &ms));
         if (bbn == 0 || ms < bs) {

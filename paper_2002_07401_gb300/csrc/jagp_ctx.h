@@ -28,6 +28,8 @@ struct jagp_ctx {
   const uint16_t *split_lam = nullptr;   // [L][5 kp]: row n slices lambda[n, :]  (Bt = lambda phi)
   const int *exp_lamT = nullptr;         // [L] exponents of those rows
   const int *exp_lam = nullptr;          // [L]
+  // non-zero K range [x, y) per 16 rows of the sliced lambda^T and lambda
+  const int2 *range_lamT = nullptr, *range_lam = nullptr;
   int *d_err = nullptr;                  // tensor-core pipeline timeout flag
   // tile choices of jagp_autotune (0 / -1: the shape heuristics)
   int tune_bn_left = 0, tune_bn_right = 0;  // tensor-core tile width of the lambda products

@@ -123,7 +123,12 @@ cudaError_t launch_increment(uint32_t *c, uint32_t by, cudaStream_t st);
 // aligned bases); rows m < *m_dev (or m_max) are written; out FP32, pitch ldo.
 // With a_exp/b_exp (row / column exponents) the terms are fixed-point slices and
 // pairs of equal a + b share an exact accumulator (see k_umma.cu).
-// stages_max: pipeline depth (0: as many as fit); -1, -2, -3: chunk-major stages (K chunks of 64, 32, 16).
+// Every slice pair a + b < ns of ns = 6, 7 or 8 slices (two-float or FP64 result)
+// runs in k_umma_tri; only there: out64, batches, an affine output, bn_max (0 or
+// 64: the widest tile the shape rule takes; 16, 32, 48: that width at most),
+// stages_max (-1, -2, -3: K chunks of 64, 32, 16; else the rule), klive (K
+// elements per term that may be non-zero; 0: kp) and krange (non-zero K range
+// [x, y) per 16 rows of B; null: [0, klive)).
 int umma_pick_bn(int n, int max_bn);
 cudaError_t launch_umma_gemm(const uint16_t *A, int m_max, const int *m_dev, int a_terms, const uint16_t *B, int n,
                              int b_terms, int kp, int npairs, const int *pair_a, const int *pair_b, float *out,
@@ -131,7 +136,8 @@ cudaError_t launch_umma_gemm(const uint16_t *A, int m_max, const int *m_dev, int
                              const int *a_exp = nullptr, const int *b_exp = nullptr, float *out_lo = nullptr,
                              int bn_max = 0, double *out64 = nullptr, int slice_bits = 8, int batch_rows = 0,
                              int batches = 0, int stages_max = 0, int b_batch_rows = 0, long long o_bstride = 0,
-                             long long o_rstride = 0, long long o_cstride = 0, const int *pair_group = nullptr);
+                             long long o_rstride = 0, long long o_cstride = 0, const int2 *krange = nullptr,
+                             int klive = 0);
 // whether two chunk-major stages (stages_max = -1, -2, -3: K chunks of 64, 32,
 // 16) of these pairs fit at tile width bn
 bool umma_chunk_fits(int npairs, const int *pair_a, const int *pair_b, int bn, int stages_max);

@@ -18,20 +18,17 @@
 // accuracy, which the lossy FP32 accumulation inside the tensor cores would
 // not give.
 //
-// One CTA computes a 128 x BN tile: warp 0 lane 0 issues the TMA loads, warp 1
-// lane 0 issues the MMAs (one per 16-wide K slice), all four warps drain the
-// accumulator from tensor memory (warp w owns TMEM lanes 32w..32w+31 = rows).
-// Stages hold one A and one B slice of a 64-wide K chunk, pair after pair; in
-// chunk-major modes (stages_max = -1, -2, -3: K chunks of 64, 32, 16) a stage holds every slice of
-// the chunk and the MMA thread issues all pairs from it.  CTAs walk kGroupM row
-// tiles of one column tile before the next, so that a wave shares operand
-// tiles in L2.  Every wait is bounded by the global timer; a timeout sets *err.
+// Two kernels.  k_umma_gemm takes any list of slice pairs: one CTA per 128 x BN
+// tile, stages of one A and one B slice of a 64-wide K chunk, pair after pair.
+// k_umma_tri takes the full triangle of pairs (a + b < NS) that every product
+// of the library uses; see there.  Every wait is bounded by the global timer; a
+// timeout sets *err.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
+#include <atomic>
 #include <mutex>
 
-#include "jagp_group.cuh"
 #include "jagp_group.cuh"
 #include "jagp_launch.h"
 
@@ -151,15 +148,6 @@ struct UmmaArgs {
   int npairs;
   int pair_a[kMaxPairs], pair_b[kMaxPairs], pair_group[kMaxPairs];
   int ngroups;           // accumulators (1 in plain mode)
-  int slice_bits;        // fixed-point mode: bits per slice (8, or 7 for long K)
-  double *out64;         // fixed-point mode: FP64 result instead of out / out_lo, or null
-  int batch_rows;        // batched mode (> 0): A and B are stacked per-batch blocks of batch_rows
-                         // rows; batch b's rows of A meet only batch b's rows of B
-  int tiles_per_batch;   // batched mode: 128-row tiles per batch
-  int b_batch_rows;      // batched mode: rows of B per batch (= batch_rows unless given)
-  int chunk_major;       // 1: one stage holds every slice of one K chunk of A (na) and B (nb),
-  int na, nb;            //    and the MMA thread issues all pairs from it (slices loaded once per chunk)
-  int cw;                // K chunk width in elements: 64, or 32 / 16 for chunk-major stages of many slices
   const int *a_exp;      // fixed-point mode: row exponents [m_max], else null
   const int *b_exp;      // fixed-point mode: column exponents [n]
   uint32_t idesc;
@@ -168,9 +156,6 @@ struct UmmaArgs {
   float *out_lo;         // fixed-point mode: low part of a two-float result, or null
   long long ldo;         // output row pitch (elements)
   const int *out_rows;   // destination row of row m, or null (= m)
-  // batched mode, affine output (o_cstride != 0): the element of local row r
-  // (within its batch b) and column c goes to out[b o_bstride + r o_rstride + c o_cstride]
-  long long o_bstride, o_rstride, o_cstride;
   int *err;
 };
 
@@ -180,8 +165,6 @@ struct UmmaGemm {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int M = g.m_dev ? *g.m_dev : g.m_max;
-    // batched mode: tile t of batch b starts at row b * batch_rows + 128 t; rows
-    // past the batch's end (read from the next batch) are computed but not written
     // grouped tile order: CTAs in launch order walk kGroupM row tiles of one
     // column tile before the next column tile, so that a wave reuses both A and
     // B tiles from L2 (with large K the operands exceed L2)
@@ -196,18 +179,12 @@ struct UmmaGemm {
       tile_y = first + r % gsize;
       tile_x = r / gsize;
     }
-    const int bb = g.batch_rows ? tile_y / g.tiles_per_batch : 0;
-    const int bt0 = g.batch_rows ? (tile_y - bb * g.tiles_per_batch) * 128 : 0;
-    const int m0 = g.batch_rows ? bb * g.batch_rows + bt0 : tile_y * 128;
-    const int bbase = bb * g.b_batch_rows;  // first B row (and column exponent) of this batch
+    const int m0 = tile_y * 128;
     if (m0 >= M) return;  // whole CTA, before any barrier or tensor-memory use
     const int n0 = tile_x * g.bn;
-    const uint32_t row_bytes = static_cast<uint32_t>(g.cw) * 2u;  // 128, 64 or 32
-    const uint32_t a_bytes = 128u * row_bytes;
-    const uint32_t b_bytes = static_cast<uint32_t>(g.bn) * row_bytes;
-    const int ksteps = g.cw / 16;  // MMAs (K = 16) per chunk
-    const uint32_t stage_bytes =
-        g.chunk_major ? static_cast<uint32_t>(g.na) * a_bytes + static_cast<uint32_t>(g.nb) * b_bytes : a_bytes + b_bytes;
+    const uint32_t a_bytes = 128u * 128u;
+    const uint32_t b_bytes = static_cast<uint32_t>(g.bn) * 128u;
+    const uint32_t stage_bytes = a_bytes + b_bytes;
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + g.stages * stage_bytes);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * g.stages + 1);
     const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8u * g.stages, done = full0 + 16u * g.stages;
@@ -230,52 +207,12 @@ struct UmmaGemm {
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    const int kchunks = g.kp / g.cw;
-    const int iters = g.chunk_major ? kchunks : g.npairs * kchunks;
+    const int kchunks = g.kp / 64;
+    const int iters = g.npairs * kchunks;
     const uint32_t tiles = smem_u32(smem);
 
     if (warp == 0 && lane == 0) tensormap_acquire(&tmA, &tmB);
-    if (warp == 0 && lane == 0 && g.chunk_major) {
-      // producer, chunk-major: every slice of A and B for one K chunk per stage
-      for (int it = 0; it < iters; ++it) {
-        const int s = it % g.stages;
-        const uint32_t use = static_cast<uint32_t>(it / g.stages);
-        if (it >= g.stages && !mbar_wait(empty0 + 8u * s, (use & 1u) ^ 1u)) {
-          atomicExch(g.err, 1);
-          break;
-        }
-        const uint32_t full = full0 + 8u * s, base = tiles + s * stage_bytes;
-        mbar_expect_tx(full, stage_bytes);
-        for (int a = 0; a < g.na; ++a) tma_load_2d(base + a * a_bytes, &tmA, a * g.kp + it * g.cw, m0, full);
-        for (int b = 0; b < g.nb; ++b)
-          tma_load_2d(base + g.na * a_bytes + b * b_bytes, &tmB, b * g.kp + it * g.cw, bbase + n0, full);
-      }
-    } else if (warp == 1 && lane == 0 && g.chunk_major) {
-      // MMA issuer, chunk-major: all pairs of the chunk from the one stage
-      uint32_t started = 0;
-      for (int it = 0; it < iters; ++it) {
-        const int s = it % g.stages;
-        const uint32_t use = static_cast<uint32_t>(it / g.stages);
-        if (!mbar_wait(full0 + 8u * s, use & 1u)) {
-          atomicExch(g.err, 2);
-          break;
-        }
-        tc_fence_after();
-        const uint32_t base = tiles + s * stage_bytes;
-        for (int p = 0; p < g.npairs; ++p) {
-          const int grp = g.pair_group[p];
-          const uint32_t a0 = base + g.pair_a[p] * a_bytes, b0 = base + g.na * a_bytes + g.pair_b[p] * b_bytes;
-          const uint32_t d_tmem = tmem + static_cast<uint32_t>(grp * g.bn);
-          for (int kk = 0; kk < ksteps; ++kk) {
-            umma_bf16(d_tmem, desc_kmajor(a0 + kk * 32, row_bytes), desc_kmajor(b0 + kk * 32, row_bytes), g.idesc,
-                      (started >> grp) & 1u);
-            started |= 1u << grp;
-          }
-        }
-        umma_commit(empty0 + 8u * s);
-      }
-      umma_commit(done);
-    } else if (warp == 0 && lane == 0) {
+    if (warp == 0 && lane == 0) {
       // producer: one A tile (128 x 64) and one B tile (bn x 64) per stage
       for (int it = 0; it < iters; ++it) {
         const int s = it % g.stages;
@@ -288,7 +225,7 @@ struct UmmaGemm {
         mbar_expect_tx(full, stage_bytes);
         const int p = it / kchunks, c = it - p * kchunks;
         tma_load_2d(tiles + s * stage_bytes, &tmA, g.pair_a[p] * g.kp + c * 64, m0, full);
-        tma_load_2d(tiles + s * stage_bytes + a_bytes, &tmB, g.pair_b[p] * g.kp + c * 64, bbase + n0, full);
+        tma_load_2d(tiles + s * stage_bytes + a_bytes, &tmB, g.pair_b[p] * g.kp + c * 64, n0, full);
       }
     } else if (warp == 1 && lane == 0) {
       // MMA issuer: four K = 16 slices per 64-wide chunk, accumulating in TMEM
@@ -321,38 +258,12 @@ struct UmmaGemm {
     tc_fence_after();
     if (ready) {
       const int row = m0 + warp * 32 + lane;
-      const bool live = row < M && (!g.batch_rows || bt0 + warp * 32 + lane < g.batch_rows);
+      const bool live = row < M;
       const long long dst = live ? (g.out_rows ? g.out_rows[row] : row) : 0;
-      // element offset of this row's column 0 and the stride between columns
-      const long long obase = g.o_cstride ? (long long)bb * g.o_bstride + (long long)(bt0 + warp * 32 + lane) * g.o_rstride
-                                          : dst * g.ldo;
-      const long long ocs = g.o_cstride ? g.o_cstride : 1;
+      const long long obase = dst * g.ldo;  // element offset of this row's column 0
       const uint32_t t_row = tmem + (static_cast<uint32_t>(warp * 32) << 16);
       const int ea = (g.a_exp && live) ? g.a_exp[row] : 0;
       for (int c = 0; c < g.bn; c += 16) {
-        if (g.out64) {
-          // FP64 result: v = S_0 + 2^-b (S_1 + 2^-b (S_2 + ...)) by Horner in FP64
-          // from the exact integer sums, then the power-of-two scale
-          double acc[16];
-  #pragma unroll
-          for (int j = 0; j < 16; ++j) acc[j] = 0.0;
-          const double wq = ldexp(1.0, -g.slice_bits);
-          for (int q = g.ngroups - 1; q >= 0; --q) {
-            float u[16];
-            tmem_ld16(t_row + static_cast<uint32_t>(q * g.bn + c), u);
-  #pragma unroll
-            for (int j = 0; j < 16; ++j) acc[j] = fma(acc[j], wq, static_cast<double>(u[j]));
-          }
-          if (live) {
-            double *o = g.out64 + obase;
-  #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              const int col = n0 + c + j;
-              if (col < g.n) o[col * ocs] = ldexp(acc[j], ea + g.b_exp[bbase + col] - 2 * (g.slice_bits - 1));
-            }
-          }
-          continue;
-        }
         float v[16];
         tmem_ld16(t_row + static_cast<uint32_t>(c), v);
         if (g.a_exp) {
@@ -382,7 +293,7 @@ struct UmmaGemm {
             const float hi = __fadd_rn(v[j], lo[j]);
             const float l2 = __fsub_rn(lo[j], __fsub_rn(hi, v[j]));
             const int col = n0 + c + j;
-            const int sh = ea + (col < g.n ? g.b_exp[bbase + col] : 0) - 14;
+            const int sh = ea + (col < g.n ? g.b_exp[col] : 0) - 14;
             v[j] = ldexpf(hi, sh);
             lo[j] = ldexpf(l2, sh);
           }
@@ -390,14 +301,14 @@ struct UmmaGemm {
             float *ol = g.out_lo + obase;
   #pragma unroll
             for (int j = 0; j < 16; ++j)
-              if (n0 + c + j < g.n) ol[(n0 + c + j) * ocs] = lo[j];
+              if (n0 + c + j < g.n) ol[n0 + c + j] = lo[j];
           }
         }
         if (live) {
           float *o = g.out + obase;
   #pragma unroll
           for (int j = 0; j < 16; ++j)
-            if (n0 + c + j < g.n) o[(n0 + c + j) * ocs] = v[j];
+            if (n0 + c + j < g.n) o[n0 + c + j] = v[j];
         }
       }
     } else if (lane == 0) {
@@ -416,6 +327,440 @@ __global__ void __launch_bounds__(128) k_umma_gemm(const __grid_constant__ CUten
                                                    const __grid_constant__ CUtensorMap tmB,
                                                    const __grid_constant__ UmmaArgs g) {
   UmmaGemm::run(tmA, tmB, g, blockIdx, gridDim);
+}
+
+// ---------------------------------------------------------------------------
+// k_umma_tri: the fixed-point product with every pair a + b < NS of NS slices.
+//
+// What bounds it: each 128 x 64 x 16 MMA takes 32 clocks of the tensor pipe but
+// reads 4 KB of A and 2 KB of B from shared memory (48 clocks), so one MMA per
+// pair is bound by operand reads.  The B slices of a K chunk are stacked in
+// shared memory, and accumulator d sits bn tensor-memory columns after
+// accumulator d - 1, so the pairs (a, 0) .. (a, NS - 1 - a) of one A slice are ONE
+// product of that slice with the stacked B slices into consecutive
+// accumulators: 6 A slices give 8 MMAs of up to 256 columns per K = 16 step
+// instead of 21 of 64, and A is read 8 times instead of 21.
+//
+// Persistent CTAs (one per SM: warp 0 TMA, warp 1 MMA, eight epilogue warps)
+// walk the tiles, so that the next tile's operands load during the epilogue.
+// Two CTAs of a cluster take neighbouring column tiles of one row tile and
+// each multicasts half of the A slices to both, which lowers the L2 reads per
+// tile from NS (128 + bn) to NS (64 + bn) rows per K.  Only the K chunks in
+// which the B tile has a non-zero element are visited (krange: [first, last)
+// per 16 rows of B, found when lambda is sliced): zeros change no exact sum, so
+// a banded pairing matrix costs its band, and the padding of K costs nothing.
+//
+// TMEM: NS accumulators of bn <= 512 / NS columns.  The CTA asks for more than
+// half of the SM's shared memory, so that two CTAs (of clusters that each hold one
+// SM of a pair) never wait for each other's tensor memory.
+//
+// Measured against one MMA per pair in CTA-per-tile launches: the six-slice
+// lambda products of the accepted rows of 4096 walkers (about 30 thousand rows,
+// K = N = 320) 403 -> 120 us (1.06 PFLOP/s of slice products); seven slices, 2048
+// walkers, FP64 result 443 -> 136 us; the six products of a 512-electron sweep
+// (64 walkers, K = N = 4096, a tenth of lambda non-zero) 39.3 -> 4.0 ms.
+// ---------------------------------------------------------------------------
+constexpr int kTriThreads = 320;
+constexpr int kTriEpiWarps = 8;
+
+struct TriArgs {
+  int m_max;             // rows the grid covers
+  const int *m_dev;      // live row count on the device, or null (= m_max)
+  int n, bn, tiles_n;    // output columns, columns per CTA, column tiles
+  int kp, klive;         // K per slice (row pitch of a slice), elements that may be non-zero
+  int cw, stages;        // K chunk width in elements (64, 32, 16), chunks in flight
+  int cl;                // CTAs per cluster (1, 2)
+  const int2 *krange;    // non-zero K range per 16 rows of B, or null (= [0, klive))
+  int slice_bits;
+  int batch_rows, tiles_per_batch, b_batch_rows;  // batched mode (batch_rows > 0): block b of A against block b of B
+  const int *a_exp, *b_exp;
+  float *out, *out_lo;
+  double *out64;
+  long long ldo;
+  const int *out_rows;
+  long long o_bstride, o_rstride, o_cstride;
+  int vec;               // output rows take 32-byte stores
+  int *err;
+};
+
+__device__ __forceinline__ void tma_load_2d_mc(uint32_t dst, const CUtensorMap *map, int x, int y, uint32_t bar,
+                                               uint16_t mask) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1, "
+      "{%2, %3}], [%4], %5;" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar), "h"(mask)
+      : "memory");
+}
+
+__device__ __forceinline__ void umma_commit_mc(uint32_t bar, uint16_t mask) {
+  asm volatile(
+      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+      "h"(mask)
+      : "memory");
+}
+
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
+// sixteen columns of this warp's lanes; valid after tmem_ld_wait
+__device__ __forceinline__ void tmem_ld16_async(uint32_t taddr, uint32_t r[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+}
+
+// v * 2^sh, rounded once: by the factor 2^sh where that is a normal number
+__device__ __forceinline__ float scale_pow2(float v, int sh) {
+  return sh >= -126 && sh <= 127 ? __fmul_rn(v, __int_as_float((sh + 127) << 23)) : ldexpf(v, sh);
+}
+__device__ __forceinline__ double scale_pow2(double v, int sh) {
+  const long long b = __double_as_longlong(v);
+  const int e = static_cast<int>((b >> 52) & 0x7ff);
+  return e > 0 && e < 0x7ff && e + sh > 0 && e + sh < 0x7ff ? __longlong_as_double(b + (static_cast<long long>(sh) << 52))
+                                                            : ldexp(v, sh);
+}
+// an integer |x| < 2^51 as FP64 (one FP64 instruction)
+__device__ __forceinline__ double small_int_to_double(long long x) {
+  return __longlong_as_double(0x4338000000000000LL + x) - 6755399441055744.0;
+}
+
+__device__ __forceinline__ void store8(float *p, const float *v) {
+  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]),
+               "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+               : "memory");
+}
+__device__ __forceinline__ void store4(double *p, const double *v) {
+  asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(v[0]), "d"(v[1]), "d"(v[2]), "d"(v[3])
+               : "memory");
+}
+
+template <int NS, bool F64>
+struct UmmaTri {
+  static __device__ __forceinline__ void run(const CUtensorMap &tmA, const CUtensorMap &tmB, const TriArgs &g,
+                                             const uint3 bid, const uint3 gdim) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    const int M = g.m_dev ? *g.m_dev : g.m_max;
+    const int cl = g.cl, rank = cl == 2 ? static_cast<int>(bid.x & 1u) : 0;
+    const int tiles_m = g.batch_rows ? (g.m_max / g.batch_rows) * g.tiles_per_batch : (M + 127) / 128;
+    const int ctiles = (g.tiles_n + cl - 1) / cl;  // column tiles in steps of the cluster
+    const int total = tiles_m * ctiles;
+    const int first = static_cast<int>(bid.x) / cl, step = static_cast<int>(gdim.x) / cl;
+    if (first >= total) return;  // both CTAs of a cluster, before any barrier or tensor-memory use
+    const uint32_t row_bytes = static_cast<uint32_t>(g.cw) * 2u;
+    const uint32_t a_bytes = 128u * row_bytes, b_bytes = static_cast<uint32_t>(g.bn) * row_bytes;
+    const uint32_t stage_bytes = NS * (a_bytes + b_bytes);
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + g.stages * stage_bytes);
+    const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8u * g.stages, tfull = full0 + 16u * g.stages,
+                   tempty = tfull + 8u;
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * g.stages + 2);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+      for (int s = 0; s < g.stages; ++s) {
+        mbar_init(full0 + 8u * s, 1);
+        mbar_init(empty0 + 8u * s, static_cast<uint32_t>(cl));
+      }
+      mbar_init(tfull, 1);
+      mbar_init(tempty, kTriEpiWarps);
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                   "r"(512)
+                   : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (cl == 2) {  // the peer's barriers exist before anything arrives there
+      asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+      asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+    const uint32_t tiles = smem_u32(smem);
+
+    // tile t of this cluster: row tile, first column of the cluster's column tiles
+    auto place = [&](int t, int &ty, int &cx) {
+      // kGroupM row tiles of one column step before the next, so that a wave
+      // shares operand tiles in L2
+      const int span = kGroupM * ctiles, q = t / span, r = t - q * span;
+      const int gsize = tiles_m - q * kGroupM < kGroupM ? tiles_m - q * kGroupM : kGroupM;
+      ty = q * kGroupM + r % gsize;
+      cx = r / gsize;
+    };
+    // K chunks [c0, c1) of the cluster's column tiles (the same in both CTAs)
+    auto chunks = [&](int cx, int &c0, int &c1) {
+      int lo = 0, hi = g.klive;
+      if (g.krange) {
+        lo = g.kp;
+        hi = 0;
+        const int b0 = cx * cl * g.bn / 16, b1 = b0 + cl * g.bn / 16, nb = (g.n + 15) / 16;
+        for (int b = b0; b < b1 && b < nb; ++b) {
+          const int2 r = g.krange[b];
+          lo = r.x < lo ? r.x : lo;
+          hi = r.y > hi ? r.y : hi;
+        }
+      }
+      c0 = lo / g.cw;
+      c1 = (hi + g.cw - 1) / g.cw;
+      if (c1 <= c0) {  // every element zero: one chunk clears the accumulators
+        c0 = 0;
+        c1 = 1;
+      }
+    };
+    auto rows_of = [&](int ty, int &bb, int &bt0, int &m0) {
+      bb = g.batch_rows ? ty / g.tiles_per_batch : 0;
+      bt0 = g.batch_rows ? (ty - bb * g.tiles_per_batch) * 128 : 0;
+      m0 = g.batch_rows ? bb * g.batch_rows + bt0 : ty * 128;
+    };
+
+    if (warp == 0) {
+      if (lane == 0) {
+        // producer: every slice of A (its share of them, to both CTAs of a
+        // cluster) and of its own B tile for one K chunk per stage
+        tensormap_acquire(&tmA, &tmB);
+        int it = 0;
+        bool ok = true;
+        for (int t = first; t < total && ok; t += step) {
+          int ty, cx, c0, c1, bb, bt0, m0;
+          place(t, ty, cx);
+          chunks(cx, c0, c1);
+          rows_of(ty, bb, bt0, m0);
+          const int brow = bb * g.b_batch_rows + (cx * cl + rank) * g.bn;
+          for (int c = c0; c < c1; ++c, ++it) {
+            const int s = it % g.stages;
+            if (it >= g.stages && !mbar_wait(empty0 + 8u * s, ((it / g.stages) & 1u) ^ 1u)) {
+              atomicExch(g.err, 1);
+              ok = false;
+              break;
+            }
+            const uint32_t full = full0 + 8u * s, base = tiles + s * stage_bytes, bbase = base + NS * a_bytes;
+            mbar_expect_tx(full, stage_bytes);
+  #pragma unroll
+            for (int a = 0; a < NS; ++a) {
+              if (cl == 1)
+                tma_load_2d(base + a * a_bytes, &tmA, a * g.kp + c * g.cw, m0, full);
+              else if ((a & 1) == rank)
+                tma_load_2d_mc(base + a * a_bytes, &tmA, a * g.kp + c * g.cw, m0, full, 3);
+            }
+  #pragma unroll
+            for (int b = 0; b < NS; ++b) tma_load_2d(bbase + b * b_bytes, &tmB, b * g.kp + c * g.cw, brow, full);
+          }
+        }
+        // the last uses of every stage: their consumers' arrivals (of both CTAs)
+        // land, and no load is in flight, before this CTA ends
+        for (int u = it > g.stages ? it - g.stages : 0; u < it; ++u)
+          if (!mbar_wait(empty0 + 8u * (u % g.stages), (u / g.stages) & 1u)) {
+            atomicExch(g.err, 1);
+            break;
+          }
+      }
+    } else if (warp == 1) {
+      if (lane == 0) {
+        int it = 0, done = 0;
+        bool ok = true;
+        const uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(128 >> 4) << 24);
+        const int ksteps = g.cw / 16;
+        for (int t = first; t < total && ok; t += step, ++done) {
+          int ty, cx, c0, c1;
+          place(t, ty, cx);
+          chunks(cx, c0, c1);
+          if (done > 0 && !mbar_wait(tempty, (done - 1) & 1u)) {
+            atomicExch(g.err, 2);
+            break;
+          }
+          tc_fence_after();
+          for (int c = c0; c < c1; ++c, ++it) {
+            const int s = it % g.stages;
+            if (!mbar_wait(full0 + 8u * s, (it / g.stages) & 1u)) {
+              atomicExch(g.err, 2);
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+            const uint32_t base = tiles + s * stage_bytes;
+            const uint64_t da = desc_kmajor(base, row_bytes), db = desc_kmajor(base + NS * a_bytes, row_bytes);
+            for (int kk = 0; kk < ksteps; ++kk) {
+              // descriptor addresses count 16-byte units
+              const uint64_t ak = da + kk * 2, bk = db + kk * 2;
+              const uint32_t init = (c > c0 || kk > 0) ? 1u : 0u;
+  #pragma unroll
+              for (int a = 0; a < NS; ++a) {
+                // slice a against stacked slices 0 .. NS - 1 - a, into accumulators a .. NS - 1
+                const int cols = (NS - a) * g.bn;
+                const uint64_t aa = ak + a * (a_bytes >> 4);
+                const uint32_t d = tmem + static_cast<uint32_t>(a * g.bn);
+                const uint32_t acc = a > 0 ? 1u : init;
+                const int n1 = cols < 256 ? cols : 256;
+                umma_bf16(d, aa, bk, idesc0 | (static_cast<uint32_t>(n1 >> 3) << 17), acc);
+                if (cols > 256)
+                  umma_bf16(d + 256u, aa, bk + ((256u * row_bytes) >> 4),
+                            idesc0 | (static_cast<uint32_t>((cols - 256) >> 3) << 17), acc);
+              }
+            }
+            if (cl == 2)
+              umma_commit_mc(empty0 + 8u * s, 3);
+            else
+              umma_commit(empty0 + 8u * s);
+          }
+          if (ok) umma_commit(tfull);
+        }
+      }
+    } else {
+      // epilogue warps 2 .. 9: tensor-memory lanes 32 (warp % 4) .. + 31 are the
+      // rows, the two warps of a lane quarter take alternate 16-column groups
+      const int quarter = warp & 3, half = (warp - 2) >> 2;
+      const int ngrp = g.bn / 16;
+      int done = 0;
+      for (int t = first; t < total; t += step, ++done) {
+        int ty, cx, bb, bt0, m0;
+        place(t, ty, cx);
+        rows_of(ty, bb, bt0, m0);
+        const int n0 = (cx * cl + rank) * g.bn;
+        const int r = quarter * 32 + lane, row = m0 + r;
+        const bool live = row < M && (!g.batch_rows || bt0 + r < g.batch_rows);
+        const long long dst = live ? (g.out_rows ? g.out_rows[row] : row) : 0;
+        const long long obase =
+            g.o_cstride ? (long long)bb * g.o_bstride + (long long)(bt0 + r) * g.o_rstride : dst * g.ldo;
+        const long long ocs = g.o_cstride ? g.o_cstride : 1;
+        const int ea = live ? g.a_exp[row] : 0;
+        const int *be = g.b_exp + bb * g.b_batch_rows;
+        const uint32_t t_row = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
+        if (!__all_sync(0xffffffffu, mbar_wait(tfull, done & 1u))) {  // warp-uniform for tcgen05.ld
+          if (lane == 0) atomicExch(g.err, 3);
+          break;
+        }
+        tc_fence_after();
+        bool released = false;
+        for (int cg = half; cg < ngrp; cg += 2) {
+          uint32_t u[NS][16];
+  #pragma unroll
+          for (int q = 0; q < NS; ++q) tmem_ld16_async(t_row + static_cast<uint32_t>(q * g.bn + cg * 16), u[q]);
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          // the values may be used from here on, not earlier
+  #pragma unroll
+          for (int q = 0; q < NS; ++q)
+  #pragma unroll
+            for (int j = 0; j < 16; ++j) asm volatile("" : "+r"(u[q][j]));
+          if (cg + 2 >= ngrp) {  // this warp's last reads: the accumulators may be overwritten
+            tc_fence_before();
+            if (lane == 0) mbar_arrive(tempty);
+            released = true;
+          }
+          const int c0 = n0 + cg * 16;
+          if constexpr (F64) {
+            // the exact sums as two integers of NS / 2 terms each (H leading, the
+            // rest below), joined by one rounding: hi 2^(b (NS - H)) + lo
+            constexpr int H = NS / 2;
+            const int b = g.slice_bits;
+            const double up = __longlong_as_double(static_cast<long long>(1023 + b * (NS - H)) << 52);
+            const int sh0 = ea - b * (NS - 1) - 2 * (b - 1);
+            double v[16];
+  #pragma unroll
+            for (int j = 0; j < 16; ++j) {
+              long long hi = 0, lo = 0;
+  #pragma unroll
+              for (int q = 0; q < H; ++q) hi = hi * (1ll << b) + __float2int_rn(__uint_as_float(u[q][j]));
+  #pragma unroll
+              for (int q = H; q < NS; ++q) lo = lo * (1ll << b) + __float2int_rn(__uint_as_float(u[q][j]));
+              double s = fma(small_int_to_double(hi), up, small_int_to_double(lo));
+              // a non-finite operand shows in its leading slice's sum
+              if (!(fabsf(__uint_as_float(u[0][j])) <= 3.0e38f)) s = __longlong_as_double(0x7ff8000000000000LL);
+              v[j] = scale_pow2(s, sh0 + (c0 + j < g.n ? be[c0 + j] : 0));
+            }
+            if (live) {
+              double *o = g.out64 + obase;
+              if (g.vec && c0 + 16 <= g.n) {
+  #pragma unroll
+                for (int j = 0; j < 16; j += 4) store4(o + c0 + j, v + j);
+              } else {
+  #pragma unroll
+                for (int j = 0; j < 16; ++j)
+                  if (c0 + j < g.n) o[(c0 + j) * ocs] = v[j];
+              }
+            }
+          } else {
+            // S_0 + S_1 / 256 + S_2 / 256^2 + ... as an unevaluated sum hi + lo of
+            // FP32 numbers: every S_d is an exact integer below 2^24 and each
+            // addition goes through an error-free transformation (TwoSum)
+            float v[16], lo[16];
+  #pragma unroll
+            for (int j = 0; j < 16; ++j) {
+              v[j] = __uint_as_float(u[0][j]);
+              lo[j] = 0.0f;
+            }
+            float scale = 1.0f;
+  #pragma unroll
+            for (int q = 1; q < NS; ++q) {
+              scale *= 0.00390625f;
+  #pragma unroll
+              for (int j = 0; j < 16; ++j) {
+                const float b = __fmul_rn(__uint_as_float(u[q][j]), scale);  // exact: power-of-two scaling
+                const float s = __fadd_rn(v[j], b);
+                const float z = __fsub_rn(s, v[j]);
+                const float e = __fadd_rn(__fsub_rn(v[j], __fsub_rn(s, z)), __fsub_rn(b, z));
+                v[j] = s;
+                lo[j] = __fadd_rn(lo[j], e);
+              }
+            }
+  #pragma unroll
+            for (int j = 0; j < 16; ++j) {
+              const float hi = __fadd_rn(v[j], lo[j]);
+              const float l2 = __fsub_rn(lo[j], __fsub_rn(hi, v[j]));
+              const int sh = ea + (c0 + j < g.n ? be[c0 + j] : 0) - 14;
+              v[j] = scale_pow2(hi, sh);
+              lo[j] = scale_pow2(l2, sh);
+            }
+            if (live) {
+              float *o = g.out + obase, *ol = g.out_lo ? g.out_lo + obase : nullptr;
+              if (g.vec && c0 + 16 <= g.n) {
+                store8(o + c0, v);
+                store8(o + c0 + 8, v + 8);
+                if (ol) {
+                  store8(ol + c0, lo);
+                  store8(ol + c0 + 8, lo + 8);
+                }
+              } else {
+  #pragma unroll
+                for (int j = 0; j < 16; ++j)
+                  if (c0 + j < g.n) {
+                    o[(c0 + j) * ocs] = v[j];
+                    if (ol) ol[(c0 + j) * ocs] = lo[j];
+                  }
+              }
+            }
+          }
+        }
+        if (!released) {  // a warp without columns
+          tc_fence_before();
+          if (lane == 0) mbar_arrive(tempty);
+        }
+      }
+    }
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    if (cl == 2) {
+      asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+      asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
+    if (warp == 1) {
+      tc_fence_after();
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+    }
+  }
+};
+
+template <int NS, bool F64>
+__global__ void __launch_bounds__(kTriThreads, 1) k_umma_tri(const __grid_constant__ CUtensorMap tmA,
+                                                             const __grid_constant__ CUtensorMap tmB,
+                                                             const __grid_constant__ TriArgs g) {
+  UmmaTri<NS, F64>::run(tmA, tmB, g, blockIdx, gridDim);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
@@ -482,38 +827,181 @@ bool umma_chunk_fits(int npairs, const int *pair_a, const int *pair_b, int bn, i
   return 2u * chunk_stage_bytes(na, nb, bn, chunk_width(stages_max)) <= chunk_budget();
 }
 
+namespace {
+// the full triangle a + b < ns of ns slices, each pair once, in any order
+bool full_triangle(int npairs, const int *pair_a, const int *pair_b, int ns) {
+  if (ns < 6 || ns > 8 || npairs != ns * (ns + 1) / 2) return false;
+  bool seen[8][8] = {};
+  for (int p = 0; p < npairs; ++p) {
+    const int a = pair_a[p], b = pair_b[p];
+    if (a < 0 || b < 0 || a + b >= ns || seen[a][b]) return false;
+    seen[a][b] = true;
+  }
+  return true;
+}
+
+int sm_count() {
+  static std::atomic<int> count[64];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 152;
+  const int slot = dev >= 0 && dev < 64 ? dev : 0;
+  int n = count[slot].load(std::memory_order_relaxed);
+  if (n == 0) {
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 152;
+    count[slot].store(n, std::memory_order_relaxed);
+  }
+  return n;
+}
+
+// K chunk width and stages of a tri tile: 32-wide chunks where three stages of
+// every slice fit (64-byte TMA rows), else 16-wide ones; pinned: 64, 32 or 16 where two fit
+void tri_stages(int ns, int bn, int pinned, int *cw, int *stages) {
+  const uint32_t budget = chunk_budget() - 128;  // (barriers of up to eight stages)
+  const uint32_t per = static_cast<uint32_t>(ns) * (128u + bn) * 2u;  // bytes per K element
+  int w = pinned;
+  if (w == 0 || 2 * per * w > budget) w = 3 * per * 32 <= budget ? 32 : 16;
+  *cw = w;
+  const uint32_t s = budget / (per * w);
+  *stages = static_cast<int>(s > 8 ? 8 : s);
+}
+
+// Columns per CTA (multiple of 16, at most limit) and CTAs per cluster: the pair
+// with the least estimated time of one CTA's share.  Clocks per K = 16 step: the
+// tensor pipe (bn / 2 per slice pair) or the operand reads (128 bytes a clock),
+// whichever is more; fixed clocks per tile for the epilogue and the pipeline's
+// fill; alone, a CTA reads twice the A slices from L2.
+void tri_tile(int ns, int n, int tiles_m, int klive, int limit, bool clusters, int *bn, int *cl) {
+  const int sms = sm_count();
+  double best = 0.0;
+  *bn = 16;
+  *cl = 1;
+  for (int w = 16; w <= limit; w += 16)
+    for (int c = 1; c <= (clusters ? 2 : 1); ++c) {
+      const int tn = (n + w - 1) / w, padded = (tn + c - 1) / c * c;
+      int reads = 0;  // A slice reads per step
+      for (int a = 0; a < ns; ++a) reads += (ns - a) * w > 256 ? 2 : 1;
+      const double pairs = 0.5 * ns * (ns + 1), math = pairs * w / 2, smem = (reads * 4096.0 + pairs * w * 32) / 128;
+      const double l2 = ns * 32.0 * (128.0 / c + w) / 32;  // about 32 bytes a clock and SM
+      double t = math > smem ? math : smem;
+      if (l2 > t) t = l2;
+      const long long tiles = (long long)tiles_m * padded;
+      const double share = static_cast<double>((tiles + sms - 1) / sms);
+      const double cost = share * (t * ((klive + 15) / 16) + 1500.0 + 40.0 * w);
+      if (best == 0.0 || cost < best) {
+        best = cost;
+        *bn = w;
+        *cl = c;
+      }
+    }
+}
+
+template <int NS, bool F64>
+cudaError_t launch_tri(const CUtensorMap &ta, const CUtensorMap &tb, const TriArgs &g, int grid, size_t smem,
+                       cudaStream_t st) {
+  if (g.cl == 1)
+    return launch_or_record<UmmaTri<NS, F64>, kTriThreads>(k_umma_tri<NS, F64>, dim3(grid), dim3(kTriThreads), smem,
+                                                           st, ta, tb, g);
+  static std::atomic<unsigned char> raised[64];
+  cudaError_t e = group_raise_smem(reinterpret_cast<const void *>(k_umma_tri<NS, F64>), raised);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = static_cast<unsigned>(g.cl);
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(kTriThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_umma_tri<NS, F64>, ta, tb, g);
+}
+}  // namespace
+
 cudaError_t launch_umma_gemm(const uint16_t *A, int m_max, const int *m_dev, int a_terms, const uint16_t *B, int n,
                              int b_terms, int kp, int npairs, const int *pair_a, const int *pair_b, float *out,
                              long long ldo, const int *out_rows, int *err, cudaStream_t st, const int *a_exp,
                              const int *b_exp, float *out_lo, int bn_max, double *out64, int slice_bits,
                              int batch_rows, int batches, int stages_max, int b_batch_rows, long long o_bstride,
-                             long long o_rstride, long long o_cstride, const int *pair_group) {
+                             long long o_rstride, long long o_cstride, const int2 *krange, int klive) {
   if (m_max <= 0 || n <= 0) return cudaSuccess;
   if (kp <= 0 || kp % 64 != 0 || npairs < 1 || npairs > kMaxPairs || a_terms < 1 || b_terms < 1)
     return cudaErrorInvalidValue;
   if (out64 && (!a_exp || (slice_bits != 7 && slice_bits != 8))) return cudaErrorInvalidValue;
   if ((reinterpret_cast<uintptr_t>(A) & 15u) || (reinterpret_cast<uintptr_t>(B) & 15u)) return cudaErrorInvalidValue;
   if ((a_exp == nullptr) != (b_exp == nullptr)) return cudaErrorInvalidValue;
+  if (bn_max < 0 || bn_max % 16) return cudaErrorInvalidValue;
+  for (int p = 0; p < npairs; ++p)
+    if (pair_a[p] < 0 || pair_a[p] >= a_terms || pair_b[p] < 0 || pair_b[p] >= b_terms) return cudaErrorInvalidValue;
+  CUtensorMap ta, tb;
+  if (a_exp && a_terms == b_terms && full_triangle(npairs, pair_a, pair_b, a_terms) && (out64 || a_terms == 6)) {
+    TriArgs g{};
+    if (b_batch_rows <= 0) b_batch_rows = batch_rows;
+    if (batch_rows < 0 || (batch_rows > 0 && (batches <= 0 || n > b_batch_rows))) return cudaErrorInvalidValue;
+    if (o_cstride != 0 && (batch_rows <= 0 || out_rows)) return cudaErrorInvalidValue;
+    if (stages_max < -3) return cudaErrorInvalidValue;
+    g.m_max = m_max;
+    g.m_dev = m_dev;
+    g.n = n;
+    g.kp = kp;
+    g.klive = klive > 0 && klive < kp ? klive : kp;
+    g.batch_rows = batch_rows;
+    g.b_batch_rows = b_batch_rows;
+    g.tiles_per_batch = batch_rows > 0 ? (batch_rows + 127) / 128 : 0;
+    const int tiles_m = batch_rows > 0 ? batches * g.tiles_per_batch : (m_max + 127) / 128;
+    // as many columns as NS accumulators leave room for in 512 (80 of six, 64
+    // of seven or eight), or the pinned width (64 stands for the widest)
+    const int widest = a_terms == 6 ? 80 : 64;
+    tri_tile(a_terms, n, tiles_m, g.klive, bn_max > 0 && bn_max < 64 ? bn_max : widest, group_recorder() == nullptr,
+             &g.bn, &g.cl);
+    tri_stages(a_terms, g.bn, stages_max < 0 ? chunk_width(stages_max) : 0, &g.cw, &g.stages);
+    g.tiles_n = (n + g.bn - 1) / g.bn;
+    g.krange = krange;
+    g.slice_bits = slice_bits;
+    g.a_exp = a_exp;
+    g.b_exp = b_exp;
+    g.out = out;
+    g.out_lo = out_lo;
+    g.out64 = out64;
+    g.ldo = ldo;
+    g.out_rows = out_rows;
+    g.o_bstride = o_bstride;
+    g.o_rstride = o_rstride;
+    g.o_cstride = o_cstride;
+    g.err = err;
+    const long long unit = out64 ? 4 : 8;  // elements of a 32-byte store
+    const uintptr_t bases = out64 ? reinterpret_cast<uintptr_t>(out64)
+                                  : reinterpret_cast<uintptr_t>(out) | reinterpret_cast<uintptr_t>(out_lo);
+    g.vec = bases % 32 == 0 && (o_cstride ? o_cstride == 1 && o_bstride % unit == 0 && o_rstride % unit == 0
+                                          : ldo % unit == 0);
+    const uint64_t rows_b = batch_rows > 0 ? static_cast<uint64_t>(b_batch_rows) * batches : static_cast<uint64_t>(n);
+    if (!make_map(&ta, A, static_cast<uint64_t>(a_terms) * kp, static_cast<uint64_t>(m_max), 128,
+                  static_cast<uint32_t>(g.cw)) ||
+        !make_map(&tb, B, static_cast<uint64_t>(b_terms) * kp, rows_b, static_cast<uint32_t>(g.bn),
+                  static_cast<uint32_t>(g.cw)))
+      return cudaErrorInvalidValue;
+    size_t smem = 1024 + static_cast<size_t>(g.stages) * a_terms * (128 + g.bn) * g.cw * 2 + 8 * (2 * g.stages + 2) + 16;
+    if (smem < 120 * 1024) smem = 120 * 1024;  // one CTA per SM (see the kernel)
+    const long long tiles = (long long)tiles_m * ((g.tiles_n + g.cl - 1) / g.cl) * g.cl;
+    const int sms = sm_count() / g.cl * g.cl;
+    const int grid = static_cast<int>(tiles < sms ? tiles : sms);
+    if (!out64) return launch_tri<6, false>(ta, tb, g, grid, smem, st);
+    if (a_terms == 6) return launch_tri<6, true>(ta, tb, g, grid, smem, st);
+    if (a_terms == 7) return launch_tri<7, true>(ta, tb, g, grid, smem, st);
+    return launch_tri<8, true>(ta, tb, g, grid, smem, st);
+  }
+  // any other list of pairs: FP32 (or two-float) rows, no batches
+  if (out64 || batch_rows != 0 || o_cstride != 0) return cudaErrorInvalidValue;
   UmmaArgs g{};
   g.ngroups = 1;
   for (int p = 0; p < npairs; ++p) {
-    if (pair_a[p] < 0 || pair_a[p] >= a_terms || pair_b[p] < 0 || pair_b[p] >= b_terms) return cudaErrorInvalidValue;
     g.pair_a[p] = pair_a[p];
     g.pair_b[p] = pair_b[p];
-    // fixed-point mode: the accumulator of weight 256^-(a + b), or the one the
-    // caller names (terms pre-scaled by powers of 256 share an accumulator)
-    g.pair_group[p] = a_exp ? (pair_group ? pair_group[p] : pair_a[p] + pair_b[p]) : 0;
-    if (g.pair_group[p] < 0 || g.pair_group[p] >= 8) return cudaErrorInvalidValue;
+    g.pair_group[p] = a_exp ? pair_a[p] + pair_b[p] : 0;  // fixed-point mode: the accumulator of weight 256^-(a + b)
+    if (g.pair_group[p] >= 8) return cudaErrorInvalidValue;
     if (g.pair_group[p] + 1 > g.ngroups) g.ngroups = g.pair_group[p] + 1;
   }
-  if (g.ngroups > 8) return cudaErrorInvalidValue;
-  g.slice_bits = slice_bits;
-  g.out64 = out64;
-  if (b_batch_rows <= 0) b_batch_rows = batch_rows;
-  if (batch_rows < 0 || (batch_rows > 0 && (batches <= 0 || n > b_batch_rows))) return cudaErrorInvalidValue;
-  g.batch_rows = batch_rows;
-  g.b_batch_rows = b_batch_rows;
-  g.tiles_per_batch = batch_rows > 0 ? (batch_rows + 127) / 128 : 0;
   g.a_exp = a_exp;
   g.b_exp = b_exp;
   g.m_max = m_max;
@@ -521,36 +1009,14 @@ cudaError_t launch_umma_gemm(const uint16_t *A, int m_max, const int *m_dev, int
   g.n = n;
   g.kp = kp;
   // the ngroups accumulators of bn columns share the 512 tensor-memory columns;
-  // bn_max (a multiple of 16, from the autotuner) may lower the limit
+  // bn_max (a multiple of 16) may lower the limit
   int limit = g.ngroups <= 2 ? 256 : (g.ngroups <= 4 ? 128 : (g.ngroups <= 5 ? 96 : 64));
-  if (bn_max > 0) {
-    if (bn_max % 16) return cudaErrorInvalidValue;
-    limit = bn_max < limit ? bn_max : limit;
-  }
+  if (bn_max > 0) limit = bn_max < limit ? bn_max : limit;
   g.bn = umma_pick_bn(n, limit);
-  g.na = g.nb = 0;
-  for (int p = 0; p < npairs; ++p) {
-    g.na = pair_a[p] + 1 > g.na ? pair_a[p] + 1 : g.na;
-    g.nb = pair_b[p] + 1 > g.nb ? pair_b[p] + 1 : g.nb;
-  }
-  uint32_t stage_bytes = 128u * 128u + static_cast<uint32_t>(g.bn) * 128u;
-  if (stages_max < -3) return cudaErrorInvalidValue;
-  // stages_max = -1, -2, -3: chunk-major, every slice of a 64-, 32- or 16-wide
-  // K chunk per stage, as many stages as fit (two to four)
-  g.chunk_major = stages_max < 0 ? 1 : 0;
-  g.cw = g.chunk_major ? chunk_width(stages_max) : 64;
-  if (g.chunk_major) {
-    stage_bytes = chunk_stage_bytes(g.na, g.nb, g.bn, g.cw);
-    if (2u * stage_bytes > chunk_budget()) return cudaErrorInvalidValue;
-    g.stages = static_cast<int>(chunk_budget() / stage_bytes);
-    if (g.stages > 4) g.stages = 4;
-  } else {
-    // pipeline depth: as many stages as fit in 200 KB, at most 6, or fewer
-    // (stages_max, from the autotuner) so that several CTAs share an SM
-    g.stages = static_cast<int>((200u * 1024u) / stage_bytes);
-    if (g.stages > 6) g.stages = 6;
-    if (stages_max > 0 && stages_max < g.stages) g.stages = stages_max < 2 ? 2 : stages_max;
-  }
+  const uint32_t stage_bytes = 128u * 128u + static_cast<uint32_t>(g.bn) * 128u;
+  // pipeline depth: as many stages as fit in 200 KB, at most 6
+  g.stages = static_cast<int>((200u * 1024u) / stage_bytes);
+  if (g.stages > 6) g.stages = 6;
   g.npairs = npairs;
   g.idesc = (1u << 4)                                   // D: FP32
             | (1u << 7) | (1u << 10)                    // A, B: BF16
@@ -564,20 +1030,12 @@ cudaError_t launch_umma_gemm(const uint16_t *A, int m_max, const int *m_dev, int
   g.out_lo = a_exp ? out_lo : nullptr;
   g.ldo = ldo;
   g.out_rows = out_rows;
-  if (o_cstride != 0 && (batch_rows <= 0 || out_rows)) return cudaErrorInvalidValue;
-  g.o_bstride = o_bstride;
-  g.o_rstride = o_rstride;
-  g.o_cstride = o_cstride;
   g.err = err;
-  CUtensorMap ta, tb;
-  const uint64_t b_rows = batch_rows > 0 ? static_cast<uint64_t>(b_batch_rows) * batches : static_cast<uint64_t>(n);
-  if (!make_map(&ta, A, static_cast<uint64_t>(a_terms) * kp, static_cast<uint64_t>(m_max), 128,
-                static_cast<uint32_t>(g.cw)) ||
-      !make_map(&tb, B, static_cast<uint64_t>(b_terms) * kp, b_rows, static_cast<uint32_t>(g.bn),
-                static_cast<uint32_t>(g.cw)))
+  if (!make_map(&ta, A, static_cast<uint64_t>(a_terms) * kp, static_cast<uint64_t>(m_max), 128, 64) ||
+      !make_map(&tb, B, static_cast<uint64_t>(b_terms) * kp, static_cast<uint64_t>(n), static_cast<uint32_t>(g.bn), 64))
     return cudaErrorInvalidValue;
   const size_t smem = 1024 + static_cast<size_t>(g.stages) * stage_bytes + 8 * (2 * g.stages + 1) + 16;
-  dim3 grid((n + g.bn - 1) / g.bn, batch_rows > 0 ? batches * g.tiles_per_batch : (m_max + 127) / 128);
+  dim3 grid((n + g.bn - 1) / g.bn, (m_max + 127) / 128);
   return launch_or_record<UmmaGemm, 128>(k_umma_gemm, grid, dim3(128), smem, st, ta, tb, g);
 }
 
