@@ -1770,18 +1770,23 @@ jagp_status_t jagp_sr_step(const double *d_O, long long ldo, const double *d_eL,
   const SrLayout L = sr_layout(M, P);
   double *w = static_cast<double *>(d_work);
   JAGP_CU(sr_prepare(d_O, ldo, d_eL, M, P, w, L, d_f, st));
-  JAGP_CU(sr_cg_init(d_f, eps, P, w, L, st));
-  double rr0 = 0.0, rr = 0.0;
-  JAGP_CU(cudaMemcpyAsync(&rr0, w + L.sc + 3, sizeof(double), cudaMemcpyDeviceToHost, st));
-  JAGP_CU(cudaStreamSynchronize(st));
-  rr = rr0;
-  int it = 0;
-  while (it < max_iter && rr > tol * tol * rr0 && rr > 0.0) {
-    JAGP_CU(sr_cg_iter(d_O, ldo, M, P, eps, w, L, st));
-    JAGP_CU(cudaMemcpyAsync(&rr, w + L.sc + 3, sizeof(double), cudaMemcpyDeviceToHost, st));
+  JAGP_CU(sr_cg_init(d_f, eps, tol, P, w, L, st));
+  // the device stops the iteration by itself (its launches then return at once),
+  // so the host looks only after every kSrAhead launched iterations
+  constexpr int kSrAhead = 8;
+  double sc[9] = {};
+  for (int launched = 0; launched < max_iter && sc[8] == 0.0;) {
+    for (int k = 0; k < kSrAhead && launched < max_iter; ++k, ++launched)
+      JAGP_CU(sr_cg_iter(d_O, ldo, M, P, eps, tol, w, L, st));
+    JAGP_CU(cudaMemcpyAsync(sc, w + L.sc, sizeof(sc), cudaMemcpyDeviceToHost, st));
     JAGP_CU(cudaStreamSynchronize(st));
-    ++it;
   }
+  if (max_iter == 0) {
+    JAGP_CU(cudaMemcpyAsync(sc, w + L.sc, sizeof(sc), cudaMemcpyDeviceToHost, st));
+    JAGP_CU(cudaStreamSynchronize(st));
+  }
+  const double rr0 = sc[6], rr = sc[3];
+  const int it = (int)sc[7];
   JAGP_CU(sr_finish(delta, P, w, L, d_dalpha, st));
   if (h_iters) *h_iters = it;
   if (h_resid) *h_resid = rr0 > 0.0 ? sqrt(rr / rr0) : 0.0;

@@ -207,17 +207,18 @@ cudaError_t launch_sr_jastrow(const DevSystem &s, const double *r, double *O, lo
                               cudaStream_t st);
 // workspace of the SR solve (offsets in doubles)
 struct SrLayout {
-  size_t obar, diag, dinv, x, r, z, p, q, u, part, ec, t, sc, total;
+  size_t obar, diag, dinv, x, r, z, p, q, u, part, ec, t, sc, dots, total;
 };
 SrLayout sr_layout(int M, int P);
 // Obar, diag S and f = -(2/M) sum_i (e_i - ebar)(O_i - Obar) from the samples
 cudaError_t sr_prepare(const double *O, long long ldo, const double *e, int M, int P, double *w, const SrLayout &L,
                        double *f, cudaStream_t st);
 // preconditioned CG on (S + eps diag S) x = f: start (x = 0), one iteration
-// (device scalars at w + L.sc: [0] r.z, [3] r.r), and dalpha = delta x
-cudaError_t sr_cg_init(const double *f, double eps, int P, double *w, const SrLayout &L, cudaStream_t st);
-cudaError_t sr_cg_iter(const double *O, long long ldo, int M, int P, double eps, double *w, const SrLayout &L,
-                       cudaStream_t st);
+// (nothing once converged), and dalpha = delta x.  Device scalars at w + L.sc:
+// [3] r.r, [6] r.r at the start, [7] iterations taken, [8] 1 once r.r <= tol^2 [6]
+cudaError_t sr_cg_init(const double *f, double eps, double tol, int P, double *w, const SrLayout &L, cudaStream_t st);
+cudaError_t sr_cg_iter(const double *O, long long ldo, int M, int P, double eps, double tol, double *w,
+                       const SrLayout &L, cudaStream_t st);
 cudaError_t sr_finish(double delta, int P, const double *w, const SrLayout &L, double *dalpha, cudaStream_t st);
 
 // Finite-variance forces (k_forces.cu).

@@ -145,7 +145,9 @@ constexpr int kRowChunks = 16;
 
 __global__ void __launch_bounds__(kThreads) k_sr_colsum(const double *__restrict__ O, long long ldo, int M, int P,
                                                         const double *__restrict__ t, const double *__restrict__ c,
-                                                        int mode, double *__restrict__ part) {
+                                                        int mode, const double *__restrict__ done,
+                                                        double *__restrict__ part) {
+  if (done && done[0] != 0.0) return;
   const int k = blockIdx.x * kThreads + threadIdx.x, z = blockIdx.y;
   if (k >= P) return;
   const int rows = (M + kRowChunks - 1) / kRowChunks, i0 = z * rows, i1 = min(M, i0 + rows);
@@ -172,42 +174,90 @@ __global__ void k_sr_colsum_finish(const double *__restrict__ part, int P, doubl
   out[k] = a * scale;
 }
 
-// t_i = sum_k O_ik v_k - (Obar . v): one CTA per sample row; the scalar
-// Obar . v (in dotc[0]) is formed once beforehand
+// sum of x[0 .. n) in the order of one CTA of kThreads (thread t takes t, t +
+// kThreads, ..., then a tree); every block that asks forms the same value
+__device__ double block_total(const double *__restrict__ x, int n, double *sh) {
+  double a = 0.0;
+  for (int k = threadIdx.x; k < n; k += kThreads) a += x[k];
+  return cta_sum(a, sh);
+}
+
+// Dot products x . y (blockIdx.y = 0) and x2 . y2 (1) over P parameters, in the
+// order of one CTA of kThreads threads: thread t's chain over t, t + kThreads,
+// ..., then a tree (dot_total, by the reader).  That order is kept because
+// conjugate gradients on ill-conditioned samples amplify a change of rounding
+// within some tens of iterations.  The CTA's eight warps go to eight CTAs with the
+// next terms' loads in flight; what is left is the latency of a chain of
+// P / 256 FMAs (P = 102403: 78 -> 33 us).
+__device__ double dot_chain(const double *__restrict__ u, const double *__restrict__ v, int t, int n) {
+  double a = 0.0;
+  // the next sixteen terms load while the present sixteen pass through the chain
+  constexpr int B = 16;
+  double p[B], q[B];
+  int k = t;
+  if (k + (B - 1) * kThreads < n) {
+#pragma unroll
+    for (int i = 0; i < B; ++i) {
+      p[i] = u[k + i * kThreads];
+      q[i] = v[k + i * kThreads];
+    }
+    for (; k + (2 * B - 1) * kThreads < n; k += B * kThreads) {
+      double pn[B], qn[B];
+#pragma unroll
+      for (int i = 0; i < B; ++i) {
+        pn[i] = u[k + (B + i) * kThreads];
+        qn[i] = v[k + (B + i) * kThreads];
+      }
+#pragma unroll
+      for (int i = 0; i < B; ++i) a = fma(p[i], q[i], a);
+#pragma unroll
+      for (int i = 0; i < B; ++i) {
+        p[i] = pn[i];
+        q[i] = qn[i];
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < B; ++i) a = fma(p[i], q[i], a);
+    k += B * kThreads;
+  }
+  for (; k < n; k += kThreads) a = fma(u[k], v[k], a);
+  return a;
+}
+__global__ void __launch_bounds__(32) k_sr_dots(const double *__restrict__ x, const double *__restrict__ y,
+                                                const double *__restrict__ x2, const double *__restrict__ y2, int n,
+                                                const double *__restrict__ done, double *__restrict__ out) {
+  if (done && done[0] != 0.0) return;
+  const int t = blockIdx.x * 32 + threadIdx.x;
+  out[blockIdx.y * kThreads + t] = dot_chain(blockIdx.y ? x2 : x, blockIdx.y ? y2 : y, t, n);
+}
+// the chains' sum, by a CTA of kThreads threads or (the same tree) by one warp
+__device__ double dot_total(const double *__restrict__ chains, double *sh) { return cta_sum(chains[threadIdx.x], sh); }
+__device__ double warp_dot_total(const double *__restrict__ chains, double *sh) {
+  for (int i = threadIdx.x; i < kThreads; i += 32) sh[i] = chains[i];
+  __syncwarp();
+  for (int o = kThreads / 2; o > 0; o >>= 1) {
+    for (int i = threadIdx.x; i < o; i += 32) sh[i] += sh[i + o];
+    __syncwarp();
+  }
+  const double r = sh[0];
+  __syncwarp();
+  return r;
+}
+
+// t_i = sum_k O_ik v_k - (Obar . v): one CTA per sample row; Obar . v from its
+// chains dotc.  *done: the iteration has converged.  (Chains beside the rows in this
+// launch share the FP64 pipe with them and then outlast them.)
 __global__ void __launch_bounds__(kThreads) k_sr_rowdot(const double *__restrict__ O, long long ldo, int P,
                                                         const double *__restrict__ v, const double *__restrict__ dotc,
-                                                        double *__restrict__ t) {
+                                                        const double *__restrict__ done, double *__restrict__ t) {
   __shared__ double sh[kThreads];
+  if (done[0] != 0.0) return;
   const int i = blockIdx.x;
   const double *row = O + (size_t)i * ldo;
   double a = 0.0;
   for (int k = threadIdx.x; k < P; k += kThreads) a = fma(row[k], v[k], a);
-  const double s = cta_sum(a, sh);
-  if (threadIdx.x == 0) t[i] = s - (dotc ? dotc[0] : 0.0);
-}
-
-// out[0] = sum_k x_k y_k (z given: sum_k x_k y_k z_k), one CTA, fixed order
-__global__ void __launch_bounds__(kThreads) k_sr_dot(const double *__restrict__ x, const double *__restrict__ y,
-                                                     const double *__restrict__ z, int n, double *__restrict__ out) {
-  __shared__ double sh[kThreads];
-  double a = 0.0;
-  for (int k = threadIdx.x; k < n; k += kThreads) a = fma(x[k], z ? y[k] * z[k] : y[k], a);
-  const double s = cta_sum(a, sh);
-  if (threadIdx.x == 0) out[0] = s;
-}
-
-// out[0] = sum_i x_i, one CTA, fixed order
-__global__ void __launch_bounds__(kThreads) k_sr_sum(const double *__restrict__ x, int n, double *__restrict__ out) {
-  __shared__ double sh[kThreads];
-  double a = 0.0;
-  for (int k = threadIdx.x; k < n; k += kThreads) a += x[k];
-  const double s = cta_sum(a, sh);
-  if (threadIdx.x == 0) out[0] = s;
-}
-
-// the new r.z becomes the old one for the next iteration
-__global__ void k_sr_roll(double *sc) {
-  if (threadIdx.x == 0) sc[0] = sc[2];
+  const double s = cta_sum(a, sh), c = dot_total(dotc, sh);
+  if (threadIdx.x == 0) t[i] = s - c;
 }
 
 // local energies: ebar = mean, ec_i = e_i - ebar, and sum_i ec_i (for the centred form)
@@ -229,12 +279,17 @@ __global__ void __launch_bounds__(kThreads) k_sr_center(const double *__restrict
   }
 }
 
-// preconditioned CG vector updates.  dinv_k = 1 / S'_kk (0 for a parameter
-// whose samples do not vary: it stays at 0)
-__global__ void k_sr_cg_init(const double *__restrict__ f, const double *__restrict__ diag, double eps, int P,
-                             double *__restrict__ dinv, double *__restrict__ x, double *__restrict__ r,
-                             double *__restrict__ z, double *__restrict__ p) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+// Preconditioned CG.  Device scalars sc: [0] r.z, [3] r.r,
+// [6] r.r at the start, [7] iterations, [8] 1 once r.r <= tol^2 of the start's
+// (later launches then change nothing).  Chains of the dot products at dots:
+// [0 .. kThreads) p.q, then r.z, r.r, Obar.p.
+
+// x = 0, r = f (0 where the samples do not vary: dinv_k = 0, else 1 / S'_kk), z = dinv r, p = z
+__global__ void __launch_bounds__(kThreads) k_sr_cg_init(const double *__restrict__ f, const double *__restrict__ diag,
+                                                         double eps, int P, double *__restrict__ dinv,
+                                                         double *__restrict__ x, double *__restrict__ r,
+                                                         double *__restrict__ z, double *__restrict__ p) {
+  const int k = blockIdx.x * kThreads + threadIdx.x;
   if (k >= P) return;
   const double d = diag[k] * (1.0 + eps);
   const double di = d > 0.0 ? 1.0 / d : 0.0;
@@ -245,34 +300,85 @@ __global__ void k_sr_cg_init(const double *__restrict__ f, const double *__restr
   p[k] = z[k];
 }
 
-// q = S' p from u = (1/M) O_c^T t:  q_k = u_k + eps diag_k p_k (0 where dinv = 0)
-__global__ void k_sr_cg_apply(const double *__restrict__ u, const double *__restrict__ diag,
-                              const double *__restrict__ dinv, const double *__restrict__ p, double eps, int P,
-                              double *__restrict__ q) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= P) return;
-  q[k] = dinv[k] > 0.0 ? u[k] + eps * diag[k] * p[k] : 0.0;
+// the scalars at the start (one CTA): r.z, r.r
+__global__ void __launch_bounds__(kThreads) k_sr_cg_start(const double *__restrict__ dots, double tol,
+                                                          double *__restrict__ sc) {
+  __shared__ double sh[kThreads];
+  const double rz = dot_total(dots + kThreads, sh), rr = dot_total(dots + 2 * kThreads, sh);
+  if (threadIdx.x == 0) {
+    sc[0] = rz;
+    sc[3] = rr;
+    sc[6] = rr;
+    sc[7] = 0.0;
+    sc[8] = rr > tol * tol * rr && rr > 0.0 ? 0.0 : 1.0;
+  }
 }
 
-// x += a p, r -= a q, z = dinv r with a = rz / pq (device scalars)
-__global__ void k_sr_cg_step(const double *__restrict__ p, const double *__restrict__ q,
-                             const double *__restrict__ dinv, const double *__restrict__ sc, int P,
-                             double *__restrict__ x, double *__restrict__ r, double *__restrict__ z) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+// q = S' p = (1/M) (O^T t - Obar sum_i t_i) + eps diag p (0 where dinv = 0), from the column sums' slabs
+__global__ void __launch_bounds__(kThreads) k_sr_cg_apply(const double *__restrict__ part, const double *__restrict__ t,
+                                                          int M, const double *__restrict__ obar,
+                                                          const double *__restrict__ diag,
+                                                          const double *__restrict__ dinv,
+                                                          const double *__restrict__ p, double eps, double scale, int P,
+                                                          const double *__restrict__ done, double *__restrict__ q) {
+  __shared__ double sh[kThreads];
+  if (done[0] != 0.0) return;
+  const double ts = block_total(t, M, sh);
+  const int k = blockIdx.x * kThreads + threadIdx.x;
   if (k >= P) return;
-  const double a = sc[1] != 0.0 ? sc[0] / sc[1] : 0.0;  // rz / pq
+  double a = 0.0;
+  for (int z = 0; z < kRowChunks; ++z) a += part[(size_t)z * P + k];
+  a = fma(-obar[k], ts, a);
+  q[k] = dinv[k] > 0.0 ? fma(__dmul_rn(eps, diag[k]), p[k], __dmul_rn(a, scale)) : 0.0;
+}
+
+// x += a p, r -= a q, z = dinv r with a = rz / pq
+__global__ void __launch_bounds__(kThreads) k_sr_cg_step(const double *__restrict__ p, const double *__restrict__ q,
+                                                         const double *__restrict__ dinv,
+                                                         const double *__restrict__ sc,
+                                                         const double *__restrict__ dots, int P,
+                                                         double *__restrict__ x, double *__restrict__ r,
+                                                         double *__restrict__ z) {
+  __shared__ double sh[kThreads];
+  if (sc[8] != 0.0) return;
+  const double pq = dot_total(dots, sh), a = pq != 0.0 ? sc[0] / pq : 0.0;
+  const int k = blockIdx.x * kThreads + threadIdx.x;
+  if (k >= P) return;
   x[k] = fma(a, p[k], x[k]);
   r[k] = fma(-a, q[k], r[k]);
   z[k] = r[k] * dinv[k];
 }
 
 // p = z + (rz_new / rz_old) p
-__global__ void k_sr_cg_dir(const double *__restrict__ z, const double *__restrict__ sc, int P,
-                            double *__restrict__ p) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= P) return;
-  const double beta = sc[0] != 0.0 ? sc[2] / sc[0] : 0.0;
-  p[k] = fma(beta, p[k], z[k]);
+__global__ void __launch_bounds__(kThreads) k_sr_cg_dir(const double *__restrict__ z, const double *__restrict__ sc,
+                                                        const double *__restrict__ dots, int P,
+                                                        double *__restrict__ p) {
+  __shared__ double sh[kThreads];
+  if (sc[8] != 0.0) return;
+  const double rz = dot_total(dots + kThreads, sh), beta = sc[0] != 0.0 ? rz / sc[0] : 0.0;
+  const int k = blockIdx.x * kThreads + threadIdx.x;
+  if (k < P) p[k] = fma(beta, p[k], z[k]);
+}
+
+// After k_sr_cg_dir (every block of which has read the old r.z): the chains of
+// Obar . p (blocks 0 .. 7) and, in block 8, the end of the iteration: the new r.z
+// and r.r, the count, and whether it has converged.
+__global__ void __launch_bounds__(32) k_sr_cg_end(const double *__restrict__ obar, const double *__restrict__ p, int P,
+                                                  double *__restrict__ dots, double tol, double *__restrict__ sc) {
+  __shared__ double sh[kThreads];
+  if (blockIdx.x < kThreads / 32) {
+    const int t = blockIdx.x * 32 + threadIdx.x;
+    dots[3 * kThreads + t] = dot_chain(obar, p, t, P);
+    return;
+  }
+  if (sc[8] != 0.0) return;
+  const double rz = warp_dot_total(dots + kThreads, sh), rr = warp_dot_total(dots + 2 * kThreads, sh);
+  if (threadIdx.x == 0) {
+    sc[0] = rz;
+    sc[3] = rr;
+    sc[7] += 1.0;
+    if (!(rr > tol * tol * sc[6] && rr > 0.0)) sc[8] = 1.0;
+  }
 }
 
 __global__ void k_sr_scale(const double *__restrict__ x, double delta, int P, double *__restrict__ out) {
@@ -317,6 +423,7 @@ SrLayout sr_layout(int M, int P) {
   l.ec = take(M);
   l.t = take(M);
   l.sc = take(32);
+  l.dots = take(4 * kThreads);
   l.total = o;
   return l;
 }
@@ -325,50 +432,48 @@ cudaError_t sr_prepare(const double *O, long long ldo, const double *e, int M, i
                        double *f, cudaStream_t st) {
   const dim3 cgrid(blocks_for(P), kRowChunks);
   // Obar_k = (1/M) sum_i O_ik
-  k_sr_colsum<<<cgrid, kThreads, 0, st>>>(O, ldo, M, P, nullptr, nullptr, 0, w + L.part);
+  k_sr_colsum<<<cgrid, kThreads, 0, st>>>(O, ldo, M, P, nullptr, nullptr, 0, nullptr, w + L.part);
   k_sr_colsum_finish<<<blocks_for(P), kThreads, 0, st>>>(w + L.part, P, 1.0 / M, nullptr, nullptr, w + L.obar);
   // diag S_kk = (1/M) sum_i (O_ik - Obar_k)^2
-  k_sr_colsum<<<cgrid, kThreads, 0, st>>>(O, ldo, M, P, nullptr, w + L.obar, 1, w + L.part);
+  k_sr_colsum<<<cgrid, kThreads, 0, st>>>(O, ldo, M, P, nullptr, w + L.obar, 1, nullptr, w + L.part);
   k_sr_colsum_finish<<<blocks_for(P), kThreads, 0, st>>>(w + L.part, P, 1.0 / M, nullptr, nullptr, w + L.diag);
   // f_k = -(2/M) sum_i (e_i - ebar)(O_ik - Obar_k)
-  k_sr_center<<<1, kThreads, 0, st>>>(e, M, w + L.ec, w + L.sc + 8);
-  k_sr_colsum<<<cgrid, kThreads, 0, st>>>(O, ldo, M, P, w + L.ec, nullptr, 0, w + L.part);
-  k_sr_colsum_finish<<<blocks_for(P), kThreads, 0, st>>>(w + L.part, P, -2.0 / M, w + L.obar, w + L.sc + 9, f);
+  k_sr_center<<<1, kThreads, 0, st>>>(e, M, w + L.ec, w + L.sc + 16);
+  k_sr_colsum<<<cgrid, kThreads, 0, st>>>(O, ldo, M, P, w + L.ec, nullptr, 0, nullptr, w + L.part);
+  k_sr_colsum_finish<<<blocks_for(P), kThreads, 0, st>>>(w + L.part, P, -2.0 / M, w + L.obar, w + L.sc + 17, f);
   return cudaGetLastError();
 }
 
-cudaError_t sr_cg_init(const double *f, double eps, int P, double *w, const SrLayout &L, cudaStream_t st) {
+cudaError_t sr_cg_init(const double *f, double eps, double tol, int P, double *w, const SrLayout &L, cudaStream_t st) {
+  double *dots = w + L.dots;
   k_sr_cg_init<<<blocks_for(P), kThreads, 0, st>>>(f, w + L.diag, eps, P, w + L.dinv, w + L.x, w + L.r, w + L.z,
                                                     w + L.p);
-  // sc[0] = r . z, sc[3] = r . r at the start
-  k_sr_dot<<<1, kThreads, 0, st>>>(w + L.r, w + L.z, nullptr, P, w + L.sc);
-  k_sr_dot<<<1, kThreads, 0, st>>>(w + L.r, w + L.r, nullptr, P, w + L.sc + 3);
+  k_sr_dots<<<dim3(kThreads / 32, 2), 32, 0, st>>>(w + L.r, w + L.z, w + L.r, w + L.r, P, nullptr, dots + kThreads);
+  k_sr_cg_start<<<1, kThreads, 0, st>>>(dots, tol, w + L.sc);
+  k_sr_dots<<<dim3(kThreads / 32, 1), 32, 0, st>>>(w + L.obar, w + L.p, nullptr, nullptr, P, nullptr,
+                                                   dots + 3 * kThreads);
   return cudaGetLastError();
 }
 
 // One preconditioned CG iteration on S' x = f, S' v = (1/M) O_c^T (O_c v) +
-// eps diag(S) v.  Device scalars sc: [0] r.z, [1] p.q, [2] new r.z, [3] new
-// r.r, [4] Obar.p, [5] sum_i t_i.
-cudaError_t sr_cg_iter(const double *O, long long ldo, int M, int P, double eps, double *w, const SrLayout &L,
-                       cudaStream_t st) {
-  double *sc = w + L.sc;
-  const dim3 cgrid(blocks_for(P), kRowChunks);
-  // t = O_c p = O p - (Obar . p)
-  k_sr_dot<<<1, kThreads, 0, st>>>(w + L.obar, w + L.p, nullptr, P, sc + 4);
-  k_sr_rowdot<<<M, kThreads, 0, st>>>(O, ldo, P, w + L.p, sc + 4, w + L.t);
-  // u = (1/M) O_c^T t = (1/M) (O^T t - Obar sum_i t_i)
-  k_sr_sum<<<1, kThreads, 0, st>>>(w + L.t, M, sc + 5);
-  k_sr_colsum<<<cgrid, kThreads, 0, st>>>(O, ldo, M, P, w + L.t, nullptr, 0, w + L.part);
-  k_sr_colsum_finish<<<blocks_for(P), kThreads, 0, st>>>(w + L.part, P, 1.0 / M, w + L.obar, sc + 5, w + L.u);
-  // q = S' p; a = r.z / p.q; x += a p, r -= a q, z = dinv r
-  k_sr_cg_apply<<<blocks_for(P), kThreads, 0, st>>>(w + L.u, w + L.diag, w + L.dinv, w + L.p, eps, P, w + L.q);
-  k_sr_dot<<<1, kThreads, 0, st>>>(w + L.p, w + L.q, nullptr, P, sc + 1);
-  k_sr_cg_step<<<blocks_for(P), kThreads, 0, st>>>(w + L.p, w + L.q, w + L.dinv, sc, P, w + L.x, w + L.r, w + L.z);
-  k_sr_dot<<<1, kThreads, 0, st>>>(w + L.r, w + L.z, nullptr, P, sc + 2);
-  k_sr_dot<<<1, kThreads, 0, st>>>(w + L.r, w + L.r, nullptr, P, sc + 3);
+// eps diag(S) v (nothing once the device's flag says converged).
+cudaError_t sr_cg_iter(const double *O, long long ldo, int M, int P, double eps, double tol, double *w,
+                       const SrLayout &L, cudaStream_t st) {
+  double *sc = w + L.sc, *dots = w + L.dots;
+  const int nb = blocks_for(P);
+  const dim3 cgrid(nb, kRowChunks), one(kThreads / 32, 1), two(kThreads / 32, 2);
+  // t = O_c p = O p - (Obar . p);  O^T t in slabs;  q = S' p
+  k_sr_rowdot<<<M, kThreads, 0, st>>>(O, ldo, P, w + L.p, dots + 3 * kThreads, sc + 8, w + L.t);
+  k_sr_colsum<<<cgrid, kThreads, 0, st>>>(O, ldo, M, P, w + L.t, nullptr, 0, sc + 8, w + L.part);
+  k_sr_cg_apply<<<nb, kThreads, 0, st>>>(w + L.part, w + L.t, M, w + L.obar, w + L.diag, w + L.dinv, w + L.p, eps,
+                                         1.0 / M, P, sc + 8, w + L.q);
+  // a = r.z / p.q; x += a p, r -= a q, z = dinv r
+  k_sr_dots<<<one, 32, 0, st>>>(w + L.p, w + L.q, nullptr, nullptr, P, sc + 8, dots);
+  k_sr_cg_step<<<nb, kThreads, 0, st>>>(w + L.p, w + L.q, w + L.dinv, sc, dots, P, w + L.x, w + L.r, w + L.z);
   // p = z + (new r.z / old r.z) p
-  k_sr_cg_dir<<<blocks_for(P), kThreads, 0, st>>>(w + L.z, sc, P, w + L.p);
-  k_sr_roll<<<1, 32, 0, st>>>(sc);
+  k_sr_dots<<<two, 32, 0, st>>>(w + L.r, w + L.z, w + L.r, w + L.r, P, sc + 8, dots + kThreads);
+  k_sr_cg_dir<<<nb, kThreads, 0, st>>>(w + L.z, sc, dots, P, w + L.p);
+  k_sr_cg_end<<<kThreads / 32 + 1, 32, 0, st>>>(w + L.obar, w + L.p, P, dots, tol, sc);
   return cudaGetLastError();
 }
 
