@@ -52,6 +52,43 @@ __global__ void __launch_bounds__(256) k_gemm_rows(const T *__restrict__ X, size
   GemmRows<T>::run(X, xw, Y, yw, ma, nb, K, Out, ow, ldo, blockIdx, gridDim);
 }
 
+// The same products for ma, nb <= NB = 2, 4 or 8: 256 / NB^2 walkers per CTA,
+// one output per thread (a 16 x 16 tile of one walker would be mostly padding:
+// 2 x 2 outputs used 1.6 % of it).  The sum over k keeps its order.
+template <typename T, int NB>
+struct GemmRowsTiny {
+  static __device__ __forceinline__ void run(const T *__restrict__ X, size_t xw, const T *__restrict__ Y, size_t yw,
+                                             int ma, int nb, int K, T *__restrict__ Out, size_t ow, int ldo, int W,
+                                             const uint3 bid, const uint3 gdim) {
+    assume_global(X, Y, Out);
+    constexpr int WK = 256 / (NB * NB), KC = 16, ROWS = WK * NB;  // walkers per CTA, staged rows per operand
+    __shared__ T Xs[ROWS][KC + 1];
+    __shared__ T Ys[ROWS][KC + 1];
+    const int tid = threadIdx.x, wl = tid / (NB * NB), a = tid / NB % NB, b = tid % NB;
+    const int w0 = bid.x * WK, w = w0 + wl;
+    T acc = T(0);
+    for (int k0 = 0; k0 < K; k0 += KC) {
+      for (int idx = tid; idx < ROWS * KC; idx += 256) {
+        const int row = idx / KC, kk = idx % KC, wr = w0 + row / NB, i = row % NB, k = k0 + kk;
+        const bool in = wr < W && k < K;
+        Xs[row][kk] = in && i < ma ? X[(size_t)wr * xw + (size_t)i * K + k] : T(0);
+        Ys[row][kk] = in && i < nb ? Y[(size_t)wr * yw + (size_t)i * K + k] : T(0);
+      }
+      __syncthreads();
+  #pragma unroll
+      for (int kk = 0; kk < KC; ++kk) acc = fma(Xs[wl * NB + a][kk], Ys[wl * NB + b][kk], acc);
+      __syncthreads();
+    }
+    if (w < W && a < ma && b < nb) Out[(size_t)w * ow + (size_t)a * ldo + b] = acc;
+}
+};
+template <typename T, int NB>
+__global__ void __launch_bounds__(256) k_gemm_rows_tiny(const T *__restrict__ X, size_t xw, const T *__restrict__ Y,
+                                                        size_t yw, int ma, int nb, int K, T *__restrict__ Out,
+                                                        size_t ow, int ldo, int W) {
+  GemmRowsTiny<T, NB>::run(X, xw, Y, yw, ma, nb, K, Out, ow, ldo, W, blockIdx, gridDim);
+}
+
 // The refresh's G~ = Phi_up Bt^T in the FP32 path: the same tile scheme with a
 // compensated dot product (error-free product by fma, error-free sum, the
 // errors summed separately; Ogita, Rump and Oishi 2005) over two-float
@@ -339,6 +376,16 @@ cudaError_t launch_gemm_rows(const T *X, size_t xw, const T *Y, size_t yw, int m
     return launch_or_record<GemmRowsBlk<T, 32, false, T>, 256>(k_gemm_rows_blk<T, 32, false, T>, grid, dim3(256), 0,
                                                                st, X, none, xw, Y, none, yw, ma, nb, K, Out, ow, ldo);
   }
+  const int m = ma > nb ? ma : nb;
+  if (m <= 2)
+    return launch_or_record<GemmRowsTiny<T, 2>, 256>(k_gemm_rows_tiny<T, 2>, dim3((W + 63) / 64), dim3(256), 0, st, X,
+                                                     xw, Y, yw, ma, nb, K, Out, ow, ldo, W);
+  if (m <= 4)
+    return launch_or_record<GemmRowsTiny<T, 4>, 256>(k_gemm_rows_tiny<T, 4>, dim3((W + 15) / 16), dim3(256), 0, st, X,
+                                                     xw, Y, yw, ma, nb, K, Out, ow, ldo, W);
+  if (m <= 8)
+    return launch_or_record<GemmRowsTiny<T, 8>, 256>(k_gemm_rows_tiny<T, 8>, dim3((W + 3) / 4), dim3(256), 0, st, X,
+                                                     xw, Y, yw, ma, nb, K, Out, ow, ldo, W);
   dim3 grid((nb + 15) / 16, (ma + 15) / 16, W);
   return launch_or_record<GemmRows<T>, 256>(k_gemm_rows<T>, grid, dim3(256), 0, st, X, xw, Y, yw, ma, nb, K, Out, ow,
                                             ldo);
