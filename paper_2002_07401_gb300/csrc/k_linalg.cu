@@ -605,160 +605,159 @@ __global__ void __launch_bounds__(128) k_refresh_inverse_reg(const double *__res
   RefreshInverseReg<T, NM>::run(gm, ginv, scal, status, n, W, check_drift, drift_tol, ginv64, blockIdx, gridDim);
 }
 
-// 32 < N_up <= 64: the same register-resident scheme on two warps per walker.
-// Warp h of a walker holds rows 32 h .. 32 h + 31, lane c the columns c and
-// c + 32 (identity past N_up); the pivot of each step is found per warp by
-// shuffles and between the two warps through shared memory, and the warp
-// holding the pivot row publishes it, scaled, for both.  Each step passes two
-// 64-thread named barriers; the exchange slots are double-buffered by step
-// parity, so no third barrier is needed.  Two walkers per CTA of 128 threads.
-template <typename T>
-struct RefreshInverseReg64 {
+// The pivot of a step over a warp: the largest |f| of the rows that are still to
+// be pivoted (key: the integer bits of |f|, 0 for the others), the lowest row on ties.
+__device__ __forceinline__ int best_row(unsigned long long key, int row) {
+  constexpr unsigned kFull = 0xffffffffu;
+  const unsigned hi = static_cast<unsigned>(key >> 32), lo = static_cast<unsigned>(key);
+  const unsigned mh = __reduce_max_sync(kFull, hi);
+  const unsigned ml = __reduce_max_sync(kFull, hi == mh ? lo : 0u);
+  return static_cast<int>(__reduce_min_sync(kFull, hi == mh && lo == ml ? static_cast<unsigned>(row) : 0xffffu));
+}
+__device__ __forceinline__ unsigned long long abs_key(double f) {
+  return static_cast<unsigned long long>(__double_as_longlong(f)) & 0x7fffffffffffffffull;
+}
+
+// log|det| and the parity of negative pivots from two pivots per lane (1 where
+// there is none): the mantissas multiplied and the exponents added over the
+// warp, one log at the end
+__device__ __forceinline__ double log_pivots(double first, double second, bool *neg) {
+  int e1, e2;
+  double m = frexp(fabs(first), &e1) * frexp(fabs(second), &e2);
+  int e = e1 + e2;
+  unsigned flips = (__double_as_longlong(first) < 0) ^ (__double_as_longlong(second) < 0);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    m *= __shfl_xor_sync(0xffffffffu, m, o);  // at most 64 factors of at least 1/2
+    e += __shfl_xor_sync(0xffffffffu, e, o);
+    flips ^= __shfl_xor_sync(0xffffffffu, flips, o);
+  }
+  *neg = flips & 1u;
+  return log(m) + e * 0.6931471805599453;
+}
+
+// 32 < N_up <= 16 CPL (CPL = 3 or 4): the same elimination on four warps of one
+// walker per CTA.  Half-warp g = 0 .. 7 holds the rows g + 8 i, its lane c the
+// columns c + 16 j (identity past N_up), so that the FP64 pipe, which bounds a
+// step, sees little padding (at N_up = 44: 66 FMA warp instructions a step
+// against 60.5 without any; two columns c, c + 32 per lane took 88).  Column k goes
+// to shared memory, every warp finds the pivot, the pivot row's half-warp
+// publishes it scaled, and all update.  Two barriers a step; the exchange
+// slots alternate with the parity of k, so no third is needed.  Measured
+// (serialised): 509 walkers of N_up = 44 342 -> 193 us against two warps per
+// walker with two columns per lane and the multipliers through shuffles;
+// the FP64 instructions alone take 110 us.
+template <typename T, int CPL>
+struct RefreshInverseCta {
+  static constexpr int kMinBlocks = 4;
   static __device__ __forceinline__ void run(const double *__restrict__ gm, T *__restrict__ ginv,
                                              double *__restrict__ scal, int *__restrict__ status, int n, int W,
                                              int check_drift, double drift_tol, double *__restrict__ ginv64,
                                              const uint3 bid, const uint3 gdim) {
     assume_global(gm, ginv, scal, status);
     constexpr unsigned kFull = 0xffffffffu;
-    __shared__ double s_prow[2][2][64];                 // [walker slot][parity][column]
-    __shared__ unsigned long long s_key[2][2][2];       // [slot][parity][half]
-    __shared__ int s_idx[2][2][2];
-    __shared__ double s_val[2][2][2];
-    __shared__ int s_q[2][64];                          // step at which each row was pivoted
-    __shared__ double s_red[2][2][2];                   // [slot][half][gmax, dmax]
-    const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5, slot = wi >> 1, h = wi & 1;
-    const int w = bid.x * 2 + slot;
-    if (w >= W) return;  // both warps of the walker leave; its barriers involve no one else
-    const int bar_id = 1 + slot;
-    const int c0 = lane, c1 = lane + 32, r0 = 32 * h;
+    constexpr int RPL = 2 * CPL;
+    __shared__ double s_f[2][64], s_prow[2][64], s_pv[64];
+    __shared__ int s_q[64], s_p[64];  // step at which each row was pivoted; pivot row of each step
+    __shared__ double s_red[4][2];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c = lane & 15, g = 2 * warp + (lane >> 4);
+    const int w = bid.x;
     const double *Gw = gm + (size_t)w * n * n;
-    double a0[32], a1[32];
+    double a[RPL][CPL];
     double gmax = 0.0;
   #pragma unroll
-    for (int i = 0; i < 32; ++i) {
-      const int r = r0 + i;
-      double v0 = r == c0 ? 1.0 : 0.0, v1 = r == c1 ? 1.0 : 0.0;
-      if (r < n) {
-        if (c0 < n) v0 = Gw[(size_t)r * n + c0];
-        if (c1 < n) v1 = Gw[(size_t)r * n + c1];
-        gmax = fmax(gmax, fmax(c0 < n ? fabs(v0) : 0.0, c1 < n ? fabs(v1) : 0.0));
+    for (int i = 0; i < RPL; ++i)
+  #pragma unroll
+      for (int j = 0; j < CPL; ++j) {
+        const int r = g + 8 * i, col = c + 16 * j;
+        double v = r == col ? 1.0 : 0.0;
+        if (r < n && col < n) {
+          v = Gw[(size_t)r * n + col];
+          gmax = fmax(gmax, fabs(v));
+        }
+        a[i][j] = v;
       }
-      a0[i] = v0;
-      a1[i] = v1;
-    }
     unsigned long long used = 0;
-    int inversions = 0, myp0 = 0, myp1 = 0;
-    PivotProduct pp;
-    bool neg = false, ok = true;
     const unsigned long long rows_n = n >= 64 ? ~0ull : ((1ull << n) - 1ull);
-    for (int k = 0; k < n; ++k) {
-      const int par = k & 1, kl = k & 31;
-      const bool hi = k >= 32;
-      // this warp's rows of column k: lane i keeps f of row r0 + i
-      double fme = 0.0;
-      if (hi) {
+    int inversions = 0;
+    bool ok = true;
   #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const double t = __shfl_sync(kFull, a1[i], kl);
-          if (lane == i) fme = t;
+    for (int jj = 0; jj < CPL; ++jj) {
+      for (int kk = 0; kk < 16; ++kk) {
+        const int k = 16 * jj + kk, par = k & 1;
+        if (k >= n) break;
+        if (c == kk) {
+  #pragma unroll
+          for (int i = 0; i < RPL; ++i) s_f[par][g + 8 * i] = a[i][jj];
         }
-      } else {
-  #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const double t = __shfl_sync(kFull, a0[i], kl);
-          if (lane == i) fme = t;
+        __syncthreads();
+        // rows lane and lane + 32: the better of the two, then over the warp
+        const double f0 = s_f[par][lane], f1 = s_f[par][lane + 32];
+        const unsigned long long k0 = !((used >> lane) & 1ull) ? abs_key(f0) : 0ull;
+        const unsigned long long k1 = lane + 32 < n && !((used >> (lane + 32)) & 1ull) ? abs_key(f1) : 0ull;
+        const int p = best_row(k1 > k0 ? k1 : k0, k1 > k0 ? lane + 32 : lane);
+        const double pv = s_f[par][p];
+        const unsigned long long pk = abs_key(pv);
+        ok = ok && !((used >> p) & 1ull) && pk != 0ull && pk < 0x7ff0000000000000ull;
+        inversions += __popcll(~used & rows_n & ((1ull << p) - 1ull));
+        used |= 1ull << p;
+        if (threadIdx.x == 0) {
+          s_q[p] = k;
+          s_p[k] = p;
+          s_pv[k] = pv;
         }
-      }
-      const int myrow = r0 + lane;
-      unsigned long long key = (myrow < n && !((used >> myrow) & 1ull))
-                                   ? static_cast<unsigned long long>(__double_as_longlong(fme)) & 0x7fffffffffffffffull
-                                   : 0ull;
-      int pi = myrow;
+        if (warp == (p & 7) >> 1) {  // the warp with the pivot row (lane half (p & 7) & 1) publishes it scaled
+          const double ip = recip_newton(pv);
+          double x[CPL];
   #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long k2 = __shfl_xor_sync(kFull, key, o);
-        const int i2 = __shfl_xor_sync(kFull, pi, o);
-        if (k2 > key || (k2 == key && i2 < pi)) {
-          key = k2;
-          pi = i2;
-        }
-      }
-      const double pval = __shfl_sync(kFull, fme, pi - r0);
-      if (lane == 0) {
-        s_key[slot][par][h] = key;
-        s_idx[slot][par][h] = pi;
-        s_val[slot][par][h] = pval;
-      }
-      asm volatile("bar.sync %0, 64;" ::"r"(bar_id) : "memory");
-      // the better of the two halves (the lower rows on ties)
-      const unsigned long long ka = s_key[slot][par][0], kb = s_key[slot][par][1];
-      const int hp = kb > ka ? 1 : 0;
-      const int p = s_idx[slot][par][hp];
-      const double pv = s_val[slot][par][hp];
-      ok = ok && !((used >> p) & 1ull) && pv != 0.0 && isfinite(pv);
-      inversions += __popcll(~used & rows_n & ((1ull << p) - 1ull));
-      used |= 1ull << p;
-      if (k == c0) myp0 = p;
-      if (k == c1) myp1 = p;
-      if (h == 0 && lane == 0) s_q[slot][p] = k;
-      pp.mul(pv);
-      neg ^= pv < 0.0;
-      const double ip = recip_newton(pv);
-      if ((p >> 5) == h) {
-        // this warp holds the pivot row: publish it scaled (column k: 1/p)
-        const int pl = p & 31;
-        double x0 = 0.0, x1 = 0.0;
+          for (int j = 0; j < CPL; ++j) x[j] = a[0][j];
   #pragma unroll
-        for (int i = 0; i < 32; ++i)
-          if (i == pl) {
-            x0 = a0[i];
-            x1 = a1[i];
+          for (int i = 1; i < RPL; ++i)
+            if (i == p >> 3) {
+  #pragma unroll
+              for (int j = 0; j < CPL; ++j) x[j] = a[i][j];
+            }
+          if (g == (p & 7)) {
+  #pragma unroll
+            for (int j = 0; j < CPL; ++j) s_prow[par][c + 16 * j] = j == jj && c == kk ? ip : x[j] * ip;
           }
-        s_prow[slot][par][c0] = c0 == k ? ip : x0 * ip;
-        s_prow[slot][par][c1] = c1 == k ? ip : x1 * ip;
-      }
-      asm volatile("bar.sync %0, 64;" ::"r"(bar_id) : "memory");
-      const double v0 = s_prow[slot][par][c0], v1 = s_prow[slot][par][c1];
-      const bool k0 = c0 == k, k1 = c1 == k;
-      if (hi) {
-  #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const int r = r0 + i;
-          if (r >= n) break;  // warp-uniform
-          const double fi = __shfl_sync(kFull, a1[i], kl);
-          a0[i] = r == p ? v0 : fma(-fi, v0, a0[i]);
-          a1[i] = r == p ? v1 : fma(-fi, v1, k1 ? 0.0 : a1[i]);
         }
-      } else {
+        __syncthreads();
+        double v[CPL];
   #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const int r = r0 + i;
-          if (r >= n) break;  // warp-uniform
-          const double fi = __shfl_sync(kFull, a0[i], kl);
-          a0[i] = r == p ? v0 : fma(-fi, v0, k0 ? 0.0 : a0[i]);
-          a1[i] = r == p ? v1 : fma(-fi, v1, a1[i]);
+        for (int j = 0; j < CPL; ++j) v[j] = s_prow[par][c + 16 * j];
+  #pragma unroll
+        for (int i = 0; i < RPL; ++i) {
+          if (2 * warp + 8 * i < n) {  // warp-uniform: at least one of the two halves' rows exists
+            const int r = g + 8 * i;
+            const double f = s_f[par][r];
+  #pragma unroll
+            for (int j = 0; j < CPL; ++j) {
+              const double base = j == jj && c == kk ? 0.0 : a[i][j];
+              a[i][j] = r == p ? v[j] : fma(-f, v[j], base);
+            }
+          }
         }
       }
     }
-    asm volatile("bar.sync %0, 64;" ::"r"(bar_id) : "memory");  // s_q complete
-    // inverse[k][p_c] = result[p_k][c]: row r of the result goes to row q_r
+    __syncthreads();  // s_q, s_p, s_pv complete
+    // inverse[k][p_c] = result[p_k][c]: row r of the result goes to row q_r, column c to column p_c
     T *gi = ginv + (size_t)w * n * n;
     double dmax = 0.0;
     if (ok) {
   #pragma unroll
-      for (int i = 0; i < 32; ++i) {
-        const int r = r0 + i;
-        if (r >= n) break;
-        const size_t row = (size_t)s_q[slot][r] * n;
-        if (c0 < n) {
-          if (check_drift) dmax = fmax(dmax, fabs(a0[i] - static_cast<double>(gi[row + myp0])));
-          gi[row + myp0] = static_cast<T>(a0[i]);
-          if (ginv64) ginv64[(size_t)w * n * n + row + myp0] = a0[i];
-        }
-        if (c1 < n) {
-          if (check_drift) dmax = fmax(dmax, fabs(a1[i] - static_cast<double>(gi[row + myp1])));
-          gi[row + myp1] = static_cast<T>(a1[i]);
-          if (ginv64) ginv64[(size_t)w * n * n + row + myp1] = a1[i];
+      for (int i = 0; i < RPL; ++i) {
+        const int r = g + 8 * i;
+        if (r >= n) continue;
+        const size_t row = (size_t)s_q[r] * n;
+  #pragma unroll
+        for (int j = 0; j < CPL; ++j) {
+          const int col = c + 16 * j;
+          if (col >= n) continue;
+          const size_t idx = row + s_p[col];
+          if (check_drift) dmax = fmax(dmax, fabs(a[i][j] - static_cast<double>(gi[idx])));
+          gi[idx] = static_cast<T>(a[i][j]);
+          if (ginv64) ginv64[(size_t)w * n * n + idx] = a[i][j];
         }
       }
     }
@@ -768,13 +767,14 @@ struct RefreshInverseReg64 {
       gmax = fmax(gmax, __shfl_xor_sync(kFull, gmax, o));
     }
     if (lane == 0) {
-      s_red[slot][h][0] = gmax;
-      s_red[slot][h][1] = dmax;
+      s_red[warp][0] = gmax;
+      s_red[warp][1] = dmax;
     }
-    asm volatile("bar.sync %0, 64;" ::"r"(bar_id) : "memory");
-    if (h != 0 || lane != 0) return;
-    gmax = fmax(s_red[slot][0][0], s_red[slot][1][0]);
-    dmax = fmax(s_red[slot][0][1], s_red[slot][1][1]);
+    __syncthreads();
+    if (warp != 0) return;
+    bool neg;
+    const double logdet = log_pivots(ok ? s_pv[lane] : 1.0, ok && lane + 32 < n ? s_pv[lane + 32] : 1.0, &neg);
+    if (lane != 0) return;
     double *sw = scal + (size_t)w * S_STRIDE;
     if (!ok) {
       status[w] |= JAGP_WS_SINGULAR;
@@ -782,21 +782,23 @@ struct RefreshInverseReg64 {
       sw[S_SIGN] = 0.0;
       return;
     }
-    sw[S_LOGDET] = pp.log_abs();
-    sw[S_SIGN] = (neg != (inversions & 1)) ? -1.0 : 1.0;
+    sw[S_LOGDET] = logdet;
+    sw[S_SIGN] = (neg != ((inversions & 1) != 0)) ? -1.0 : 1.0;
     if (check_drift) {
-      const double drift = dmax * gmax;
+      const double gm4 = fmax(fmax(s_red[0][0], s_red[1][0]), fmax(s_red[2][0], s_red[3][0]));
+      const double dm4 = fmax(fmax(s_red[0][1], s_red[1][1]), fmax(s_red[2][1], s_red[3][1]));
+      const double drift = dm4 * gm4;
       sw[S_DRIFT] = drift;
       if (!(drift <= drift_tol)) status[w] |= JAGP_WS_DRIFT;
     }
 }
 };
-template <typename T>
-__global__ void __launch_bounds__(128) k_refresh_inverse_reg64(const double *__restrict__ gm, T *__restrict__ ginv,
-                                                               double *__restrict__ scal, int *__restrict__ status,
-                                                               int n, int W, int check_drift, double drift_tol,
-                                                               double *__restrict__ ginv64) {
-  RefreshInverseReg64<T>::run(gm, ginv, scal, status, n, W, check_drift, drift_tol, ginv64, blockIdx, gridDim);
+template <typename T, int CPL>
+__global__ void __launch_bounds__(128, 4) k_refresh_inverse_cta(const double *__restrict__ gm, T *__restrict__ ginv,
+                                                                double *__restrict__ scal, int *__restrict__ status,
+                                                                int n, int W, int check_drift, double drift_tol,
+                                                                double *__restrict__ ginv64) {
+  RefreshInverseCta<T, CPL>::run(gm, ginv, scal, status, n, W, check_drift, drift_tol, ginv64, blockIdx, gridDim);
 }
 
 // In-place Gauss-Jordan (N_up > 32): step k scales the pivot row, stores
@@ -984,11 +986,12 @@ cudaError_t launch_refresh_inverse(double *gm, T *ginv, double *scal, int *statu
   if (W <= 0) return cudaSuccess;
   const size_t aux = (size_t)n * (2 * sizeof(double) + sizeof(int));
   const size_t inplace_smem = (size_t)n * (n + 1) * sizeof(double) + aux;
-  if (n > 32 && n <= 64) {
-    return launch_or_record<RefreshInverseReg64<T>, 128>(k_refresh_inverse_reg64<T>, dim3((W + 1) / 2), dim3(128), 0,
-                                                         st, gm, ginv, scal, status, n, W, check_drift, drift_tol,
-                                                         ginv64);
-  }
+  if (n > 32 && n <= 48)
+    return launch_or_record<RefreshInverseCta<T, 3>, 128>(k_refresh_inverse_cta<T, 3>, dim3(W), dim3(128), 0, st, gm,
+                                                          ginv, scal, status, n, W, check_drift, drift_tol, ginv64);
+  if (n > 48 && n <= 64)
+    return launch_or_record<RefreshInverseCta<T, 4>, 128>(k_refresh_inverse_cta<T, 4>, dim3(W), dim3(128), 0, st, gm,
+                                                          ginv, scal, status, n, W, check_drift, drift_tol, ginv64);
   if (n > 32 && inplace_smem <= kRefreshSmemMax) {
     return launch_or_record<RefreshInverseInplace<T>, 512>(k_refresh_inverse_inplace<T>, dim3(W), dim3(256),
                                                            inplace_smem, st, gm, ginv, scal, status, n, n, check_drift,
