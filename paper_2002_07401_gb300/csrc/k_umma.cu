@@ -1111,52 +1111,107 @@ cudaError_t launch_pack_fixed(const float *P, const float *P_lo, const int *list
                                           reinterpret_cast<__nv_bfloat16 *>(A), rows_out, exps);
 }
 
-// FP64 rows -> nsl exact slices of `bits` bits (|t| <= 2^(bits-1), BF16) per
-// element relative to 2^e, e = 1 + the binary exponent of the row's largest
-// magnitude, for the FP64-equivalent products (every step exact in FP64).
+// An FP64 value v, |v| < 2^e, as NSL slices of BITS bits: the integer nearest to
+// v 2^(NSL BITS - 1 - e) cut from the top, each slice the nearest integer
+// (|t| <= 2^(BITS - 1), exact in BF16).  Integer instructions only: as FP64
+// arithmetic (scale, round, subtract, multiply per slice) the cut was bound by
+// the FP64 pipe, which takes 16 clocks per warp instruction.  A value that is not
+// finite gives NaN slices.
+template <int NSL, int BITS>
+__device__ __forceinline__ void cut_slices(double v, int e, uint16_t t[NSL]) {
+  const long long b = __double_as_longlong(v);
+  const int ef = static_cast<int>((b >> 52) & 0x7ff);
+  long long m = b & 0xfffffffffffffll;
+  if (ef) m |= 1ll << 52;
+  // v = +-m 2^(max(ef, 1) - 1075); shift to units of 2^(e + 1 - NSL BITS)
+  const int sh = (ef ? ef : 1) - 1075 + NSL * BITS - 1 - e;
+  if (sh >= 0) {
+    m <<= sh < 10 ? sh : 10;  // |v| < 2^e leaves at most 55 bits
+  } else {
+    const int r = -sh;
+    m = r > 54 ? 0 : (m + (1ll << (r - 1))) >> r;
+  }
+  if (b < 0) m = -m;
+#pragma unroll
+  for (int q = 0; q < NSL; ++q) {
+    constexpr int kLast = (NSL - 1) * BITS;
+    const int s = kLast - q * BITS;
+    const int d = static_cast<int>(s ? (m + (1ll << (s ? s - 1 : 0))) >> s : m);
+    m -= static_cast<long long>(d) << s;
+    // a small integer's BF16 bits: the leading half of its FP32 number
+    t[q] = ef == 0x7ff ? static_cast<uint16_t>(0x7fc0)
+                       : static_cast<uint16_t>(__float_as_uint(__int_as_float(0x4B400000 + d) - 12582912.0f) >> 16);
+  }
+}
+// the exponent e with |v| < 2^e from the largest leading word of |v| (0 where a
+// value is not finite: the products are then NaN whatever the scale)
+__device__ __forceinline__ unsigned abs_hi(double v) {
+  return static_cast<unsigned>(static_cast<unsigned long long>(__double_as_longlong(v)) >> 32) & 0x7fffffffu;
+}
+__device__ __forceinline__ int exponent_of(unsigned hi) {
+  const int ef = static_cast<int>(hi >> 20);
+  return ef == 0x7ff || hi == 0u ? 0 : (ef ? ef : 1) - 1022;
+}
+
+// FP64 rows -> NSL exact slices of BITS bits per element relative to 2^e, e = 1 +
+// the binary exponent of the row's largest magnitude.  A warp per row, two
+// consecutive elements per lane; bound by its writes (2 NSL bytes per element).
+// 16 thousand rows of L = 320 into seven slices: 278 us with FP64 arithmetic.
+template <int NSL, int BITS>
 struct PackFixed64 {
   static __device__ __forceinline__ void run(const double *__restrict__ P, const int *__restrict__ list,
                                              const int *__restrict__ count, int nrows, int nsub, int stride, int L,
-                                             int kp, int nsl, int bits, __nv_bfloat16 *__restrict__ A,
-                                             int *__restrict__ rows_out, int *__restrict__ exps, long dst_stride,
-                                             long dst_off, const uint3 bid, const uint3 gdim) {
+                                             int kp, uint16_t *__restrict__ A, int *__restrict__ rows_out,
+                                             int *__restrict__ exps, long dst_stride, long dst_off, const uint3 bid,
+                                             const uint3 gdim) {
     assume_global(P, A, rows_out, exps);
     const int rows = count ? *count : nrows;
     const int lane = threadIdx.x & 31;
     const long nw = (long)gdim.x * (blockDim.x >> 5);
-    const double step = ldexp(1.0, bits);
     for (long m = (long)bid.x * (blockDim.x >> 5) + (threadIdx.x >> 5); m < rows; m += nw) {
       const long phys = list ? (long)list[m] : (m / nsub) * stride + (m % nsub);
       const double *src = P + phys * L;
-      double mx = 0.0;
-      for (int k = lane; k < L; k += 32) mx = fmax(mx, fabs(src[k]));
-  #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      const int e = (mx > 0.0) ? ilogb(mx) + 1 : 0;
+      unsigned mx = 0;
+      for (int k = lane; k < L; k += 32) {
+        const unsigned h = abs_hi(src[k]) | (src[k] != 0.0 ? 1u : 0u);  // (a subnormal's leading word may be 0)
+        mx = h > mx ? h : mx;
+      }
+      mx = __reduce_max_sync(0xffffffffu, mx);
+      const int e = exponent_of(mx);
       if (lane == 0) {
         // the row of the result: the source row, or (m / nsub) * dst_stride + dst_off + m % nsub
         rows_out[m] = dst_stride > 0 ? (int)((m / nsub) * dst_stride + dst_off + m % nsub) : (int)phys;
         exps[m] = e;
       }
-      __nv_bfloat16 *dst = A + m * nsl * (long)kp;
-      for (int k = lane; k < kp; k += 32) {
-        double x = k < L ? ldexp(src[k], bits - 1 - e) : 0.0;  // |x| < 2^(bits-1)
-        for (int t = 0; t < nsl; ++t) {
-          const double q = rint(x);
-          dst[t * kp + k] = __float2bfloat16_rn(static_cast<float>(q));
-          x = (x - q) * step;
-        }
+      uint16_t *dst = A + m * NSL * (long)kp;
+      for (int k = 2 * lane; k < kp; k += 64) {
+        uint16_t t0[NSL], t1[NSL];
+        cut_slices<NSL, BITS>(k < L ? src[k] : 0.0, e, t0);
+        cut_slices<NSL, BITS>(k + 1 < L ? src[k + 1] : 0.0, e, t1);
+  #pragma unroll
+        for (int t = 0; t < NSL; ++t)
+          *reinterpret_cast<uint32_t *>(dst + t * kp + k) = t0[t] | (static_cast<uint32_t>(t1[t]) << 16);
       }
     }
 }
 };
+template <int NSL, int BITS>
 __global__ void __launch_bounds__(256) k_pack_fixed64(const double *__restrict__ P, const int *__restrict__ list,
                                                       const int *__restrict__ count, int nrows, int nsub, int stride,
-                                                      int L, int kp, int nsl, int bits, __nv_bfloat16 *__restrict__ A,
+                                                      int L, int kp, uint16_t *__restrict__ A,
                                                       int *__restrict__ rows_out, int *__restrict__ exps,
                                                       long dst_stride, long dst_off) {
-  PackFixed64::run(P, list, count, nrows, nsub, stride, L, kp, nsl, bits, A, rows_out, exps, dst_stride, dst_off,
-                   blockIdx, gridDim);
+  PackFixed64<NSL, BITS>::run(P, list, count, nrows, nsub, stride, L, kp, A, rows_out, exps, dst_stride, dst_off,
+                              blockIdx, gridDim);
+}
+
+template <int NSL, int BITS>
+static cudaError_t pack_fixed64(const double *P, const int *list, const int *count, int nrows, int nsub, int stride,
+                                int L, int kp, uint16_t *A, int *rows_out, int *exps, int blocks, cudaStream_t st,
+                                long dst_stride, long dst_off) {
+  return launch_or_record<PackFixed64<NSL, BITS>, 256>(k_pack_fixed64<NSL, BITS>, dim3(blocks), dim3(256), 0, st, P,
+                                                       list, count, nrows, nsub > 0 ? nsub : 1, stride, L, kp, A,
+                                                       rows_out, exps, dst_stride, dst_off);
 }
 
 cudaError_t launch_pack_fixed64(const double *P, const int *list, const int *count, int nrows, int nsub, int stride,
@@ -1165,9 +1220,14 @@ cudaError_t launch_pack_fixed64(const double *P, const int *list, const int *cou
   if (max_rows <= 0) return cudaSuccess;
   long blocks = (max_rows + 7) / 8;
   if (blocks > 152 * 16) blocks = 152 * 16;
-  return launch_or_record<PackFixed64, 256>(k_pack_fixed64, dim3((int)blocks), dim3(256), 0, st, P, list, count, nrows,
-                                            nsub > 0 ? nsub : 1, stride, L, kp, nsl, bits,
-                                            reinterpret_cast<__nv_bfloat16 *>(A), rows_out, exps, dst_stride, dst_off);
+  const int nb = (int)blocks;
+  if (nsl == 6 && bits == 8)
+    return pack_fixed64<6, 8>(P, list, count, nrows, nsub, stride, L, kp, A, rows_out, exps, nb, st, dst_stride, dst_off);
+  if (nsl == 7 && bits == 8)
+    return pack_fixed64<7, 8>(P, list, count, nrows, nsub, stride, L, kp, A, rows_out, exps, nb, st, dst_stride, dst_off);
+  if (nsl == 8 && bits == 7)
+    return pack_fixed64<8, 7>(P, list, count, nrows, nsub, stride, L, kp, A, rows_out, exps, nb, st, dst_stride, dst_off);
+  return cudaErrorInvalidValue;
 }
 
 // ---------------------------------------------------------------------------
@@ -1185,61 +1245,51 @@ cudaError_t launch_pack_fixed64(const double *P, const int *list, const int *cou
 // row) and the writes (64 consecutive entries of one slice of an operand row)
 // are both coalesced.
 // ---------------------------------------------------------------------------
-template <bool kF64>
+template <bool kF64, int NSL, int BITS>
 struct PackCols {
   static __device__ __forceinline__ void run(const double *__restrict__ X64, const float *__restrict__ X32,
                                              const float *__restrict__ Xlo, size_t xw, int R, int C, int kp,
-                                             __nv_bfloat16 *__restrict__ A, int *__restrict__ exps,
-                                             int *__restrict__ rows_out, long dst_stride, long dst_off, int nsl,
-                                             int bits, const uint3 bid, const uint3 gdim) {
+                                             uint16_t *__restrict__ A, int *__restrict__ exps,
+                                             int *__restrict__ rows_out, long dst_stride, long dst_off,
+                                             const uint3 bid, const uint3 gdim) {
     assume_global(A, exps);
     if constexpr (kF64) assume_global(X64); else assume_global(X32);
-    constexpr int kMaxSl = 8;
     __shared__ double t64[kF64 ? 64 : 1][33];
     __shared__ float th[kF64 ? 1 : 64][33], tl[kF64 ? 1 : 64][33];
-    __shared__ float cmax[8][32];
+    __shared__ unsigned cmax[8][32];
     __shared__ int cexp[32];
     const int tid = threadIdx.x, cl = tid & 31, jr = tid >> 5;
     const int w = bid.y, c0 = bid.x * 32;
     const int c = c0 + cl;
     const size_t base = (size_t)w * xw;
-    float mx = 0.0f;
-    double mx64 = 0.0;
+    // the columns' largest magnitudes, as integer bits (FP64: the leading words)
+    unsigned mx = 0;
     if (c < C)
       for (int j = jr; j < R; j += 8) {
-        if constexpr (kF64)
-          mx64 = fmax(mx64, fabs(X64[base + (size_t)j * C + c]));
-        else
-          mx = fmaxf(mx, fabsf(X32[base + (size_t)j * C + c]));
-      }
-    if constexpr (kF64) {
-      // exponents from the FP64 maxima: compare through the exponent only
-      cmax[jr][cl] = 0.0f;
-      __shared__ double cmax64[8][32];
-      cmax64[jr][cl] = mx64;
-      __syncthreads();
-      if (jr == 0) {
-        double m = cmax64[0][cl];
-        for (int q = 1; q < 8; ++q) m = fmax(m, cmax64[q][cl]);
-        const int e = m > 0.0 ? ilogb(m) + 1 : 0;
-        cexp[cl] = e;
-        if (c < C) {
-          exps[(size_t)w * C + c] = e;
-          if (rows_out) rows_out[(size_t)w * C + c] = (int)(w * dst_stride + dst_off + c);
+        unsigned h;
+        if constexpr (kF64) {
+          const double v = X64[base + (size_t)j * C + c];
+          h = abs_hi(v) | (v != 0.0 ? 1u : 0u);
+        } else {
+          h = __float_as_uint(fmaxf(0.0f, fabsf(X32[base + (size_t)j * C + c])));  // (NaN: 0)
         }
+        mx = h > mx ? h : mx;
       }
-    } else {
-      cmax[jr][cl] = mx;
-      __syncthreads();
-      if (jr == 0) {
-        float m = cmax[0][cl];
-        for (int q = 1; q < 8; ++q) m = fmaxf(m, cmax[q][cl]);
-        const int e = m > 0.0f ? ilogbf(m) + 1 : 0;
-        cexp[cl] = e;
-        if (c < C) {
-          exps[(size_t)w * C + c] = e;
-          if (rows_out) rows_out[(size_t)w * C + c] = (int)(w * dst_stride + dst_off + c);
-        }
+    cmax[jr][cl] = mx;
+    __syncthreads();
+    if (jr == 0) {
+      for (int q = 1; q < 8; ++q) mx = cmax[q][cl] > mx ? cmax[q][cl] : mx;
+      int e;
+      if constexpr (kF64) {
+        e = exponent_of(mx);
+      } else {
+        const float m = __uint_as_float(mx);
+        e = m > 0.0f ? ilogbf(m) + 1 : 0;
+      }
+      cexp[cl] = e;
+      if (c < C) {
+        exps[(size_t)w * C + c] = e;
+        if (rows_out) rows_out[(size_t)w * C + c] = (int)(w * dst_stride + dst_off + c);
       }
     }
     __syncthreads();
@@ -1263,55 +1313,49 @@ struct PackCols {
         const int col = jr + 8 * cc, cg = c0 + col;
         if (cg >= C) continue;
         const int e = cexp[col];
-        __nv_bfloat16 sl[2][kMaxSl];
+        uint16_t sl[2][NSL];
   #pragma unroll
         for (int h = 0; h < 2; ++h) {
           const int jj = 2 * (tid & 31) + h;
           if constexpr (kF64) {
-            const double step = ldexp(1.0, bits);
-            double x = ldexp(t64[jj][col], bits - 1 - e);  // |x| < 2^(bits - 1)
-  #pragma unroll
-            for (int t = 0; t < kMaxSl; ++t) {
-              if (t >= nsl) break;
-              const double q = rint(x);
-              sl[h][t] = __float2bfloat16_rn(static_cast<float>(q));
-              x = (x - q) * step;
-            }
+            cut_slices<NSL, BITS>(t64[jj][col], e, sl[h]);
           } else {
             float x = ldexpf(th[jj][col], 7 - e), xl = ldexpf(tl[jj][col], 7 - e);
   #pragma unroll
-            for (int t = 0; t < kMaxSl; ++t) {
-              if (t >= nsl) break;
+            for (int t = 0; t < NSL; ++t) {
               const float q = rintf(x);
-              sl[h][t] = __float2bfloat16_rn(q);
+              sl[h][t] = __bfloat16_as_ushort(__float2bfloat16_rn(q));
               const fdw r = two_sum(__fsub_rn(x, q), xl);
               x = __fmul_rn(r.hi, 256.0f);
               xl = __fmul_rn(r.lo, 256.0f);
             }
           }
         }
-        __nv_bfloat16 *dst = A + ((size_t)w * C + cg) * nsl * (size_t)kp + j0 + 2 * (tid & 31);
+        uint16_t *dst = A + ((size_t)w * C + cg) * NSL * (size_t)kp + j0 + 2 * (tid & 31);
   #pragma unroll
-        for (int t = 0; t < kMaxSl; ++t) {
-          if (t >= nsl) break;
-          __nv_bfloat162 v;
-          v.x = sl[0][t];
-          v.y = sl[1][t];
-          *reinterpret_cast<__nv_bfloat162 *>(dst + (size_t)t * kp) = v;
-        }
+        for (int t = 0; t < NSL; ++t)
+          *reinterpret_cast<uint32_t *>(dst + (size_t)t * kp) = sl[0][t] | (static_cast<uint32_t>(sl[1][t]) << 16);
       }
       __syncthreads();
     }
 }
 };
-template <bool kF64>
+template <bool kF64, int NSL, int BITS>
 __global__ void __launch_bounds__(256) k_pack_cols(const double *__restrict__ X64, const float *__restrict__ X32,
                                                    const float *__restrict__ Xlo, size_t xw, int R, int C, int kp,
-                                                   __nv_bfloat16 *__restrict__ A, int *__restrict__ exps,
-                                                   int *__restrict__ rows_out, long dst_stride, long dst_off, int nsl,
-                                                   int bits) {
-  PackCols<kF64>::run(X64, X32, Xlo, xw, R, C, kp, A, exps, rows_out, dst_stride, dst_off, nsl, bits, blockIdx,
-                      gridDim);
+                                                   uint16_t *__restrict__ A, int *__restrict__ exps,
+                                                   int *__restrict__ rows_out, long dst_stride, long dst_off) {
+  PackCols<kF64, NSL, BITS>::run(X64, X32, Xlo, xw, R, C, kp, A, exps, rows_out, dst_stride, dst_off, blockIdx,
+                                 gridDim);
+}
+
+template <bool kF64, int NSL, int BITS>
+static cudaError_t pack_cols(const double *X64, const float *X32, const float *Xlo, size_t xw, int R, int C, int kp,
+                             int W, uint16_t *A, int *exps, int *rows_out, long dst_stride, long dst_off,
+                             cudaStream_t st) {
+  return launch_or_record<PackCols<kF64, NSL, BITS>, 256>(k_pack_cols<kF64, NSL, BITS>, dim3((C + 31) / 32, W),
+                                                          dim3(256), 0, st, X64, X32, Xlo, xw, R, C, kp, A, exps,
+                                                          rows_out, dst_stride, dst_off);
 }
 
 cudaError_t launch_pack_cols(const double *X64, const float *X32, const float *Xlo, size_t xw, int R, int C, int kp,
@@ -1319,17 +1363,13 @@ cudaError_t launch_pack_cols(const double *X64, const float *X32, const float *X
                              cudaStream_t st, int nsl, int bits) {
   if (W <= 0 || C <= 0) return cudaSuccess;
   if (kp % 64 != 0 || kp < R || (X64 == nullptr) == (X32 == nullptr)) return cudaErrorInvalidValue;
-  if (nsl < 1 || nsl > 8 || (bits != 8 && (bits != 7 || !X64))) return cudaErrorInvalidValue;
-  dim3 grid((C + 31) / 32, W);
-  const float *nf = nullptr;
-  const double *nd = nullptr;
-  if (X64)
-    return launch_or_record<PackCols<true>, 256>(k_pack_cols<true>, grid, dim3(256), 0, st, X64, nf, nf, xw, R, C, kp,
-                                                 reinterpret_cast<__nv_bfloat16 *>(A), exps, rows_out, dst_stride,
-                                                 dst_off, nsl, bits);
-  return launch_or_record<PackCols<false>, 256>(k_pack_cols<false>, grid, dim3(256), 0, st, nd, X32, Xlo, xw, R, C, kp,
-                                                reinterpret_cast<__nv_bfloat16 *>(A), exps, rows_out, dst_stride,
-                                                dst_off, nsl, bits);
+  if (X32 && nsl == 6 && bits == 8)
+    return pack_cols<false, 6, 8>(X64, X32, Xlo, xw, R, C, kp, W, A, exps, rows_out, dst_stride, dst_off, st);
+  if (X64 && nsl == 6 && bits == 8)
+    return pack_cols<true, 6, 8>(X64, X32, Xlo, xw, R, C, kp, W, A, exps, rows_out, dst_stride, dst_off, st);
+  if (X64 && nsl == 8 && bits == 7)
+    return pack_cols<true, 8, 7>(X64, X32, Xlo, xw, R, C, kp, W, A, exps, rows_out, dst_stride, dst_off, st);
+  return cudaErrorInvalidValue;
 }
 
 cudaError_t setup_umma_attributes() {
