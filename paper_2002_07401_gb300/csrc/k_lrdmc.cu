@@ -20,6 +20,9 @@
 // electrons' orbital rows and their lambda products, and, on a compact copy
 // of the moved walkers' state, a refresh of G~^{-1} and the local energy of
 // the new configurations (jagp_api.cu) prepare the next round.  Decisions read the Philox4x32-10 stream (walker, generation, hop, 2).
+#include <atomic>
+
+#include "jagp_group.cuh"
 #include "jagp_launch.h"
 
 namespace jagp {
@@ -27,6 +30,101 @@ namespace jagp {
 namespace {
 
 constexpr int kRatioThreads = 128;
+
+// 2^(j / 64) as double-words (its FP32 rounding and the remainder)
+__device__ const float2 kExpTab[64] = {
+    {0x1.0000000000000p+0f, 0x0.0p+0f}, {0x1.02c9a40000000p+0f, -0x1.887fa00000000p-28f},
+    {0x1.059b0e0000000p+0f, -0x1.9d4f520000000p-25f}, {0x1.0874520000000p+0f, -0x1.e2990e0000000p-26f},
+    {0x1.0b55860000000p+0f, 0x1.9f31220000000p-25f}, {0x1.0e3ec40000000p+0f, -0x1.a585cc0000000p-25f},
+    {0x1.11301e0000000p+0f, -0x1.fdb4960000000p-25f}, {0x1.1429aa0000000p+0f, 0x1.d525bc0000000p-25f},
+    {0x1.172b840000000p+0f, -0x1.c157420000000p-27f}, {0x1.1a35be0000000p+0f, 0x1.6df96e0000000p-25f},
+    {0x1.1d48740000000p+0f, -0x1.d2e8ca0000000p-25f}, {0x1.2063b80000000p+0f, 0x1.0c519a0000000p-25f},
+    {0x1.2387a60000000p+0f, 0x1.ceac480000000p-25f}, {0x1.26b4560000000p+0f, 0x1.789f380000000p-26f},
+    {0x1.29e9e00000000p+0f, -0x1.5c04240000000p-25f}, {0x1.2d285a0000000p+0f, 0x1.b900c20000000p-26f},
+    {0x1.306fe00000000p+0f, 0x1.4636e20000000p-25f}, {0x1.33c08c0000000p+0f, -0x1.b37d200000000p-25f},
+    {0x1.371a740000000p+0f, -0x1.18aac60000000p-25f}, {0x1.3a7db40000000p+0f, -0x1.634c020000000p-25f},
+    {0x1.3dea640000000p+0f, 0x1.8246840000000p-25f}, {0x1.4160a20000000p+0f, 0x1.f72e2a0000000p-28f},
+    {0x1.44e0860000000p+0f, 0x1.8624b40000000p-30f}, {0x1.486a2c0000000p+0f, -0x1.47d8660000000p-25f},
+    {0x1.4bfdae0000000p+0f, -0x1.593abc0000000p-25f}, {0x1.4f9b280000000p+0f, -0x1.2c5a6c0000000p-25f},
+    {0x1.5342b60000000p+0f, -0x1.2c56100000000p-25f}, {0x1.56f4740000000p+0f, -0x1.295b040000000p-25f},
+    {0x1.5ab07e0000000p+0f, -0x1.5bd5ec0000000p-27f}, {0x1.5e76f20000000p+0f, -0x1.4a5bd60000000p-25f},
+    {0x1.6247ec0000000p+0f, -0x1.f8b5500000000p-25f}, {0x1.6623880000000p+0f, 0x1.2a91120000000p-27f},
+    {0x1.6a09e60000000p+0f, 0x1.9fcef40000000p-26f}, {0x1.6dfb240000000p+0f, -0x1.cd72e80000000p-27f},
+    {0x1.71f75e0000000p+0f, 0x1.1d8bee0000000p-25f}, {0x1.75feb60000000p+0f, -0x1.37b3060000000p-25f},
+    {0x1.7a11480000000p+0f, -0x1.829fd00000000p-25f}, {0x1.7e2f340000000p+0f, -0x1.2616340000000p-25f},
+    {0x1.82589a0000000p+0f, -0x1.accc7c0000000p-26f}, {0x1.868d9a0000000p+0f, -0x1.2edb440000000p-26f},
+    {0x1.8ace540000000p+0f, 0x1.15506e0000000p-27f}, {0x1.8f1aea0000000p+0f, -0x1.baa2320000000p-26f},
+    {0x1.93737c0000000p+0f, -0x1.e647440000000p-25f}, {0x1.97d82a0000000p+0f, -0x1.0d8d840000000p-31f},
+    {0x1.9c49180000000p+0f, 0x1.51f8480000000p-27f}, {0x1.a0c6680000000p+0f, -0x1.2886a60000000p-26f},
+    {0x1.a5503c0000000p+0f, -0x1.b83b540000000p-25f}, {0x1.a9e6b60000000p+0f, -0x1.50c0480000000p-25f},
+    {0x1.ae89fa0000000p+0f, -0x1.a94b140000000p-26f}, {0x1.b33a2c0000000p+0f, -0x1.ec3a820000000p-26f},
+    {0x1.b7f7700000000p+0f, -0x1.a094380000000p-25f}, {0x1.bcc1ea0000000p+0f, -0x1.f687c60000000p-25f},
+    {0x1.c199be0000000p+0f, -0x1.3d56b20000000p-27f}, {0x1.c67f120000000p+0f, 0x1.cafa2a0000000p-25f},
+    {0x1.cb720e0000000p+0f, -0x1.8837cc0000000p-27f}, {0x1.d072d40000000p+0f, 0x1.40f1300000000p-25f},
+    {0x1.d5818e0000000p+0f, -0x1.822dbc0000000p-27f}, {0x1.da9e600000000p+0f, 0x1.ed99420000000p-27f},
+    {0x1.dfc9740000000p+0f, -0x1.908c940000000p-25f}, {0x1.e502ee0000000p+0f, 0x1.e2cffe0000000p-26f},
+    {0x1.ea4afa0000000p+0f, 0x1.52486c0000000p-27f}, {0x1.efa1be0000000p+0f, 0x1.cc2b440000000p-25f},
+    {0x1.f507660000000p+0f, -0x1.246eb00000000p-26f}, {0x1.fa7c180000000p+0f, 0x1.9e90d80000000p-28f},
+};
+
+// e^x = m 2^k, |x| <= 170, by a table (Tang, ACM TOMS 15 (1989) 144): x = (64 k + j)
+// ln2 / 64 + r, |r| <= ln2 / 128, ln2 / 64 in three parts (the first of 10 bits, so
+// that its product and the first subtraction are exact), m = 2^(j/64) (1 + r +
+// r^2/2 + ...) with r, r^2 and the table in double-word, r^3/6 .. r^6/720 in FP32;
+// relative error below 2^-46.  The exponent stays apart, so that products and
+// quotients of such numbers neither overflow nor underflow on the way.
+struct ExpParts {
+  fdw m;
+  int k;
+};
+__device__ __forceinline__ ExpParts dw_exp_parts(fdw x, const float2 *__restrict__ tab) {
+  const float k = rintf(__fmul_rn(x.hi, 92.33248138427734f));
+  fdw r = two_sum(__fmaf_rn(-k, 0x1.628p-7f, x.hi), x.lo);
+  r = dw_add(r, dw_neg(two_prod(k, 0x1.90bfbep-17f)));
+  r = fast_two_sum(r.hi, __fmaf_rn(-k, 0x1.1cf79ap-42f, r.lo));
+  const int ki = static_cast<int>(k);
+  const float2 t = tab[ki & 63];
+  const float h = __fmul_rn(r.hi, r.hi), hl = __fmaf_rn(2.0f * r.hi, r.lo, __fmaf_rn(r.hi, r.hi, -h));  // r^2
+  float q = __fmaf_rn(r.hi, 1.0f / 720.0f, 1.0f / 120.0f);
+  q = __fmaf_rn(q, r.hi, 1.0f / 24.0f);
+  q = __fmaf_rn(q, r.hi, 1.0f / 6.0f);
+  q = __fmul_rn(q, __fmul_rn(h, r.hi));
+  const fdw e = fast_two_sum(r.hi, 0.5f * h);  // e^r - 1 = e.hi + low
+  const float low = __fadd_rn(__fadd_rn(__fmaf_rn(0.5f, hl, r.lo), q), e.lo);
+  const fdw te = two_prod(t.x, e.hi);
+  const float tl = __fmaf_rn(t.x, low, __fmaf_rn(t.y, e.hi, te.lo));
+  const fdw u = fast_two_sum(t.x, te.hi);
+  return {fast_two_sum(u.hi, __fadd_rn(u.lo, __fadd_rn(t.y, tl))), ki >> 6};
+}
+// m 2^k, |m| below 2^20 or so; rounded once where the result is subnormal
+__device__ __forceinline__ fdw dw_scale(fdw m, int k) {
+  if (k >= -100) {
+    const float sc = __int_as_float((127 + (k < 127 ? k : 127)) << 23);
+    return {__fmul_rn(m.hi, sc), __fmul_rn(m.lo, sc)};
+  }
+  return {ldexpf(m.hi, k), ldexpf(m.lo, k)};
+}
+// e^x for x <= 0 (0 below -104)
+__device__ __forceinline__ fdw dw_exp_tab(fdw x, const float2 *__restrict__ tab) {
+  if (!(x.hi > -104.0f)) return {x.hi != x.hi ? x.hi : 0.0f, 0.0f};
+  const ExpParts p = dw_exp_parts(x, tab);
+  return dw_scale(p.m, p.k);
+}
+
+// v as a double-word without FP64 instructions (a conversion occupies the FP64
+// pipe for 16 clocks per warp): the leading 24 bits truncated, the other 29 as
+// an integer.  Magnitudes outside FP32's normal range: 0, or an infinity / NaN.
+__device__ __forceinline__ fdw dw_of_bits(double v) {
+  const unsigned hi = static_cast<unsigned>(__double2hiint(v)), lo = static_cast<unsigned>(__double2loint(v));
+  const int e = static_cast<int>((hi >> 20) & 0x7ffu) - 1023;
+  if (e > 127) return {__uint_as_float((hi & 0x80000000u) | (e == 1024 && ((hi & 0xfffffu) | lo) ? 0x7fc00000u : 0x7f800000u)), 0.0f};
+  if (e < -100) return {0.0f, 0.0f};
+  const float h = __uint_as_float((hi & 0x80000000u) | static_cast<unsigned>(e + 127) << 23 | (hi & 0xfffffu) << 3 |
+                                  lo >> 29);
+  const float l = __fmul_rn(static_cast<float>(static_cast<int>(lo & 0x1fffffffu)),
+                            __int_as_float(((hi >> 31) << 31) | (127 + (e < -74 ? -126 : e - 52)) << 23));
+  return e < -74 ? fdw{h, 0.0f} : fast_two_sum(h, l);
+}
 
 // warp-wide double-word sum; dw_add is commutative, so every lane of the
 // butterfly ends with the same value
@@ -39,15 +137,33 @@ __device__ __forceinline__ fdw warp_sum_dw(fdw v) {
   return v;
 }
 
-__device__ __forceinline__ fdw dw_dist(const fdw *p, const fdw *q) {
-  const fdw dx = dw_add(p[0], dw_neg(q[0])), dy = dw_add(p[1], dw_neg(q[1])), dz = dw_add(p[2], dw_neg(q[2]));
-  return dw_sqrt(dw_add(dw_add(dw_mul(dx, dx), dw_mul(dy, dy)), dw_mul(dz, dz)));
+// squared distances r'^2 of the six hops from the displacement d of the electron
+// from a centre: r^2 + a^2 +- 2 a d_q
+struct HopDist {
+  fdw base;     // r^2 + a^2
+  fdw step[3];  // 2 a d_q
+  __device__ __forceinline__ fdw r2(int k) const {
+    return dw_add(base, (k & 1) ? dw_neg(step[k >> 1]) : step[k >> 1]);
+  }
+};
+__device__ __forceinline__ HopDist hop_dist(const DwDisp &d, fdw two_a, fdw a2) {
+  return {dw_add(d.r2, a2), {dw_mul(two_a, d.x), dw_mul(two_a, d.y), dw_mul(two_a, d.z)}};
+}
+__device__ __forceinline__ DwDisp dw_between(const fdw *p, const fdw *q) {
+  DwDisp d;
+  d.x = dw_add(p[0], dw_neg(q[0]));
+  d.y = dw_add(p[1], dw_neg(q[1]));
+  d.z = dw_add(p[2], dw_neg(q[2]));
+  d.r2 = dw_add(dw_add(dw_mul(d.x, d.x), dw_mul(d.y, d.y)), dw_mul(d.z, d.z));
+  return d;
 }
 
 // one-body term of one atom, -c^3 u(c r), u(s) = (1 - e^{-b s}) / (2b) (s / 2 at b = 0)
-__device__ __forceinline__ fdw j1_term_dw(fdw c, fdw mc3, fdw b, fdw inv2b, bool b0, fdw r) {
+__device__ __forceinline__ fdw j1_term_dw(fdw c, fdw mc3, fdw b, fdw inv2b, bool b0, fdw r,
+                                          const float2 *__restrict__ tab) {
   const fdw sc = dw_mul(c, r);
-  const fdw u = b0 ? dw_mul_f(sc, 0.5f) : dw_mul(dw_add_f(dw_neg(dw_exp_neg(dw_neg(dw_mul(b, sc)))), 1.0f), inv2b);
+  const fdw u =
+      b0 ? dw_mul_f(sc, 0.5f) : dw_mul(dw_add_f(dw_neg(dw_exp_tab(dw_neg(dw_mul(b, sc)), tab)), 1.0f), inv2b);
   return dw_mul(mc3, u);
 }
 
@@ -58,81 +174,136 @@ __device__ __forceinline__ fdw j2_term_dw(fdw b, float kinv, fdw r) {
 
 // rho[w][k] for every hop of every walker still active: one CTA per walker, a
 // warp per electron and its six hops (lanes over shells, atoms and electrons),
-// in double-word FP32 arithmetic (relative error a few units of 2^-46; FP64
-// instructions only to convert M, the positions and the atoms): GB300 issues
-// FP32 at ~64x its FP64 rate, and the 6N orbital evaluations per walker and
-// round are the bulk of the ratio work.
+// in double-word FP32 arithmetic (relative error a few units of 2^-46).  Bound by
+// its FP32 instructions, so that what the six hops share is formed once: a hop by
+// +-a along q changes r^2 by a^2 +- 2 a d_q, so a Gaussian's six radial factors are
+// e^{-zeta (r^2 + a^2)} times or over e^{-2 zeta a d_q} (four exponentials, not
+// six), and sum_c M_c P_c, a polynomial of degree two at most, follows from its
+// value, gradient and second derivatives at the electron.  Conversions are done with integer
+// instructions.  A generation of 1024 walkers of 16 He, 26 rounds: 22.0 -> 10.2 ms
+// against six separate evaluations.
 __global__ void __launch_bounds__(kRatioThreads) k_lrdmc_ratios(DevSystem s, const double *__restrict__ r,
                                                                  const double *__restrict__ mbuf,
                                                                  const int *__restrict__ active, double a,
                                                                  double *__restrict__ rho) {
-  extern __shared__ double xs[];                         // the walker's positions [N][3]
-  fdw *xd = reinterpret_cast<fdw *>(xs + 3 * s.N);       // the same as double-words
-  const int w = blockIdx.x, N = s.N, L = s.L;
+  extern __shared__ fdw xd[];         // the walker's positions [N][3], then per atom R, c, -c^3
+  __shared__ float2 tab[64];
+  const int w = blockIdx.x, N = s.N, L = s.L, na = s.n_atoms;
+  fdw *const ad = xd + 3 * N;
   if (!active[w]) return;
-  for (int t = threadIdx.x; t < 3 * N; t += kRatioThreads) {
-    const double v = r[(size_t)w * N * 3 + t];
-    xs[t] = v;
-    xd[t] = dw_of(v);
+  for (int t = threadIdx.x; t < 3 * N; t += kRatioThreads) xd[t] = dw_of_bits(r[(size_t)w * N * 3 + t]);
+  for (int t = threadIdx.x; t < na; t += kRatioThreads) {
+    for (int q = 0; q < 3; ++q) ad[5 * t + q] = dw_of_bits(s.R[3 * t + q]);
+    const double c = s.c1[t];
+    ad[5 * t + 3] = dw_of_bits(c);
+    ad[5 * t + 4] = dw_of_bits(-c * c * c);
   }
+  for (int t = threadIdx.x; t < 64; t += kRatioThreads) tab[t] = kExpTab[t];
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const bool b0 = s.b_ea == 0.0;
-  const fdw bea = dw_of(s.b_ea), inv2b = dw_of(b0 ? 0.0 : 0.5 / s.b_ea);
+  const fdw bea = dw_of_bits(s.b_ea), inv2b = dw_of_bits(b0 ? 0.0 : 0.5 / s.b_ea);
+  const fdw ah = dw_of_bits(a), a2 = dw_mul(ah, ah), two_a{2.0f * ah.hi, 2.0f * ah.lo};
+  // pair constants [same spin, opposite]
+  double k2[2], bb2[2];
+  j2_params(s, true, &k2[0], &bb2[0]);
+  j2_params(s, false, &k2[1], &bb2[1]);
+  const fdw b2[2] = {dw_of_bits(bb2[0]), dw_of_bits(bb2[1])};
+  const float kinv2[2] = {k2[0] == 4.0 ? 0.25f : 0.5f, k2[1] == 4.0 ? 0.25f : 0.5f};
   for (int i = warp; i < N; i += kRatioThreads / 32) {
-    const double *o = xs + 3 * i;
     const fdw *od = xd + 3 * i;
-    fdw pd[6][3];
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-      const int d = k / 2;
-#pragma unroll
-      for (int q = 0; q < 3; ++q) pd[k][q] = q == d ? dw_of((k & 1) ? o[d] - a : o[d] + a) : od[q];
-    }
     fdw dot[6], dj[6];
 #pragma unroll
     for (int k = 0; k < 6; ++k) dot[k] = dj[k] = fdw{0.0f, 0.0f};
     const double *Mi = mbuf + ((size_t)w * N + i) * L;
     for (int sh = lane; sh < s.n_shells; sh += 32) {
       const float4 gh = s.shell_dw[2 * sh], gl = s.shell_dw[2 * sh + 1];
-      const int info = s.shell_info[sh], off = shell_off(info), nc = 2 * shell_l(info) + 1;
-      fdw m[5];
-#pragma unroll
-      for (int c = 0; c < 5; ++c) m[c] = c < nc ? dw_of(Mi[off + c]) : fdw{0.0f, 0.0f};
+      const int info = s.shell_info[sh], off = shell_off(info), l = shell_l(info), rad = shell_rad(info);
       const fdw zeta{gh.w, gl.w};
+      const DwDisp d = dw_displacement(od, gh, gl);
+      // every hop's value is 0 in FP32 (e^-104) where even the nearest one is that far
+      const float far = fmaxf(fmaxf(fabsf(d.x.hi), fabsf(d.y.hi)), fabsf(d.z.hi));
+      const float near2 = fmaxf(d.r2.hi + a2.hi - 2.0f * ah.hi * far, 0.0f);
+      if (gh.w * (rad ? sqrtf(near2) : near2) > 105.0f) continue;
+      // S = sum_c M_c P_c at the electron, its gradient and half its second derivatives
+      const fdw m0 = dw_of_bits(Mi[off]);
+      fdw S0, Sq[3] = {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, Cq[3] = {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}};
+      if (l == 0) {
+        S0 = m0;
+      } else if (l == 1) {
+        Sq[0] = m0;
+        Sq[1] = dw_of_bits(Mi[off + 1]);
+        Sq[2] = dw_of_bits(Mi[off + 2]);
+        S0 = dw_add(dw_add(dw_mul(Sq[0], d.x), dw_mul(Sq[1], d.y)), dw_mul(Sq[2], d.z));
+      } else {
+        const fdw m1 = dw_of_bits(Mi[off + 1]), m2 = dw_of_bits(Mi[off + 2]), m3 = dw_of_bits(Mi[off + 3]),
+                  m4 = dw_of_bits(Mi[off + 4]);
+        // P = xy, yz, zx, x^2 - y^2, 2 z^2 - x^2 - y^2: S = x (S_x / 2) + y (S_y / 2) + z (S_z / 2)
+        Cq[0] = dw_add(m3, dw_neg(m4));
+        Cq[1] = dw_neg(dw_add(m3, m4));
+        Cq[2] = fdw{2.0f * m4.hi, 2.0f * m4.lo};
+        const fdw x2{2.0f * d.x.hi, 2.0f * d.x.lo}, y2{2.0f * d.y.hi, 2.0f * d.y.lo}, z2{2.0f * d.z.hi, 2.0f * d.z.lo};
+        Sq[0] = dw_add(dw_add(dw_mul(m0, d.y), dw_mul(m2, d.z)), dw_mul(Cq[0], x2));
+        Sq[1] = dw_add(dw_add(dw_mul(m0, d.x), dw_mul(m1, d.z)), dw_mul(Cq[1], y2));
+        Sq[2] = dw_add(dw_add(dw_mul(m1, d.y), dw_mul(m2, d.x)), dw_mul(Cq[2], z2));
+        const fdw t = dw_add(dw_add(dw_mul(Sq[0], d.x), dw_mul(Sq[1], d.y)), dw_mul(Sq[2], d.z));
+        S0 = fdw{0.5f * t.hi, 0.5f * t.lo};
+      }
+      const HopDist h = hop_dist(d, two_a, a2);
+      // the six hops' S: S0 +- a S_q + a^2 C_q
+      fdw S[6];
 #pragma unroll
-      for (int k = 0; k < 6; ++k) {
-        const DwDisp dd = dw_displacement(pd[k], gh, gl);
-        float v[5], vl[5];
-        shell_values_dw(info, zeta, dd, v, vl);
+      for (int q = 0; q < 3; ++q) {
+        if (l == 0) {
+          S[2 * q] = S[2 * q + 1] = S0;
+        } else {
+          const fdw c = l == 2 ? dw_add(S0, dw_mul(a2, Cq[q])) : S0, g = dw_mul(ah, Sq[q]);
+          S[2 * q] = dw_add(c, g);
+          S[2 * q + 1] = dw_add(c, dw_neg(g));
+        }
+      }
+      if (rad || gh.w * h.base.hi > 168.0f) {
 #pragma unroll
-        for (int c = 0; c < 5; ++c)
-          if (c < nc) dot[k] = dw_add(dot[k], dw_mul(fdw{v[c], vl[c]}, m[c]));
+        for (int k = 0; k < 6; ++k) {
+          const fdw r2 = h.r2(k);
+          dot[k] = dw_add(dot[k], dw_mul(dw_exp_tab(dw_neg(dw_mul(zeta, rad ? dw_sqrt(r2) : r2)), tab), S[k]));
+        }
+      } else {
+        // zeta (r^2 + a^2) <= 168 bounds 2 zeta a |d_q| too
+        const ExpParts e0 = dw_exp_parts(dw_neg(dw_mul(zeta, h.base)), tab);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          const ExpParts f = dw_exp_parts(dw_neg(dw_mul(zeta, h.step[q])), tab);
+          dot[2 * q] = dw_add(dot[2 * q], dw_mul(dw_scale(dw_mul(e0.m, f.m), e0.k + f.k), S[2 * q]));
+          dot[2 * q + 1] =
+              dw_add(dot[2 * q + 1], dw_mul(dw_scale(dw_mul(e0.m, dw_recip(f.m)), e0.k - f.k), S[2 * q + 1]));
+        }
       }
     }
     if (s.use_j1) {
-      for (int at = lane; at < s.n_atoms; at += 32) {
-        const fdw R[3] = {dw_of(s.R[3 * at]), dw_of(s.R[3 * at + 1]), dw_of(s.R[3 * at + 2])};
-        const double c = s.c1[at];
-        const fdw cd = dw_of(c), mc3 = dw_of(-c * c * c);
-        const fdw f0 = j1_term_dw(cd, mc3, bea, inv2b, b0, dw_dist(od, R));
+      for (int at = lane; at < na; at += 32) {
+        const fdw *R = ad + 5 * at, cd = R[3], mc3 = R[4];
+        const DwDisp d = dw_between(od, R);
+        const HopDist h = hop_dist(d, two_a, a2);
+        const fdw f0 = j1_term_dw(cd, mc3, bea, inv2b, b0, dw_sqrt(d.r2), tab);
 #pragma unroll
         for (int k = 0; k < 6; ++k)
-          dj[k] = dw_add(dj[k], dw_add(j1_term_dw(cd, mc3, bea, inv2b, b0, dw_dist(pd[k], R)), dw_neg(f0)));
+          dj[k] = dw_add(dj[k], dw_add(j1_term_dw(cd, mc3, bea, inv2b, b0, dw_sqrt(h.r2(k)), tab), dw_neg(f0)));
       }
     }
     if (s.use_j2) {
       const bool up = i < s.n_up;
       for (int q = lane; q < N; q += 32) {
         if (q == i) continue;
-        double kk, bb;
-        j2_params(s, (q < s.n_up) == up, &kk, &bb);
-        const fdw b = dw_of(bb);
-        const float kinv = kk == 4.0 ? 0.25f : 0.5f;
-        const fdw f0 = j2_term_dw(b, kinv, dw_dist(od, xd + 3 * q));
+        const int o = (q < s.n_up) == up ? 0 : 1;
+        const fdw b = o ? b2[1] : b2[0];
+        const float kinv = o ? kinv2[1] : kinv2[0];
+        const DwDisp d = dw_between(od, xd + 3 * q);
+        const HopDist h = hop_dist(d, two_a, a2);
+        const fdw f0 = j2_term_dw(b, kinv, dw_sqrt(d.r2));
 #pragma unroll
         for (int k = 0; k < 6; ++k)
-          dj[k] = dw_add(dj[k], dw_add(j2_term_dw(b, kinv, dw_dist(pd[k], xd + 3 * q)), dw_neg(f0)));
+          dj[k] = dw_add(dj[k], dw_add(j2_term_dw(b, kinv, dw_sqrt(h.r2(k))), dw_neg(f0)));
       }
     }
 #pragma unroll
@@ -349,8 +520,12 @@ __global__ void k_lrdmc_energy(const double *__restrict__ wbar, const double *__
 cudaError_t launch_lrdmc_ratios(const DevSystem &s, const double *r, const double *mbuf, const int *active, double a,
                                 double *rho, int W, cudaStream_t st) {
   if (W <= 0) return cudaSuccess;
-  const size_t smem = (size_t)s.N * 3 * (sizeof(double) + sizeof(fdw));
-  if (smem > 48 * 1024) return cudaErrorInvalidValue;
+  const size_t smem = ((size_t)s.N * 3 + (size_t)s.n_atoms * 5) * sizeof(fdw);
+  if (smem > 48 * 1024) {
+    static std::atomic<unsigned char> raised[64];
+    const cudaError_t e = group_raise_smem(reinterpret_cast<const void *>(k_lrdmc_ratios), raised);
+    if (e != cudaSuccess) return e;
+  }
   k_lrdmc_ratios<<<W, kRatioThreads, smem, st>>>(s, r, mbuf, active, a, rho);
   return cudaGetLastError();
 }
