@@ -1969,9 +1969,10 @@ jagp_status_t lrdmc_project(jagp_ctx *h, double *d_r, void *d_state, int W, uint
     in.c[5] = {status, at<int>(k.sub_state, C.status), 4};
     in.n = 6;
     LAUNCH(0, 1, launch_walker_copy(in, k.list_w, Wc, false, st));
-    s = run_refresh<double>(h, k.r_sub, k.sub_state, Wc, 0, true, st);
+    // (the local-energy pass also forms J, so the refresh skips its Jastrow pass)
+    s = run_refresh<double>(h, k.r_sub, k.sub_state, Wc, 0, false, st);
     if (s != JAGP_OK) return s;
-    s = run_local_energy<double>(h, k.r_sub, k.sub_state, Wc, k.eL_sub, nullptr, st);
+    s = run_local_energy<double>(h, k.r_sub, k.sub_state, Wc, k.eL_sub, nullptr, st, true);
     if (s != JAGP_OK) return s;
     WalkerCopies out{};
     out.c[0] = {at<double>(k.sub_state, C.ginv), at<double>(d_state, L.ginv), n * n * 8};
@@ -2052,7 +2053,7 @@ static jagp_status_t jagp_lrdmc_branch_impl(jagp_handle_t h, double *d_r, int W,
   const size_t bytes = (size_t)W * h->ds.N * 3 * sizeof(double);
   JAGP_CU(cudaMemcpyAsync(k.r_tmp, d_r, bytes, cudaMemcpyDeviceToDevice, st));
   LAUNCH(0, 2,
-         launch_lrdmc_branch(W, h->ds.N, (uint32_t)generation, h->ds.key0, h->ds.key1, d_weight, d_eL,
+         launch_lrdmc_branch(W, h->ds.N, (uint32_t)generation, h->ds.key0, h->ds.key1, d_weight, d_eL, k.left,
                              d_parent ? d_parent : k.moved, d_stats, k.r_tmp, d_r, st));
   return JAGP_OK;
 }

@@ -275,8 +275,8 @@ cudaError_t launch_lrdmc_finish(int W, const double *lw, const double *eL_cur, d
 // parents by systematic resampling, (wbar, ebar) into stats, weights reset to
 // 1, r_new[j] = r_old[parent[j]]
 cudaError_t launch_lrdmc_branch(int W, int N, uint32_t gen, uint32_t key0, uint32_t key1, double *weight,
-                                const double *eL, int *parent, double *stats, const double *r_old, double *r_new,
-                                cudaStream_t st);
+                                const double *eL, double *run, int *parent, double *stats, const double *r_old,
+                                double *r_new, cudaStream_t st);
 cudaError_t launch_lrdmc_energy(const double *wbar, const double *ebar, int T, int p, double *E, cudaStream_t st);
 
 // one-time kernel attribute set-up (dynamic shared memory limits), per file

@@ -116,14 +116,18 @@ __device__ __forceinline__ fdw dw_exp_tab(fdw x, const float2 *__restrict__ tab)
 // an integer.  Magnitudes outside FP32's normal range: 0, or an infinity / NaN.
 __device__ __forceinline__ fdw dw_of_bits(double v) {
   const unsigned hi = static_cast<unsigned>(__double2hiint(v)), lo = static_cast<unsigned>(__double2loint(v));
+  const unsigned sign = hi & 0x80000000u;
   const int e = static_cast<int>((hi >> 20) & 0x7ffu) - 1023;
-  if (e > 127) return {__uint_as_float((hi & 0x80000000u) | (e == 1024 && ((hi & 0xfffffu) | lo) ? 0x7fc00000u : 0x7f800000u)), 0.0f};
-  if (e < -100) return {0.0f, 0.0f};
-  const float h = __uint_as_float((hi & 0x80000000u) | static_cast<unsigned>(e + 127) << 23 | (hi & 0xfffffu) << 3 |
-                                  lo >> 29);
-  const float l = __fmul_rn(static_cast<float>(static_cast<int>(lo & 0x1fffffffu)),
-                            __int_as_float(((hi >> 31) << 31) | (127 + (e < -74 ? -126 : e - 52)) << 23));
-  return e < -74 ? fdw{h, 0.0f} : fast_two_sum(h, l);
+  if (e > 127) {
+    const bool nan = e == 1024 && ((hi & 0xfffffu) | lo) != 0u;
+    return {__uint_as_float(sign | (nan ? 0x7fc00000u : 0x7f800000u)), 0.0f};
+  }
+  if (e < -126) return {0.0f, 0.0f};
+  const unsigned scale = sign | static_cast<unsigned>(e + 127) << 23;  // +-2^e
+  const float h = __uint_as_float(scale | (hi & 0xfffffu) << 3 | lo >> 29);
+  const float l = __fmul_rn(__fmul_rn(static_cast<float>(static_cast<int>(lo & 0x1fffffffu)), 0x1p-52f),
+                            __uint_as_float(scale));
+  return fast_two_sum(h, l);
 }
 
 // warp-wide double-word sum; dw_add is commutative, so every lane of the
@@ -332,68 +336,91 @@ __global__ void k_lrdmc_start(const int *__restrict__ status, int W, double tau,
   active[w] = bad ? 0 : 1;
 }
 
-// One round's decision per walker (one thread each, in the order the oracle
-// takes the steps): the rates and Gamma from rho in hop order, the wait
-// tau_xi = -ln(1 - xi) / Gamma; the walker ends (log-weight less the time
-// left times e_L - e_ref) or hops to the first k whose running rate sum
-// exceeds u Gamma (a non-finite Gamma or e_L ends the walker with flag 4).
-// A moved electron's row goes to the up or down list
-// (w n_up + row) for the lambda products, the walker to list_w; cnt[2]
-// counts the walkers that moved (those still active).
-__global__ void k_lrdmc_decide(DevSystem s, double *__restrict__ r, const double *__restrict__ rho,
-                               const double *__restrict__ eL, const int *__restrict__ status, int W, uint32_t walker0,
-                               uint32_t gen, double a, double gamma, double e_ref, int max_hops,
-                               double *__restrict__ left, double *__restrict__ lw, int *__restrict__ hops,
-                               int *__restrict__ flags, int *__restrict__ active, int *__restrict__ moved,
-                               int *__restrict__ list_up, int *__restrict__ list_dn, int *__restrict__ list_w,
-                               int *__restrict__ cnt) {
-  const int w = blockIdx.x * blockDim.x + threadIdx.x;
+// One round's decision per walker, a warp each: the rates and Gamma from rho, the
+// wait tau_xi = -ln(1 - xi) / Gamma; the walker ends (log-weight less the time
+// left times e_L - e_ref) or hops to the first k in hop order whose running rate
+// sum exceeds u Gamma (a non-finite Gamma or e_L ends the walker with flag 4).
+// A lane takes consecutive hops and the running sums come from a warp scan: one
+// thread adding 12 N rates one after another took 86 us a round at N = 32, this 13.  A moved electron's row goes to the up or down list (w n_up + row)
+// for the lambda products, the walker to list_w; cnt[2] counts the walkers
+// that moved (those still active).
+__global__ void __launch_bounds__(128) k_lrdmc_decide(
+    DevSystem s, double *__restrict__ r, const double *__restrict__ rho, const double *__restrict__ eL,
+    const int *__restrict__ status, int W, uint32_t walker0, uint32_t gen, double a, double gamma, double e_ref,
+    int max_hops, double *__restrict__ left, double *__restrict__ lw, int *__restrict__ hops, int *__restrict__ flags,
+    int *__restrict__ active, int *__restrict__ moved, int *__restrict__ list_up, int *__restrict__ list_dn,
+    int *__restrict__ list_w, int *__restrict__ cnt) {
+  const int w = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)), lane = threadIdx.x & 31;
   if (w >= W) return;
-  moved[w] = -1;
+  const bool first = lane == 0;
+  if (first) moved[w] = -1;
   if (!active[w]) return;
   if (status[w] & (JAGP_WS_SINGULAR | JAGP_WS_NONFINITE)) {
-    flags[w] |= 2;
-    active[w] = 0;
+    if (first) {
+      flags[w] |= 2;
+      active[w] = 0;
+    }
     return;
   }
-  const int N = s.N, n = s.n_up;
-  const double *q = rho + (size_t)w * 6 * N;
+  const int N = s.N, n = s.n_up, K = 6 * N, per = (K + 31) / 32, k0 = lane * per, k1 = min(K, k0 + per);
+  const double *q = rho + (size_t)w * K;
   const double c = 1.0 / (2.0 * a * a);
-  double G = 0.0;
-  for (int k = 0; k < 6 * N; ++k) G += (q[k] > 0.0 ? q[k] : -gamma * q[k]) * c;
+  double mine = 0.0;
+  for (int k = k0; k < k1; ++k) mine += (q[k] > 0.0 ? q[k] : -gamma * q[k]) * c;
+  double incl = mine;  // sums up to and with this lane's hops
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const double t = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += t;
+  }
+  const double before = __shfl_up_sync(0xffffffffu, incl, 1), G = __shfl_sync(0xffffffffu, incl, 31);
   const double e = eL[w];
   if (!isfinite(G) || !isfinite(e)) {
-    flags[w] |= 4;
-    active[w] = 0;
+    if (first) {
+      flags[w] |= 4;
+      active[w] = 0;
+    }
     return;
   }
   const int h = hops[w];
+  const double time = left[w];
   if (h >= max_hops) {
-    flags[w] |= 1;
-    lw[w] -= left[w] * (e - e_ref);
-    active[w] = 0;
+    if (first) {
+      flags[w] |= 1;
+      lw[w] -= time * (e - e_ref);
+      active[w] = 0;
+    }
     return;
   }
   uint32_t o[4] = {walker0 + (uint32_t)w, gen, (uint32_t)h, 2u};
   philox4x32_10(o, s.key0, s.key1);
   const double xi = ((double)o[0] + 0.5) * 0x1p-32;
   const double wait = G > 0.0 ? -log(1.0 - xi) / G : INFINITY;
-  if (wait >= left[w]) {
-    lw[w] -= left[w] * (e - e_ref);
-    active[w] = 0;
+  if (wait >= time) {
+    if (first) {
+      lw[w] -= time * (e - e_ref);
+      active[w] = 0;
+    }
     return;
   }
-  lw[w] -= wait * (e - e_ref);
-  left[w] -= wait;
+  // the first hop whose running sum exceeds thr, else the last one with a rate
   const double thr = ((double)o[1] + 0.5) * 0x1p-32 * G;
-  double run = 0.0;
-  int k = -1;
-  for (int j = 0; j < 6 * N; ++j) {
-    const double t = (q[j] > 0.0 ? q[j] : -gamma * q[j]) * c;
+  double run = lane ? before : 0.0;
+  int hit = K, last = -1;
+  for (int k = k0; k < k1 && hit == K; ++k) {
+    const double t = (q[k] > 0.0 ? q[k] : -gamma * q[k]) * c;
     run += t;
-    if (t > 0.0) k = j;
-    if (run > thr) break;
+    if (t > 0.0) {
+      last = k;
+      if (run > thr) hit = k;
+    }
   }
+  hit = static_cast<int>(__reduce_min_sync(0xffffffffu, static_cast<unsigned>(hit)));
+  last = __reduce_max_sync(0xffffffffu, last);
+  if (!first) return;
+  const int k = hit < K ? hit : last;
+  lw[w] -= wait * (e - e_ref);
+  left[w] = time - wait;
   const int i = k / 6, d = (k % 6) / 2;
   double *x = r + ((size_t)w * N + i) * 3 + d;
   *x = (k & 1) ? *x - a : *x + a;
@@ -452,36 +479,76 @@ __global__ void k_lrdmc_finish(int W, const double *__restrict__ lw, const doubl
   if (eL_out) eL_out[w] = eL_cur[w];
 }
 
-// Reconfiguration (Eqs. branching-1, branching-2) by systematic resampling,
-// one thread, every sum in walker order: z from Philox (0, g, 0, 3); new
-// walker j takes the first old walker whose running weight sum exceeds
-// (j + z) S / W; stats = (wbar, ebar).  Weights reset to 1.
-__global__ void k_lrdmc_select(int W, uint32_t gen, uint32_t key0, uint32_t key1, double *__restrict__ weight,
-                               const double *__restrict__ eL, int *__restrict__ parent, double *__restrict__ stats) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// Reconfiguration (Eqs. branching-1, branching-2) by systematic resampling, one
+// CTA: z from Philox (0, g, 0, 3); new walker j takes the first old walker whose
+// running weight sum exceeds (j + z) S / W; stats = (wbar, ebar).  Weights reset
+// to 1.  Threads take consecutive walkers and scan their sums (run [W], scratch);
+// one thread alone took 0.67 ms at W = 1024.
+constexpr int kSelectThreads = 1024;
+__global__ void __launch_bounds__(kSelectThreads) k_lrdmc_select(int W, uint32_t gen, uint32_t key0, uint32_t key1,
+                                                                 double *__restrict__ weight,
+                                                                 const double *__restrict__ eL,
+                                                                 double *__restrict__ run, int *__restrict__ parent,
+                                                                 double *__restrict__ stats) {
+  __shared__ double ws[32], we[32];
+  __shared__ int wl[32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int per = (W + kSelectThreads - 1) / kSelectThreads, b0 = min(W, tid * per), b1 = min(W, b0 + per);
+  double sum = 0.0, se = 0.0;
+  int last = 0;  // the last walker with a weight
+  for (int b = b0; b < b1; ++b) {
+    sum += weight[b];
+    se += weight[b] * eL[b];
+    if (weight[b] > 0.0) last = b;
+  }
+  double incl = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const double t = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += t;
+  }
+  se = warp_sum(se);
+  last = __reduce_max_sync(0xffffffffu, last);
+  if (lane == 31) ws[warp] = incl;
+  if (lane == 0) {
+    we[warp] = se;
+    wl[warp] = last;
+  }
+  __syncthreads();
+  double base = 0.0, S = 0.0, Se = 0.0;
+  last = 0;
+  for (int q = 0; q < kSelectThreads / 32; ++q) {
+    if (q < warp) base += ws[q];
+    S += ws[q];
+    Se += we[q];
+    last = max(last, wl[q]);
+  }
+  double acc = base + (incl - sum);
+  for (int b = b0; b < b1; ++b) {
+    acc += weight[b];
+    run[b] = acc;
+  }
   uint32_t o[4] = {0u, gen, 0u, 3u};
   philox4x32_10(o, key0, key1);
   const double z = ((double)o[0] + 0.5) * 0x1p-32;
-  double S = 0.0, Se = 0.0;
-  int last = 0;
-  for (int b = 0; b < W; ++b) {
-    S += weight[b];
-    Se += weight[b] * eL[b];
-    if (weight[b] > 0.0) last = b;
-  }
-  int b = 0;
-  double run = weight[0];
-  for (int j = 0; j < W; ++j) {
+  __syncthreads();  // run[] complete (one CTA: its own writes)
+  for (int j = tid; j < W; j += kSelectThreads) {
     const double thr = ((double)j + z) * S / W;
-    while (b < W && !(run > thr)) {
-      b++;
-      if (b < W) run += weight[b];
+    int lo = 0, hi = W;  // the first b with run[b] > thr
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (run[mid] > thr)
+        hi = mid;
+      else
+        lo = mid + 1;
     }
-    parent[j] = b < W ? b : last;
+    parent[j] = lo < W ? lo : last;
+    weight[j] = 1.0;
   }
-  stats[0] = S / W;
-  stats[1] = Se / S;
-  for (int j = 0; j < W; ++j) weight[j] = 1.0;
+  if (tid == 0) {
+    stats[0] = S / W;
+    stats[1] = Se / S;
+  }
 }
 
 // r_new[j] = r_old[parent[j]] (positions of the new population)
@@ -540,7 +607,7 @@ cudaError_t launch_lrdmc_decide(const DevSystem &s, double *r, const double *eL,
                                 uint32_t walker0, uint32_t gen, double a, double gamma, double e_ref, int max_hops,
                                 LrdmcWork &lw, cudaStream_t st) {
   if (W <= 0) return cudaSuccess;
-  k_lrdmc_decide<<<(W + 127) / 128, 128, 0, st>>>(s, r, lw.rho, eL, status, W, walker0, gen, a, gamma, e_ref,
+  k_lrdmc_decide<<<(W + 3) / 4, 128, 0, st>>>(s, r, lw.rho, eL, status, W, walker0, gen, a, gamma, e_ref,
                                                    max_hops, lw.left, lw.lw, lw.hops, lw.flags, lw.active, lw.moved,
                                                    lw.list_up, lw.list_dn, lw.list_w, lw.cnt);
   return cudaGetLastError();
@@ -569,10 +636,10 @@ cudaError_t launch_lrdmc_finish(int W, const double *lw, const double *eL_cur, d
 }
 
 cudaError_t launch_lrdmc_branch(int W, int N, uint32_t gen, uint32_t key0, uint32_t key1, double *weight,
-                                const double *eL, int *parent, double *stats, const double *r_old, double *r_new,
-                                cudaStream_t st) {
+                                const double *eL, double *run, int *parent, double *stats, const double *r_old,
+                                double *r_new, cudaStream_t st) {
   if (W <= 0) return cudaSuccess;
-  k_lrdmc_select<<<1, 32, 0, st>>>(W, gen, key0, key1, weight, eL, parent, stats);
+  k_lrdmc_select<<<1, kSelectThreads, 0, st>>>(W, gen, key0, key1, weight, eL, run, parent, stats);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const long tot = (long)W * N * 3;
