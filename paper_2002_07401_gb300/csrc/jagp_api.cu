@@ -1465,9 +1465,9 @@ jagp_status_t batch_build_grouped(jagp_batch *b) {
   b->blob = nullptr;
   JAGP_CU(cudaMalloc(&b->blob, std::max<size_t>(host.size(), 256)));
   JAGP_CU(cudaMemcpy(b->blob, host.data(), host.size(), cudaMemcpyHostToDevice));
-  // dynamic shared memory beyond 48 KB: the kernel's limit raised to the device's
+  // dynamic shared memory near 48 KB or beyond: the kernel's limit raised to the device's
   for (const auto &gl : b->glaunch)
-    if (gl.smem > 48 * 1024) {
+    if (gl.smem > kRaiseSmem) {
       std::atomic<unsigned char> done[64];
       for (auto &d : done) d.store(0, std::memory_order_relaxed);
       JAGP_CU(group_raise_smem(gl.fn, done));

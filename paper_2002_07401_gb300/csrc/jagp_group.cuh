@@ -178,6 +178,10 @@ inline void group_subkey(int e) {
   }
 }
 
+// dynamic shared memory above this raises a kernel's limit: 48 KB hold the static
+// shared memory (up to 8 KB beside dynamic memory, the arguments of a grouped
+// launch among it) as well
+constexpr size_t kRaiseSmem = 40 * 1024;
 // allow kernel fn dynamic shared memory up to the current device's opt-in
 // limit less its static shared memory; done[device] records that it was set
 // (setting it twice from two threads is harmless)
@@ -212,7 +216,7 @@ cudaError_t launch_or_record(K kernel, dim3 grid, dim3 block, size_t smem, cudaS
     R->recs.push_back(std::move(r));
     return cudaSuccess;
   }
-  if (smem > 48 * 1024) {
+  if (smem > kRaiseSmem) {
     static std::atomic<unsigned char> raised[64];  // per device (zero at start)
     const cudaError_t e = group_raise_smem(reinterpret_cast<const void *>(kernel), raised);
     if (e != cudaSuccess) return e;

@@ -110,7 +110,9 @@ cudaError_t launch_lambda_rows(const double *P, const double *Lam, double *Out, 
   if (max_rows <= 0) return cudaSuccess;
   // the tile whose fullest SM has the least FP64 work (the sums of an output
   // run over k in the same order in each, so the choice changes no result);
-  // the factors are the smaller tiles' extra loads and barriers
+  // the factors are the smaller tiles' extra loads and barriers.  A grouped launch
+  // fills the SMs with many systems' tiles: one tile for all, so that they share it.
+  if (group_recorder()) return launch_tile<32>(P, Lam, Out, list, count, nrows, nsub, stride, L, max_rows, st);
   auto work = [&](int t, double f) {
     const long long tiles = (long long)((L + t - 1) / t) * ((max_rows + t - 1) / t);
     return f * (double)((tiles + 151) / 152) * t * t;
