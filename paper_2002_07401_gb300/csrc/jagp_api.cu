@@ -191,13 +191,18 @@ jagp_status_t lambda_products(jagp_ctx *h, const float *P, const float *P_lo, fl
                               const int *count, int nrows, int nsub, int stride, int max_rows, void *state, int W,
                               cudaStream_t st) {
   // mixed path: cut the two-float rows P + P_lo into fixed-point slices, then
-  // the exact tensor-core contraction against the sliced lambda
+  // the exact tensor-core contraction against the sliced lambda.  Listed rows are
+  // those of accepted moves: where the refresh takes its operands from slices of the
+  // tables (tc_refresh), the rows that changed are cut again there, up rows of
+  // Phi_up with the operand here, down rows of Bt from the result.
   const Layout L = layout_of(h, W);
+  const bool keep = list && tc_refresh(h);
   uint16_t *pack = at<uint16_t>(state, L.pack);
   int *rows = at<int>(state, L.rows), *exps = at<int>(state, L.exps);
   LAUNCH(0, 1,
          launch_pack_fixed(P, P_lo, list, count, nrows, nsub, stride, h->ds.L, h->kp, pack, rows, exps, max_rows,
-                            st));
+                           st, keep && left ? at<uint16_t>(state, L.gpack_a) : nullptr,
+                           keep && left ? at<int>(state, L.gexp_a) : nullptr));
   // the rows keep their low parts (two-float Bt and A_up tables)
   float *out_lo = at<float>(state, left ? L.a_up_lo : L.bt_lo);
   LAUNCH(JAGP_KERNEL_LAMBDA_ROWS, 1,
@@ -207,6 +212,10 @@ jagp_status_t lambda_products(jagp_ctx *h, const float *P, const float *P_lo, fl
                           left ? h->tune_bn_left : h->tune_bn_right, nullptr, 8, 0, 0,
                           left ? h->tune_st_left : h->tune_st_right, 0, 0, 0, 0,
                           left ? h->range_lamT : h->range_lam, h->ds.L));
+  if (keep && !left)
+    LAUNCH(0, 1,
+           launch_pack_fixed(out, out_lo, list, count, nrows, nsub, stride, h->ds.L, h->kp, nullptr, nullptr, nullptr,
+                             max_rows, st, at<uint16_t>(state, L.gpack_b), at<int>(state, L.gexp_b)));
   return JAGP_OK;
 }
 
@@ -311,9 +320,11 @@ jagp_status_t run_local_energy(jagp_ctx *h, const double *r, void *state, int W,
 }
 
 // G~ = Phi_up Bt^T, its inverse (FP64 elimination), log|det| and (optionally) J
+// (cut_tables: the tables are new as a whole, so that their slices are all cut here;
+// in a sweep lambda_products has kept them current)
 template <typename T>
 jagp_status_t run_refresh(jagp_ctx *h, const double *r, void *state, int W, int check_drift, bool jastrow,
-                          cudaStream_t st) {
+                          cudaStream_t st, bool cut_tables = false) {
   const Layout L = layout_of(h, W);
   const int n = h->ds.n_up, Lb = h->ds.L;
   double *gm = refresh_g(L, state);
@@ -321,15 +332,16 @@ jagp_status_t run_refresh(jagp_ctx *h, const double *r, void *state, int W, int 
   if (tc_refresh(h)) {
     // G~ = (Phi_up + lo)(Bt + lo)^T per walker on the tensor cores: both tables
     // cut into six fixed-point slices, twenty-one pairs, FP64 epilogue
-    int *rows = at<int>(state, L.grows);
     uint16_t *pa = at<uint16_t>(state, L.gpack_a), *pb = at<uint16_t>(state, L.gpack_b);
     int *ea = at<int>(state, L.gexp_a), *eb = at<int>(state, L.gexp_b);
-    LAUNCH(0, 1,
-           launch_pack_fixed(at<float>(state, L.phi_up), lo_table(h, state, L.phi_lo), nullptr, nullptr, W * n, 1, 1,
-                             Lb, h->kp, pa, rows, ea, W * n, st));
-    LAUNCH(0, 1,
-           launch_pack_fixed(at<float>(state, L.bt), lo_table(h, state, L.bt_lo), nullptr, nullptr, W * n, 1, 1, Lb,
-                             h->kp, pb, rows, eb, W * n, st));
+    if (cut_tables) {
+      LAUNCH(0, 1,
+             launch_pack_fixed(at<float>(state, L.phi_up), lo_table(h, state, L.phi_lo), nullptr, nullptr, W * n, 1, 1,
+                               Lb, h->kp, nullptr, nullptr, nullptr, W * n, st, pa, ea));
+      LAUNCH(0, 1,
+             launch_pack_fixed(at<float>(state, L.bt), lo_table(h, state, L.bt_lo), nullptr, nullptr, W * n, 1, 1, Lb,
+                               h->kp, nullptr, nullptr, nullptr, W * n, st, pb, eb));
+    }
     group_subkey(1);
     LAUNCH(JAGP_KERNEL_GEMM_ROWS, 1,
            launch_umma_gemm(pa, W * n, nullptr, kFixedSlices, pb, n, kFixedSlices, h->kp, kFixedPairs, kPairA, kPairB,
@@ -378,7 +390,7 @@ jagp_status_t run_eval(jagp_ctx *h, const double *d_r, int W, void *d_state, dou
   LAUNCH(0, d.n_up > d.n_dn, launch_fill_unpaired<T>(d, at<T>(d_state, L.bt), W, st));
   if (h->precision == JAGP_PREC_MIXED)
     LAUNCH(0, d.n_up > d.n_dn, launch_fill_unpaired_lo(d, at<float>(d_state, L.bt_lo), W, st));
-  s = run_refresh<T>(h, d_r, d_state, W, 0, true, st);
+  s = run_refresh<T>(h, d_r, d_state, W, 0, true, st, true);
   if (s != JAGP_OK) return s;
   LAUNCH(0, (d_logabs || d_sign), launch_logpsi_out(at<double>(d_state, L.scal), W, d_logabs, d_sign, st));
   return JAGP_OK;

@@ -84,11 +84,11 @@ struct Layout {
   size_t bt_lo;    // float  [W][n_up][L]    mixed path: low parts of Bt (Bt + bt_lo is a two-float table)
   size_t phi_lo;   // float  [W][n_up][L]    mixed path: low parts of phi_up
   size_t pprop_lo; // float  [W][n_up][L]    mixed path: low parts of pprop
-  size_t gpack_a;  // BF16   [W n_up][5 kp]  mixed path, large N_up: slices of Phi_up + lo for G~ on the tensor cores
-  size_t gpack_b;  // BF16   [W n_up][5 kp]  ... and of Bt + lo
+  size_t gpack_a;  // BF16   [W n_up][6 kp]  mixed path, large N_up: slices of Phi_up + lo for G~ on the tensor cores
+                   //                        (all rows cut by jagp_eval, a row again when its move is accepted)
+  size_t gpack_b;  // BF16   [W n_up][6 kp]  ... and of Bt + lo
   size_t gexp_a;   // int    [W n_up]        their row exponents
   size_t gexp_b;   // int    [W n_up]
-  size_t grows;    // int    [W n_up]        scratch row map of the packing
   // mixed path, local energy: the M vectors as exact fixed-point tensor-core
   // products of the FP64 inverse with the two-float tables (kpn = N_up padded to 64)
   size_t ginv64;   // double [W][n_up][n_up] G~^{-1} of the last refresh in FP64
@@ -139,7 +139,6 @@ inline Layout make_layout(size_t W, size_t nu, size_t N, size_t L, size_t esz = 
   l.gpack_b = take(gp);
   l.gexp_a = take(gi);
   l.gexp_b = take(gi);
-  l.grows = take(gi);
   const bool mx = esz == 4;
   const size_t kpn = (nu + 63) / 64 * 64;
   l.ginv64 = take(mx ? W * nu * nu * 8 : 0);

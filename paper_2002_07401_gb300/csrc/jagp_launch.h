@@ -155,10 +155,11 @@ cudaError_t launch_pack_cols(const double *X64, const float *X32, const float *X
                              int W, uint16_t *A, int *exps, int *rows_out, long dst_stride, long dst_off,
                              cudaStream_t st, int nsl = kFixedSlices, int bits = 8);
 // FP32 rows (two-float rows P + P_lo when P_lo is given) -> kFixedSlices exact
-// 8-bit slices per element (BF16) plus a row exponent
+// 8-bit slices per element (BF16) plus a row exponent, compacted into A / rows_out /
+// exps (unless A is null) and, when given, at each row's own place in A_at / exps_at
 cudaError_t launch_pack_fixed(const float *P, const float *P_lo, const int *list, const int *count, int nrows,
-                               int nsub, int stride, int L, int kp, uint16_t *A, int *rows_out, int *exps,
-                               int max_rows, cudaStream_t st);
+                              int nsub, int stride, int L, int kp, uint16_t *A, int *rows_out, int *exps,
+                              int max_rows, cudaStream_t st, uint16_t *A_at = nullptr, int *exps_at = nullptr);
 cudaError_t setup_umma_attributes();
 
 // Reverse-mode derivatives (k_adjoint.cu); see that file for the formulas.

@@ -1050,15 +1050,18 @@ cudaError_t launch_umma_gemm(const uint16_t *A, int m_max, const int *m_dev, int
 // BF16 side by side, with e in exps[m].  Every step of the cut is exact in
 // FP32.  A two-float row P + P_lo is cut the same way, its remainder carried
 // from slice to slice as an exact two-float sum (TwoSum), so that the slices
-// take the low part's bits as well.
+// take the low part's bits as well.  A_at / exps_at (or null) receive the same
+// slices and exponent at the table row's own place (the refresh's operands,
+// kept current row by row as moves are accepted); A null writes only those.
 // ---------------------------------------------------------------------------
 struct PackFixed {
   static __device__ __forceinline__ void run(const float *__restrict__ P, const float *__restrict__ P_lo,
                                              const int *__restrict__ list, const int *__restrict__ count, int nrows,
-                                             int nsub, int stride, int L, int kp, __nv_bfloat16 *__restrict__ A,
-                                             int *__restrict__ rows_out, int *__restrict__ exps, const uint3 bid,
+                                             int nsub, int stride, int L, int kp, uint16_t *__restrict__ A,
+                                             int *__restrict__ rows_out, int *__restrict__ exps,
+                                             uint16_t *__restrict__ A_at, int *__restrict__ exps_at, const uint3 bid,
                                              const uint3 gdim) {
-    assume_global(P, A, rows_out, exps);
+    assume_global(P);
     const int rows = count ? *count : nrows;
     const int lane = threadIdx.x & 31;
     const long nw = (long)gdim.x * (blockDim.x >> 5);
@@ -1072,21 +1075,37 @@ struct PackFixed {
       for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
       const int e = (mx > 0.0f) ? ilogbf(mx) + 1 : 0;
       if (lane == 0) {
-        rows_out[m] = (int)phys;
-        exps[m] = e;
+        if (A) {
+          rows_out[m] = (int)phys;
+          exps[m] = e;
+        }
+        if (exps_at) exps_at[phys] = e;
       }
-      __nv_bfloat16 *dst = A + m * kFixedSlices * (long)kp;
-      for (int k = lane; k < kp; k += 32) {
-        float x = k < L ? ldexpf(src[k], 7 - e) : 0.0f;  // |x| < 128
-        // the low part, in the same scale
-        float xl = (srl && k < L) ? ldexpf(srl[k], 7 - e) : 0.0f;
+      uint16_t *dst = A ? A + m * kFixedSlices * (long)kp : nullptr;
+      uint16_t *at = A_at ? A_at + phys * kFixedSlices * (long)kp : nullptr;
+      // two consecutive elements per lane
+      for (int k = 2 * lane; k < kp; k += 64) {
+        float x[2], xl[2];
+  #pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const bool in = k + h < L;
+          x[h] = in ? scale_pow2(src[k + h], 7 - e) : 0.0f;             // |x| < 128
+          xl[h] = in && srl ? scale_pow2(srl[k + h], 7 - e) : 0.0f;     // the low part, in the same scale
+        }
   #pragma unroll
         for (int t = 0; t < kFixedSlices; ++t) {
-          const float q = rintf(x);
-          dst[t * kp + k] = __float2bfloat16_rn(q);
-          const fdw r = two_sum(__fsub_rn(x, q), xl);  // remainder + low part, exactly
-          x = __fmul_rn(r.hi, 256.0f);
-          xl = __fmul_rn(r.lo, 256.0f);
+          uint32_t v = 0;
+  #pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const float q = rintf(x[h]);
+            // a small integer's BF16 bits: the leading half of its FP32 number
+            v |= (__float_as_uint(q) >> 16) << (16 * h);
+            const fdw r = two_sum(__fsub_rn(x[h], q), xl[h]);  // remainder + low part, exactly
+            x[h] = __fmul_rn(r.hi, 256.0f);
+            xl[h] = __fmul_rn(r.lo, 256.0f);
+          }
+          if (dst) *reinterpret_cast<uint32_t *>(dst + t * kp + k) = v;
+          if (at) *reinterpret_cast<uint32_t *>(at + t * kp + k) = v;
         }
       }
     }
@@ -1095,20 +1114,21 @@ struct PackFixed {
 __global__ void __launch_bounds__(256) k_pack_fixed(const float *__restrict__ P, const float *__restrict__ P_lo,
                                                     const int *__restrict__ list, const int *__restrict__ count,
                                                     int nrows, int nsub, int stride, int L, int kp,
-                                                    __nv_bfloat16 *__restrict__ A, int *__restrict__ rows_out,
-                                                    int *__restrict__ exps) {
-  PackFixed::run(P, P_lo, list, count, nrows, nsub, stride, L, kp, A, rows_out, exps, blockIdx, gridDim);
+                                                    uint16_t *__restrict__ A, int *__restrict__ rows_out,
+                                                    int *__restrict__ exps, uint16_t *__restrict__ A_at,
+                                                    int *__restrict__ exps_at) {
+  PackFixed::run(P, P_lo, list, count, nrows, nsub, stride, L, kp, A, rows_out, exps, A_at, exps_at, blockIdx,
+                 gridDim);
 }
 
 cudaError_t launch_pack_fixed(const float *P, const float *P_lo, const int *list, const int *count, int nrows,
-                               int nsub, int stride, int L, int kp, uint16_t *A, int *rows_out, int *exps,
-                               int max_rows, cudaStream_t st) {
+                              int nsub, int stride, int L, int kp, uint16_t *A, int *rows_out, int *exps,
+                              int max_rows, cudaStream_t st, uint16_t *A_at, int *exps_at) {
   if (max_rows <= 0) return cudaSuccess;
   long blocks = (max_rows + 7) / 8;
   if (blocks > 152 * 16) blocks = 152 * 16;
   return launch_or_record<PackFixed, 256>(k_pack_fixed, dim3((int)blocks), dim3(256), 0, st, P, P_lo, list, count,
-                                          nrows, nsub > 0 ? nsub : 1, stride, L, kp,
-                                          reinterpret_cast<__nv_bfloat16 *>(A), rows_out, exps);
+                                          nrows, nsub > 0 ? nsub : 1, stride, L, kp, A, rows_out, exps, A_at, exps_at);
 }
 
 // An FP64 value v, |v| < 2^e, as NSL slices of BITS bits: the integer nearest to
