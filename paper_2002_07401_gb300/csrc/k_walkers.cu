@@ -194,9 +194,10 @@ __device__ __forceinline__ void block_sum2(double &a, double &b, double *red) {
 
 // ---------------------------------------------------------------------------
 // Sequential single-electron Metropolis for one spin species (Sec. VMC).
-// One CTA per walker; G~^{-1} lives in shared memory for the whole
-// half-sweep (in global memory, L2-resident, when it does not fit).  Move m of an up electron replaces row m of G~ by the proposed
-// row g' (already computed from the frozen down-spin table):
+// One CTA per walker; G~^{-1} lives in shared memory for the whole half-sweep
+// (when it does not fit: MetropolisBig below).  Move m of an up electron
+// replaces row m of G~ by the proposed row g' (already computed from the frozen
+// down-spin table):
 //   ratio R = g' . G~^{-1}[:, m],
 //   G~^{-1} <- G~^{-1} - G~^{-1}[:, m] (g'^T G~^{-1} - e_m^T) / R   (Sherman-Morrison);
 // a down electron replaces column m, with the transposed formulas.  The
@@ -225,7 +226,7 @@ __host__ __device__ inline size_t metro_smem_per_walker(int n, int N) {
   return ((size_t)N * 3 * sizeof(double) + (size_t)(n * n + 3 * n) * sizeof(T) + mirror + 15) & ~size_t(15);
 }
 
-template <bool UP, typename T, bool GLOB>
+template <bool UP, typename T>
 struct Metropolis {
   static __device__ __forceinline__ void run(DevSystem s, double *__restrict__ r, const double *__restrict__ rprop,
                                              const T *__restrict__ gprop, T *__restrict__ ginv,
@@ -241,10 +242,8 @@ struct Metropolis {
     const int w = bid.x;
     T *gw = ginv + (size_t)w * n * n;
     double *xs = sm;                                  // N * 3 positions (FP64)
-    // G~^{-1} in shared memory, or (GLOB, too large for it) in place in global
-    // memory, where a CTA's n x n block stays resident in L2 for the half-sweep
-    T *Gi = GLOB ? gw : reinterpret_cast<T *>(xs + N * 3);
-    T *gp = GLOB ? reinterpret_cast<T *>(xs + N * 3) : Gi + n * n;  // n
+    T *Gi = reinterpret_cast<T *>(xs + N * 3);        // n * n  G~^{-1}
+    T *gp = Gi + n * n;                               // n
     T *vv = gp + n;                                   // n
     T *cc = vv + n;                                   // n
     float *xf = reinterpret_cast<float *>(cc + n);    // mixed path: N * 3 positions rounded to FP32
@@ -252,7 +251,7 @@ struct Metropolis {
     // three-body Jastrow (G~^{-1} in shared memory; its change in FP64 in both
     // paths): the walker's j3 vectors [6][LJ] and chi at the old and the
     // proposed position, chi change, after the per-walker block
-    const bool j3 = !GLOB && s.use_j3 && j3buf;
+    const bool j3 = s.use_j3 && j3buf;
     const int LJ = s.LJ;
     double *j3v = reinterpret_cast<double *>(reinterpret_cast<char *>(sm) + metro_smem_per_walker<T>(n, N));
     double *chi_o = j3v + 6 * LJ, *chi_n = chi_o + LJ, *dchi = chi_n + LJ;
@@ -261,8 +260,7 @@ struct Metropolis {
     __shared__ double red[64];
     __shared__ int s_acc;
     __shared__ double s_R;
-    if (!GLOB)
-      for (int t = tid; t < n * n; t += bs) Gi[t] = gw[t];
+    for (int t = tid; t < n * n; t += bs) Gi[t] = gw[t];
     for (int t = tid; t < N * 3; t += bs) {
       xs[t] = r[(size_t)w * N * 3 + t];
       if constexpr (kF32) xf[t] = static_cast<float>(xs[t]);
@@ -341,28 +339,16 @@ struct Metropolis {
       }
       __syncthreads();
       if (s_acc) {
-        if (GLOB && !UP) {
-          // rows of G~^{-1} against g': one warp per row, coalesced loads
-          const int lane = tid & 31, nw = bs >> 5;
-          for (int t = tid >> 5; t < n; t += nw) {
-            T a = T(0);
-            for (int i = lane; i < n; i += 32) a += Gi[t * n + i] * gp[i];
-            a = warp_sum(a);
-            if (lane == 0) vv[t] = a;
+        for (int t = tid; t < n; t += bs) {
+          T a = T(0);
+          if (UP) {
+            for (int j = 0; j < n; ++j) a += gp[j] * Gi[j * n + t];
+            cc[t] = Gi[t * n + m];
+          } else {
+            for (int i = 0; i < n; ++i) a += Gi[t * n + i] * gp[i];
+            cc[t] = Gi[m * n + t];
           }
-          for (int t = tid; t < n; t += bs) cc[t] = Gi[m * n + t];
-        } else {
-          for (int t = tid; t < n; t += bs) {
-            T a = T(0);
-            if (UP) {
-              for (int j = 0; j < n; ++j) a += gp[j] * Gi[j * n + t];
-              cc[t] = Gi[t * n + m];
-            } else {
-              for (int i = 0; i < n; ++i) a += Gi[t * n + i] * gp[i];
-              cc[t] = Gi[m * n + t];
-            }
-            vv[t] = a;
-          }
+          vv[t] = a;
         }
         __syncthreads();
         const T invR = T(1) / static_cast<T>(s_R);
@@ -410,8 +396,7 @@ struct Metropolis {
     }
     if (j3)
       for (int t = tid; t < 6 * LJ; t += bs) j3buf[(size_t)w * 6 * LJ + t] = j3v[t];
-    if (!GLOB)
-      for (int t = tid; t < n * n; t += bs) gw[t] = Gi[t];
+    for (int t = tid; t < n * n; t += bs) gw[t] = Gi[t];
     for (int t = tid; t < N * 3; t += bs) r[(size_t)w * N * 3 + t] = xs[t];
     if (tid == 0) {
       scal[(size_t)w * S_STRIDE + S_SIGN] = sgn;
@@ -421,7 +406,7 @@ struct Metropolis {
     }
 }
 };
-template <bool UP, typename T, bool GLOB>
+template <bool UP, typename T>
 __global__ void __launch_bounds__(512) k_metropolis(DevSystem s, double *__restrict__ r,
                                                     const double *__restrict__ rprop, const T *__restrict__ gprop,
                                                     T *__restrict__ ginv, double *__restrict__ scal,
@@ -430,8 +415,213 @@ __global__ void __launch_bounds__(512) k_metropolis(DevSystem s, double *__restr
                                                     int *__restrict__ count, const float *__restrict__ pprop_lo,
                                                     float *__restrict__ phi_lo, int m_begin, int m_end,
                                                     int *__restrict__ total, double *__restrict__ j3buf) {
-  Metropolis<UP, T, GLOB>::run(s, r, rprop, gprop, ginv, scal, status, pprop, phi_up, list, count, pprop_lo, phi_lo,
-                               m_begin, m_end, total, j3buf, blockIdx, gridDim);
+  Metropolis<UP, T>::run(s, r, rprop, gprop, ginv, scal, status, pprop, phi_up, list, count, pprop_lo, phi_lo,
+                         m_begin, m_end, total, j3buf, blockIdx, gridDim);
+}
+
+// ---------------------------------------------------------------------------
+// The same acceptance loop for a G~^{-1} that does not fit in shared memory: its
+// first rs rows live there (as many as fit), the others in global memory, where
+// they stay resident in L2.  The moves of a walker follow one another, so an
+// accepted move is bound by the three passes over G~^{-1} (one to form v, a read
+// and a write of the update): the shared rows go at shared-memory speed, the
+// others with sixteen independent loads in flight per thread, a warp per row
+// where the pass allows it.  Sums run in the order of the kernel above (v of an
+// up move, the ratio) or over a warp's lanes (v of a down move).
+// ---------------------------------------------------------------------------
+template <bool UP, typename T>
+struct MetropolisBig {
+  static constexpr int kLoads = 16;
+  static __device__ __forceinline__ void run(DevSystem s, double *__restrict__ r, const double *__restrict__ rprop,
+                                             const T *__restrict__ gprop, T *__restrict__ ginv,
+                                             double *__restrict__ scal, int *__restrict__ status,
+                                             const T *__restrict__ pprop, T *__restrict__ phi_up,
+                                             int *__restrict__ list, int *__restrict__ count,
+                                             const float *__restrict__ pprop_lo, float *__restrict__ phi_lo,
+                                             int m_begin, int m_end, int *__restrict__ total, int rs, const uint3 bid,
+                                             const uint3 gdim) {
+    assume_global(r, rprop, gprop, ginv, scal, status, pprop, phi_up, list, count);
+    extern __shared__ double sm[];
+    const int n = s.n_up, N = s.N, tid = threadIdx.x, bs = blockDim.x;
+    const int lane = tid & 31, warp = tid >> 5, nw = bs >> 5;
+    const int w = bid.x;
+    T *const gw = ginv + (size_t)w * n * n;
+    double *xs = sm;                                  // N * 3 positions (FP64)
+    T *const Gs = reinterpret_cast<T *>(xs + N * 3);  // rs * n: the first rows of G~^{-1}
+    T *gp = Gs + (size_t)rs * n;                      // n
+    T *vv = gp + n;                                   // n
+    T *cc = vv + n;                                   // n
+    float *xf = reinterpret_cast<float *>(cc + n);    // mixed path: N * 3 positions rounded to FP32
+    constexpr bool kF32 = std::is_same<T, float>::value;
+    __shared__ double red[64];
+    __shared__ int s_acc;
+    __shared__ double s_R;
+    for (int t = tid; t < rs * n; t += bs) Gs[t] = gw[t];
+    for (int t = tid; t < N * 3; t += bs) {
+      xs[t] = r[(size_t)w * N * 3 + t];
+      if constexpr (kF32) xf[t] = static_cast<float>(xs[t]);
+    }
+    double sgn = 1.0, J = 0.0, nacc = 0.0;
+    int st_bits = 0;
+    if (tid == 0) {
+      sgn = scal[(size_t)w * S_STRIDE + S_SIGN];
+      J = scal[(size_t)w * S_STRIDE + S_J];
+      nacc = scal[(size_t)w * S_STRIDE + S_NACC];
+      st_bits = status[w];
+    }
+    const int nmoves = m_end < (UP ? s.n_up : s.n_dn) ? m_end : (UP ? s.n_up : s.n_dn);
+    const int e0 = UP ? 0 : s.n_up;
+    __syncthreads();
+    for (int m = m_begin; m < nmoves; ++m) {
+      const int e = e0 + m;
+      const double *rp4 = rprop + ((size_t)w * n + m) * kPropStride;
+      const double px = rp4[0], py = rp4[1], pz = rp4[2];
+      // the move's column (up) or row (down) of G~^{-1} and the proposed row or column of G~
+      T prt = T(0);
+      for (int t = tid; t < n; t += bs) {
+        const T g = gprop[((size_t)w * n + m) * n + t];
+        T c;
+        if (UP)
+          c = t < rs ? Gs[t * n + m] : gw[(size_t)t * n + m];
+        else
+          c = m < rs ? Gs[m * n + t] : gw[(size_t)m * n + t];
+        gp[t] = g;
+        cc[t] = c;
+        prt += UP ? g * c : c * g;
+      }
+      double pr = static_cast<double>(prt), pj = 0.0;
+      const double ox = xs[3 * e], oy = xs[3 * e + 1], oz = xs[3 * e + 2];
+      if (tid == 0) pj = rp4[4];   // one-body Jastrow change, from the proposal kernel
+      if (s.use_j2) {
+        if constexpr (kF32) {
+          const float pf[3] = {static_cast<float>(px), static_cast<float>(py), static_cast<float>(pz)};
+          const float of[3] = {xf[3 * e], xf[3 * e + 1], xf[3 * e + 2]};
+          pj += static_cast<double>(j2_move_change_f<UP>(s, xf, e, pf, of, tid, bs));
+        } else {
+          pj += j2_move_change<T, UP>(s, xs, e, px, py, pz, ox, oy, oz, tid, bs);
+        }
+      }
+      block_sum2(pr, pj, red);
+      if (tid == 0) {
+        const double u = rp4[3];
+        const double p = accept_prob<T>(pr, pj);
+        int acc = 0;
+        if (!isfinite(p) || !isfinite(pr)) {
+          st_bits |= JAGP_WS_NONFINITE;
+        } else if (pr != 0.0 && u < p) {
+          acc = 1;
+          if (pr < 0.0) sgn = -sgn;
+          J += pj;
+          nacc += 1.0;
+          list[atomicAdd(count, 1)] = w * n + m;
+          if (total) atomicAdd(total, 1);
+        }
+        s_acc = acc;
+        s_R = pr;
+      }
+      __syncthreads();  // (also: gp, cc complete)
+      if (s_acc) {
+        if (UP) {
+          // v = g'^T G~^{-1}: a thread per column, rows in order
+          for (int t = tid; t < n; t += bs) {
+            T q[kLoads];  // the first global rows, loading while the shared ones are summed
+  #pragma unroll
+            for (int i = 0; i < kLoads; ++i) q[i] = rs + i < n ? gw[(size_t)(rs + i) * n + t] : T(0);
+            T a = T(0);
+  #pragma unroll 8
+            for (int j = 0; j < rs; ++j) a = fma(gp[j], Gs[j * n + t], a);
+            for (int j = rs; j < n; j += kLoads) {
+              T next[kLoads];
+  #pragma unroll
+              for (int i = 0; i < kLoads; ++i)
+                next[i] = j + kLoads + i < n ? gw[(size_t)(j + kLoads + i) * n + t] : T(0);
+  #pragma unroll
+              for (int i = 0; i < kLoads; ++i)
+                if (j + i < n) a = fma(gp[j + i], q[i], a);
+  #pragma unroll
+              for (int i = 0; i < kLoads; ++i) q[i] = next[i];
+            }
+            vv[t] = a;
+          }
+        } else {
+          // v = G~^{-1} g': a warp per row
+  #pragma unroll 4
+          for (int t = warp; t < n; t += nw) {
+            const T *row = t < rs ? Gs + t * n : gw + (size_t)t * n;
+            T a = T(0);
+  #pragma unroll 8
+            for (int i = lane; i < n; i += 32) a = fma(row[i], gp[i], a);
+            a = warp_sum(a);
+            if (lane == 0) vv[t] = a;
+          }
+        }
+        __syncthreads();
+        const T invR = T(1) / static_cast<T>(s_R);
+        // rank-one update, a warp per row
+        auto update = [&](T *row, int j) {
+          const T vj = vv[j] - (j == m ? T(1) : T(0)), cj = cc[j];
+          for (int k0 = 0; k0 < n; k0 += 32 * 8) {
+            T g[8];
+  #pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              const int k = k0 + lane + 32 * i;
+              g[i] = k < n ? row[k] : T(0);
+            }
+  #pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              const int k = k0 + lane + 32 * i;
+              if (k < n) {
+                const T x = UP ? cj * (vv[k] - (k == m ? T(1) : T(0))) : vj * cc[k];
+                row[k] = fma(-x, invR, g[i]);
+              }
+            }
+          }
+        };
+        for (int j = warp; j < rs; j += nw) update(Gs + j * n, j);
+  #pragma unroll 2
+        for (int j = rs + warp; j < n; j += nw) update(gw + (size_t)j * n, j);
+        if (tid == 0) {
+          xs[3 * e] = px;
+          xs[3 * e + 1] = py;
+          xs[3 * e + 2] = pz;
+          if constexpr (kF32) {
+            xf[3 * e] = static_cast<float>(px);
+            xf[3 * e + 1] = static_cast<float>(py);
+            xf[3 * e + 2] = static_cast<float>(pz);
+          }
+        }
+        if (UP) {
+          const size_t row = ((size_t)w * n + m) * s.L;
+  #pragma unroll 4
+          for (int t = tid; t < s.L; t += bs) phi_up[row + t] = pprop[row + t];
+          if (phi_lo)
+  #pragma unroll 4
+            for (int t = tid; t < s.L; t += bs) phi_lo[row + t] = pprop_lo[row + t];
+        }
+      }
+      __syncthreads();
+    }
+    for (int t = tid; t < rs * n; t += bs) gw[t] = Gs[t];
+    for (int t = tid; t < N * 3; t += bs) r[(size_t)w * N * 3 + t] = xs[t];
+    if (tid == 0) {
+      scal[(size_t)w * S_STRIDE + S_SIGN] = sgn;
+      scal[(size_t)w * S_STRIDE + S_J] = J;
+      scal[(size_t)w * S_STRIDE + S_NACC] = nacc;
+      status[w] = st_bits;
+    }
+}
+};
+template <bool UP, typename T>
+__global__ void __launch_bounds__(512) k_metropolis_big(DevSystem s, double *__restrict__ r,
+                                                        const double *__restrict__ rprop, const T *__restrict__ gprop,
+                                                        T *__restrict__ ginv, double *__restrict__ scal,
+                                                        int *__restrict__ status, const T *__restrict__ pprop,
+                                                        T *__restrict__ phi_up, int *__restrict__ list,
+                                                        int *__restrict__ count, const float *__restrict__ pprop_lo,
+                                                        float *__restrict__ phi_lo, int m_begin, int m_end,
+                                                        int *__restrict__ total, int rs) {
+  MetropolisBig<UP, T>::run(s, r, rprop, gprop, ginv, scal, status, pprop, phi_up, list, count, pprop_lo, phi_lo,
+                            m_begin, m_end, total, rs, blockIdx, gridDim);
 }
 
 // ---------------------------------------------------------------------------
@@ -838,30 +1028,21 @@ cudaError_t launch_metropolis(const DevSystem &s, bool up, double *r, const doub
   if (m_end < 0) m_end = up ? s.n_up : s.n_dn;
   if (m_begin >= m_end) return cudaSuccess;
   const int n = s.n_up;
-  // one CTA per walker (threads per CTA, shared memory, G~^{-1} in shared or global memory)
-  auto cta = [&](int threads, size_t smem, bool glob, double *j3) -> cudaError_t {
-    if (glob) {
-      if (up)
-        return launch_or_record<Metropolis<true, T, true>, 512>(k_metropolis<true, T, true>, dim3(W), dim3(threads), smem, st, s, r, rprop, gprop,
-                                                                ginv, scal, status, pprop, phi_up, list, count,
-                                                                pprop_lo, phi_lo, m_begin, m_end, total, j3);
-      return launch_or_record<Metropolis<false, T, true>, 512>(k_metropolis<false, T, true>, dim3(W), dim3(threads), smem, st, s, r, rprop, gprop,
-                                                               ginv, scal, status, pprop, phi_up, list, count,
-                                                               pprop_lo, phi_lo, m_begin, m_end, total, j3);
-    }
+  // one CTA per walker (threads per CTA, shared memory)
+  auto cta = [&](int threads, size_t smem, double *j3) -> cudaError_t {
     if (up)
-      return launch_or_record<Metropolis<true, T, false>, 512>(k_metropolis<true, T, false>, dim3(W), dim3(threads), smem, st, s, r, rprop, gprop,
-                                                               ginv, scal, status, pprop, phi_up, list, count,
-                                                               pprop_lo, phi_lo, m_begin, m_end, total, j3);
-    return launch_or_record<Metropolis<false, T, false>, 512>(k_metropolis<false, T, false>, dim3(W), dim3(threads), smem, st, s, r, rprop, gprop,
-                                                              ginv, scal, status, pprop, phi_up, list, count,
-                                                              pprop_lo, phi_lo, m_begin, m_end, total, j3);
+      return launch_or_record<Metropolis<true, T>, 512>(k_metropolis<true, T>, dim3(W), dim3(threads), smem, st, s, r,
+                                                        rprop, gprop, ginv, scal, status, pprop, phi_up, list, count,
+                                                        pprop_lo, phi_lo, m_begin, m_end, total, j3);
+    return launch_or_record<Metropolis<false, T>, 512>(k_metropolis<false, T>, dim3(W), dim3(threads), smem, st, s, r,
+                                                       rprop, gprop, ginv, scal, status, pprop, phi_up, list, count,
+                                                       pprop_lo, phi_lo, m_begin, m_end, total, j3);
   };
   if (s.use_j3) {
     // the three-body Jastrow's change is formed in the CTA-per-walker kernel
     const size_t per3 = metro_smem_per_walker<T>(n, s.N) + (size_t)9 * s.LJ * sizeof(double);
     if (!j3buf || per3 > kMetroSmemMax) return cudaErrorInvalidValue;
-    return cta(n <= 64 ? 128 : 256, per3, false, j3buf);
+    return cta(n <= 64 ? 128 : 256, per3, j3buf);
   }
   const size_t per = metro_smem_per_walker<T>(n, s.N);
   if (n <= 32) {
@@ -874,10 +1055,19 @@ cudaError_t launch_metropolis(const DevSystem &s, bool up, double *r, const doub
         dim3(blocks), dim3(kMetroWarps * 32), per * kMetroWarps, st, s, r, rprop, gprop, ginv, scal, status, pprop,
         phi_up, list, count, W, pprop_lo, phi_lo, m_begin, m_end, total);
   }
-  if (per <= kMetroSmemMax) return cta(n <= 64 ? 128 : 256, per, false, nullptr);
-  const size_t glob = (size_t)s.N * 3 * sizeof(double) + (size_t)3 * n * sizeof(T) +
+  if (per <= kMetroSmemMax) return cta(n <= 64 ? 128 : 256, per, nullptr);
+  // as many rows of G~^{-1} in shared memory as fit beside the rest
+  const size_t rest = (size_t)s.N * 3 * sizeof(double) + (size_t)3 * n * sizeof(T) +
                       (std::is_same<T, float>::value ? (size_t)s.N * 3 * sizeof(float) : 0);
-  return cta(512, glob, true, nullptr);
+  const int rs = rest < kMetroSmemMax ? (int)((kMetroSmemMax - rest) / ((size_t)n * sizeof(T))) : 0;
+  const size_t smem = rest + (size_t)rs * n * sizeof(T);
+  if (up)
+    return launch_or_record<MetropolisBig<true, T>, 512>(k_metropolis_big<true, T>, dim3(W), dim3(512), smem, st, s, r,
+                                                         rprop, gprop, ginv, scal, status, pprop, phi_up, list, count,
+                                                         pprop_lo, phi_lo, m_begin, m_end, total, rs);
+  return launch_or_record<MetropolisBig<false, T>, 512>(k_metropolis_big<false, T>, dim3(W), dim3(512), smem, st, s, r,
+                                                        rprop, gprop, ginv, scal, status, pprop, phi_up, list, count,
+                                                        pprop_lo, phi_lo, m_begin, m_end, total, rs);
 }
 template cudaError_t launch_metropolis<double>(const DevSystem &, bool, double *, const double *, const double *,
                                                double *, double *, int *, const double *, double *, int *, int *,
