@@ -1,6 +1,10 @@
 // k_linalg.cu -- the dense contractions and the FP64 inverse refresh of the
 // geminal matrix (Sec. AGP, Eq. agp_expansion: G~ = Phi_up lambda Phi_dn^T | Phi_up C).
+#include <cooperative_groups.h>
 #include <math.h>
+
+#include <algorithm>
+#include <atomic>
 
 #include "jagp_group.cuh"
 #include "jagp_launch.h"
@@ -801,7 +805,212 @@ __global__ void __launch_bounds__(128, 4) k_refresh_inverse_cta(const double *__
   RefreshInverseCta<T, CPL>::run(gm, ginv, scal, status, n, W, check_drift, drift_tol, ginv64, blockIdx, gridDim);
 }
 
-// In-place Gauss-Jordan (N_up > 32): step k scales the pivot row, stores
+// N_up > 64 while a cluster's shared memory holds the matrix: the same elimination
+// (no row swaps) on a cluster of cl CTAs per walker, CTA c with the columns c C ..
+// c C + C - 1 of every row in shared memory.  The owner of column k finds the
+// pivot row and sends the column and the row's index to every CTA; the rest of a
+// step is local (each CTA has its columns of the pivot row), so a step costs one
+// cluster barrier, and the column buffers alternate with the parity of k.  A
+// thread keeps one column and takes every R-th row, R = threads / C, so that
+// consecutive threads touch consecutive elements and none of the FP64 pipe, which
+// bounds an update (n C / 2 clocks), goes to padding.  Several CTAs share an SM and
+// hide each other's barriers and pivot searches.
+constexpr int kClusterThreads = 256;
+struct ClusterSmem {
+  static __host__ __device__ size_t bytes(int n, int C) {
+    // the columns, two column buffers, the scaled pivot row, pivots; pivot rows, steps, used flags
+    return ((size_t)n * C + 3 * (size_t)n + C) * sizeof(double) + (size_t)3 * n * sizeof(int);
+  }
+};
+
+template <typename T>
+struct RefreshInverseCluster {
+  static __device__ __forceinline__ void run(const double *__restrict__ gm, T *__restrict__ ginv,
+                                             double *__restrict__ scal, int *__restrict__ status, int n, int cl,
+                                             int check_drift, double drift_tol, double *__restrict__ ginv64,
+                                             const uint3 bid, const uint3 gdim) {
+    assume_global(gm, ginv, scal, status);
+    namespace cg = cooperative_groups;
+    extern __shared__ double sm[];
+    const int C = (n + cl - 1) / cl, w = (int)bid.x / cl, rank = (int)bid.x - w * cl;
+    double *const S = sm;                      // [n][C]
+    double *const F = S + (size_t)n * C;       // [2][n] column k before the step
+    double *const prow = F + 2 * n;            // [C]
+    double *const pvs = prow + C;              // [n] pivots
+    int *const sp = reinterpret_cast<int *>(pvs + n);  // [n] pivot row of each step
+    int *const sq = sp + n;                    // [n] step at which each row was pivoted
+    int *const used = sq + n;                  // [n]
+    __shared__ int s_piv[2];
+    __shared__ double red[kClusterThreads / 32][2];
+    __shared__ double s_max[8][2];             // rank 0: every CTA's largest |G~| and drift
+    __shared__ unsigned s_par[kClusterThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    auto cluster_sync = [&] {
+      if (cl > 1) {
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+      } else {
+        __syncthreads();
+      }
+    };
+    // the CTA's copy of p in rank r's shared memory
+    auto remote = [&](auto *q, int r) { return cl > 1 ? cg::this_cluster().map_shared_rank(q, r) : q; };
+    const int j0 = rank * C, nc = n - j0 < C ? (n - j0 > 0 ? n - j0 : 0) : C;  // this CTA's columns
+    const int R = kClusterThreads / C, g = tid / C, jc = tid - g * C;  // (C <= kClusterThreads)
+    const double *Gw = gm + (size_t)w * n * n;
+    double gmax = 0.0;
+    for (int i = warp; i < n; i += kClusterThreads / 32)
+      for (int j = lane; j < C; j += 32) {
+        const double v = j < nc ? Gw[(size_t)i * n + j0 + j] : 0.0;
+        gmax = fmax(gmax, fabs(v));
+        S[(size_t)i * C + j] = v;
+      }
+    for (int i = tid; i < n; i += kClusterThreads) used[i] = 0;
+    bool ok = true;
+    cluster_sync();  // (every CTA of the cluster runs, its buffers may be written)
+    for (int k = 0; k < n; ++k) {
+      const int par = k & 1, owner = k / C, kc = k - owner * C;
+      double *const f = F + par * n;
+      if (rank == owner) {
+        // column k to every CTA; the pivot among the rows not yet used
+        for (int i = tid; i < n; i += kClusterThreads) {
+          const double v = S[(size_t)i * C + kc];
+          for (int r = 0; r < cl; ++r) remote(f, r)[i] = v;
+        }
+        if (warp == 0) {
+          unsigned long long key = 0ull;
+          int row = lane;
+          for (int i = lane; i < n; i += 32) {
+            const unsigned long long ki = used[i] ? 0ull : abs_key(S[(size_t)i * C + kc]);
+            if (ki > key) {
+              key = ki;
+              row = i;
+            }
+          }
+          const int p = best_row(key, row);
+          if (lane < cl) *remote(&s_piv[par], lane) = p;
+        }
+      }
+      cluster_sync();
+      const int p = s_piv[par];
+      const double pv = f[p];
+      const unsigned long long pk = abs_key(pv);
+      if (used[p] || pk == 0ull || pk >= 0x7ff0000000000000ull) {  // the same in every CTA
+        ok = false;
+        break;
+      }
+      const double ip = recip_newton(pv);
+      const bool mine = rank == owner;
+      for (int j = tid; j < C; j += kClusterThreads)
+        prow[j] = mine && j == kc ? ip : S[(size_t)p * C + j] * ip;
+      __syncthreads();
+      if (tid == 0) {
+        sp[k] = p;
+        sq[p] = k;
+        pvs[k] = pv;
+        used[p] = 1;
+      }
+      if (g < R) {
+        const double x = prow[jc];
+        const bool ck = mine && jc == kc;
+        double *Sj = S + jc;
+#pragma unroll 8
+        for (int i = g; i < n; i += R) {
+          const double base = ck ? 0.0 : Sj[i * C];
+          Sj[i * C] = i == p ? x : fma(-f[i], x, base);
+        }
+      }
+      __syncthreads();
+    }
+    T *gi = ginv + (size_t)w * n * n;
+    double dmax = 0.0;
+    if (ok) {
+      // inverse[k][p_c] = result[p_k][c]: row i of the result goes to row q_i, column c to column p_c
+      for (int i = warp; i < n; i += kClusterThreads / 32) {
+        const size_t row = (size_t)sq[i] * n;
+        for (int j = lane; j < nc; j += 32) {
+          const double v = S[(size_t)i * C + j];
+          const size_t idx = row + sp[j0 + j];
+          if (check_drift) dmax = fmax(dmax, fabs(v - static_cast<double>(gi[idx])));
+          gi[idx] = static_cast<T>(v);
+          if (ginv64) ginv64[(size_t)w * n * n + idx] = v;
+        }
+      }
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      dmax = fmax(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
+      gmax = fmax(gmax, __shfl_xor_sync(0xffffffffu, gmax, o));
+    }
+    if (lane == 0) {
+      red[warp][0] = gmax;
+      red[warp][1] = dmax;
+    }
+    // parity of the pivot order
+    unsigned inv = 0;
+    if (ok && rank == 0)
+      for (int k = tid; k < n; k += kClusterThreads)
+        for (int q = k + 1; q < n; ++q) inv ^= sp[q] < sp[k];
+    inv = __reduce_xor_sync(0xffffffffu, inv);
+    if (lane == 0) s_par[warp] = inv;
+    __syncthreads();
+    if (tid == 0) {
+      for (int q = 1; q < kClusterThreads / 32; ++q) {
+        gmax = fmax(gmax, red[q][0]);
+        dmax = fmax(dmax, red[q][1]);
+      }
+      double *m = remote(&s_max[0][0], 0);
+      m[2 * rank] = gmax;
+      m[2 * rank + 1] = dmax;
+    }
+    cluster_sync();
+    if (rank != 0 || warp != 0) return;
+    double *sw = scal + (size_t)w * S_STRIDE;
+    if (!ok) {
+      if (lane == 0) {
+        status[w] |= JAGP_WS_SINGULAR;
+        sw[S_LOGDET] = -INFINITY;
+        sw[S_SIGN] = 0.0;
+      }
+      return;
+    }
+    // log|det|: each lane's pivots as a mantissa and an exponent, then the warp's
+    PivotProduct pp;
+    unsigned flips = 0;
+    for (int k = lane; k < n; k += 32) {
+      pp.mul(pvs[k]);
+      flips ^= pvs[k] < 0.0;
+    }
+    double mant = pp.m;
+    int e = pp.e;
+    for (int o = 16; o > 0; o >>= 1) {
+      mant *= __shfl_xor_sync(0xffffffffu, mant, o);
+      e += __shfl_xor_sync(0xffffffffu, e, o);
+    }
+    flips = __reduce_xor_sync(0xffffffffu, flips);
+    if (lane != 0) return;
+    for (int q = 0; q < kClusterThreads / 32; ++q) flips ^= s_par[q];
+    sw[S_LOGDET] = log(mant) + e * 0.6931471805599453;
+    sw[S_SIGN] = flips ? -1.0 : 1.0;
+    if (check_drift) {
+      double g = 0.0, d = 0.0;
+      for (int r = 0; r < cl; ++r) {
+        g = fmax(g, s_max[r][0]);
+        d = fmax(d, s_max[r][1]);
+      }
+      const double drift = d * g;
+      sw[S_DRIFT] = drift;
+      if (!(drift <= drift_tol)) status[w] |= JAGP_WS_DRIFT;
+    }
+}
+};
+template <typename T>
+__global__ void __launch_bounds__(kClusterThreads) k_refresh_inverse_cluster(
+    const double *__restrict__ gm, T *__restrict__ ginv, double *__restrict__ scal, int *__restrict__ status, int n,
+    int cl, int check_drift, double drift_tol, double *__restrict__ ginv64) {
+  RefreshInverseCluster<T>::run(gm, ginv, scal, status, n, cl, check_drift, drift_tol, ginv64, blockIdx, gridDim);
+}
+
+// In-place Gauss-Jordan (larger N_up): step k scales the pivot row, stores
 // -f_i / p in column k and updates the rest, so the inverse takes the place of
 // G~ (half the work of eliminating [G~ | I]); the row swaps of the partial
 // pivoting become column swaps of the result, undone in reverse order at the
@@ -984,23 +1193,50 @@ template <typename T>
 cudaError_t launch_refresh_inverse(double *gm, T *ginv, double *scal, int *status, int n, int W,
                                    int check_drift, double drift_tol, cudaStream_t st, double *ginv64) {
   if (W <= 0) return cudaSuccess;
-  const size_t aux = (size_t)n * (2 * sizeof(double) + sizeof(int));
-  const size_t inplace_smem = (size_t)n * (n + 1) * sizeof(double) + aux;
-  if (n > 32 && n <= 48)
+  if (n > 32 && n <= 48 && !group_recorder())  // (grouped launches: one kernel for both sizes)
     return launch_or_record<RefreshInverseCta<T, 3>, 128>(k_refresh_inverse_cta<T, 3>, dim3(W), dim3(128), 0, st, gm,
                                                           ginv, scal, status, n, W, check_drift, drift_tol, ginv64);
-  if (n > 48 && n <= 64)
+  if (n > 32 && n <= 64)
     return launch_or_record<RefreshInverseCta<T, 4>, 128>(k_refresh_inverse_cta<T, 4>, dim3(W), dim3(128), 0, st, gm,
                                                           ginv, scal, status, n, W, check_drift, drift_tol, ginv64);
-  if (n > 32 && inplace_smem <= kRefreshSmemMax) {
-    return launch_or_record<RefreshInverseInplace<T>, 512>(k_refresh_inverse_inplace<T>, dim3(W), dim3(256),
-                                                           inplace_smem, st, gm, ginv, scal, status, n, n, check_drift,
-                                                           drift_tol, ginv64);
-  }
-  if (n > 32) {
+  // a cluster per walker whose CTAs together hold the matrix: as few CTAs as fit, or
+  // more (up to eight) while that leaves SMs idle or keeps a second CTA off an SM
+  // (grouped launches: one CTA, up to N_up = 156)
+  if (n > 64) {
+    int cl = 1;
+    auto fits = [&](int c, size_t limit) {
+      return (n + c - 1) / c <= kClusterThreads && ClusterSmem::bytes(n, (n + c - 1) / c) <= limit;
+    };
+    const int most = group_recorder() ? 1 : 8;
+    while (cl < most && (!fits(cl, kRefreshSmemMax) || (long long)W * cl < 2 * 152 || !fits(cl, kRefreshSmemMax / 2)))
+      cl *= 2;
+    if (fits(cl, kRefreshSmemMax)) {
+      const size_t smem = ClusterSmem::bytes(n, (n + cl - 1) / cl);
+      if (cl == 1)
+        return launch_or_record<RefreshInverseCluster<T>, kClusterThreads>(
+            k_refresh_inverse_cluster<T>, dim3(W), dim3(kClusterThreads), smem, st, (const double *)gm, ginv, scal,
+            status, n, 1, check_drift, drift_tol, ginv64);
+      static std::atomic<unsigned char> raised[64];
+      cudaError_t e = group_raise_smem(reinterpret_cast<const void *>(k_refresh_inverse_cluster<T>), raised);
+      if (e != cudaSuccess) return e;
+      cudaLaunchConfig_t cfg = {};
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = static_cast<unsigned>(cl);
+      at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+      cfg.gridDim = dim3(W * cl);
+      cfg.blockDim = dim3(kClusterThreads);
+      cfg.dynamicSmemBytes = smem;
+      cfg.stream = st;
+      cfg.attrs = at;
+      cfg.numAttrs = 1;
+      return cudaLaunchKernelEx(&cfg, k_refresh_inverse_cluster<T>, (const double *)gm, ginv, scal, status, n, cl,
+                                check_drift, drift_tol, ginv64);
+    }
     // as many leading rows in shared memory as fit in kRefreshSmemMax (which
     // also keeps one CTA per SM), the rest in global memory
-    const int rs = static_cast<int>((kRefreshSmemMax - aux) / ((size_t)(n + 1) * sizeof(double)));
+    const size_t aux = (size_t)n * (2 * sizeof(double) + sizeof(int));
+    const int rs = std::min(n, static_cast<int>((kRefreshSmemMax - aux) / ((size_t)(n + 1) * sizeof(double))));
     const size_t smem = (size_t)rs * (n + 1) * sizeof(double) + aux;
     return launch_or_record<RefreshInverseInplace<T>, 512>(k_refresh_inverse_inplace<T>, dim3(W), dim3(512), smem, st,
                                                            gm, ginv, scal, status, n, rs, check_drift, drift_tol,

@@ -19,7 +19,7 @@ def torch_cuda():
     return torch
 
 
-@pytest.mark.parametrize("n_up", [1, 8, 9, 17, 32, 33, 47, 48, 49, 63, 64, 65])
+@pytest.mark.parametrize("n_up", [1, 8, 9, 17, 32, 33, 47, 48, 49, 63, 64, 65, 111, 157, 200])
 @pytest.mark.parametrize("unpaired", [0, 1])
 def test_log_det_and_sign(torch_cuda, n_up, unpaired):
     import paper_2002_07401_gb300 as pg
@@ -36,7 +36,7 @@ def test_log_det_and_sign(torch_cuda, n_up, unpaired):
     g.close()
 
 
-@pytest.mark.parametrize("n_up", [33, 48, 49, 64])
+@pytest.mark.parametrize("n_up", [33, 48, 49, 64, 65, 160])
 def test_singular_matrix_is_flagged(torch_cuda, n_up):
     """A walker with a NaN coordinate among sound ones: its bits, and only its, are set."""
     import paper_2002_07401_gb300 as pg
