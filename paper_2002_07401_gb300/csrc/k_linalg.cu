@@ -5,6 +5,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <type_traits>
 
 #include "jagp_group.cuh"
 #include "jagp_launch.h"
@@ -93,68 +94,264 @@ __global__ void __launch_bounds__(256) k_gemm_rows_tiny(const T *__restrict__ X,
   GemmRowsTiny<T, NB>::run(X, xw, Y, yw, ma, nb, K, Out, ow, ldo, W, blockIdx, gridDim);
 }
 
-// The refresh's G~ = Phi_up Bt^T in the FP32 path: the same tile scheme with a
-// compensated dot product (error-free product by fma, error-free sum, the
-// errors summed separately; Ogita, Rump and Oishi 2005) over two-float
+// The FP32 path's per-walker products of up to 32 rows (the proposed rows and
+// columns, plain; the refresh's G~ = Phi_up Bt^T, DOT2): 4 x 4 outputs per
+// thread, Q x Q threads per walker (Q = ceil(rows / 4)), as many walkers as fill
+// 128 threads; operands through shared memory in k-chunks of 16, transposed, so
+// that sixteen outputs take two 16-byte reads per term (one output per thread was
+// bound by its two or four reads), the next chunk loading into registers
+// meanwhile.  Every output sums over k in order.
+// DOT2: a compensated dot product (error-free product by fma, error-free sum,
+// the errors summed separately; Ogita, Rump and Oishi 2005) over two-float
 // operands X + Xlo and Y + Ylo (the low parts' products with the high parts go
 // into the error sum; lo * lo is below the result's precision), so that G~ is
-// as accurate as the double-word tables rather than FP32.  The _rn intrinsics
-// keep the compiler from fusing the steps.
-struct GemmRowsDot2 {
+// as accurate as the double-word tables rather than FP32, kept in FP64.  The _rn
+// intrinsics keep the compiler from fusing the steps.
+// Plain, 4096 walkers of 16 x 16, K = 320: 107 us with one output per thread, this 46.
+// DOT2, 1021 walkers of 24 x 24, K = 460: 324 us with one output per thread, this 203
+// (its FP32 instructions alone: 94); up to 16 rows the 2 x 2 kernel below, whose
+// fewer registers keep more warps, is as fast (204 us for 4096 walkers of 16 x 16,
+// K = 320, against 220).
+constexpr int kSmallKC = 16, kSmallThreads = 128;
+constexpr int small_walkers(int q) { return q == 1 ? 32 : (q == 2 ? 16 : kSmallThreads / (q * q)); }
+constexpr int small_pitch(int q) { return 4 * q + 4; }  // floats per staged k: the transposing stores spread over banks
+
+template <bool DOT2, int Q>
+struct GemmSmallF32 {
+  using OutT = std::conditional_t<DOT2, double, float>;
   static __device__ __forceinline__ void run(const float *__restrict__ X, const float *__restrict__ Xlo, size_t xw,
                                              const float *__restrict__ Y, const float *__restrict__ Ylo, size_t yw,
-                                             int ma, int nb, int K, double *__restrict__ Out, size_t ow, int ldo,
-                                             const uint3 bid, const uint3 gdim) {
+                                             int ma, int nb, int K, OutT *__restrict__ Out, size_t ow, int ldo, int W,
+                                             int vec, const uint3 bid, const uint3 gdim) {
     assume_global(X, Y, Out);
-    __shared__ float Xs[16][65];
-    __shared__ float Xl[16][65];
-    __shared__ float Ys[16][65];
-    __shared__ float Yl[16][65];
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int w = bid.z, a0 = bid.y * 16, b0 = bid.x * 16;
-    float s = 0.0f, c = 0.0f;
-    for (int k0 = 0; k0 < K; k0 += 64) {
+    extern __shared__ float4 smf4[];
+    constexpr int KC = kSmallKC, kOps = DOT2 ? 4 : 2, rows = 4 * Q, wpc = small_walkers(Q), P = small_pitch(Q);
+    constexpr int per = kOps * KC * P;  // floats per walker: X, Y (and their low parts), each [KC][P]
+    constexpr int kQuads = wpc * kOps * rows * (KC / 4), kLoads = (kQuads + kSmallThreads - 1) / kSmallThreads;
+    const int tid = threadIdx.x;
+    float *sm = reinterpret_cast<float *>(smf4);
+    const int wl = tid / (Q * Q), t = tid - wl * Q * Q, ty = t / Q, tx = t - ty * Q;
+    const int w0 = (int)bid.x * wpc, w = w0 + wl;
+    const bool active = wl < wpc && w < W;  // idle threads still load and take part in the barriers
+    float acc[4][4], cmp[DOT2 ? 4 : 1][DOT2 ? 4 : 1];
   #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int idx = threadIdx.x + q * 256, row = idx >> 6, col = idx & 63;
-        const int k = k0 + col;
-        const int a = a0 + row, b = b0 + row;
-        const bool xa = a < ma && k < K, yb = b < nb && k < K;
-        const size_t xi = (size_t)w * xw + (size_t)a * K + k, yi = (size_t)w * yw + (size_t)b * K + k;
-        Xs[row][col] = xa ? X[xi] : 0.0f;
-        Xl[row][col] = (Xlo && xa) ? Xlo[xi] : 0.0f;
-        Ys[row][col] = yb ? Y[yi] : 0.0f;
-        Yl[row][col] = (Ylo && yb) ? Ylo[yi] : 0.0f;
+    for (int i = 0; i < 4; ++i)
+  #pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        acc[i][j] = 0.0f;
+        if constexpr (DOT2) cmp[i][j] = 0.0f;
       }
+    // quad idx: four consecutive k of one row; consecutive threads take a row's quads
+    auto fetch = [&](int idx, int k0) {
+      const int k = k0 + 4 * (idx % (KC / 4)), row = idx / (KC / 4) % rows, op = idx / (KC / 4 * rows) % kOps,
+                wr = idx / (KC / 4 * rows * kOps);
+      const bool y = op & 1;
+      const float *src = op >= 2 ? (y ? Ylo : Xlo) : (y ? Y : X);
+      float4 f = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      if (idx < kQuads && w0 + wr < W && row < (y ? nb : ma) && src) {
+        const float *g = src + (size_t)(w0 + wr) * (y ? yw : xw) + (size_t)row * K + k;
+        if (vec) {  // (K % 4 = 0: a quad is whole or absent)
+          if (k < K) f = *reinterpret_cast<const float4 *>(g);
+        } else {
+          if (k < K) f.x = g[0];
+          if (k + 1 < K) f.y = g[1];
+          if (k + 2 < K) f.z = g[2];
+          if (k + 3 < K) f.w = g[3];
+        }
+      }
+      return f;
+    };
+    auto put = [&](int idx, const float4 f) {
+      const int k4 = idx % (KC / 4), row = idx / (KC / 4) % rows, op = idx / (KC / 4 * rows) % kOps,
+                wr = idx / (KC / 4 * rows * kOps);
+      if (idx < kQuads) {
+        float *d = sm + wr * per + (op * KC + 4 * k4) * P + row;
+        d[0] = f.x;
+        d[P] = f.y;
+        d[2 * P] = f.z;
+        d[3 * P] = f.w;
+      }
+    };
+    float4 pre[kLoads];
+  #pragma unroll
+    for (int l = 0; l < kLoads; ++l) pre[l] = fetch(tid + l * kSmallThreads, 0);
+    const float *xs = sm + wl * per + 4 * ty, *ys = sm + wl * per + KC * P + 4 * tx;
+    for (int k0 = 0; k0 < K; k0 += KC) {
+  #pragma unroll
+      for (int l = 0; l < kLoads; ++l) put(tid + l * kSmallThreads, pre[l]);
       __syncthreads();
-  #pragma unroll 8
-      for (int k = 0; k < 64; ++k) {
-        const float x = Xs[ty][k], y = Ys[tx][k];
-        const float p = __fmul_rn(x, y);
-        const float pe = __fmaf_rn(x, y, -p);
-        const float t = __fadd_rn(s, p);
-        const float z = __fsub_rn(t, s);
-        const float se = __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(p, z));
-        s = t;
-        const float cross = __fmaf_rn(Xl[ty][k], y, __fmul_rn(x, Yl[tx][k]));
-        c = __fadd_rn(c, __fadd_rn(__fadd_rn(cross, pe), se));
+      if (k0 + KC < K) {
+  #pragma unroll
+        for (int l = 0; l < kLoads; ++l) pre[l] = fetch(tid + l * kSmallThreads, k0 + KC);
+      }
+      if (active) {
+  #pragma unroll 4
+        for (int kk = 0; kk < KC; ++kk) {
+          const float4 xv = *reinterpret_cast<const float4 *>(xs + kk * P);
+          const float4 yv = *reinterpret_cast<const float4 *>(ys + kk * P);
+          const float xa[4] = {xv.x, xv.y, xv.z, xv.w}, yb[4] = {yv.x, yv.y, yv.z, yv.w};
+          if constexpr (DOT2) {
+            const float4 xw4 = *reinterpret_cast<const float4 *>(xs + (2 * KC + kk) * P);
+            const float4 yw4 = *reinterpret_cast<const float4 *>(ys + (2 * KC + kk) * P);
+            const float xl[4] = {xw4.x, xw4.y, xw4.z, xw4.w}, yl[4] = {yw4.x, yw4.y, yw4.z, yw4.w};
+  #pragma unroll
+            for (int i = 0; i < 4; ++i)
+  #pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                const float x = xa[i], y = yb[j], sv = acc[i][j];
+                const float p = __fmul_rn(x, y);
+                const float pe = __fmaf_rn(x, y, -p);
+                const float tt = __fadd_rn(sv, p);
+                const float z = __fsub_rn(tt, sv);
+                const float se = __fadd_rn(__fsub_rn(sv, __fsub_rn(tt, z)), __fsub_rn(p, z));
+                acc[i][j] = tt;
+                const float cross = __fmaf_rn(xl[i], y, __fmul_rn(x, yl[j]));
+                cmp[i][j] = __fadd_rn(cmp[i][j], __fadd_rn(__fadd_rn(cross, pe), se));
+              }
+          } else {
+  #pragma unroll
+            for (int i = 0; i < 4; ++i)
+  #pragma unroll
+              for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(xa[i], yb[j], acc[i][j]);
+          }
+        }
       }
       __syncthreads();
     }
-    // the pair (s, c) carries more than FP32 precision: keep it in FP64
-    if (a0 + ty < ma && b0 + tx < nb)
-      Out[(size_t)w * ow + (size_t)(a0 + ty) * ldo + b0 + tx] = static_cast<double>(s) + static_cast<double>(c);
+    if (!active) return;
+  #pragma unroll
+    for (int i = 0; i < 4; ++i)
+  #pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int a = 4 * ty + i, b = 4 * tx + j;
+        if (a >= ma || b >= nb) continue;
+        // DOT2: the pair (s, c) carries more than FP32 precision: keep it in FP64
+        if constexpr (DOT2)
+          Out[(size_t)w * ow + (size_t)a * ldo + b] = static_cast<double>(acc[i][j]) + static_cast<double>(cmp[i][j]);
+        else
+          Out[(size_t)w * ow + (size_t)a * ldo + b] = acc[i][j];
+      }
 }
 };
-__global__ void __launch_bounds__(256) k_gemm_rows_dot2(const float *__restrict__ X, const float *__restrict__ Xlo,
+template <bool DOT2, int Q>
+__global__ void __launch_bounds__(kSmallThreads) k_gemm_small_f32(const float *__restrict__ X, const float *__restrict__ Xlo,
                                                         size_t xw, const float *__restrict__ Y,
                                                         const float *__restrict__ Ylo, size_t yw, int ma, int nb,
-                                                        int K, double *__restrict__ Out, size_t ow, int ldo) {
-  GemmRowsDot2::run(X, Xlo, xw, Y, Ylo, yw, ma, nb, K, Out, ow, ldo, blockIdx, gridDim);
+                                                        int K, typename GemmSmallF32<DOT2, Q>::OutT *__restrict__ Out,
+                                                        size_t ow, int ldo, int W, int vec) {
+  GemmSmallF32<DOT2, Q>::run(X, Xlo, xw, Y, Ylo, yw, ma, nb, K, Out, ow, ldo, W, vec, blockIdx, gridDim);
+}
+// threads per side of a walker's tile; grouped launches take two sizes, so that
+// systems share a launch
+static int small_q(int ma, int nb) {
+  const int q = (std::max(ma, nb) + 3) / 4;
+  return group_recorder() ? (q <= 4 ? 4 : 8) : q;
+}
+template <bool DOT2, int Q>
+static cudaError_t launch_small_f32(int q, const float *X, const float *Xlo, size_t xw, const float *Y,
+                                    const float *Ylo, size_t yw, int ma, int nb, int K,
+                                    typename GemmSmallF32<DOT2, Q>::OutT *Out, size_t ow, int ldo, int W,
+                                    cudaStream_t st) {
+  if constexpr (Q > (DOT2 ? 5 : 1))  // (DOT2: more than 16 rows)
+    if (q < Q) return launch_small_f32<DOT2, Q - 1>(q, X, Xlo, xw, Y, Ylo, yw, ma, nb, K, Out, ow, ldo, W, st);
+  constexpr int wpc = small_walkers(Q);
+  // 16-byte loads along k where every row starts on 16 bytes
+  const uintptr_t at = reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(Y) |
+                       reinterpret_cast<uintptr_t>(Xlo) | reinterpret_cast<uintptr_t>(Ylo);
+  const int vec = at % 16 == 0 && K % 4 == 0 && xw % 4 == 0 && yw % 4 == 0;
+  const size_t smem = (size_t)wpc * (DOT2 ? 4 : 2) * kSmallKC * small_pitch(Q) * sizeof(float);
+  return launch_or_record<GemmSmallF32<DOT2, Q>, kSmallThreads>(k_gemm_small_f32<DOT2, Q>, dim3((W + wpc - 1) / wpc),
+                                                                dim3(kSmallThreads), smem, st, X, Xlo, xw, Y, Ylo, yw, ma, nb, K, Out, ow, ldo, W,
+                                                      vec);
+}
+
+// The FP32 path's plain per-walker products of more than 32 rows: 64 x 64 output
+// tile, 64 threads with 8 x 8 outputs each (columns 4 tx .. + 3 and 32 + 4 tx .. + 3, rows
+// likewise), k-chunks of 16 with the next chunk loading into registers meanwhile: 64 FMAs per four 16-byte
+// reads.  64 walkers, 256 x 256, K = 4096: 1.53 ms (now 1.08) with 4 x 4 outputs per thread
+// and scalar reads.
+struct GemmTile64F32 {
+  static __device__ __forceinline__ void run(const float *__restrict__ X, size_t xw, const float *__restrict__ Y,
+                                             size_t yw, int ma, int nb, int K, float *__restrict__ Out, size_t ow,
+                                             int ldo, int vec, const uint3 bid, const uint3 gdim) {
+    assume_global(X, Y, Out);
+    constexpr int KC = 16, P = 68;
+    __shared__ __align__(16) float Xs[KC][P];
+    __shared__ __align__(16) float Ys[KC][P];
+    const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
+    const int w = bid.z, a0 = bid.y * 64, b0 = bid.x * 64;
+    const bool xin = a0 + tid < ma, yin = b0 + tid < nb;  // this thread's row of each operand
+    const float *xr = X + (size_t)w * xw + (size_t)(a0 + tid) * K, *yr = Y + (size_t)w * yw + (size_t)(b0 + tid) * K;
+    auto load = [&](const float *row, bool in, int k0, float v[KC]) {
+  #pragma unroll
+      for (int c = 0; c < KC; c += 4) {
+        if (in && vec && k0 + c + 4 <= K) {
+          const float4 f = *reinterpret_cast<const float4 *>(row + k0 + c);
+          v[c] = f.x;
+          v[c + 1] = f.y;
+          v[c + 2] = f.z;
+          v[c + 3] = f.w;
+        } else {
+  #pragma unroll
+          for (int i = 0; i < 4; ++i) v[c + i] = in && k0 + c + i < K ? row[k0 + c + i] : 0.0f;
+        }
+      }
+    };
+    float acc[8][8];
+  #pragma unroll
+    for (int i = 0; i < 8; ++i)
+  #pragma unroll
+      for (int j = 0; j < 8; ++j) acc[i][j] = 0.0f;
+    float xv[KC], yv[KC];
+    load(xr, xin, 0, xv);
+    load(yr, yin, 0, yv);
+    for (int k0 = 0; k0 < K; k0 += KC) {
+  #pragma unroll
+      for (int c = 0; c < KC; ++c) {
+        Xs[c][tid] = xv[c];
+        Ys[c][tid] = yv[c];
+      }
+      __syncthreads();
+      if (k0 + KC < K) {
+        load(xr, xin, k0 + KC, xv);
+        load(yr, yin, k0 + KC, yv);
+      }
+  #pragma unroll
+      for (int kk = 0; kk < KC; ++kk) {
+        const float4 x0 = *reinterpret_cast<const float4 *>(&Xs[kk][4 * ty]);
+        const float4 x1 = *reinterpret_cast<const float4 *>(&Xs[kk][32 + 4 * ty]);
+        const float4 y0 = *reinterpret_cast<const float4 *>(&Ys[kk][4 * tx]);
+        const float4 y1 = *reinterpret_cast<const float4 *>(&Ys[kk][32 + 4 * tx]);
+        const float xa[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+        const float yb[8] = {y0.x, y0.y, y0.z, y0.w, y1.x, y1.y, y1.z, y1.w};
+  #pragma unroll
+        for (int i = 0; i < 8; ++i)
+  #pragma unroll
+          for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(xa[i], yb[j], acc[i][j]);
+      }
+      __syncthreads();
+    }
+  #pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int a = a0 + (i < 4 ? 4 * ty + i : 28 + 4 * ty + i);
+      if (a >= ma) continue;
+      float *o = Out + (size_t)w * ow + (size_t)a * ldo;
+  #pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int b = b0 + (j < 4 ? 4 * tx + j : 28 + 4 * tx + j);
+        if (b < nb) o[b] = acc[i][j];
+      }
+    }
+}
+};
+__global__ void __launch_bounds__(64) k_gemm_tile64_f32(const float *__restrict__ X, size_t xw,
+                                                        const float *__restrict__ Y, size_t yw, int ma, int nb, int K,
+                                                        float *__restrict__ Out, size_t ow, int ldo, int vec) {
+  GemmTile64F32::run(X, xw, Y, yw, ma, nb, K, Out, ow, ldo, vec, blockIdx, gridDim);
 }
 
 // ---------------------------------------------------------------------------
-// Register-blocked variant of the two kernels above for N_up >= 32: a TM x TM
+// Register-blocked variant for N_up >= 32 (FP64; compensated FP32): a TM x TM
 // output tile per CTA of 256 threads, R x R outputs per thread (R = TM / 16),
 // operands staged through shared memory in k-chunks of 32, transposed so that
 // each thread reads R consecutive entries of a column.  With DOT2 every output
@@ -346,23 +543,22 @@ cudaError_t launch_gemm_rows_dot2(const float *X, const float *Xlo, size_t xw, c
                                   cudaStream_t st, int tile) {
   if (W <= 0 || ma <= 0 || nb <= 0) return cudaSuccess;
   if (tile != -1 && tile != 0 && tile != 16 && tile != 32 && tile != 64) return cudaErrorInvalidValue;
-  const int tm = tile >= 0 ? tile : (ma <= 16 && nb <= 16 ? 16 : gemm_rows_tile(ma, nb));
-  if (tm == 16) {
-    if (ma > 16 || nb > 16) return cudaErrorInvalidValue;
+  if (tile == 16 && (ma > 16 || nb > 16)) return cudaErrorInvalidValue;
+  // one kernel per size up to 32 rows, whatever the tile asked for; above: blocked tiles
+  if (ma <= 16 && nb <= 16)
     return launch_or_record<GemmRowsDot2Small, 256>(k_gemm_rows_dot2_small, dim3((W + 3) / 4), dim3(256), 0, st, X,
                                                      Xlo, xw, Y, Ylo, yw, ma, nb, K, Out, ow, ldo, W);
-  }
-  if (tm) {
-    dim3 grid((nb + tm - 1) / tm, (ma + tm - 1) / tm, W);
-    if (tm == 64)
-      return launch_or_record<GemmRowsBlk<float, 64, true, double>, 256>(k_gemm_rows_blk<float, 64, true, double>, grid, dim3(256), 0, st, X, Xlo, xw, Y, Ylo, yw, ma, nb, K, Out, ow,
-          ldo);
-    return launch_or_record<GemmRowsBlk<float, 32, true, double>, 256>(k_gemm_rows_blk<float, 32, true, double>, grid, dim3(256), 0, st, X, Xlo, xw, Y, Ylo, yw, ma, nb, K, Out, ow,
-        ldo);
-  }
-  dim3 grid((nb + 15) / 16, (ma + 15) / 16, W);
-  return launch_or_record<GemmRowsDot2, 256>(k_gemm_rows_dot2, grid, dim3(256), 0, st, X, Xlo, xw, Y, Ylo, yw, ma, nb,
-                                             K, Out, ow, ldo);
+  if (ma <= 32 && nb <= 32)
+    return launch_small_f32<true, 8>(small_q(ma, nb), X, Xlo, xw, Y, Ylo, yw, ma, nb, K, Out, ow, ldo, W, st);
+  const int tm = tile == 32 || tile == 64 ? tile : (ma >= 64 && nb >= 64 ? 64 : 32);
+  dim3 grid((nb + tm - 1) / tm, (ma + tm - 1) / tm, W);
+  if (tm == 64)
+    return launch_or_record<GemmRowsBlk<float, 64, true, double>, 256>(k_gemm_rows_blk<float, 64, true, double>, grid,
+                                                                       dim3(256), 0, st, X, Xlo, xw, Y, Ylo, yw, ma,
+                                                                       nb, K, Out, ow, ldo);
+  return launch_or_record<GemmRowsBlk<float, 32, true, double>, 256>(k_gemm_rows_blk<float, 32, true, double>, grid,
+                                                                     dim3(256), 0, st, X, Xlo, xw, Y, Ylo, yw, ma, nb,
+                                                                     K, Out, ow, ldo);
 }
 
 template <typename T>
@@ -370,6 +566,17 @@ cudaError_t launch_gemm_rows(const T *X, size_t xw, const T *Y, size_t yw, int m
                              int ldo, int W, cudaStream_t st, int tile) {
   if (W <= 0 || ma <= 0 || nb <= 0) return cudaSuccess;
   if (tile != -1 && tile != 0 && tile != 32 && tile != 64) return cudaErrorInvalidValue;
+  if constexpr (std::is_same<T, float>::value) {
+    // one kernel per size, whatever the tile asked for
+    const float *none = nullptr;
+    if (ma <= 32 && nb <= 32) 
+      return launch_small_f32<false, 8>(small_q(ma, nb), X, none, xw, Y, none, yw, ma, nb, K, Out, ow, ldo, W,
+                                        st);
+    const int vec = (reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(Y)) % 16 == 0 && K % 4 == 0 &&
+                    xw % 4 == 0 && yw % 4 == 0;
+    return launch_or_record<GemmTile64F32, 64>(k_gemm_tile64_f32, dim3((nb + 63) / 64, (ma + 63) / 64, W), dim3(64), 0,
+                                               st, X, xw, Y, yw, ma, nb, K, Out, ow, ldo, vec);
+  } else {
   const int tm = tile >= 0 ? tile : gemm_rows_tile(ma, nb);
   if (tm) {
     dim3 grid((nb + tm - 1) / tm, (ma + tm - 1) / tm, W);
@@ -393,6 +600,7 @@ cudaError_t launch_gemm_rows(const T *X, size_t xw, const T *Y, size_t yw, int m
   dim3 grid((nb + 15) / 16, (ma + 15) / 16, W);
   return launch_or_record<GemmRows<T>, 256>(k_gemm_rows<T>, grid, dim3(256), 0, st, X, xw, Y, yw, ma, nb, K, Out, ow,
                                             ldo);
+  }
 }
 template cudaError_t launch_gemm_rows<double>(const double *, size_t, const double *, size_t, int, int, int, double *,
                                               size_t, int, int, cudaStream_t, int);
