@@ -634,7 +634,7 @@ static jagp_status_t jagp_grad_impl(jagp_handle_t h, const double *d_r, void *d_
   if (s != JAGP_OK) return s;
   LAUNCH(0, 1,
          launch_adj_positions(d, d_r, d_seed_eL, wp(G.jg), at<double>(d_state, L.mbuf), wp(G.phibar_a),
-                              wp(G.phibar_b), wp(G.phibar_dn), d.shell_atom, wp(G.rbar), wp(G.part), W, st));
+                              wp(G.phibar_b), wp(G.phibar_dn), wp(G.rbar), wp(G.part), W, st));
   LAUNCH(0, 1,
          launch_adj_jastrow(d, d_r, d_seed_logpsi, d_seed_eL, wp(G.jg), at<double>(d_state, L.kin), wp(G.rbar),
                             wp(G.rbar_at), wp(G.jpar), W, st));
@@ -749,6 +749,14 @@ jagp_status_t jagp_create(jagp_handle_t *out, const jagp_system_t *sys, const ja
         satom.push_back(a);
       }
   const int na = sys->n_atoms, k_unp = sys->n_up - sys->n_dn;
+  // the shell table's positions atom by atom
+  std::vector<int> afirst(na + 1, 0), ashell(sys->n_shells);
+  for (int a : satom) ++afirst[a + 1];
+  for (int a = 0; a < na; ++a) afirst[a + 1] += afirst[a];
+  {
+    std::vector<int> next(afirst.begin(), afirst.end() - 1);
+    for (int k = 0; k < sys->n_shells; ++k) ashell[next[satom[k]]++] = k;
+  }
   std::vector<double> c1(na), lamT((size_t)L * L);
   double vii = 0.0;
   for (int a = 0; a < na; ++a) {
@@ -815,7 +823,7 @@ jagp_status_t jagp_create(jagp_handle_t *out, const jagp_system_t *sys, const ja
   const size_t oR = take(na * 3 * 8), oZ = take(na * 8), oC = take(na * 8);
   const size_t oG = take(sys->n_shells * sizeof(double4)), oI = take(sys->n_shells * sizeof(int));
   const size_t oGd = take(sys->n_shells * 2 * sizeof(float4));
-  const size_t oSa = take(sys->n_shells * sizeof(int));
+  const size_t oSa = take(sys->n_shells * sizeof(int)), oSf = take((na + 1) * sizeof(int));
   const size_t oAf = take(na * sizeof(float4));
   const size_t oL = take((size_t)L * L * 8), oT = take((size_t)L * L * 8);
   const size_t oU = take((size_t)(k_unp > 0 ? k_unp : 1) * L * 8);
@@ -875,7 +883,8 @@ jagp_status_t jagp_create(jagp_handle_t *out, const jagp_system_t *sys, const ja
             cudaMemcpy(b + oGd, geo_dw.data(), sys->n_shells * 2 * sizeof(float4), cudaMemcpyHostToDevice) ==
                 cudaSuccess &&
             cudaMemcpy(b + oI, info.data(), sys->n_shells * sizeof(int), cudaMemcpyHostToDevice) == cudaSuccess &&
-            cudaMemcpy(b + oSa, satom.data(), sys->n_shells * sizeof(int), cudaMemcpyHostToDevice) == cudaSuccess &&
+            cudaMemcpy(b + oSa, ashell.data(), sys->n_shells * sizeof(int), cudaMemcpyHostToDevice) == cudaSuccess &&
+            cudaMemcpy(b + oSf, afirst.data(), (na + 1) * sizeof(int), cudaMemcpyHostToDevice) == cudaSuccess &&
             cudaMemcpy(b + oAf, atom_f.data(), na * sizeof(float4), cudaMemcpyHostToDevice) == cudaSuccess &&
             cudaMemcpy(b + oL, sys->lambda, (size_t)L * L * 8, cudaMemcpyHostToDevice) == cudaSuccess &&
             cudaMemcpy(b + oT, lamT.data(), (size_t)L * L * 8, cudaMemcpyHostToDevice) == cudaSuccess &&
@@ -911,7 +920,8 @@ jagp_status_t jagp_create(jagp_handle_t *out, const jagp_system_t *sys, const ja
   d.shell_geo = reinterpret_cast<const double4 *>(b + oG);
   d.shell_dw = reinterpret_cast<const float4 *>(b + oGd);
   d.shell_info = reinterpret_cast<const int *>(b + oI);
-  d.shell_atom = reinterpret_cast<const int *>(b + oSa);
+  d.atom_shells = reinterpret_cast<const int *>(b + oSa);
+  d.atom_first = reinterpret_cast<const int *>(b + oSf);
   d.lam = reinterpret_cast<const double *>(b + oL);
   d.lamT = reinterpret_cast<const double *>(b + oT);
   d.unpaired = reinterpret_cast<const double *>(b + oU);

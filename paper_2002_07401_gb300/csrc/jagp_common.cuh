@@ -40,7 +40,8 @@ struct DevSystem {
   const double4 *shell_geo; // [n_shells]
   const float4 *shell_dw;   // [n_shells][2]: (x, y, z, zeta) rounded to FP32, then the remainders
   const int *shell_info;    // [n_shells]
-  const int *shell_atom;    // [n_shells] owning atom, in the same (evaluation) order
+  // an atom's shells as positions in the shell table: atom_shells[atom_first[a]] .. [atom_first[a + 1] - 1]
+  const int *atom_first, *atom_shells;
   const double *lam;        // [L][L]
   const double *lamT;       // [L][L] = lambda^T
   const double *unpaired;   // [n_up - n_dn][L]

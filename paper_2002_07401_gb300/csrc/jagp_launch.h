@@ -178,7 +178,7 @@ cudaError_t launch_adj_rows_gemm(const DevSystem &s, const double *ginv, double 
 int adj_position_parts(const DevSystem &s);
 cudaError_t launch_adj_positions(const DevSystem &s, const double *r, const double *sE, const double *jg,
                                  const double *mbuf, const double *phibar_a, const double *phibar_b,
-                                 const double *phibar_dn, const int *shell_atom, double *rbar, double *part, int W,
+                                 const double *phibar_dn, double *rbar, double *part, int W,
                                  cudaStream_t st);
 cudaError_t launch_adj_jastrow(const DevSystem &s, const double *r, const double *sL, const double *sE,
                                const double *jg, const double *kin, double *rbar, double *rbar_at, double *jpar, int W,

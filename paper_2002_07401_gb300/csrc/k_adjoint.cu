@@ -24,112 +24,113 @@
 namespace jagp {
 
 // ---------------------------------------------------------------------------
-// orbital values, gradients, Hessians (xx, yy, zz, xy, yz, zx) and gradients
-// of the Laplacian of one shell at displacement d (FP64)
+// The angular polynomials P_c of a shell are harmonic and homogeneous of degree
+// l, so sums over its components need only their coefficients' polynomial and
+// its derivatives.  For S = sum_c m_c P_c: value, gradient, and (with b) the
+// product of its constant Hessian with a vector.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ int shell_third(int info, double zeta, double dx, double dy, double dz, double val[5],
-                                           double grad[5][3], double hess[5][6], double glap[5][3]) {
-  const int l = shell_l(info);
-  const double d[3] = {dx, dy, dz};
-  const double r2 = dx * dx + dy * dy + dz * dz;
-  double g, gg[3], Hg[3][3], lapg, glg[3];
-  if (shell_rad(info)) {
-    const double r = sqrt(r2);
-    g = exp(-zeta * r);
-    for (int a = 0; a < 3; ++a) gg[a] = -zeta * d[a] / r * g;
-    for (int a = 0; a < 3; ++a)
-      for (int b = 0; b < 3; ++b)
-        Hg[a][b] = (zeta * zeta * d[a] * d[b] / r2 + zeta * d[a] * d[b] / (r2 * r) - (a == b ? zeta / r : 0.0)) * g;
-    lapg = (zeta * zeta - 2.0 * zeta / r) * g;
-    const double q = (2.0 * zeta / (r2 * r) - zeta * (zeta * zeta - 2.0 * zeta / r) / r) * g;
-    for (int a = 0; a < 3; ++a) glg[a] = q * d[a];
+struct ShellPoly {
+  double v, g[3];
+};
+__device__ __forceinline__ ShellPoly shell_poly(int l, const double m[5], double x, double y, double z) {
+  ShellPoly s;
+  if (l == 0) {
+    s.v = m[0];
+    s.g[0] = s.g[1] = s.g[2] = 0.0;
+  } else if (l == 1) {
+    s.g[0] = m[0];
+    s.g[1] = m[1];
+    s.g[2] = m[2];
+    s.v = m[0] * x + m[1] * y + m[2] * z;
   } else {
-    g = exp(-zeta * r2);
-    for (int a = 0; a < 3; ++a) gg[a] = -2.0 * zeta * d[a] * g;
-    for (int a = 0; a < 3; ++a)
-      for (int b = 0; b < 3; ++b) Hg[a][b] = (4.0 * zeta * zeta * d[a] * d[b] - (a == b ? 2.0 * zeta : 0.0)) * g;
-    lapg = (4.0 * zeta * zeta * r2 - 6.0 * zeta) * g;
-    const double q = (8.0 * zeta * zeta - 2.0 * zeta * (4.0 * zeta * zeta * r2 - 6.0 * zeta)) * g;
-    for (int a = 0; a < 3; ++a) glg[a] = q * d[a];
+    // xy, yz, zx, x^2 - y^2, 2 z^2 - x^2 - y^2; S = (x S_x + y S_y + z S_z) / 2
+    s.g[0] = m[0] * y + m[2] * z + 2.0 * (m[3] - m[4]) * x;
+    s.g[1] = m[0] * x + m[1] * z - 2.0 * (m[3] + m[4]) * y;
+    s.g[2] = m[1] * y + m[2] * x + 4.0 * m[4] * z;
+    s.v = 0.5 * (s.g[0] * x + s.g[1] * y + s.g[2] * z);
   }
-  const int nc = 2 * l + 1;
-  for (int c = 0; c < nc; ++c) {
-    double P, gP[3] = {0.0, 0.0, 0.0}, HP[3][3] = {{0.0, 0.0, 0.0}, {0.0, 0.0, 0.0}, {0.0, 0.0, 0.0}};
-    if (l == 0) {
-      P = 1.0;
-    } else if (l == 1) {
-      P = d[c];
-      gP[c] = 1.0;
-    } else if (c == 0) {
-      P = dx * dy; gP[0] = dy; gP[1] = dx; HP[0][1] = HP[1][0] = 1.0;
-    } else if (c == 1) {
-      P = dy * dz; gP[1] = dz; gP[2] = dy; HP[1][2] = HP[2][1] = 1.0;
-    } else if (c == 2) {
-      P = dz * dx; gP[0] = dz; gP[2] = dx; HP[0][2] = HP[2][0] = 1.0;
-    } else if (c == 3) {
-      P = dx * dx - dy * dy; gP[0] = 2.0 * dx; gP[1] = -2.0 * dy; HP[0][0] = 2.0; HP[1][1] = -2.0;
-    } else {
-      P = 3.0 * dz * dz - r2; gP[0] = -2.0 * dx; gP[1] = -2.0 * dy; gP[2] = 4.0 * dz;
-      HP[0][0] = -2.0; HP[1][1] = -2.0; HP[2][2] = 4.0;
-    }
-    val[c] = P * g;
-    for (int q = 0; q < 3; ++q) grad[c][q] = gP[q] * g + P * gg[q];
-    const int pa[6] = {0, 1, 2, 0, 1, 2}, pb[6] = {0, 1, 2, 1, 2, 0};
-    for (int k = 0; k < 6; ++k) {
-      const int a = pa[k], b = pb[k];
-      hess[c][k] = HP[a][b] * g + gP[a] * gg[b] + gP[b] * gg[a] + P * Hg[a][b];
-    }
-    for (int q = 0; q < 3; ++q) {
-      double t = 0.0;
-      for (int p = 0; p < 3; ++p) t += HP[q][p] * gg[p] + gP[p] * Hg[q][p];
-      glap[c][q] = 2.0 * t + gP[q] * lapg + P * glg[q];
-    }
+  return s;
+}
+
+// Radial factor g (e^{-zeta r^2} or e^{-zeta r}) through what its derivatives need:
+// grad g = -al g d, lap(P g) = P g h for degree l, grad h = et d, and be with
+// grad al = -be d (0 for a Gaussian).
+struct Radial {
+  double g, al, h, et, be;
+};
+__device__ __forceinline__ Radial radial_parts(int rad, int l, double zeta, double r2) {
+  Radial p;
+  if (rad) {
+    const double ri = rsqrt(r2), r = r2 * ri, zr = zeta * ri, zr3 = zr * ri * ri;
+    p.g = exp(-zeta * r);
+    p.al = zr;
+    p.h = zeta * zeta - 2.0 * (l + 1) * zr;
+    p.et = 2.0 * (l + 1) * zr3;
+    p.be = zr3;
+  } else {
+    p.g = exp(-zeta * r2);
+    p.al = 2.0 * zeta;
+    p.h = 4.0 * zeta * zeta * r2 - (4 * l + 6) * zeta;
+    p.et = 8.0 * zeta * zeta;
+    p.be = 0.0;
   }
-  return nc;
+  return p;
 }
 
 // ---------------------------------------------------------------------------
-// Jastrow derivatives of one radial function F(r), r = |d|: F', F'', F''' .
+// Jastrow derivatives of one radial function F(r), r = |d|: the first three.
 // J1 term of an atom: F = -c^3 u(c r), u = (1 - e^{-b s}) / (2b);
 // J2 pair term: F = r / (k (1 + b r)).
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void j1_d3(double c, double b, double r, double *f1, double *f2, double *f3) {
-  const double c4 = c * c * c * c;
+// (and dF/db of the J1 term)
+__device__ __forceinline__ void j1_d3(double c, double b, double r, double *f1, double *f2, double *f3, double *fb) {
+  const double c3 = c * c * c, c4 = c3 * c, s = c * r;
   if (b == 0.0) {
     *f1 = -0.5 * c4;
     *f2 = 0.0;
     *f3 = 0.0;
+    *fb = 0.25 * c3 * s * s;
     return;
   }
-  const double e = exp(-b * c * r);
+  const double e = exp(-b * s), ib = 0.5 / b;
   *f1 = -0.5 * c4 * e;
-  *f2 = 0.5 * c4 * c * b * e;
-  *f3 = -0.5 * c4 * c * c * b * b * e;
+  *f2 = -c * b * *f1;
+  *f3 = -c * b * *f2;
+  *fb = -c3 * ib * (s * e - (1.0 - e) * 2.0 * ib);
 }
-__device__ __forceinline__ void j2_d3(double k, double b, double r, double *v1, double *v2, double *v3) {
-  const double q = 1.0 + b * r;
-  *v1 = 1.0 / (k * q * q);
-  *v2 = -2.0 * b / (k * q * q * q);
-  *v3 = 6.0 * b * b / (k * q * q * q * q);
+__device__ __forceinline__ void j2_d3(double ik, double b, double iq, double *v1, double *v2, double *v3) {
+  *v1 = ik * iq * iq;  // iq = 1 / (1 + b r), ik = 1 / k
+  const double t = b * iq;
+  *v2 = -2.0 * t * *v1;
+  *v3 = -3.0 * t * *v2;
 }
 
-// gradient F' dhat, Hessian-vector product H v, and gradient of the Laplacian
-// (F''' + 2F''/r - 2F'/r^2) dhat of F(|d|)
-__device__ __forceinline__ void radial_adj(double f1, double f2, double f3, const double d[3], double r,
-                                           const double v[3], double hv[3], double glap[3]) {
-  const double dh[3] = {d[0] / r, d[1] / r, d[2] / r};
-  const double dv = dh[0] * v[0] + dh[1] * v[1] + dh[2] * v[2];
-  const double gl = f3 + 2.0 * f2 / r - 2.0 * f1 / (r * r);
-  for (int q = 0; q < 3; ++q) {
-    hv[q] = f2 * dh[q] * dv + (f1 / r) * (v[q] - dh[q] * dv);
-    glap[q] = gl * dh[q];
-  }
+// Hessian-vector product H v and gradient of the Laplacian, gl d with gl =
+// (f3 + 2 f2/r - 2 f1/r^2) / r, of F(|d|); ri = 1/r
+__device__ __forceinline__ void radial_adj(double f1, double f2, double f3, const double d[3], double ri,
+                                           const double v[3], double hv[3], double *gl) {
+  const double f1r = f1 * ri, dv = (d[0] * v[0] + d[1] * v[1] + d[2] * v[2]) * ri * ri, q = (f2 - f1r) * dv;
+  for (int k = 0; k < 3; ++k) hv[k] = q * d[k] + f1r * v[k];
+  *gl = (f3 + 2.0 * (f2 - f1r) * ri) * ri;
+}
+
+// lanes per group of a warp that takes n items at a time: the power of two >= n, at most 32
+__host__ __device__ inline int group_lanes(int n) {
+  int g = 1;
+  while (g < n && g < 32) g *= 2;
+  return g;
+}
+__device__ __forceinline__ double group_sum(double v, int g) {
+  for (int o = g / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
 }
 
 // ---------------------------------------------------------------------------
 // 1. Jastrow gradient at every electron and the kinetic adjoint vectors
 //    Mbar_e = sE (-1/2 lap phi - grad phi . grad J_e); also the orbital values
-//    at the down electrons (rows of dnphi).  One warp per electron.
+//    at the down electrons (rows of dnphi).  One warp per electron.  Bound by the
+//    FP64 pipe: per component P (-h/2 + al b.d) - grad P . b, b = grad J, times g
+//    (1000 walkers of 16 He: 0.53 ms; 0.85 with each component's full gradient and Laplacian).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_adj_kvec(DevSystem s, const double *__restrict__ r,
                                                   const double *__restrict__ sE, double *__restrict__ jg,
@@ -153,25 +154,23 @@ __global__ void __launch_bounds__(256) k_adj_kvec(DevSystem s, const double *__r
     if (s.use_j1)
       for (int a = lane; a < s.n_atoms; a += 32) {
         const double dx = ex - s.R[3 * a], dy = ey - s.R[3 * a + 1], dz = ez - s.R[3 * a + 2];
-        const double rr = sqrt(dx * dx + dy * dy + dz * dz);
-        double fp, fpp;
-        j1_d(s.c1[a], s.b_ea, rr, &fp, &fpp);
-        gx += fp * dx / rr;
-        gy += fp * dy / rr;
-        gz += fp * dz / rr;
+        const double r2 = dx * dx + dy * dy + dz * dz, ri = rsqrt(r2), c = s.c1[a], c4 = c * c * c * c;
+        const double fp = -0.5 * c4 * (s.b_ea == 0.0 ? 1.0 : exp(-s.b_ea * c * r2 * ri)) * ri;
+        gx += fp * dx;
+        gy += fp * dy;
+        gz += fp * dz;
       }
     if (s.use_j2)
       for (int k = lane; k < s.N; k += 32) {
         if (k == e) continue;
         const double dx = ex - xw[3 * k], dy = ey - xw[3 * k + 1], dz = ez - xw[3 * k + 2];
-        const double rr = sqrt(dx * dx + dy * dy + dz * dz);
+        const double r2 = dx * dx + dy * dy + dz * dz, ri = rsqrt(r2);
         double kk, bb;
         j2_params(s, (e < s.n_up) == (k < s.n_up), &kk, &bb);
-        const double q1 = 1.0 + bb * rr;
-        const double vp = 1.0 / (kk * q1 * q1);
-        gx += vp * dx / rr;
-        gy += vp * dy / rr;
-        gz += vp * dz / rr;
+        const double iq = 1.0 / (1.0 + bb * r2 * ri), vp = (kk == 4.0 ? 0.25 : 0.5) * iq * iq * ri;
+        gx += vp * dx;
+        gy += vp * dy;
+        gz += vp * dz;
       }
     gx = warp_sum(gx);
     gy = warp_sum(gy);
@@ -185,14 +184,33 @@ __global__ void __launch_bounds__(256) k_adj_kvec(DevSystem s, const double *__r
     double *kb = kbar + pt * s.L;
     double *dp = (e >= s.n_up) ? dnphi + ((size_t)w * s.n_up + (e - s.n_up)) * s.L : nullptr;
     for (int k = lane; k < s.n_shells; k += 32) {
-      const double4 g = sh_geo[k];
-      const int info = sh_info[k];
-      double o[5][5];
-      const int nc = shell_derivs(info, g.w, ex - g.x, ey - g.y, ez - g.z, o);
-      const int off = shell_off(info);
-      for (int c = 0; c < nc; ++c) {
-        kb[off + c] = se * (-0.5 * o[c][4] - (o[c][1] * gx + o[c][2] * gy + o[c][3] * gz));
-        if (dp) dp[off + c] = o[c][0];
+      const double4 G = sh_geo[k];
+      const int info = sh_info[k], l = shell_l(info), off = shell_off(info);
+      const double x = ex - G.x, y = ey - G.y, z = ez - G.z, r2 = x * x + y * y + z * z;
+      const Radial p = radial_parts(shell_rad(info), l, G.w, r2);
+      const double t = p.al * (gx * x + gy * y + gz * z) - 0.5 * p.h, sg = se * p.g;
+      if (l == 0) {
+        kb[off] = sg * t;
+        if (dp) dp[off] = p.g;
+      } else if (l == 1) {
+        kb[off] = sg * (x * t - gx);
+        kb[off + 1] = sg * (y * t - gy);
+        kb[off + 2] = sg * (z * t - gz);
+        if (dp) {
+          dp[off] = x * p.g;
+          dp[off + 1] = y * p.g;
+          dp[off + 2] = z * p.g;
+        }
+      } else {
+        const double P[5] = {x * y, y * z, z * x, x * x - y * y, 3.0 * z * z - r2};
+        const double xg = x * gx, yg = y * gy;
+        const double D[5] = {y * gx + x * gy, z * gy + y * gz, x * gz + z * gx, 2.0 * (xg - yg),
+                             4.0 * z * gz - 2.0 * (xg + yg)};
+#pragma unroll
+        for (int c = 0; c < 5; ++c) {
+          kb[off + c] = sg * (P[c] * t - D[c]);
+          if (dp) dp[off + c] = P[c] * p.g;
+        }
       }
     }
   }
@@ -276,185 +294,245 @@ __global__ void __launch_bounds__(256) k_adj_rows(DevSystem s, const double *__r
 }
 
 // ---------------------------------------------------------------------------
-// 4. orbital tables -> positions.  One warp per electron e; per orbital mu:
-//    c = phibar_mu grad phi_mu + M_mu (Hess phi_mu) gbarD + lbarD M_mu grad(lap phi_mu)
-//    with gbarD = -sE grad J_e, lbarD = -sE / 2; rbar_e += c, Rbar_atom(mu) -= c.
-//    The per-atom sums of the CTA's electrons go to part[w][blockIdx.x][atom].
+// 4. orbital tables -> positions.  Per shell at displacement d, with b =
+//    -sE grad J_e, lb = -sE / 2, Q = sum_c phibar_c P_c and S = sum_c M_c P_c,
+//      grad(Q g) + Hess(S g) b + lb grad(lap(S g))
+//        = g [grad Q + (Hess S) b + (lb h - al b.d) grad S - al S b + ka d],
+//      ka = -al (Q + u) + be S b.d + lb S (et - al h),  u = b.grad S - al S b.d
+//    goes to the electron and, negated, to the shell's atom.  A lane takes an
+//    atom and all its shells (lanes in groups of the next power of two, so that
+//    a few atoms leave room for several electrons per warp), so the atoms' sums
+//    stay in registers: per-component third derivatives with FP64 atomics in
+//    shared memory took 2.2 ms for 1000 walkers of 16 He, these 0.58.  A CTA takes kAdjElectrons
+//    electrons of one walker; its per-atom sums go to part[w][blockIdx.x][atom].
 // ---------------------------------------------------------------------------
 constexpr int kAdjWarps = 8;
+constexpr int kAdjElectrons = 32;
 
 __global__ void __launch_bounds__(kAdjWarps * 32) k_adj_positions(
     DevSystem s, const double *__restrict__ r, const double *__restrict__ sE, const double *__restrict__ jg,
     const double *__restrict__ mbuf, const double *__restrict__ phibar_a, const double *__restrict__ phibar_b,
-    const double *__restrict__ phibar_dn, const int *__restrict__ shell_atom, double *__restrict__ rbar,
-    double *__restrict__ part) {
-  extern __shared__ double sm[];
-  double *Rb = sm;                                           // n_atoms * 3
-  int *s_atom = reinterpret_cast<int *>(Rb + 3 * s.n_atoms);   // n_shells
-  for (int t = threadIdx.x; t < 3 * s.n_atoms; t += blockDim.x) Rb[t] = 0.0;
-  for (int t = threadIdx.x; t < s.n_shells; t += blockDim.x) s_atom[t] = shell_atom[t];
+    const double *__restrict__ phibar_dn, double *__restrict__ rbar, double *__restrict__ part) {
+  __shared__ double s_re[kAdjElectrons][3];  // electrons' sums over the atoms so far
+  __shared__ double s_at[kAdjWarps][32][3];   // a chunk of atoms: each warp's lanes
+  const int w = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int e0 = blockIdx.x * kAdjElectrons, ne = min(kAdjElectrons, s.N - e0);
+  const int G = group_lanes(s.n_atoms), per = 32 / G;  // electrons of a warp at a time
+  const int sub = lane / G, ga = lane - sub * G;
+  const double se = sE ? sE[w] : 0.0, lb = -0.5 * se;
+  for (int t = tid; t < 3 * kAdjElectrons; t += kAdjWarps * 32) s_re[t / 3][t % 3] = 0.0;
   __syncthreads();
-  const int w = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int e = blockIdx.x * kAdjWarps + warp;
-  if (e < s.N) {
-    const size_t pt = (size_t)w * s.N + e;
-    const double ex = r[pt * 3], ey = r[pt * 3 + 1], ez = r[pt * 3 + 2];
-    const double se = sE ? sE[w] : 0.0;
-    const double gb[3] = {-se * jg[pt * 3], -se * jg[pt * 3 + 1], -se * jg[pt * 3 + 2]};
-    const double lb = -0.5 * se;
-    const double *M = mbuf + pt * s.L;
-    const bool up = e < s.n_up;
-    const double *pa = up ? phibar_a + ((size_t)w * s.n_up + e) * s.L : phibar_dn + ((size_t)w * s.n_up + e - s.n_up) * s.L;
-    const double *pb2 = up ? phibar_b + ((size_t)w * s.n_up + e) * s.L : nullptr;
-    double re[3] = {0.0, 0.0, 0.0};
-    for (int k = lane; k < s.n_shells; k += 32) {
-      const double4 g = s.shell_geo[k];
-      const int info = s.shell_info[k];
-      double val[5], grad[5][3], hs[5][6], gl[5][3];
-      const int nc = shell_third(info, g.w, ex - g.x, ey - g.y, ez - g.z, val, grad, hs, gl);
-      const int off = shell_off(info);
+  for (int a0 = 0; a0 < s.n_atoms; a0 += G) {
+    const int a = a0 + ga;
+    const int k0 = a < s.n_atoms ? s.atom_first[a] : 0, k1 = a < s.n_atoms ? s.atom_first[a + 1] : 0;
+    double ra[3] = {0.0, 0.0, 0.0};
+    const double Rx = a < s.n_atoms ? s.R[3 * a] : 0.0, Ry = a < s.n_atoms ? s.R[3 * a + 1] : 0.0,
+                 Rz = a < s.n_atoms ? s.R[3 * a + 2] : 0.0;
+    for (int q0 = warp * per; q0 < ne; q0 += kAdjWarps * per) {
+      const int q = q0 + sub, e = e0 + q;
       double c[3] = {0.0, 0.0, 0.0};
-      for (int q = 0; q < nc; ++q) {
-        const double pbar = pa[off + q] + (pb2 ? pb2[off + q] : 0.0);
-        const double m = M[off + q];
-        // Hessian (xx, yy, zz, xy, yz, zx) times gb
-        const double h0 = hs[q][0] * gb[0] + hs[q][3] * gb[1] + hs[q][5] * gb[2];
-        const double h1 = hs[q][3] * gb[0] + hs[q][1] * gb[1] + hs[q][4] * gb[2];
-        const double h2 = hs[q][5] * gb[0] + hs[q][4] * gb[1] + hs[q][2] * gb[2];
-        c[0] += pbar * grad[q][0] + m * h0 + lb * m * gl[q][0];
-        c[1] += pbar * grad[q][1] + m * h1 + lb * m * gl[q][1];
-        c[2] += pbar * grad[q][2] + m * h2 + lb * m * gl[q][2];
+      if (q < ne) {
+        const size_t pt = (size_t)w * s.N + e;
+        const double x = r[pt * 3] - Rx, y = r[pt * 3 + 1] - Ry, z = r[pt * 3 + 2] - Rz;
+        const double b[3] = {-se * jg[pt * 3], -se * jg[pt * 3 + 1], -se * jg[pt * 3 + 2]};
+        const double r2 = x * x + y * y + z * z, bd = b[0] * x + b[1] * y + b[2] * z;
+        const double *M = mbuf + pt * s.L;
+        const bool up = e < s.n_up;
+        const size_t row = (size_t)w * s.n_up + (up ? e : e - s.n_up);
+        const double *pa = (up ? phibar_a : phibar_dn) + row * s.L, *pb = up ? phibar_b + row * s.L : nullptr;
+        for (int k = k0; k < k1; ++k) {
+          const int sh = s.atom_shells[k], info = s.shell_info[sh], l = shell_l(info), off = shell_off(info);
+          double m[5], f[5];
+#pragma unroll
+          for (int i = 0; i < 5; ++i)
+            if (i < 2 * l + 1) {
+              m[i] = M[off + i];
+              f[i] = pa[off + i] + (pb ? pb[off + i] : 0.0);
+            }
+          const Radial p = radial_parts(shell_rad(info), l, s.shell_geo[sh].w, r2);
+          const ShellPoly S = shell_poly(l, m, x, y, z), Q = shell_poly(l, f, x, y, z);
+          double H[3] = {0.0, 0.0, 0.0};  // (Hess S) b
+          if (l == 2) {
+            H[0] = 2.0 * (m[3] - m[4]) * b[0] + m[0] * b[1] + m[2] * b[2];
+            H[1] = m[0] * b[0] - 2.0 * (m[3] + m[4]) * b[1] + m[1] * b[2];
+            H[2] = m[2] * b[0] + m[1] * b[1] + 4.0 * m[4] * b[2];
+          }
+          const double aS = p.al * S.v, u = b[0] * S.g[0] + b[1] * S.g[1] + b[2] * S.g[2] - aS * bd;
+          const double cs = lb * p.h - p.al * bd;
+          const double ka = S.v * (p.be * bd + lb * (p.et - p.al * p.h)) - p.al * (Q.v + u);
+          c[0] += p.g * (Q.g[0] + H[0] + cs * S.g[0] - aS * b[0] + ka * x);
+          c[1] += p.g * (Q.g[1] + H[1] + cs * S.g[1] - aS * b[1] + ka * y);
+          c[2] += p.g * (Q.g[2] + H[2] + cs * S.g[2] - aS * b[2] + ka * z);
+        }
       }
-      const int a = s_atom[k];
-      atomicAdd(&Rb[3 * a], -c[0]);
-      atomicAdd(&Rb[3 * a + 1], -c[1]);
-      atomicAdd(&Rb[3 * a + 2], -c[2]);
-      re[0] += c[0];
-      re[1] += c[1];
-      re[2] += c[2];
+#pragma unroll
+      for (int t = 0; t < 3; ++t) {
+        ra[t] -= c[t];
+        const double v = group_sum(c[t], G);
+        if (ga == 0 && q < ne) s_re[q][t] += v;  // (this warp's electrons in every chunk)
+      }
     }
-    re[0] = warp_sum(re[0]);
-    re[1] = warp_sum(re[1]);
-    re[2] = warp_sum(re[2]);
-    if (lane == 0) {
-      rbar[pt * 3] = re[0];
-      rbar[pt * 3 + 1] = re[1];
-      rbar[pt * 3 + 2] = re[2];
+    // the chunk's atoms over the CTA's electrons
+#pragma unroll
+    for (int t = 0; t < 3; ++t) s_at[warp][lane][t] = ra[t];
+    __syncthreads();
+    for (int t = tid; t < 3 * G; t += kAdjWarps * 32) {
+      const int i = t / 3, q = t - 3 * i;
+      if (a0 + i < s.n_atoms) {
+        double v = 0.0;
+        for (int ww = 0; ww < kAdjWarps; ++ww)
+          for (int h = 0; h < per; ++h) v += s_at[ww][h * G + i][q];
+        part[((size_t)w * gridDim.x + blockIdx.x) * 3 * s.n_atoms + 3 * (a0 + i) + q] = v;
+      }
     }
+    __syncthreads();
   }
-  __syncthreads();
-  double *po = part + ((size_t)w * gridDim.x + blockIdx.x) * 3 * s.n_atoms;
-  for (int t = threadIdx.x; t < 3 * s.n_atoms; t += blockDim.x) po[t] = Rb[t];
+  for (int t = tid; t < 3 * ne; t += kAdjWarps * 32) rbar[((size_t)w * s.N + e0) * 3 + t] = s_re[t / 3][t % 3];
 }
 
 // ---------------------------------------------------------------------------
 // 5. Jastrow and Coulomb adjoints, Jastrow parameter derivatives.  One CTA per
-//    walker; electrons first (their grad J adjoints in shared memory), then
-//    atoms.  rbar[e] += ..., rbar_at[w][a] = ..., jpar[w][3] = ...
+//    walker.  Electron-atom pairs: lanes on atoms (in groups, as above), a pair's
+//    terms added to its electron (over the group) and, negated, to its atom (in
+//    the lane); electron-electron pairs: a warp per electron, lanes on the others.
+//    rbar[e] += ..., rbar_at[w][a] = ..., jpar[w][3] = ...  Bound by the FP64 pipe:
+//    one reciprocal square root and one division per pair (1000 walkers of 16 He:
+//    0.31 ms; 1.05 with a thread per electron and atomics for the atoms).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(128) k_adj_jastrow(DevSystem s, const double *__restrict__ r,
-                                                     const double *__restrict__ sL, const double *__restrict__ sE,
-                                                     const double *__restrict__ jg, const double *__restrict__ kin,
-                                                     double *__restrict__ rbar, double *__restrict__ rbar_at,
-                                                     double *__restrict__ jpar) {
+constexpr int kJasWarps = 8;
+
+__global__ void __launch_bounds__(kJasWarps * 32) k_adj_jastrow(DevSystem s, const double *__restrict__ r,
+                                                                const double *__restrict__ sL,
+                                                                const double *__restrict__ sE,
+                                                                const double *__restrict__ jg,
+                                                                const double *__restrict__ kin,
+                                                                double *__restrict__ rbar,
+                                                                double *__restrict__ rbar_at,
+                                                                double *__restrict__ jpar) {
   extern __shared__ double sm[];
-  const int w = blockIdx.x, N = s.N, tid = threadIdx.x, bs = blockDim.x;
-  double *xs = sm, *gJb = xs + 3 * N;  // electron positions; adjoint of grad J_e
+  __shared__ double s_at[kJasWarps][32][3];
+  __shared__ double red[3][kJasWarps];
+  const int w = blockIdx.x, N = s.N, tid = threadIdx.x, bs = kJasWarps * 32, lane = tid & 31, warp = tid >> 5;
+  double *xs = sm, *gJb = xs + 3 * N, *re_s = gJb + 3 * N;  // positions; adjoint of grad J_e; electrons' sums
   const double sl = sL ? sL[w] : 0.0, se = sE ? sE[w] : 0.0;
   const double lJb = -0.5 * se;        // adjoint of lap J_e (the same for all e)
   for (int t = tid; t < 3 * N; t += bs) {
     xs[t] = r[(size_t)w * N * 3 + t];
-    // gbarJ_e = -sE (gD_e + gJ_e)
+    // gbarJ_e = -sE (gD_e + gJ_e); sL grad J_e from J itself
     const int e = t / 3, q = t - 3 * e;
-    gJb[t] = -se * (kin[((size_t)w * N + e) * 4 + q] + jg[((size_t)w * N + e) * 3 + q]);
+    const double gj = jg[((size_t)w * N + e) * 3 + q];
+    gJb[t] = -se * (kin[((size_t)w * N + e) * 4 + q] + gj);
+    re_s[t] = sl * gj;
   }
   __syncthreads();
   double pb_ea = 0.0, pb_para = 0.0, pb_anti = 0.0;
-  for (int e = tid; e < N; e += bs) {
-    const double *xe = xs + 3 * e;
-    const double gje[3] = {jg[((size_t)w * N + e) * 3], jg[((size_t)w * N + e) * 3 + 1], jg[((size_t)w * N + e) * 3 + 2]};
-    double re[3] = {sl * gje[0], sl * gje[1], sl * gje[2]};  // from J itself
-    for (int a = 0; a < s.n_atoms; ++a) {
-      const double d[3] = {xe[0] - s.R[3 * a], xe[1] - s.R[3 * a + 1], xe[2] - s.R[3 * a + 2]};
-      const double rr = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-      const double z3 = s.Z[a] / (rr * rr * rr);
-      for (int q = 0; q < 3; ++q) re[q] += se * z3 * d[q];  // V_ei
-      if (s.use_j1) {
-        double f1, f2, f3, hv[3], gl[3];
-        j1_d3(s.c1[a], s.b_ea, rr, &f1, &f2, &f3);
-        radial_adj(f1, f2, f3, d, rr, gJb + 3 * e, hv, gl);
-        for (int q = 0; q < 3; ++q) re[q] += hv[q] + lJb * gl[q];
-        pb_ea += sl * j1_db(s.c1[a], s.b_ea, rr);
+  const int G = group_lanes(s.n_atoms), per = 32 / G, sub = lane / G, ga = lane - sub * G;
+  for (int a0 = 0; a0 < s.n_atoms; a0 += G) {
+    const int a = a0 + ga;
+    const bool have = a < s.n_atoms;
+    double ra[3] = {0.0, 0.0, 0.0};
+    const double R[3] = {have ? s.R[3 * a] : 0.0, have ? s.R[3 * a + 1] : 0.0, have ? s.R[3 * a + 2] : 0.0};
+    const double Z = have ? s.Z[a] : 0.0, c1 = have ? s.c1[a] : 0.0;
+    for (int q0 = warp * per; q0 < N; q0 += kJasWarps * per) {
+      const int e = q0 + sub;
+      double re[3] = {0.0, 0.0, 0.0};
+      if (have && e < N) {
+        const double d[3] = {xs[3 * e] - R[0], xs[3 * e + 1] - R[1], xs[3 * e + 2] - R[2]};
+        const double r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2], ri = rsqrt(r2);
+        const double z3 = se * Z * ri * ri * ri;  // V_ei
+        double f1r = 0.0;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) re[q] = z3 * d[q];
+        if (s.use_j1) {
+          double f1, f2, f3, fb, hv[3], gl;
+          j1_d3(c1, s.b_ea, r2 * ri, &f1, &f2, &f3, &fb);
+          radial_adj(f1, f2, f3, d, ri, gJb + 3 * e, hv, &gl);
+          gl *= lJb;
+#pragma unroll
+          for (int q = 0; q < 3; ++q) re[q] += hv[q] + gl * d[q];
+          pb_ea += sl * fb;
+          f1r = sl * f1 * ri;
+        }
+#pragma unroll
+        for (int q = 0; q < 3; ++q) ra[q] -= re[q] + f1r * d[q];
+      }
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        const double v = group_sum(re[q], G);
+        if (ga == 0 && e < N) re_s[3 * e + q] += v;  // (an electron belongs to one warp in every chunk)
       }
     }
-    for (int k = 0; k < N; ++k) {
+#pragma unroll
+    for (int q = 0; q < 3; ++q) s_at[warp][lane][q] = ra[q];
+    __syncthreads();
+    for (int t = tid; t < 3 * G; t += bs) {
+      const int i = t / 3, q = t - 3 * i, at = a0 + i;
+      if (at < s.n_atoms) {
+        double v = 0.0;
+        for (int ww = 0; ww < kJasWarps; ++ww)
+          for (int h = 0; h < per; ++h) v += s_at[ww][h * G + i][q];
+        for (int bb = 0; bb < s.n_atoms; ++bb) {  // V_ii
+          if (bb == at) continue;
+          const double d[3] = {s.R[3 * at] - s.R[3 * bb], s.R[3 * at + 1] - s.R[3 * bb + 1],
+                               s.R[3 * at + 2] - s.R[3 * bb + 2]};
+          const double ri = rsqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
+          v -= se * s.Z[at] * s.Z[bb] * d[q] * ri * ri * ri;
+        }
+        rbar_at[((size_t)w * s.n_atoms + at) * 3 + q] = v;
+      }
+    }
+    __syncthreads();
+  }
+  for (int e = warp; e < N; e += kJasWarps) {
+    const double ex = xs[3 * e], ey = xs[3 * e + 1], ez = xs[3 * e + 2];
+    const bool eup = e < s.n_up;
+    double re[3] = {0.0, 0.0, 0.0};
+    for (int k = lane; k < N; k += 32) {
       if (k == e) continue;
-      const double d[3] = {xe[0] - xs[3 * k], xe[1] - xs[3 * k + 1], xe[2] - xs[3 * k + 2]};
-      const double rr = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-      const double r3 = 1.0 / (rr * rr * rr);
-      for (int q = 0; q < 3; ++q) re[q] -= se * r3 * d[q];  // V_ee
+      const double d[3] = {ex - xs[3 * k], ey - xs[3 * k + 1], ez - xs[3 * k + 2]};
+      const double r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2], ri = rsqrt(r2);
+      double t = -se * ri * ri * ri;  // V_ee
       if (s.use_j2) {
-        const bool same = (e < s.n_up) == (k < s.n_up);
-        double kk, bb, v1, v2, v3, hv[3], gl[3];
+        const bool same = eup == (k < s.n_up);
+        double kk, bb, v1, v2, v3, hv[3], gl;
         j2_params(s, same, &kk, &bb);
-        j2_d3(kk, bb, rr, &v1, &v2, &v3);
+        const double ik = kk == 4.0 ? 0.25 : 0.5, rr = r2 * ri, iq = 1.0 / (1.0 + bb * rr);
+        j2_d3(ik, bb, iq, &v1, &v2, &v3);
         const double dg[3] = {gJb[3 * e] - gJb[3 * k], gJb[3 * e + 1] - gJb[3 * k + 1], gJb[3 * e + 2] - gJb[3 * k + 2]};
-        radial_adj(v1, v2, v3, d, rr, dg, hv, gl);
-        for (int q = 0; q < 3; ++q) re[q] += hv[q] + 2.0 * lJb * gl[q];
+        radial_adj(v1, v2, v3, d, ri, dg, hv, &gl);
+        t += 2.0 * lJb * gl;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) re[q] += hv[q];
         if (k > e) {
-          const double q1 = 1.0 + bb * rr;
-          const double vdb = -rr * rr / (kk * q1 * q1);
+          const double vdb = -r2 * ik * iq * iq;
           if (same && !s.j2_si) pb_para += sl * vdb;
           else pb_anti += sl * vdb;
         }
       }
+#pragma unroll
+      for (int q = 0; q < 3; ++q) re[q] += t * d[q];
     }
-    for (int q = 0; q < 3; ++q) rbar[((size_t)w * N + e) * 3 + q] += re[q];
-  }
-  for (int a = tid; a < s.n_atoms; a += bs) {
-    double ra[3] = {0.0, 0.0, 0.0};
-    for (int e = 0; e < N; ++e) {
-      const double *xe = xs + 3 * e;
-      const double d[3] = {xe[0] - s.R[3 * a], xe[1] - s.R[3 * a + 1], xe[2] - s.R[3 * a + 2]};
-      const double rr = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-      const double z3 = s.Z[a] / (rr * rr * rr);
-      for (int q = 0; q < 3; ++q) ra[q] -= se * z3 * d[q];
-      if (s.use_j1) {
-        double f1, f2, f3, hv[3], gl[3];
-        j1_d3(s.c1[a], s.b_ea, rr, &f1, &f2, &f3);
-        radial_adj(f1, f2, f3, d, rr, gJb + 3 * e, hv, gl);
-        for (int q = 0; q < 3; ++q) ra[q] -= hv[q] + lJb * gl[q] + sl * f1 * d[q] / rr;
-      }
+#pragma unroll
+    for (int q = 0; q < 3; ++q) re[q] = warp_sum(re[q]);
+    if (lane < 3) {
+      const double v = lane == 0 ? re[0] : (lane == 1 ? re[1] : re[2]);
+      rbar[((size_t)w * N + e) * 3 + lane] += re_s[3 * e + lane] + v;
     }
-    for (int b = 0; b < s.n_atoms; ++b) {  // V_ii
-      if (b == a) continue;
-      const double d[3] = {s.R[3 * a] - s.R[3 * b], s.R[3 * a + 1] - s.R[3 * b + 1], s.R[3 * a + 2] - s.R[3 * b + 2]};
-      const double rr = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-      for (int q = 0; q < 3; ++q) ra[q] -= se * s.Z[a] * s.Z[b] * d[q] / (rr * rr * rr);
-    }
-    for (int q = 0; q < 3; ++q) rbar_at[((size_t)w * s.n_atoms + a) * 3 + q] = ra[q];
   }
   // Jastrow parameter adjoints (from log|Psi| only): block sums
-  __shared__ double red[3][4];
   pb_ea = warp_sum(pb_ea);
   pb_para = warp_sum(pb_para);
   pb_anti = warp_sum(pb_anti);
-  if ((tid & 31) == 0) {
-    red[0][tid >> 5] = pb_ea;
-    red[1][tid >> 5] = pb_para;
-    red[2][tid >> 5] = pb_anti;
+  if (lane == 0) {
+    red[0][warp] = pb_ea;
+    red[1][warp] = pb_para;
+    red[2][warp] = pb_anti;
   }
   __syncthreads();
-  if (tid == 0) {
-    double a0 = 0.0, a1 = 0.0, a2 = 0.0;
-    for (int q = 0; q < (bs >> 5); ++q) {
-      a0 += red[0][q];
-      a1 += red[1][q];
-      a2 += red[2][q];
-    }
-    jpar[(size_t)w * 3] = a0;
-    jpar[(size_t)w * 3 + 1] = a1;
-    jpar[(size_t)w * 3 + 2] = a2;
+  if (tid < 3) {
+    double a0 = 0.0;
+    for (int q = 0; q < kJasWarps; ++q) a0 += red[tid][q];
+    jpar[(size_t)w * 3 + tid] = a0;
   }
 }
 
@@ -696,24 +774,21 @@ cudaError_t launch_adj_rows_gemm(const DevSystem &s, const double *ginv, double 
   return e;
 }
 
-int adj_position_parts(const DevSystem &s) { return (s.N + kAdjWarps - 1) / kAdjWarps; }
+int adj_position_parts(const DevSystem &s) { return (s.N + kAdjElectrons - 1) / kAdjElectrons; }
 
 cudaError_t launch_adj_positions(const DevSystem &s, const double *r, const double *sE, const double *jg,
                                  const double *mbuf, const double *phibar_a, const double *phibar_b,
-                                 const double *phibar_dn, const int *shell_atom, double *rbar, double *part, int W,
-                                 cudaStream_t st) {
+                                 const double *phibar_dn, double *rbar, double *part, int W, cudaStream_t st) {
   dim3 grid(adj_position_parts(s), W);
-  const size_t smem = (size_t)3 * s.n_atoms * sizeof(double) + (size_t)s.n_shells * sizeof(int);
-  k_adj_positions<<<grid, kAdjWarps * 32, smem, st>>>(s, r, sE, jg, mbuf, phibar_a, phibar_b, phibar_dn, shell_atom,
-                                                      rbar, part);
+  k_adj_positions<<<grid, kAdjWarps * 32, 0, st>>>(s, r, sE, jg, mbuf, phibar_a, phibar_b, phibar_dn, rbar, part);
   return cudaGetLastError();
 }
 
 cudaError_t launch_adj_jastrow(const DevSystem &s, const double *r, const double *sL, const double *sE,
                                const double *jg, const double *kin, double *rbar, double *rbar_at, double *jpar, int W,
                                cudaStream_t st) {
-  const size_t smem = (size_t)6 * s.N * sizeof(double);
-  k_adj_jastrow<<<W, 128, smem, st>>>(s, r, sL, sE, jg, kin, rbar, rbar_at, jpar);
+  const size_t smem = (size_t)9 * s.N * sizeof(double);
+  k_adj_jastrow<<<W, kJasWarps * 32, smem, st>>>(s, r, sL, sE, jg, kin, rbar, rbar_at, jpar);
   return cudaGetLastError();
 }
 
@@ -765,7 +840,7 @@ cudaError_t setup_adjoint_attributes() {
   if ((e = cudaFuncSetAttribute(k_adj_kvec, cudaFuncAttributeMaxDynamicSharedMemorySize, big))) return e;
   if ((e = cudaFuncSetAttribute(k_adj_gbar, cudaFuncAttributeMaxDynamicSharedMemorySize, big))) return e;
   if ((e = cudaFuncSetAttribute(k_adj_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, big))) return e;
-  return cudaFuncSetAttribute(k_adj_positions, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+  return cudaFuncSetAttribute(k_adj_jastrow, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
 }
 
 }  // namespace jagp

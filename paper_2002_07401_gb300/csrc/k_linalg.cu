@@ -268,8 +268,8 @@ static cudaError_t launch_small_f32(int q, const float *X, const float *Xlo, siz
 // The FP32 path's plain per-walker products of more than 32 rows: 64 x 64 output
 // tile, 64 threads with 8 x 8 outputs each (columns 4 tx .. + 3 and 32 + 4 tx .. + 3, rows
 // likewise), k-chunks of 16 with the next chunk loading into registers meanwhile: 64 FMAs per four 16-byte
-// reads.  64 walkers, 256 x 256, K = 4096: 1.53 ms (now 1.08) with 4 x 4 outputs per thread
-// and scalar reads.
+// reads.  64 walkers, 256 x 256, K = 4096: 1.08 ms (1.53 with 4 x 4 outputs per
+// thread and scalar reads).
 struct GemmTile64F32 {
   static __device__ __forceinline__ void run(const float *__restrict__ X, size_t xw, const float *__restrict__ Y,
                                              size_t yw, int ma, int nb, int K, float *__restrict__ Out, size_t ow,
