@@ -87,11 +87,33 @@ struct LaunchScope {
 
 bool tc_refresh(const jagp_ctx *h) { return h->precision == JAGP_PREC_MIXED && h->ds.n_up >= kTcRefreshMinUp; }
 
+// FP64-equivalent handles: the products with G~^{-1} (K = N_up) and of kinetic
+// rows take the tensor cores as the lambda products do, from N_up = 32 on: below,
+// the slices of a column padded to 64 terms cost as much to write as the FP64
+// product itself (N_up = 16, L = 320, 2048 walkers: 275 us either way); at N_up = 64, L = 1536 a
+// product of 256 walkers takes 0.3 ms instead of 2.7.
+bool tc_products(const jagp_ctx *h) {
+  return h->precision == JAGP_PREC_FP64 && h->tc_lambda && h->ds.n_up >= kTcProductsMinUp;
+}
+// slices and bits of operands with K = N_up (exact leading sums, as for lambda)
+int cols_slices(const jagp_ctx *h) { return h->ds.n_up <= 512 ? 7 : 8; }
+int cols_bits(const jagp_ctx *h) { return h->ds.n_up <= 512 ? 8 : 7; }
+// walkers at a time: packed operands of about 96 MB, which the product then reads from L2
+int tc_chunk(const jagp_ctx *h, int W, size_t bytes_per_walker) {
+  const size_t c = (size_t)96 * 1024 * 1024 / bytes_per_walker;
+  return c < 1 ? 1 : (c < (size_t)W ? (int)c : W);
+}
+int cols_chunk(const jagp_ctx *h, int W) {
+  const size_t kpn = (h->ds.n_up + 63) / 64 * 64;
+  return tc_chunk(h, W, (size_t)h->ds.L * cols_slices(h) * kpn * 2);
+}
+
 Layout layout_of(const jagp_ctx *h, int W) {
   const bool mixed = h->precision == JAGP_PREC_MIXED;
   return make_layout((size_t)W, (size_t)h->ds.n_up, (size_t)h->ds.N, (size_t)h->ds.L, mixed ? 4 : 8,
                      h->tc_lambda ? (size_t)h->kp : 0, (size_t)h->tc_slices, tc_refresh(h),
-                     h->ds.use_j3 ? (size_t)h->ds.LJ : 0);
+                     h->ds.use_j3 ? (size_t)h->ds.LJ : 0, tc_products(h) ? (size_t)cols_chunk(h, W) : 0,
+                     (size_t)cols_slices(h));
 }
 
 // the twenty-one slice pairs (a, b) with a + b <= 5 of the six-slice
@@ -293,6 +315,53 @@ jagp_status_t run_kinetic_mixed(jagp_ctx *h, const double *r, void *state, int W
   return JAGP_OK;
 }
 
+// FP64-equivalent tensor-core product over K rows of per-walker tables,
+//   out_w[y][c] (+)= sum_{k < K} X_w[k][c] Y_w(k, y),  c < L, y < ny,
+// X_w = X + w xw of row pitch L, out_w = out + w ow of row pitch L; Y_w = Y + w
+// N_up^2 of row pitch N_up, Y_w(k, y) = Y_w[y][k] (y_rows; K = N_up) or Y_w[k][y].
+// The columns of X and the rows or columns of Y are cut into exact slices.
+jagp_status_t cols_product64(jagp_ctx *h, void *state, int W, const double *X, size_t xw, int K, const double *Y,
+                             bool y_rows, int ny, double *out, size_t ow, bool add, cudaStream_t st) {
+  const Layout L = layout_of(h, W);
+  const int n = h->ds.n_up, Lb = h->ds.L, kpn = (n + 63) / 64 * 64, nsl = cols_slices(h), bits = cols_bits(h),
+            chunk = cols_chunk(h, W);
+  uint16_t *pa = at<uint16_t>(state, L.mpack_a), *pb = at<uint16_t>(state, L.mpack_b);
+  int *ea = at<int>(state, L.mexp_a), *eb = at<int>(state, L.mexp_b), *mr = at<int>(state, L.mrows);
+  int qa[kMaxPairs], qb[kMaxPairs];
+  const int np = slice_pairs(nsl, qa, qb);
+  for (int w0 = 0; w0 < W; w0 += chunk) {
+    const int wc = std::min(chunk, W - w0);
+    const double *Yc = Y + (size_t)w0 * n * n;
+    LAUNCH(0, 1, launch_pack_cols(X + w0 * xw, nullptr, nullptr, xw, K, Lb, kpn, wc, pb, eb, nullptr, 0, 0, st, nsl, bits));
+    if (y_rows)
+      LAUNCH(0, 1, launch_pack_fixed64(Yc, nullptr, nullptr, wc * ny, ny, n, n, kpn, nsl, bits, pa, mr, ea, wc * ny, st));
+    else
+      LAUNCH(0, 1,
+             launch_pack_cols(Yc, nullptr, nullptr, (size_t)n * n, K, n, kpn, wc, pa, ea, nullptr, 0, 0, st, nsl, bits));
+    LAUNCH(JAGP_KERNEL_ENERGY, 1,
+           launch_umma_gemm(pb, wc * Lb, nullptr, nsl, pa, ny, nsl, kpn, np, qa, qb, nullptr, 0, nullptr, h->d_err, st,
+                            eb, ea, nullptr, 0, out + w0 * ow, bits, Lb, wc, 0, y_rows ? ny : n, (long long)ow, 1, Lb,
+                            nullptr, K, add));
+  }
+  return JAGP_OK;
+}
+
+// the M vectors of an FP64 handle
+jagp_status_t run_mmat64(jagp_ctx *h, void *state, int W, cudaStream_t st) {
+  const Layout L = layout_of(h, W);
+  const double *gi = at<double>(state, L.ginv), *bt = at<double>(state, L.bt), *a_up = at<double>(state, L.a_up);
+  double *m = at<double>(state, L.mbuf);
+  if (!tc_products(h)) {
+    LAUNCH(JAGP_KERNEL_ENERGY, 1, launch_mmat<double>(h->ds, gi, bt, a_up, m, W, st));
+    return JAGP_OK;
+  }
+  const int n = h->ds.n_up, nd = h->ds.n_dn;
+  const size_t nL = (size_t)n * h->ds.L, NL = (size_t)h->ds.N * h->ds.L;
+  jagp_status_t s = cols_product64(h, state, W, bt, nL, n, gi, false, n, m, NL, false, st);
+  if (s == JAGP_OK && nd > 0) s = cols_product64(h, state, W, a_up, nL, n, gi, true, nd, m + nL, NL, false, st);
+  return s;
+}
+
 template <typename T>
 jagp_status_t run_local_energy(jagp_ctx *h, const double *r, void *state, int W, double *eL, double *parts,
                                cudaStream_t st, bool write_jastrow = false) {
@@ -303,9 +372,8 @@ jagp_status_t run_local_energy(jagp_ctx *h, const double *r, void *state, int W,
     if (s != JAGP_OK) return s;
   } else {
     if (h->ds.use_j3) LAUNCH(0, 1, launch_j3_prep(h->ds, r, j3_vectors(h, L, state), W, st));
-    LAUNCH(JAGP_KERNEL_ENERGY, 1,
-           launch_mmat<T>(h->ds, at<T>(state, L.ginv), at<T>(state, L.bt), at<T>(state, L.a_up), at<T>(state, L.mbuf),
-                          W, st));
+    const jagp_status_t s = run_mmat64(h, state, W, st);
+    if (s != JAGP_OK) return s;
     LAUNCH(JAGP_KERNEL_ENERGY, 1,
            launch_kinetic<T>(h->ds, r, at<T>(state, L.mbuf), at<double>(state, L.kin), W, st));
   }
@@ -509,6 +577,9 @@ struct GradLayout {
   // columns of both operands, their exponents and the per-segment products
   int tc_lam, seg_w, nseg, kpseg;
   size_t tc_u, tc_v, tc_eu, tc_ev, tc_part;
+  // FP64-equivalent row products (tc_products): one packed operand of hw walkers
+  int hw;
+  size_t h_pack, h_exp, h_rows;
 };
 constexpr int kLamBarSlices = 8, kLamBarBits = 7;  // 7-bit slices: K <= 2048 sums stay below 2^24
 GradLayout grad_layout(const jagp_ctx *h, int W) {
@@ -546,8 +617,41 @@ GradLayout grad_layout(const jagp_ctx *h, int W) {
   g.tc_eu = take(g.tc_lam ? (size_t)g.nseg * L * 4 : 0);
   g.tc_ev = take(g.tc_lam ? (size_t)g.nseg * L * 4 : 0);
   g.tc_part = take(g.tc_lam ? (size_t)g.nseg * L * L * 8 : 0);
+  const size_t hb = n * h->tc_slices * (size_t)h->kp * 2;  // bytes per walker
+  g.hw = tc_products(h) ? tc_chunk(h, W, hb) : 0;
+  g.h_pack = take(g.hw * hb);
+  g.h_exp = take(g.hw * n * 4);
+  g.h_rows = take(g.hw * n * 4);
   g.total = o;
   return g;
+}
+
+// FP64-equivalent tensor-core product of per-walker rows of length L,
+//   out_w[a][b] = sum_k X_w[a][k] Y_w[b][k],  a < N_up, b < nb,
+// X_w, Y_w: rows of pitch L, xs and ys rows per walker; out_w [N_up][N_up]
+jagp_status_t rows_product64(jagp_ctx *h, void *state, int W, const GradLayout &G, char *wk, const double *X, int xs,
+                             const double *Y, int ys, int nb, double *out, cudaStream_t st) {
+  const Layout L = layout_of(h, W);
+  const int n = h->ds.n_up, Lb = h->ds.L;
+  uint16_t *pa = at<uint16_t>(state, L.pack), *pb = reinterpret_cast<uint16_t *>(wk + G.h_pack);
+  int *ea = at<int>(state, L.exps), *ra = at<int>(state, L.rows);
+  int *eb = reinterpret_cast<int *>(wk + G.h_exp), *rb = reinterpret_cast<int *>(wk + G.h_rows);
+  int qa[kMaxPairs], qb[kMaxPairs];
+  const int np = slice_pairs(h->tc_slices, qa, qb);
+  for (int w0 = 0; w0 < W; w0 += G.hw) {
+    const int wc = std::min(G.hw, W - w0);
+    LAUNCH(0, 1,
+           launch_pack_fixed64(X + (size_t)w0 * xs * Lb, nullptr, nullptr, wc * n, n, xs, Lb, h->kp, h->tc_slices,
+                               h->tc_bits, pa, ra, ea, wc * n, st));
+    LAUNCH(0, 1,
+           launch_pack_fixed64(Y + (size_t)w0 * ys * Lb, nullptr, nullptr, wc * nb, nb, ys, Lb, h->kp, h->tc_slices,
+                               h->tc_bits, pb, rb, eb, wc * nb, st));
+    LAUNCH(JAGP_KERNEL_GEMM_ROWS, 1,
+           launch_umma_gemm(pa, wc * n, nullptr, h->tc_slices, pb, nb, h->tc_slices, h->kp, np, qa, qb, nullptr, n,
+                            nullptr, h->d_err, st, ea, eb, nullptr, 0, out + (size_t)w0 * n * n, h->tc_bits, n, wc, 0,
+                            nb, 0, 0, 0, nullptr, Lb));
+  }
+  return JAGP_OK;
 }
 
 }  // namespace
@@ -603,24 +707,46 @@ static jagp_status_t jagp_grad_impl(jagp_handle_t h, const double *d_r, void *d_
   if (s != JAGP_OK) return s;
   double *kbar = wp(G.kbar), *dnphi = wp(G.dnphi);
   LAUNCH(0, 1, launch_adj_kvec(d, d_r, d_seed_eL, wp(G.jg), kbar, dnphi, W, st));
-  LAUNCH(JAGP_KERNEL_GEMM_ROWS, 1,
-         launch_gemm_rows<double>(kbar, (size_t)N * Lb, at<double>(d_state, L.bt), (size_t)n * Lb, n, n, Lb,
-                                  wp(G.h1), (size_t)n * n, n, W, st));
-  if (nd > 0)
-    LAUNCH(JAGP_KERNEL_GEMM_ROWS, 1,
-           launch_gemm_rows<double>(at<double>(d_state, L.a_up), (size_t)n * Lb, kbar + (size_t)n * Lb,
-                                    (size_t)N * Lb, n, nd, Lb, wp(G.h2), (size_t)n * n, n, W, st));
-  if (n <= kMaxUpGrad) {
-    LAUNCH(0, 1, launch_adj_gbar(at<double>(d_state, L.ginv), wp(G.h1), wp(G.h2), d_seed_logpsi, n, nd, wp(G.gbar),
-                                 W, st));
-    LAUNCH(0, 1,
-           launch_adj_rows(d, at<double>(d_state, L.ginv), wp(G.gbar), at<double>(d_state, L.phi_up),
-                           at<double>(d_state, L.bt), kbar, wp(G.btbar), wp(G.abar), wp(G.phibar_a), W, st));
+  const double *ginv = at<double>(d_state, L.ginv), *phi_up = at<double>(d_state, L.phi_up),
+               *bt = at<double>(d_state, L.bt), *a_up = at<double>(d_state, L.a_up);
+  const size_t nL = (size_t)n * Lb, NL = (size_t)N * Lb;
+  if (tc_products(h)) {
+    // the same products on the tensor cores; G~-sized ones with FP64 instructions
+    s = rows_product64(h, d_state, W, G, wk, kbar, N, bt, n, n, wp(G.h1), st);
+    if (s == JAGP_OK && nd > 0) s = rows_product64(h, d_state, W, G, wk, a_up, n, kbar + nL, N, nd, wp(G.h2), st);
+    if (s != JAGP_OK) return s;
+    const bool small = n <= kMaxUpGrad;  // Gbar as it is, or transposed
+    if (small)
+      LAUNCH(0, 1, launch_adj_gbar(ginv, wp(G.h1), wp(G.h2), d_seed_logpsi, n, nd, wp(G.gbar), W, st));
+    else
+      LAUNCH(0, 3,
+             launch_adj_rows_gemm(d, ginv, wp(G.h1), wp(G.h2), d_seed_logpsi, phi_up, bt, kbar, wp(G.gbar),
+                                  wp(G.btbar), wp(G.abar), wp(G.phibar_a), W, st, true));
+    const double *gb = wp(G.gbar);
+    if (nd > 0) {
+      s = cols_product64(h, d_state, W, phi_up, nL, n, gb, !small, nd, wp(G.btbar), nL, false, st);
+      if (s == JAGP_OK) s = cols_product64(h, d_state, W, kbar, NL, n, ginv, true, nd, wp(G.btbar), nL, true, st);
+      if (s == JAGP_OK) s = cols_product64(h, d_state, W, kbar + nL, NL, nd, ginv, false, n, wp(G.abar), nL, false, st);
+    } else {
+      JAGP_CU(cudaMemsetAsync(wp(G.abar), 0, (size_t)W * nL * sizeof(double), st));
+    }
+    if (s == JAGP_OK) s = cols_product64(h, d_state, W, bt, nL, n, gb, small, n, wp(G.phibar_a), nL, false, st);
+    if (s != JAGP_OK) return s;
   } else {
-    LAUNCH(0, 8,
-           launch_adj_rows_gemm(d, at<double>(d_state, L.ginv), wp(G.h1), wp(G.h2), d_seed_logpsi,
-                                at<double>(d_state, L.phi_up), at<double>(d_state, L.bt), kbar, wp(G.gbar),
-                                wp(G.btbar), wp(G.abar), wp(G.phibar_a), W, st));
+    LAUNCH(JAGP_KERNEL_GEMM_ROWS, 1,
+           launch_gemm_rows<double>(kbar, NL, bt, nL, n, n, Lb, wp(G.h1), (size_t)n * n, n, W, st));
+    if (nd > 0)
+      LAUNCH(JAGP_KERNEL_GEMM_ROWS, 1,
+             launch_gemm_rows<double>(a_up, nL, kbar + nL, NL, n, nd, Lb, wp(G.h2), (size_t)n * n, n, W, st));
+    if (n <= kMaxUpGrad) {
+      LAUNCH(0, 1, launch_adj_gbar(ginv, wp(G.h1), wp(G.h2), d_seed_logpsi, n, nd, wp(G.gbar), W, st));
+      LAUNCH(0, 1,
+             launch_adj_rows(d, ginv, wp(G.gbar), phi_up, bt, kbar, wp(G.btbar), wp(G.abar), wp(G.phibar_a), W, st));
+    } else {
+      LAUNCH(0, 8,
+             launch_adj_rows_gemm(d, ginv, wp(G.h1), wp(G.h2), d_seed_logpsi, phi_up, bt, kbar, wp(G.gbar),
+                                  wp(G.btbar), wp(G.abar), wp(G.phibar_a), W, st));
+    }
   }
   // phibar_dn = Btbar^T lambda rows, phibar_b = lambda Abar rows (on the tensor
   // cores when the handle has FP64-equivalent products)

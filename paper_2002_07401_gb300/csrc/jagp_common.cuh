@@ -18,6 +18,7 @@ constexpr int kPropStride = 8;     // doubles per proposal record
 constexpr int kFixedSlices = 6;    // 8-bit slices per element of the fixed-point lambda products (mixed path)
 constexpr int kFixedPairs = 21;    // slice pairs (a, b) with a + b < kFixedSlices
 constexpr int kMaxPairs = 36;      // slice pairs of the FP64-equivalent products (eight slices)
+constexpr int kTcProductsMinUp = 32; // FP64-equivalent handles: products with G~^{-1} and of kinetic rows on the tensor cores from this N_up on
 constexpr int kTcRefreshMinUp = 32;  // mixed path: G~ of a refresh on the tensor cores from this N_up on
 constexpr int kGuidedMaxUp = 64;     // guided sampling: G~ and G~^{-1} in shared memory up to this N_up
 constexpr int kMmatDwMaxUp = 32;     // mixed path: exact M vectors on the CUDA cores up to this N_up (tensor cores above)
@@ -91,7 +92,8 @@ struct Layout {
   size_t gexp_a;   // int    [W n_up]        their row exponents
   size_t gexp_b;   // int    [W n_up]
   // mixed path, local energy: the M vectors as exact fixed-point tensor-core
-  // products of the FP64 inverse with the two-float tables (kpn = N_up padded to 64)
+  // products of the FP64 inverse with the two-float tables (kpn = N_up padded to 64);
+  // the packed operands also serve FP64-equivalent handles (some walkers at a time)
   size_t ginv64;   // double [W][n_up][n_up] G~^{-1} of the last refresh in FP64
   size_t a_up_lo;  // float  [W][n_up][L]    low parts of A_up (A_up + a_up_lo is a two-float table)
   size_t mbuf_lo;  // float  [W][N][L]       low parts of the M vectors
@@ -109,9 +111,11 @@ enum { S_LOGDET = 0, S_SIGN = 1, S_J = 2, S_NACC = 3, S_DRIFT = 4, S_STRIDE = 8 
 
 inline size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
-// esz: bytes per table element (8 or 4); kp: padded K of the packed operand (0 = none)
+// esz: bytes per table element (8 or 4); kp: padded K of the packed operand (0 = none);
+// tc_w, tc_nsl: walkers at a time and slices of the FP64-equivalent products with G~^{-1} (0: none)
 inline Layout make_layout(size_t W, size_t nu, size_t N, size_t L, size_t esz = 8, size_t kp = 0,
-                          size_t nsl = kFixedSlices, bool tc_refresh = false, size_t lj = 0) {
+                          size_t nsl = kFixedSlices, bool tc_refresh = false, size_t lj = 0, size_t tc_w = 0,
+                          size_t tc_nsl = 0) {
   Layout l;
   size_t o = 0;
   auto take = [&](size_t bytes) { size_t r = o; o = align256(o + bytes); return r; };
@@ -145,11 +149,13 @@ inline Layout make_layout(size_t W, size_t nu, size_t N, size_t L, size_t esz = 
   l.ginv64 = take(mx ? W * nu * nu * 8 : 0);
   l.a_up_lo = take(mx ? W * nu * L * 4 : 0);
   l.mbuf_lo = take(mx ? W * N * L * 4 : 0);
-  l.mpack_a = take(mx ? W * nu * kFixedSlices * kpn * 2 : 0);
-  l.mpack_b = take(mx ? W * L * kFixedSlices * kpn * 2 : 0);
-  l.mexp_a = take(mx ? W * nu * 4 : 0);
-  l.mexp_b = take(mx ? W * L * 4 : 0);
-  l.mrows = take(mx ? W * nu * 4 : 0);
+  // walkers and slices of the packed operands (FP64-equivalent: tc_w walkers at a time)
+  const size_t mw = mx ? W : tc_w, ms = mx ? (size_t)kFixedSlices : tc_nsl;
+  l.mpack_a = take(mw * nu * ms * kpn * 2);
+  l.mpack_b = take(mw * L * ms * kpn * 2);
+  l.mexp_a = take(mw * nu * 4);
+  l.mexp_b = take(mw * L * 4);
+  l.mrows = take(mw * nu * 4);
   l.j3buf = take(W * 6 * lj * 8);
   l.total = o;
   return l;

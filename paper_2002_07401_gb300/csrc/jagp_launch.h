@@ -127,8 +127,8 @@ cudaError_t launch_increment(uint32_t *c, uint32_t by, cudaStream_t st);
 // runs in k_umma_tri; only there: out64, batches, an affine output, bn_max (0 or
 // 64: the widest tile the shape rule takes; 16, 32, 48: that width at most),
 // stages_max (-1, -2, -3: K chunks of 64, 32, 16; else the rule), klive (K
-// elements per term that may be non-zero; 0: kp) and krange (non-zero K range
-// [x, y) per 16 rows of B; null: [0, klive)).
+// elements per term that may be non-zero; 0: kp), krange (non-zero K range
+// [x, y) per 16 rows of B; null: [0, klive)) and add (out64 += instead of =).
 int umma_pick_bn(int n, int max_bn);
 cudaError_t launch_umma_gemm(const uint16_t *A, int m_max, const int *m_dev, int a_terms, const uint16_t *B, int n,
                              int b_terms, int kp, int npairs, const int *pair_a, const int *pair_b, float *out,
@@ -137,7 +137,7 @@ cudaError_t launch_umma_gemm(const uint16_t *A, int m_max, const int *m_dev, int
                              int bn_max = 0, double *out64 = nullptr, int slice_bits = 8, int batch_rows = 0,
                              int batches = 0, int stages_max = 0, int b_batch_rows = 0, long long o_bstride = 0,
                              long long o_rstride = 0, long long o_cstride = 0, const int2 *krange = nullptr,
-                             int klive = 0);
+                             int klive = 0, bool add = false);
 // whether two chunk-major stages (stages_max = -1, -2, -3: K chunks of 64, 32,
 // 16) of these pairs fit at tile width bn
 bool umma_chunk_fits(int npairs, const int *pair_a, const int *pair_b, int bn, int stages_max);
@@ -174,7 +174,8 @@ cudaError_t launch_adj_rows(const DevSystem &s, const double *ginv, const double
 // (h1, h2 are overwritten; gbarT receives Gbar transposed)
 cudaError_t launch_adj_rows_gemm(const DevSystem &s, const double *ginv, double *h1, double *h2, const double *sL,
                                  const double *phi_up, const double *bt, const double *kbar, double *gbarT,
-                                 double *btbar, double *abar, double *phibar, int W, cudaStream_t st);
+                                 double *btbar, double *abar, double *phibar, int W, cudaStream_t st,
+                                 bool gbar_only = false);
 int adj_position_parts(const DevSystem &s);
 cudaError_t launch_adj_positions(const DevSystem &s, const double *r, const double *sE, const double *jg,
                                  const double *mbuf, const double *phibar_a, const double *phibar_b,

@@ -753,7 +753,7 @@ __global__ void k_adj_gbar_init(const double *__restrict__ ginv, double *__restr
 
 cudaError_t launch_adj_rows_gemm(const DevSystem &s, const double *ginv, double *h1, double *h2, const double *sL,
                                  const double *phi_up, const double *bt, const double *kbar, double *gbarT,
-                                 double *btbar, double *abar, double *phibar, int W, cudaStream_t st) {
+                                 double *btbar, double *abar, double *phibar, int W, cudaStream_t st, bool gbar_only) {
   const int n = s.n_up, nd = s.n_dn, N = s.N, L = s.L;
   const size_t nn = (size_t)n * n, nL = (size_t)n * L, NL = (size_t)N * L;
   long blocks = ((long)W * nn + 255) / 256;
@@ -763,6 +763,7 @@ cudaError_t launch_adj_rows_gemm(const DevSystem &s, const double *ginv, double 
   // T = Ginv H (into h2), GbarT -= T Ginv
   if (!e) e = bgemm(false, ginv, nn, n, h1, nn, n, h2, nn, n, n, n, n, 1.0, 0, W, st);
   if (!e) e = bgemm(false, h2, nn, n, ginv, nn, n, gbarT, nn, n, n, n, n, -1.0, 1, W, st);
+  if (gbar_only) return e;
   // Btbar (rows j < n_dn) = GbarT Phi_up + Ginv Mbar_up
   if (!e && nd > 0) e = bgemm(false, gbarT, nn, n, phi_up, nL, L, btbar, nL, L, nd, L, n, 1.0, 0, W, st);
   if (!e && nd > 0) e = bgemm(false, ginv, nn, n, kbar, NL, L, btbar, nL, L, nd, L, n, 1.0, 1, W, st);

@@ -380,6 +380,7 @@ struct TriArgs {
   const int *out_rows;
   long long o_bstride, o_rstride, o_cstride;
   int vec;               // output rows take 32-byte stores
+  int add;               // out64 += (scalar stores)
   int *err;
 };
 
@@ -675,7 +676,11 @@ struct UmmaTri {
             }
             if (live) {
               double *o = g.out64 + obase;
-              if (g.vec && c0 + 16 <= g.n) {
+              if (g.add) {
+  #pragma unroll
+                for (int j = 0; j < 16; ++j)
+                  if (c0 + j < g.n) o[(c0 + j) * ocs] += v[j];
+              } else if (g.vec && c0 + 16 <= g.n) {
   #pragma unroll
                 for (int j = 0; j < 16; j += 4) store4(o + c0 + j, v + j);
               } else {
@@ -924,7 +929,8 @@ cudaError_t launch_umma_gemm(const uint16_t *A, int m_max, const int *m_dev, int
                              long long ldo, const int *out_rows, int *err, cudaStream_t st, const int *a_exp,
                              const int *b_exp, float *out_lo, int bn_max, double *out64, int slice_bits,
                              int batch_rows, int batches, int stages_max, int b_batch_rows, long long o_bstride,
-                             long long o_rstride, long long o_cstride, const int2 *krange, int klive) {
+                             long long o_rstride, long long o_cstride, const int2 *krange, int klive,
+                             bool add) {
   if (m_max <= 0 || n <= 0) return cudaSuccess;
   if (kp <= 0 || kp % 64 != 0 || npairs < 1 || npairs > kMaxPairs || a_terms < 1 || b_terms < 1)
     return cudaErrorInvalidValue;
@@ -970,6 +976,7 @@ cudaError_t launch_umma_gemm(const uint16_t *A, int m_max, const int *m_dev, int
     g.o_rstride = o_rstride;
     g.o_cstride = o_cstride;
     g.err = err;
+    g.add = add && out64;
     const long long unit = out64 ? 4 : 8;  // elements of a 32-byte store
     const uintptr_t bases = out64 ? reinterpret_cast<uintptr_t>(out64)
                                   : reinterpret_cast<uintptr_t>(out) | reinterpret_cast<uintptr_t>(out_lo);
@@ -1387,6 +1394,8 @@ cudaError_t launch_pack_cols(const double *X64, const float *X32, const float *X
     return pack_cols<false, 6, 8>(X64, X32, Xlo, xw, R, C, kp, W, A, exps, rows_out, dst_stride, dst_off, st);
   if (X64 && nsl == 6 && bits == 8)
     return pack_cols<true, 6, 8>(X64, X32, Xlo, xw, R, C, kp, W, A, exps, rows_out, dst_stride, dst_off, st);
+  if (X64 && nsl == 7 && bits == 8)
+    return pack_cols<true, 7, 8>(X64, X32, Xlo, xw, R, C, kp, W, A, exps, rows_out, dst_stride, dst_off, st);
   if (X64 && nsl == 8 && bits == 7)
     return pack_cols<true, 8, 7>(X64, X32, Xlo, xw, R, C, kp, W, A, exps, rows_out, dst_stride, dst_off, st);
   return cudaErrorInvalidValue;
