@@ -586,8 +586,7 @@ GradLayout grad_layout(const jagp_ctx *h, int W) {
   const size_t w = (size_t)W, n = h->ds.n_up, N = h->ds.N, L = h->ds.L, na = h->ds.n_atoms;
   GradLayout g;
   g.nparts = adj_position_parts(h->ds);
-  const size_t rows = w * (n + h->ds.n_dn);
-  g.nz = (int)std::max<size_t>(1, std::min<size_t>(64, rows / 1024));
+  g.nz = adj_lambda_splits(W, h->ds.n_up, h->ds.n_dn, h->ds.L);
   size_t o = 0;
   auto take = [&](size_t bytes) { size_t r = o; o = align256(o + bytes); return r; };
   g.jg = take(w * N * 3 * 8);

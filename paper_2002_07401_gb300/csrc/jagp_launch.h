@@ -184,8 +184,17 @@ cudaError_t launch_adj_positions(const DevSystem &s, const double *r, const doub
 cudaError_t launch_adj_jastrow(const DevSystem &s, const double *r, const double *sL, const double *sE,
                                const double *jg, const double *kin, double *rbar, double *rbar_at, double *jpar, int W,
                                cudaStream_t st);
+// out[k] = sum over walkers of in[w][k], k < n
+cudaError_t launch_walker_sum(const double *in, int W, int n, double *out, cudaStream_t st);
 cudaError_t launch_adj_reduce(const double *part, int nparts, int n_atoms, double *rbar_at, const double *jpar,
                               int W, double *dR, double *djas, cudaStream_t st);
+// ranges of rows (at most 64) for launch_adj_lambda: those whose fullest SM has the
+// least FP64 work (rows, and about 8 rows' worth per tile for its start and its sums),
+// among those that leave more than three CTAs per SM to cover one another's barriers
+// (as many as there are, of at least 64 rows, if none does).
+// 32000 rows at L = 320: 30 ranges, 750 tiles, five on the fullest SM, 5.4 ms; one
+// range per 1024 rows gave 775, six on the fullest SM (6.0 ms)
+int adj_lambda_splits(int W, int n, int nd, int L);
 cudaError_t launch_adj_lambda(const double *btbar, const double *dnphi, const double *phi_up, const double *abar,
                               int W, int n, int nd, int L, double *part, int nz, double *dlam, cudaStream_t st);
 // dlam[i] = sum_{z < nz} part[z][i] (fixed order), i < L^2

@@ -551,14 +551,6 @@ __global__ void k_adj_reduce_walker(const double *__restrict__ part, int nparts,
   }
 }
 
-__global__ void k_adj_reduce_total(const double *__restrict__ per_w, int W, int width, double *__restrict__ out) {
-  for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < width; q += gridDim.x * blockDim.x) {
-    double a = 0.0;
-    for (int w = 0; w < W; ++w) a += per_w[(size_t)w * width + q];
-    out[q] = a;
-  }
-}
-
 // ---------------------------------------------------------------------------
 // 7. lambdabar = sum_rows U[row]^T V[row] for two stacked row sets; split over
 //    row ranges (blockIdx.z), partial sums to part[z][L][L].
@@ -801,21 +793,29 @@ cudaError_t launch_adj_reduce(const double *part, int nparts, int n_atoms, doubl
   k_adj_reduce_walker<<<(int)blocks, 256, 0, st>>>(part, nparts, n_atoms, rbar_at, W);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  if (dR) {
-    k_adj_reduce_total<<<(3 * n_atoms + 255) / 256, 256, 0, st>>>(rbar_at, W, 3 * n_atoms, dR);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
-  if (djas) {
-    k_adj_reduce_total<<<1, 32, 0, st>>>(jpar, W, 3, djas);
-    e = cudaGetLastError();
-  }
+  if (dR && (e = launch_walker_sum(rbar_at, W, 3 * n_atoms, dR, st)) != cudaSuccess) return e;
+  if (djas) e = launch_walker_sum(jpar, W, 3, djas, st);
   return e;
+}
+
+static int adj_lambda_rows_per_z(long rows, int nz) { return (int)(((rows + nz - 1) / nz + 15) / 16 * 16); }
+
+int adj_lambda_splits(int W, int n, int nd, int L) {
+  const long rows = (long)W * (n + nd), tiles = (long)((L + 63) / 64) * ((L + 63) / 64);
+  const int most = (int)(rows < 128 ? 1 : (rows / 64 < 64 ? rows / 64 : 64));
+  int best = most;
+  long least = 0;
+  for (int nz = most; nz >= 1 && (nz == most || tiles * nz > 3 * 152); --nz) {
+    const long c = ((tiles * nz + 151) / 152) * (adj_lambda_rows_per_z(rows, nz) + 8);
+    if (nz == most || c <= least) best = nz, least = c;
+  }
+  return best;
 }
 
 cudaError_t launch_adj_lambda(const double *btbar, const double *dnphi, const double *phi_up, const double *abar,
                               int W, int n, int nd, int L, double *part, int nz, double *dlam, cudaStream_t st) {
   const long rows = (long)W * (n + nd);
-  const int rows_per_z = (int)(((rows + nz - 1) / nz + 15) / 16 * 16);
+  const int rows_per_z = adj_lambda_rows_per_z(rows, nz);
   dim3 grid((L + 63) / 64, (L + 63) / 64, nz);
   k_adj_lambda<<<grid, 256, 0, st>>>(btbar, dnphi, phi_up, abar, W, n, nd, L, rows_per_z, part);
   cudaError_t e = cudaGetLastError();
