@@ -424,33 +424,53 @@ __global__ void __launch_bounds__(128) k_elocal(DevSystem s, const double *__res
 // gradient multiplies grad D / D in the kinetic term, so FP32 there was not
 // enough).  One CTA per walker; the per-thread sums are double-words,
 // combined in FP64 at the end.
+//
+// Bound by FP32 issue (about 650 instructions per electron-atom pair, 450 per
+// electron pair), so that lanes are kept busy and a pair is formed once: R =
+// threads / N threads per electron share its atoms and its distances o to a
+// partner (e + o) mod N, o = 1 .. N/2.  An electron's sums stay in its thread's
+// registers; a partner's go to shared memory, which is free of conflicts because
+// the partners of one o differ (a barrier between two o).  A warp per electron
+// with lanes over the partners formed each pair twice, half filled at N = 32,
+// and reduced four sums per electron (sweeps of 4096 walkers of 16 He 2.94 ms, of 64
+// walkers of 256 He 26.9; 2.70 and 25.5 with this kernel, before in 345 us and 2.2 ms).
 // ---------------------------------------------------------------------------
+constexpr int kElocalDwThreads = 512;  // at most
 struct ElocalDw {
+  static __host__ __device__ int splits(int N, int threads) { return threads >= 2 * N ? threads / N : 1; }
+  // floats: coordinates, atoms' constants, sums of the electrons per split
+  static size_t smem(const DevSystem &s, int threads) {
+    return sizeof(float) * (((size_t)(s.N + s.n_atoms) * 6 + (size_t)s.n_atoms * 8 + 3) / 4 * 4 +
+                            (size_t)splits(s.N, threads) * s.N * 8);
+  }
   static __device__ __forceinline__ void run(DevSystem s, const double *__restrict__ r,
                                              const double *__restrict__ kin, double *__restrict__ eL,
                                              double *__restrict__ parts, double *__restrict__ scal,
                                              const double *__restrict__ j3buf, const uint3 bid, const uint3 gdim) {
     assume_global(r, kin, eL);
-    const int w = bid.x, N = s.N, tid = threadIdx.x, na = s.n_atoms;
-    const int lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-    extern __shared__ float sf[];
-    float *xh = sf, *xl = xh + 3 * N;           // electron coordinates as double-words
-    float *ah = xl + 3 * N, *al = ah + 3 * na;  // atom coordinates
+    const int w = bid.x, N = s.N, tid = threadIdx.x, bs = blockDim.x, na = s.n_atoms;
+    const int lane = tid & 31, warp = tid >> 5, nw = bs >> 5;
+    extern __shared__ float4 sf4[];
+    float *xh = reinterpret_cast<float *>(sf4), *xl = xh + 3 * N;  // electron coordinates as double-words
+    float *ah = xl + 3 * N, *al = ah + 3 * na;                     // atom coordinates
     // per atom, as double-words: -Z, and for J1 -c^4/2, c^3/(2b), -b c
     float *ac = al + 3 * na;
+    // grad J (x, y) and (z), lap J of electron e in split k: jg[k N + e], jl[k N + e]
+    const int R = splits(N, bs);
+    float4 *jg = sf4 + (6 * (N + na) + 8 * na + 3) / 4, *jl = jg + R * N;
     // two-body Jastrow constants [same spin, opposite spin]: b k (dw), k, -2 b (dw)
     __shared__ float j2c[2][5];
-    for (int t = tid; t < N * 3; t += blockDim.x) {
+    for (int t = tid; t < N * 3; t += bs) {
       const fdw v = dw_of(r[(size_t)w * N * 3 + t]);
       xh[t] = v.hi;
       xl[t] = v.lo;
     }
-    for (int t = tid; t < na * 3; t += blockDim.x) {
+    for (int t = tid; t < na * 3; t += bs) {
       const fdw v = dw_of(s.R[t]);
       ah[t] = v.hi;
       al[t] = v.lo;
     }
-    for (int a = tid; a < na; a += blockDim.x) {
+    for (int a = tid; a < na; a += bs) {
       const double c = s.c1[a], b = s.b_ea;
       const fdw z = dw_of(-s.Z[a]), c4 = dw_of(-0.5 * c * c * c * c);
       const fdw c3 = dw_of(b == 0.0 ? 0.0 : c * c * c / (2.0 * b)), bc = dw_of(-b * c);
@@ -474,23 +494,20 @@ struct ElocalDw {
       j2c[tid][3] = m2b.hi;
       j2c[tid][4] = m2b.lo;
     }
+    for (int t = tid; t < R * N; t += bs) jg[t] = jl[t] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     __syncthreads();
-    // a warp per electron, its lanes over the partners (atoms, then electrons);
     // every constant comes from shared memory, so the loops are FP32 only
-    fdw tkin{0.0f, 0.0f}, vee{0.0f, 0.0f}, vei{0.0f, 0.0f}, jv{0.0f, 0.0f};
-    const int P = na + N;
-    // lane j keeps the Jastrow gradient and Laplacian of the warp's j-th electron
-    // of the current group of 32, so that the FP64 assembly of the kinetic term
-    // is issued once per group instead of once per electron
-    fdw kx{0.0f, 0.0f}, ky{0.0f, 0.0f}, kz{0.0f, 0.0f}, kl{0.0f, 0.0f};
-    int mine = -1, slot = 0;
-    for (int e = warp; e < N; e += nw) {
-      const fdw pe[3] = {{xh[3 * e], xl[3 * e]}, {xh[3 * e + 1], xl[3 * e + 1]}, {xh[3 * e + 2], xl[3 * e + 2]}};
-      const bool eup = e < s.n_up;
-      fdw gJx{0.0f, 0.0f}, gJy{0.0f, 0.0f}, gJz{0.0f, 0.0f}, lJ{0.0f, 0.0f};
-      for (int p = lane; p < P; p += 32) {
-        if (p < na) {
-          const int a = p;
+    const fdw zero{0.0f, 0.0f};
+    fdw tkin = zero, vee = zero, vei = zero, jv = zero;
+    const int half = N / 2;
+    for (int e0 = 0; e0 < N; e0 += bs) {  // (one pass while the CTA has a thread per electron)
+      const int split = R > 1 ? tid / N : 0, e = e0 + tid - split * N;
+      const bool have = split < R && e < N;
+      fdw pe[3] = {zero, zero, zero}, gJx = zero, gJy = zero, gJz = zero, lJ = zero;
+      if (have) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) pe[k] = fdw{xh[3 * e + k], xl[3 * e + k]};
+        for (int a = split; a < na; a += R) {
           const float *q = ac + 8 * a;
           const fdw dx = dw_add(pe[0], fdw{-ah[3 * a], -al[3 * a]});
           const fdw dy = dw_add(pe[1], fdw{-ah[3 * a + 1], -al[3 * a + 1]});
@@ -517,76 +534,82 @@ struct ElocalDw {
             gJz = dw_add(gJz, dw_mul(qq, dz));
             lJ = dw_add(lJ, dw_add(fpp, dw_add(qq, qq)));
           }
-          continue;
-        }
-        const int k = p - na;
-        if (k == e) continue;
-        const fdw dx = dw_add(pe[0], fdw{-xh[3 * k], -xl[3 * k]});
-        const fdw dy = dw_add(pe[1], fdw{-xh[3 * k + 1], -xl[3 * k + 1]});
-        const fdw dz = dw_add(pe[2], fdw{-xh[3 * k + 2], -xl[3 * k + 2]});
-        const fdw r2 = dw_add(dw_add(dw_mul(dx, dx), dw_mul(dy, dy)), dw_mul(dz, dz));
-        const fdw rr = dw_sqrt(r2), rinv = dw_recip(rr);
-        if (k > e) vee = dw_add(vee, rinv);
-        if (s.use_j2) {
-          const float *jc = j2c[eup == (k < s.n_up) ? 0 : 1];
-          const float kk = jc[2];
-          const fdw den = dw_add_f(dw_mul(rr, fdw{jc[0], jc[1]}), kk);  // k (1 + b r), k exact
-          const fdw iq = dw_recip(den);                                  // 1 / (k (1 + b r))
-          if (k > e) jv = dw_add(jv, dw_mul(rr, iq));
-          const fdw qi = dw_mul_f(iq, kk);                               // 1/q (k exact)
-          const fdw vp = dw_mul(iq, qi);                                 // 1 / (k q^2)
-          const fdw vpp = dw_mul(dw_mul(vp, qi), fdw{jc[3], jc[4]});      // -2b / (k q^3)
-          const fdw qq = dw_mul(vp, rinv);
-          gJx = dw_add(gJx, dw_mul(qq, dx));
-          gJy = dw_add(gJy, dw_mul(qq, dy));
-          gJz = dw_add(gJz, dw_mul(qq, dz));
-          lJ = dw_add(lJ, dw_add(vpp, dw_add(qq, qq)));
         }
       }
-      // the electron's Jastrow gradient and Laplacian over the warp
-  #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        gJx = dw_add(gJx, fdw{__shfl_xor_sync(0xffffffffu, gJx.hi, o), __shfl_xor_sync(0xffffffffu, gJx.lo, o)});
-        gJy = dw_add(gJy, fdw{__shfl_xor_sync(0xffffffffu, gJy.hi, o), __shfl_xor_sync(0xffffffffu, gJy.lo, o)});
-        gJz = dw_add(gJz, fdw{__shfl_xor_sync(0xffffffffu, gJz.hi, o), __shfl_xor_sync(0xffffffffu, gJz.lo, o)});
-        lJ = dw_add(lJ, fdw{__shfl_xor_sync(0xffffffffu, lJ.hi, o), __shfl_xor_sync(0xffffffffu, lJ.lo, o)});
+      const bool eup = e < s.n_up;
+      for (int o0 = 1; o0 <= half; o0 += R) {
+        const int o = o0 + split;
+        // (N even: the pairs at distance N / 2 belong to the first half of the electrons)
+        if (have && o <= half && (2 * o != N || e < half)) {
+          const int k = e + o < N ? e + o : e + o - N;
+          const fdw dx = dw_add(pe[0], fdw{-xh[3 * k], -xl[3 * k]});
+          const fdw dy = dw_add(pe[1], fdw{-xh[3 * k + 1], -xl[3 * k + 1]});
+          const fdw dz = dw_add(pe[2], fdw{-xh[3 * k + 2], -xl[3 * k + 2]});
+          const fdw r2 = dw_add(dw_add(dw_mul(dx, dx), dw_mul(dy, dy)), dw_mul(dz, dz));
+          const fdw rr = dw_sqrt(r2), rinv = dw_recip(rr);
+          vee = dw_add(vee, rinv);
+          if (s.use_j2) {
+            const float *jc = j2c[eup == (k < s.n_up) ? 0 : 1];
+            const float kk = jc[2];
+            const fdw den = dw_add_f(dw_mul(rr, fdw{jc[0], jc[1]}), kk);  // k (1 + b r), k exact
+            const fdw iq = dw_recip(den);                                  // 1 / (k (1 + b r))
+            jv = dw_add(jv, dw_mul(rr, iq));
+            const fdw qi = dw_mul_f(iq, kk);                               // 1/q (k exact)
+            const fdw vp = dw_mul(iq, qi);                                 // 1 / (k q^2)
+            const fdw vpp = dw_mul(dw_mul(vp, qi), fdw{jc[3], jc[4]});      // -2b / (k q^3)
+            const fdw qq = dw_mul(vp, rinv);
+            const fdw gx = dw_mul(qq, dx), gy = dw_mul(qq, dy), gz = dw_mul(qq, dz), gl = dw_add(vpp, dw_add(qq, qq));
+            gJx = dw_add(gJx, gx);
+            gJy = dw_add(gJy, gy);
+            gJz = dw_add(gJz, gz);
+            lJ = dw_add(lJ, gl);
+            const float4 pg = jg[split * N + k], pl = jl[split * N + k];
+            const fdw kx = dw_add(fdw{pg.x, pg.y}, dw_neg(gx)), ky = dw_add(fdw{pg.z, pg.w}, dw_neg(gy));
+            const fdw kz = dw_add(fdw{pl.x, pl.y}, dw_neg(gz)), kl = dw_add(fdw{pl.z, pl.w}, gl);
+            jg[split * N + k] = make_float4(kx.hi, kx.lo, ky.hi, ky.lo);
+            jl[split * N + k] = make_float4(kz.hi, kz.lo, kl.hi, kl.lo);
+          }
+        }
+        if (s.use_j2) __syncthreads();
+      }
+      if (have) {  // the thread's own sums to its slot, which only it uses after the barrier
+        const float4 pg = jg[split * N + e], pl = jl[split * N + e];
+        const fdw kx = dw_add(fdw{pg.x, pg.y}, gJx), ky = dw_add(fdw{pg.z, pg.w}, gJy);
+        const fdw kz = dw_add(fdw{pl.x, pl.y}, gJz), kl = dw_add(fdw{pl.z, pl.w}, lJ);
+        jg[split * N + e] = make_float4(kx.hi, kx.lo, ky.hi, ky.lo);
+        jl[split * N + e] = make_float4(kz.hi, kz.lo, kl.hi, kl.lo);
+      }
+      __syncthreads();
+    }
+    // kinetic term of each electron in FP64
+    for (int e = tid; e < N; e += bs) {
+      fdw sx = zero, sy = zero, sz = zero, sl = zero;
+      for (int k = 0; k < R; ++k) {
+        const float4 pg = jg[k * N + e], pl = jl[k * N + e];
+        sx = dw_add(sx, fdw{pg.x, pg.y});
+        sy = dw_add(sy, fdw{pg.z, pg.w});
+        sz = dw_add(sz, fdw{pl.x, pl.y});
+        sl = dw_add(sl, fdw{pl.z, pl.w});
       }
       if (s.use_j3 && j3buf) {
-        // three/four-body Jastrow of this electron in FP64 on one lane (its
-        // value to J, gradient and Laplacian to the Jastrow sums of every lane)
+        // three/four-body Jastrow of this electron in FP64
         double v3 = 0.0, g3[3] = {0.0, 0.0, 0.0}, l3 = 0.0;
-        if (lane == 0) {
-          const double *pr = r + ((size_t)w * N + e) * 3;
-          j3_electron(s, j3buf + (size_t)w * 6 * s.LJ, eup, pr[0], pr[1], pr[2], &v3, g3, &l3);
-          jv = dw_add(jv, dw_of(v3));
-        }
-        gJx = dw_add(gJx, dw_of(__shfl_sync(0xffffffffu, g3[0], 0)));
-        gJy = dw_add(gJy, dw_of(__shfl_sync(0xffffffffu, g3[1], 0)));
-        gJz = dw_add(gJz, dw_of(__shfl_sync(0xffffffffu, g3[2], 0)));
-        lJ = dw_add(lJ, dw_of(__shfl_sync(0xffffffffu, l3, 0)));
+        const double *pr = r + ((size_t)w * N + e) * 3;
+        j3_electron(s, j3buf + (size_t)w * 6 * s.LJ, e < s.n_up, pr[0], pr[1], pr[2], &v3, g3, &l3);
+        jv = dw_add(jv, dw_of(v3));
+        sx = dw_add(sx, dw_of(g3[0]));
+        sy = dw_add(sy, dw_of(g3[1]));
+        sz = dw_add(sz, dw_of(g3[2]));
+        sl = dw_add(sl, dw_of(l3));
       }
-      if (lane == slot) {
-        kx = gJx;
-        ky = gJy;
-        kz = gJz;
-        kl = lJ;
-        mine = e;
-      }
-      if (++slot == 32 || e + nw >= N) {  // warp-uniform
-        if (mine >= 0) {
-          const double *kd = kin + ((size_t)w * N + mine) * 4;
-          const double gx = static_cast<double>(kx.hi) + kx.lo, gy = static_cast<double>(ky.hi) + ky.lo,
-                       gz = static_cast<double>(kz.hi) + kz.lo, lj = static_cast<double>(kl.hi) + kl.lo;
-          const double t =
-              kd[3] + lj + 2.0 * (kd[0] * gx + kd[1] * gy + kd[2] * gz) + (gx * gx + gy * gy + gz * gz);
-          tkin = dw_add(tkin, dw_of(-0.5 * t));
-        }
-        mine = -1;
-        slot = 0;
-      }
+      const double *kd = kin + ((size_t)w * N + e) * 4;
+      const double gx = static_cast<double>(sx.hi) + sx.lo, gy = static_cast<double>(sy.hi) + sy.lo,
+                   gz = static_cast<double>(sz.hi) + sz.lo, lj = static_cast<double>(sl.hi) + sl.lo;
+      const double t = kd[3] + lj + 2.0 * (kd[0] * gx + kd[1] * gy + kd[2] * gz) + (gx * gx + gy * gy + gz * gz);
+      tkin = dw_add(tkin, dw_of(-0.5 * t));
     }
     // the four sums over the block as double-words (FP32 instructions), FP64 at the end
-    __shared__ float red[4][4][2];
+    __shared__ float red[4][kElocalDwThreads / 32][2];
     fdw a4[4] = {tkin, vee, vei, jv};
   #pragma unroll
     for (int q = 0; q < 4; ++q)
@@ -619,10 +642,9 @@ struct ElocalDw {
     }
 }
 };
-__global__ void __launch_bounds__(128) k_elocal_dw(DevSystem s, const double *__restrict__ r,
-                                                   const double *__restrict__ kin, double *__restrict__ eL,
-                                                   double *__restrict__ parts, double *__restrict__ scal,
-                                                   const double *__restrict__ j3buf) {
+__global__ void __launch_bounds__(kElocalDwThreads)
+    k_elocal_dw(DevSystem s, const double *__restrict__ r, const double *__restrict__ kin, double *__restrict__ eL,
+                double *__restrict__ parts, double *__restrict__ scal, const double *__restrict__ j3buf) {
   ElocalDw::run(s, r, kin, eL, parts, scal, j3buf, blockIdx, gridDim);
 }
 
@@ -630,9 +652,16 @@ cudaError_t launch_elocal_dw(const DevSystem &s, const double *r, const double *
                              cudaStream_t st, double *scal, const double *j3buf) {
   if (W <= 0) return cudaSuccess;
   if (s.use_j3 && !j3buf) return cudaErrorInvalidValue;
-  const size_t smem = ((size_t)(s.N + s.n_atoms) * 6 + (size_t)s.n_atoms * 8) * sizeof(float);
-  return launch_or_record<ElocalDw, 128>(k_elocal_dw, dim3(W), dim3(128), smem, st, s, r, kin, eL, parts, scal,
-                                         j3buf);
+  // threads: 128 where the walkers fill the SMs (32 warps each), more where they do
+  // not; 256 also where a whole number of threads per electron leaves over a
+  // quarter of 128 idle (N = 85: a third).  Grouped launches: 256, one kernel for all.
+  int threads = 128;
+  while (threads < kElocalDwThreads && (long)W * threads < 152L * 1024) threads *= 2;
+  if (threads == 128 && (s.N <= 128 ? 128 / s.N * s.N : 64) < 96) threads = 256;
+  if (group_recorder()) threads = 256;
+  const size_t smem = ElocalDw::smem(s, threads);
+  return launch_or_record<ElocalDw, kElocalDwThreads>(k_elocal_dw, dim3(W), dim3(threads), smem, st, s, r, kin, eL,
+                                                      parts, scal, j3buf);
 }
 
 cudaError_t launch_elocal(const DevSystem &s, const double *r, const double *kin, double *eL, double *parts, int W,
