@@ -192,6 +192,33 @@ __device__ __forceinline__ void block_sum2(double &a, double &b, double *red) {
   }
 }
 
+// The sums over the block of a (non-zero only in the first na threads) and b (the
+// first nb), in FP64, valid in warp 0; pa, pb: a number per thread each.  The FP64
+// pipe takes 16 clocks per warp instruction and 165 to its result, so one warp adds
+// all the numbers, a few chains per lane (each of sixteen warps reducing its own,
+// then one thread adding theirs: 10 thousand clocks per move at N = 512; now 2).
+template <typename P>
+__device__ __forceinline__ void block_sum2_first(P a, P b, P *pa, P *pb, int na, int nb, double &sa, double &sb) {
+  pa[threadIdx.x] = a;
+  pb[threadIdx.x] = b;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    double x[2] = {0.0, 0.0}, y[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int k = threadIdx.x; k < na; k += 64) {
+#pragma unroll
+      for (int q = 0; q < 2; ++q)
+        if (k + 32 * q < na) x[q] += static_cast<double>(pa[k + 32 * q]);
+    }
+    for (int k = threadIdx.x; k < nb; k += 128) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (k + 32 * q < nb) y[q] += static_cast<double>(pb[k + 32 * q]);
+    }
+    sa = warp_sum(x[0] + x[1]);
+    sb = warp_sum((y[0] + y[1]) + (y[2] + y[3]));
+  }
+}
+
 // ---------------------------------------------------------------------------
 // Sequential single-electron Metropolis for one spin species (Sec. VMC).
 // One CTA per walker; G~^{-1} lives in shared memory for the whole half-sweep
@@ -218,16 +245,45 @@ __device__ __forceinline__ double accept_prob(double pr, double pj) {
   return pr * pr * exp(2.0 * pj);
 }
 
+// A warp copies a row of L numbers, eight loads in flight per lane (of 16 bytes where
+// the rows allow it).
+template <typename V>
+__device__ __forceinline__ void copy_vec(V *__restrict__ dst, const V *__restrict__ src, int L, int lane) {
+  for (int t0 = lane; t0 < L; t0 += 256) {
+    V v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (t0 + 32 * i < L) v[i] = src[t0 + 32 * i];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (t0 + 32 * i < L) dst[t0 + 32 * i] = v[i];
+  }
+}
+template <typename T>
+__device__ __forceinline__ void copy_row(T *__restrict__ dst, const T *__restrict__ src, int L, int lane) {
+  constexpr int kPer = 16 / sizeof(T);
+  if (L % kPer == 0)  // (every row then starts on a 16-byte boundary, as the tables do)
+    copy_vec(reinterpret_cast<float4 *>(dst), reinterpret_cast<const float4 *>(src), L / kPer, lane);
+  else
+    copy_vec(dst, src, L, lane);
+}
+
+// pitch of G~^{-1} in shared memory: odd, so that a column's entries (the ratio of
+// an up move, the rows summed by a down move's threads) lie in different banks
+__host__ __device__ inline int metro_pitch(int n) { return n | 1; }
+
 template <typename T>
 __host__ __device__ inline size_t metro_smem_per_walker(int n, int N) {
   // positions (FP64), G~^{-1}, three n-vectors, and in the mixed path the FP32
   // mirror of the positions
   const size_t mirror = std::is_same<T, float>::value ? (size_t)N * 3 * sizeof(float) : 0;
-  return ((size_t)N * 3 * sizeof(double) + (size_t)(n * n + 3 * n) * sizeof(T) + mirror + 15) & ~size_t(15);
+  return ((size_t)N * 3 * sizeof(double) + (size_t)(n * metro_pitch(n) + 3 * n) * sizeof(T) + mirror + 15) & ~size_t(15);
 }
 
 template <bool UP, typename T>
 struct Metropolis {
+  // at most 256 threads; 80 registers, so that 900 walkers of N_up <= 64 are resident
+  static constexpr int kMinBlocks = 3;
   static __device__ __forceinline__ void run(DevSystem s, double *__restrict__ r, const double *__restrict__ rprop,
                                              const T *__restrict__ gprop, T *__restrict__ ginv,
                                              double *__restrict__ scal, int *__restrict__ status,
@@ -239,11 +295,12 @@ struct Metropolis {
     assume_global(r, rprop, gprop, ginv, scal, status, pprop, phi_up, list, count);
     extern __shared__ double sm[];
     const int n = s.n_up, N = s.N, tid = threadIdx.x, bs = blockDim.x;
+    const int np = metro_pitch(n);
     const int w = bid.x;
     T *gw = ginv + (size_t)w * n * n;
     double *xs = sm;                                  // N * 3 positions (FP64)
-    T *Gi = reinterpret_cast<T *>(xs + N * 3);        // n * n  G~^{-1}
-    T *gp = Gi + n * n;                               // n
+    T *Gi = reinterpret_cast<T *>(xs + N * 3);        // n * np  G~^{-1}
+    T *gp = Gi + n * np;                              // n
     T *vv = gp + n;                                   // n
     T *cc = vv + n;                                   // n
     float *xf = reinterpret_cast<float *>(cc + n);    // mixed path: N * 3 positions rounded to FP32
@@ -257,10 +314,29 @@ struct Metropolis {
     double *chi_o = j3v + 6 * LJ, *chi_n = chi_o + LJ, *dchi = chi_n + LJ;
     if (j3)
       for (int t = tid; t < 6 * LJ; t += bs) j3v[t] = j3buf[(size_t)w * 6 * LJ + t];
-    __shared__ double red[64];
-    __shared__ int s_acc;
+    // per-thread (at most 256) terms of the ratio and of dJ: T, or FP64 with a
+    // three-body Jastrow
+    __shared__ double part[512];
+    __shared__ int s_acc, s_base;
+    __shared__ short moves[256];  // accepted (at most n <= bs)
+    int nmv = 0;
     __shared__ double s_R;
-    for (int t = tid; t < n * n; t += bs) Gi[t] = gw[t];
+    // entry (j, k) of a thread's first element of G~^{-1}, and the steps to its next
+    const int j0 = tid / n, k0 = tid - j0 * n, dj = bs / n, dk = bs - dj * n;
+    auto entries = [&](auto f) {
+      int j = j0, k = k0;
+#pragma unroll 2
+      for (int idx = tid; idx < n * n; idx += bs) {
+        f(idx, j, k);
+        j += dj;
+        k += dk;
+        if (k >= n) {
+          k -= n;
+          ++j;
+        }
+      }
+    };
+    entries([&](int idx, int j, int k) { Gi[j * np + k] = gw[idx]; });
     for (int t = tid; t < N * 3; t += bs) {
       xs[t] = r[(size_t)w * N * 3 + t];
       if constexpr (kF32) xf[t] = static_cast<float>(xs[t]);
@@ -275,24 +351,37 @@ struct Metropolis {
     }
     const int nmoves = m_end < (UP ? s.n_up : s.n_dn) ? m_end : (UP ? s.n_up : s.n_dn);
     const int e0 = UP ? 0 : s.n_up;
+    // the next move's record and proposed row or column load while a move is decided
+    // (n <= bs: a thread per element)
+    double rec[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    T gq = T(0);
+    auto fetch = [&](int m) {
+      const double *q = rprop + ((size_t)w * n + m) * kPropStride;
+#pragma unroll
+      for (int i = 0; i < 5; ++i) rec[i] = q[i];
+      if (tid < n) gq = gprop[((size_t)w * n + m) * n + tid];
+    };
+    if (m_begin < nmoves) fetch(m_begin);
     __syncthreads();
     for (int m = m_begin; m < nmoves; ++m) {
       const int e = e0 + m;
-      const double *rp4 = rprop + ((size_t)w * n + m) * kPropStride;
-      const double px = rp4[0], py = rp4[1], pz = rp4[2];
-      for (int t = tid; t < n; t += bs) gp[t] = gprop[((size_t)w * n + m) * n + t];
-      __syncthreads();
+      const double px = rec[0], py = rec[1], pz = rec[2], u = rec[3], dj1 = rec[4];
       T prt = T(0);
       double pj = 0.0;
-      for (int t = tid; t < n; t += bs) prt += UP ? gp[t] * Gi[t * n + m] : Gi[m * n + t] * gp[t];
-      double pr = static_cast<double>(prt);
+      if (tid < n) {
+        const T c = UP ? Gi[tid * np + m] : Gi[m * np + tid];
+        gp[tid] = gq;
+        cc[tid] = c;
+        prt = gq * c;
+      }
+      if (m + 1 < nmoves) fetch(m + 1);
       const double ox = xs[3 * e], oy = xs[3 * e + 1], oz = xs[3 * e + 2];
-      if (tid == 0) pj = rp4[4];   // one-body Jastrow change, from the proposal kernel
+      float pjf = 0.0f;
       if (s.use_j2) {
         if constexpr (kF32) {
           const float pf[3] = {static_cast<float>(px), static_cast<float>(py), static_cast<float>(pz)};
           const float of[3] = {xf[3 * e], xf[3 * e + 1], xf[3 * e + 2]};
-          pj += static_cast<double>(j2_move_change_f<UP>(s, xf, e, pf, of, tid, bs));
+          pjf = j2_move_change_f<UP>(s, xf, e, pf, of, tid, bs);
         } else {
           pj += j2_move_change<T, UP>(s, xs, e, px, py, pz, ox, oy, oz, tid, bs);
         }
@@ -319,9 +408,16 @@ struct Metropolis {
           pj = fma(chi_n[mu] - chi_o[mu], Vs[mu] + Va[mu] - mc, pj);
         }
       }
-      block_sum2(pr, pj, red);
+      double pr = 0.0, pjs = 0.0;
+      if (kF32 && !j3) {
+        float *pt = reinterpret_cast<float *>(part);
+        block_sum2_first<float>(static_cast<float>(prt), pjf, pt, pt + bs, n, min(N, bs), pr, pjs);
+      } else {
+        if constexpr (kF32) pj += static_cast<double>(pjf);
+        block_sum2_first<double>(static_cast<double>(prt), pj, part, part + bs, n, j3 ? bs : min(N, bs), pr, pjs);
+      }
       if (tid == 0) {
-        const double u = rp4[3];
+        pj = pjs + dj1;  // with the one-body Jastrow change, from the proposal kernel
         const double p = accept_prob<T>(pr, pj);
         int acc = 0;
         if (!isfinite(p) || !isfinite(pr)) {
@@ -331,34 +427,32 @@ struct Metropolis {
           if (pr < 0.0) sgn = -sgn;
           J += pj;
           nacc += 1.0;
-          list[atomicAdd(count, 1)] = w * n + m;
-          if (total) atomicAdd(total, 1);
+          moves[nmv++] = m;
         }
         s_acc = acc;
         s_R = pr;
       }
       __syncthreads();
       if (s_acc) {
-        for (int t = tid; t < n; t += bs) {
+        if (tid < n) {
           T a = T(0);
           if (UP) {
-            for (int j = 0; j < n; ++j) a += gp[j] * Gi[j * n + t];
-            cc[t] = Gi[t * n + m];
+#pragma unroll 8
+            for (int j = 0; j < n; ++j) a += gp[j] * Gi[j * np + tid];
           } else {
-            for (int i = 0; i < n; ++i) a += Gi[t * n + i] * gp[i];
-            cc[t] = Gi[m * n + t];
+#pragma unroll 8
+            for (int i = 0; i < n; ++i) a += Gi[tid * np + i] * gp[i];
           }
-          vv[t] = a;
+          vv[tid] = a;
         }
         __syncthreads();
         const T invR = T(1) / static_cast<T>(s_R);
-        for (int idx = tid; idx < n * n; idx += bs) {
-          const int j = idx / n, k = idx - j * n;
+        entries([&](int, int j, int k) {
           if (UP)
-            Gi[idx] -= cc[j] * (vv[k] - (k == m ? T(1) : T(0))) * invR;
+            Gi[j * np + k] -= cc[j] * (vv[k] - (k == m ? T(1) : T(0))) * invR;
           else
-            Gi[idx] -= (vv[j] - (j == m ? T(1) : T(0))) * cc[k] * invR;
-        }
+            Gi[j * np + k] -= (vv[j] - (j == m ? T(1) : T(0))) * cc[k] * invR;
+        });
         if (tid == 0) {
           xs[3 * e] = px;
           xs[3 * e + 1] = py;
@@ -368,12 +462,6 @@ struct Metropolis {
             xf[3 * e + 1] = static_cast<float>(py);
             xf[3 * e + 2] = static_cast<float>(pz);
           }
-        }
-        if (UP) {
-          const size_t row = ((size_t)w * n + m) * s.L;
-          for (int t = tid; t < s.L; t += bs) phi_up[row + t] = pprop[row + t];
-          if (phi_lo)
-            for (int t = tid; t < s.L; t += bs) phi_lo[row + t] = pprop_lo[row + t];
         }
         if (j3) {
           // the spin sum and its two products follow the moved electron
@@ -391,12 +479,29 @@ struct Metropolis {
             Ua[mu] += aa;
           }
         }
+        __syncthreads();
       }
-      __syncthreads();
     }
+    // the accepted moves: one entry each in the list of changed rows, and (up) the
+    // proposed orbitals to the table.  After the loop, because the atomic's and the
+    // copies' latency there held up every accepted move of the chain.
+    if (tid == 0) {
+      s_acc = nmv;
+      s_base = nmv ? atomicAdd(count, nmv) : 0;
+      if (total && nmv) atomicAdd(total, nmv);
+    }
+    __syncthreads();
+    const int na = s_acc;
+    for (int t = tid; t < na; t += bs) list[s_base + t] = w * n + moves[t];
+    if (UP)
+      for (int q = tid >> 5; q < na; q += bs >> 5) {
+        const size_t row = ((size_t)w * n + moves[q]) * s.L;
+        copy_row(phi_up + row, pprop + row, s.L, tid & 31);
+        if (phi_lo) copy_row(phi_lo + row, pprop_lo + row, s.L, tid & 31);
+      }
     if (j3)
       for (int t = tid; t < 6 * LJ; t += bs) j3buf[(size_t)w * 6 * LJ + t] = j3v[t];
-    for (int t = tid; t < n * n; t += bs) gw[t] = Gi[t];
+    entries([&](int idx, int j, int k) { gw[idx] = Gi[j * np + k]; });
     for (int t = tid; t < N * 3; t += bs) r[(size_t)w * N * 3 + t] = xs[t];
     if (tid == 0) {
       scal[(size_t)w * S_STRIDE + S_SIGN] = sgn;
@@ -407,7 +512,7 @@ struct Metropolis {
 }
 };
 template <bool UP, typename T>
-__global__ void __launch_bounds__(512) k_metropolis(DevSystem s, double *__restrict__ r,
+__global__ void __launch_bounds__(256, (Metropolis<UP, T>::kMinBlocks)) k_metropolis(DevSystem s, double *__restrict__ r,
                                                     const double *__restrict__ rprop, const T *__restrict__ gprop,
                                                     T *__restrict__ ginv, double *__restrict__ scal,
                                                     int *__restrict__ status, const T *__restrict__ pprop,
@@ -451,10 +556,12 @@ struct MetropolisBig {
     T *gp = Gs + (size_t)rs * n;                      // n
     T *vv = gp + n;                                   // n
     T *cc = vv + n;                                   // n
-    float *xf = reinterpret_cast<float *>(cc + n);    // mixed path: N * 3 positions rounded to FP32
+    int *moves = reinterpret_cast<int *>(cc + n);     // n accepted moves
+    float *xf = reinterpret_cast<float *>(moves + n);  // mixed path: N * 3 positions rounded to FP32
     constexpr bool kF32 = std::is_same<T, float>::value;
-    __shared__ double red[64];
-    __shared__ int s_acc;
+    __shared__ T part[2 * 512];  // per-thread terms of the ratio and of dJ
+    __shared__ int s_acc, s_base;
+    int nmv = 0;
     __shared__ double s_R;
     for (int t = tid; t < rs * n; t += bs) Gs[t] = gw[t];
     for (int t = tid; t < N * 3; t += bs) {
@@ -471,15 +578,25 @@ struct MetropolisBig {
     }
     const int nmoves = m_end < (UP ? s.n_up : s.n_dn) ? m_end : (UP ? s.n_up : s.n_dn);
     const int e0 = UP ? 0 : s.n_up;
+    // the next move's record and proposed row or column (a thread's first element)
+    // load while a move is decided
+    double rec[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    T gq = T(0);
+    auto fetch = [&](int m) {
+      const double *q = rprop + ((size_t)w * n + m) * kPropStride;
+#pragma unroll
+      for (int i = 0; i < 5; ++i) rec[i] = q[i];
+      if (tid < n) gq = gprop[((size_t)w * n + m) * n + tid];
+    };
+    if (m_begin < nmoves) fetch(m_begin);
     __syncthreads();
     for (int m = m_begin; m < nmoves; ++m) {
       const int e = e0 + m;
-      const double *rp4 = rprop + ((size_t)w * n + m) * kPropStride;
-      const double px = rp4[0], py = rp4[1], pz = rp4[2];
+      const double px = rec[0], py = rec[1], pz = rec[2], u = rec[3], dj1 = rec[4];
       // the move's column (up) or row (down) of G~^{-1} and the proposed row or column of G~
       T prt = T(0);
       for (int t = tid; t < n; t += bs) {
-        const T g = gprop[((size_t)w * n + m) * n + t];
+        const T g = t == tid ? gq : gprop[((size_t)w * n + m) * n + t];
         T c;
         if (UP)
           c = t < rs ? Gs[t * n + m] : gw[(size_t)t * n + m];
@@ -489,21 +606,22 @@ struct MetropolisBig {
         cc[t] = c;
         prt += UP ? g * c : c * g;
       }
-      double pr = static_cast<double>(prt), pj = 0.0;
+      if (m + 1 < nmoves) fetch(m + 1);
+      T pjt = T(0);
       const double ox = xs[3 * e], oy = xs[3 * e + 1], oz = xs[3 * e + 2];
-      if (tid == 0) pj = rp4[4];   // one-body Jastrow change, from the proposal kernel
       if (s.use_j2) {
         if constexpr (kF32) {
           const float pf[3] = {static_cast<float>(px), static_cast<float>(py), static_cast<float>(pz)};
           const float of[3] = {xf[3 * e], xf[3 * e + 1], xf[3 * e + 2]};
-          pj += static_cast<double>(j2_move_change_f<UP>(s, xf, e, pf, of, tid, bs));
+          pjt = j2_move_change_f<UP>(s, xf, e, pf, of, tid, bs);
         } else {
-          pj += j2_move_change<T, UP>(s, xs, e, px, py, pz, ox, oy, oz, tid, bs);
+          pjt = j2_move_change<T, UP>(s, xs, e, px, py, pz, ox, oy, oz, tid, bs);
         }
       }
-      block_sum2(pr, pj, red);
+      double pr = 0.0, pj = 0.0;
+      block_sum2_first<T>(prt, pjt, part, part + 512, min(n, bs), min(N, bs), pr, pj);
       if (tid == 0) {
-        const double u = rp4[3];
+        pj += dj1;  // the one-body Jastrow change, from the proposal kernel
         const double p = accept_prob<T>(pr, pj);
         int acc = 0;
         if (!isfinite(p) || !isfinite(pr)) {
@@ -513,8 +631,7 @@ struct MetropolisBig {
           if (pr < 0.0) sgn = -sgn;
           J += pj;
           nacc += 1.0;
-          list[atomicAdd(count, 1)] = w * n + m;
-          if (total) atomicAdd(total, 1);
+          moves[nmv++] = m;
         }
         s_acc = acc;
         s_R = pr;
@@ -590,17 +707,26 @@ struct MetropolisBig {
             xf[3 * e + 2] = static_cast<float>(pz);
           }
         }
-        if (UP) {
-          const size_t row = ((size_t)w * n + m) * s.L;
-  #pragma unroll 4
-          for (int t = tid; t < s.L; t += bs) phi_up[row + t] = pprop[row + t];
-          if (phi_lo)
-  #pragma unroll 4
-            for (int t = tid; t < s.L; t += bs) phi_lo[row + t] = pprop_lo[row + t];
-        }
+        __syncthreads();
       }
-      __syncthreads();
     }
+    // the accepted moves: one entry each in the list of changed rows, and (up) the
+    // proposed orbitals to the table.  After the loop, because the atomic's and the
+    // copies' latency there held up every accepted move of the chain.
+    if (tid == 0) {
+      s_acc = nmv;
+      s_base = nmv ? atomicAdd(count, nmv) : 0;
+      if (total && nmv) atomicAdd(total, nmv);
+    }
+    __syncthreads();
+    const int na = s_acc;
+    for (int t = tid; t < na; t += bs) list[s_base + t] = w * n + moves[t];
+    if (UP)
+      for (int q = tid >> 5; q < na; q += bs >> 5) {
+        const size_t row = ((size_t)w * n + moves[q]) * s.L;
+        copy_row(phi_up + row, pprop + row, s.L, tid & 31);
+        if (phi_lo) copy_row(phi_lo + row, pprop_lo + row, s.L, tid & 31);
+      }
     for (int t = tid; t < rs * n; t += bs) gw[t] = Gs[t];
     for (int t = tid; t < N * 3; t += bs) r[(size_t)w * N * 3 + t] = xs[t];
     if (tid == 0) {
@@ -883,9 +1009,10 @@ constexpr size_t kMetroSmemMax = 200 * 1024;  // G~^{-1} kept in shared memory u
 
 template <bool UP, typename T>
 struct MetropolisWarp {
-  // latency-bound (one walker's sequential moves per warp): keep six CTAs of
-  // four warps resident per SM
-  static constexpr int kMinBlocks = 6;
+  // latency-bound (one walker's sequential moves per warp): keep eight CTAs of four
+  // warps resident per SM, six in FP64 (4096 walkers in one wave; with five the
+  // second wave of 16 He was a third full)
+  static constexpr int kMinBlocks = std::is_same<T, float>::value ? 8 : 6;
   static __device__ __forceinline__ void run(DevSystem s, double *__restrict__ r, const double *__restrict__ rprop,
                                              const T *__restrict__ gprop, T *__restrict__ ginv,
                                              double *__restrict__ scal, int *__restrict__ status,
@@ -896,18 +1023,33 @@ struct MetropolisWarp {
                                              const uint3 gdim) {
     assume_global(r, rprop, gprop, ginv, scal, status, pprop, phi_up, list, count);
     extern __shared__ double sm[];
-    const int n = s.n_up, N = s.N, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int n = s.n_up, N = s.N, np = metro_pitch(n), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int w = bid.x * kMetroWarps + warp;
     if (w >= W) return;  // warp-uniform; the kernel has no block-wide barrier
     double *xs = reinterpret_cast<double *>(reinterpret_cast<char *>(sm) + warp * metro_smem_per_walker<T>(n, N));
     T *Gi = reinterpret_cast<T *>(xs + N * 3);
-    T *gp = Gi + n * n;
+    T *gp = Gi + n * np;
     T *vv = gp + n;
     T *cc = vv + n;
     float *xf = reinterpret_cast<float *>(cc + n);  // mixed path: N * 3 positions rounded to FP32
     constexpr bool kF32 = std::is_same<T, float>::value;
     T *gw = ginv + (size_t)w * n * n;
-    for (int t = lane; t < n * n; t += 32) Gi[t] = gw[t];
+    // entry (j, k) of a lane's first element of G~^{-1}, and the steps to its next
+    const int j0 = lane / n, k0 = lane - j0 * n, dj = 32 / n, dk = 32 - dj * n;
+    auto entries = [&](auto f) {
+      int j = j0, k = k0;
+#pragma unroll 2
+      for (int idx = lane; idx < n * n; idx += 32) {
+        f(idx, j, k);
+        j += dj;
+        k += dk;
+        if (k >= n) {
+          k -= n;
+          ++j;
+        }
+      }
+    };
+    entries([&](int idx, int j, int k) { Gi[j * np + k] = gw[idx]; });
     for (int t = lane; t < N * 3; t += 32) {
       xs[t] = r[(size_t)w * N * 3 + t];
       if constexpr (kF32) xf[t] = static_cast<float>(xs[t]);
@@ -915,21 +1057,36 @@ struct MetropolisWarp {
     double *sw = scal + (size_t)w * S_STRIDE;
     double sgn = sw[S_SIGN], J = sw[S_J], nacc = sw[S_NACC];
     int st_bits = status[w];
+    unsigned moves = 0u;  // accepted
     const int nmoves = m_end < (UP ? s.n_up : s.n_dn) ? m_end : (UP ? s.n_up : s.n_dn);
     const int e0 = UP ? 0 : s.n_up;
+    // the next move's record and proposed row or column (n <= 32: an element per
+    // lane) load while a move is decided
+    double rnext[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    T gq = T(0);
+    auto fetch = [&](int m) {
+      const double *q = rprop + ((size_t)w * n + m) * kPropStride;
+#pragma unroll
+      for (int i = 0; i < 5; ++i) rnext[i] = q[i];
+      if (lane < n) gq = gprop[((size_t)w * n + m) * n + lane];
+    };
+    if (m_begin < nmoves) fetch(m_begin);
     __syncwarp();
     for (int m = m_begin; m < nmoves; ++m) {
       const int e = e0 + m;
-      const double *rec = rprop + ((size_t)w * n + m) * kPropStride;
+      double rec[5];
+#pragma unroll
+      for (int i = 0; i < 5; ++i) rec[i] = rnext[i];
       const double px = rec[0], py = rec[1], pz = rec[2];
-      const T *grow = gprop + ((size_t)w * n + m) * n;
       T prt = T(0);
       double pj = 0.0;
-      for (int t = lane; t < n; t += 32) {
-        const T g = grow[t];
-        gp[t] = g;
-        prt += UP ? g * Gi[t * n + m] : Gi[m * n + t] * g;
+      if (lane < n) {
+        const T c = UP ? Gi[lane * np + m] : Gi[m * np + lane];
+        gp[lane] = gq;
+        cc[lane] = c;
+        prt = gq * c;
       }
+      if (m + 1 < nmoves) fetch(m + 1);
       double pr;
       if constexpr (kF32) {
         // ratio and two-body change summed in FP32 (the acceptance test's precision)
@@ -961,45 +1118,50 @@ struct MetropolisWarp {
         if (pr < 0.0) sgn = -sgn;
         J += pj;
         nacc += 1.0;
-        if (lane == 0) {
-          list[atomicAdd(count, 1)] = w * n + m;
-          if (total) atomicAdd(total, 1);
-        }
-        for (int t = lane; t < n; t += 32) {
+        moves |= 1u << m;
+        if (lane < n) {
           T a = T(0);
           if (UP) {
-            for (int j = 0; j < n; ++j) a = fma(gp[j], Gi[j * n + t], a);
-            cc[t] = Gi[t * n + m];
+#pragma unroll 8
+            for (int j = 0; j < n; ++j) a = fma(gp[j], Gi[j * np + lane], a);
           } else {
-            for (int i = 0; i < n; ++i) a = fma(Gi[t * n + i], gp[i], a);
-            cc[t] = Gi[m * n + t];
+#pragma unroll 8
+            for (int i = 0; i < n; ++i) a = fma(Gi[lane * np + i], gp[i], a);
           }
-          vv[t] = a;
+          vv[lane] = a;
         }
         __syncwarp();
         const T invR = T(1) / static_cast<T>(pr);
-        for (int idx = lane; idx < n * n; idx += 32) {
-          const int j = idx / n, k = idx - j * n;
+        entries([&](int, int j, int k) {
           if (UP)
-            Gi[idx] -= cc[j] * (vv[k] - (k == m ? T(1) : T(0))) * invR;
+            Gi[j * np + k] -= cc[j] * (vv[k] - (k == m ? T(1) : T(0))) * invR;
           else
-            Gi[idx] -= (vv[j] - (j == m ? T(1) : T(0))) * cc[k] * invR;
-        }
+            Gi[j * np + k] -= (vv[j] - (j == m ? T(1) : T(0))) * cc[k] * invR;
+        });
         if (lane < 3) {
           const double v = lane == 0 ? px : (lane == 1 ? py : pz);
           xs[3 * e + lane] = v;
           if constexpr (kF32) xf[3 * e + lane] = static_cast<float>(v);
         }
-        if (UP) {
-          const size_t row = ((size_t)w * n + m) * s.L;
-          for (int t = lane; t < s.L; t += 32) phi_up[row + t] = pprop[row + t];
-          if (phi_lo)
-            for (int t = lane; t < s.L; t += 32) phi_lo[row + t] = pprop_lo[row + t];
-        }
         __syncwarp();
       }
     }
-    for (int t = lane; t < n * n; t += 32) gw[t] = Gi[t];
+    // the accepted moves' entries in the list of changed rows and their orbitals,
+    // after the loop as in the kernel above
+    int base = 0;
+    if (lane == 0 && moves) {
+      base = atomicAdd(count, __popc(moves));
+      if (total) atomicAdd(total, __popc(moves));
+    }
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if ((moves >> lane) & 1u) list[base + __popc(moves & ((1u << lane) - 1u))] = w * n + lane;
+    if (UP)
+      for (unsigned q = moves; q; q &= q - 1u) {
+        const size_t row = ((size_t)w * n + (__ffs(q) - 1)) * s.L;
+        copy_row(phi_up + row, pprop + row, s.L, lane);
+        if (phi_lo) copy_row(phi_lo + row, pprop_lo + row, s.L, lane);
+      }
+    entries([&](int idx, int j, int k) { gw[idx] = Gi[j * np + k]; });
     for (int t = lane; t < N * 3; t += 32) r[(size_t)w * N * 3 + t] = xs[t];
     if (lane == 0) {
       sw[S_SIGN] = sgn;
@@ -1010,7 +1172,7 @@ struct MetropolisWarp {
 }
 };
 template <bool UP, typename T>
-__global__ void __launch_bounds__(kMetroWarps * 32) k_metropolis_warp(DevSystem s, double *__restrict__ r,
+__global__ void __launch_bounds__(kMetroWarps * 32, (MetropolisWarp<UP, T>::kMinBlocks)) k_metropolis_warp(DevSystem s, double *__restrict__ r,
     const double *__restrict__ rprop, const T *__restrict__ gprop, T *__restrict__ ginv, double *__restrict__ scal,
     int *__restrict__ status, const T *__restrict__ pprop, T *__restrict__ phi_up, int *__restrict__ list,
     int *__restrict__ count, int W, const float *__restrict__ pprop_lo, float *__restrict__ phi_lo, int m_begin,
@@ -1031,10 +1193,10 @@ cudaError_t launch_metropolis(const DevSystem &s, bool up, double *r, const doub
   // one CTA per walker (threads per CTA, shared memory)
   auto cta = [&](int threads, size_t smem, double *j3) -> cudaError_t {
     if (up)
-      return launch_or_record<Metropolis<true, T>, 512>(k_metropolis<true, T>, dim3(W), dim3(threads), smem, st, s, r,
+      return launch_or_record<Metropolis<true, T>, 256>(k_metropolis<true, T>, dim3(W), dim3(threads), smem, st, s, r,
                                                         rprop, gprop, ginv, scal, status, pprop, phi_up, list, count,
                                                         pprop_lo, phi_lo, m_begin, m_end, total, j3);
-    return launch_or_record<Metropolis<false, T>, 512>(k_metropolis<false, T>, dim3(W), dim3(threads), smem, st, s, r,
+    return launch_or_record<Metropolis<false, T>, 256>(k_metropolis<false, T>, dim3(W), dim3(threads), smem, st, s, r,
                                                        rprop, gprop, ginv, scal, status, pprop, phi_up, list, count,
                                                        pprop_lo, phi_lo, m_begin, m_end, total, j3);
   };
@@ -1057,7 +1219,7 @@ cudaError_t launch_metropolis(const DevSystem &s, bool up, double *r, const doub
   }
   if (per <= kMetroSmemMax) return cta(n <= 64 ? 128 : 256, per, nullptr);
   // as many rows of G~^{-1} in shared memory as fit beside the rest
-  const size_t rest = (size_t)s.N * 3 * sizeof(double) + (size_t)3 * n * sizeof(T) +
+  const size_t rest = (size_t)s.N * 3 * sizeof(double) + (size_t)n * (3 * sizeof(T) + sizeof(int)) +
                       (std::is_same<T, float>::value ? (size_t)s.N * 3 * sizeof(float) : 0);
   const int rs = rest < kMetroSmemMax ? (int)((kMetroSmemMax - rest) / ((size_t)n * sizeof(T))) : 0;
   const size_t smem = rest + (size_t)rs * n * sizeof(T);
@@ -1092,9 +1254,10 @@ __global__ void __launch_bounds__(128) k_jastrow_full(DevSystem s, const double 
       j1 += j1_val(s.c1[a], s.b_ea, sqrt(dx * dx + dy * dy + dz * dz));
     }
   if (s.use_j2)
-    for (int idx = threadIdx.x; idx < N * N; idx += blockDim.x) {
-      const int i = idx / N, j = idx - i * N;
-      if (j <= i) continue;
+    // every pair once: electron i and the one at distance o = 1 .. N / 2 around the
+    // list (N even: the pairs at N / 2 from the first half of the electrons only)
+    for (int idx = threadIdx.x; idx < N * (N - 1) / 2; idx += blockDim.x) {
+      const int o = idx / N + 1, i = idx - (o - 1) * N, j = i + o < N ? i + o : i + o - N;
       double kk, bb;
       j2_params(s, (i < s.n_up) == (j < s.n_up), &kk, &bb);
       const double dx = x[3 * i] - x[3 * j], dy = x[3 * i + 1] - x[3 * j + 1], dz = x[3 * i + 2] - x[3 * j + 2];
