@@ -1088,6 +1088,7 @@ struct RefreshInverseCluster {
         if (warp == 0) {
           unsigned long long key = 0ull;
           int row = lane;
+#pragma unroll 4
           for (int i = lane; i < n; i += 32) {
             const unsigned long long ki = used[i] ? 0ull : abs_key(S[(size_t)i * C + kc]);
             if (ki > key) {
@@ -1107,8 +1108,10 @@ struct RefreshInverseCluster {
         ok = false;
         break;
       }
-      const double ip = recip_newton(pv);
       const bool mine = rank == owner;
+      // (the reciprocal only where a warp has elements of the pivot row: it costs as
+      // much of the FP64 pipe as a third of an update when every warp forms it)
+      const double ip = tid < C ? recip_newton(pv) : 0.0;
       for (int j = tid; j < C; j += kClusterThreads)
         prow[j] = mine && j == kc ? ip : S[(size_t)p * C + j] * ip;
       __syncthreads();
