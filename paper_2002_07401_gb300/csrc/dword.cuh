@@ -69,6 +69,9 @@ __device__ __forceinline__ fdw dw_mul_f(fdw x, float y) {
   return fast_two_sum(c.hi, __fmaf_rn(x.lo, y, c.lo));
 }
 
+// x c, c a power of two: exact
+__device__ __forceinline__ fdw dw_scale(fdw x, float c) { return {__fmul_rn(x.hi, c), __fmul_rn(x.lo, c)}; }
+
 // square root: s = sqrt(hi) refined by one Newton step on the residual
 __device__ __forceinline__ fdw dw_sqrt(fdw x) {
   if (!(x.hi > 0.0f)) return {0.0f, 0.0f};

@@ -366,7 +366,7 @@ template <typename T>
 jagp_status_t run_local_energy(jagp_ctx *h, const double *r, void *state, int W, double *eL, double *parts,
                                cudaStream_t st, bool write_jastrow = false) {
   const Layout L = layout_of(h, W);
-  if (std::is_same<T, float>::value) {
+  if constexpr (std::is_same<T, float>::value) {
     if (h->ds.use_j3) LAUNCH(0, 1, launch_j3_prep(h->ds, r, j3_vectors(h, L, state), W, st));
     const jagp_status_t s = run_kinetic_mixed(h, r, state, W, st);
     if (s != JAGP_OK) return s;
@@ -375,7 +375,7 @@ jagp_status_t run_local_energy(jagp_ctx *h, const double *r, void *state, int W,
     const jagp_status_t s = run_mmat64(h, state, W, st);
     if (s != JAGP_OK) return s;
     LAUNCH(JAGP_KERNEL_ENERGY, 1,
-           launch_kinetic<T>(h->ds, r, at<T>(state, L.mbuf), at<double>(state, L.kin), W, st));
+           launch_kinetic(h->ds, r, at<double>(state, L.mbuf), at<double>(state, L.kin), W, st));
   }
   double *sc = write_jastrow ? at<double>(state, L.scal) : nullptr;
   if (std::is_same<T, float>::value)
@@ -948,6 +948,7 @@ jagp_status_t jagp_create(jagp_handle_t *out, const jagp_system_t *sys, const ja
   const size_t oR = take(na * 3 * 8), oZ = take(na * 8), oC = take(na * 8);
   const size_t oG = take(sys->n_shells * sizeof(double4)), oI = take(sys->n_shells * sizeof(int));
   const size_t oGd = take(sys->n_shells * 2 * sizeof(float4));
+  const size_t oSt = take(sys->n_shells * sizeof(int));
   const size_t oSa = take(sys->n_shells * sizeof(int)), oSf = take((na + 1) * sizeof(int));
   const size_t oAf = take(na * sizeof(float4));
   const size_t oL = take((size_t)L * L * 8), oT = take((size_t)L * L * 8);
@@ -1008,6 +1009,7 @@ jagp_status_t jagp_create(jagp_handle_t *out, const jagp_system_t *sys, const ja
             cudaMemcpy(b + oGd, geo_dw.data(), sys->n_shells * 2 * sizeof(float4), cudaMemcpyHostToDevice) ==
                 cudaSuccess &&
             cudaMemcpy(b + oI, info.data(), sys->n_shells * sizeof(int), cudaMemcpyHostToDevice) == cudaSuccess &&
+            cudaMemcpy(b + oSt, satom.data(), sys->n_shells * sizeof(int), cudaMemcpyHostToDevice) == cudaSuccess &&
             cudaMemcpy(b + oSa, ashell.data(), sys->n_shells * sizeof(int), cudaMemcpyHostToDevice) == cudaSuccess &&
             cudaMemcpy(b + oSf, afirst.data(), (na + 1) * sizeof(int), cudaMemcpyHostToDevice) == cudaSuccess &&
             cudaMemcpy(b + oAf, atom_f.data(), na * sizeof(float4), cudaMemcpyHostToDevice) == cudaSuccess &&
@@ -1045,6 +1047,7 @@ jagp_status_t jagp_create(jagp_handle_t *out, const jagp_system_t *sys, const ja
   d.shell_geo = reinterpret_cast<const double4 *>(b + oG);
   d.shell_dw = reinterpret_cast<const float4 *>(b + oGd);
   d.shell_info = reinterpret_cast<const int *>(b + oI);
+  d.shell_atom = reinterpret_cast<const int *>(b + oSt);
   d.atom_shells = reinterpret_cast<const int *>(b + oSa);
   d.atom_first = reinterpret_cast<const int *>(b + oSf);
   d.lam = reinterpret_cast<const double *>(b + oL);

@@ -3,6 +3,7 @@
 // Everything here is the GPU path's own code; the CPU oracle shares none of it.
 #pragma once
 
+#include <type_traits>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -41,6 +42,7 @@ struct DevSystem {
   const double4 *shell_geo; // [n_shells]
   const float4 *shell_dw;   // [n_shells][2]: (x, y, z, zeta) rounded to FP32, then the remainders
   const int *shell_info;    // [n_shells]
+  const int *shell_atom;    // [n_shells]
   // an atom's shells as positions in the shell table: atom_shells[atom_first[a]] .. [atom_first[a + 1] - 1]
   const int *atom_first, *atom_shells;
   const double *lam;        // [L][L]
@@ -212,10 +214,10 @@ __device__ __forceinline__ double radial_factor(int rad, double zeta, double r2)
 }
 
 // FP64 path: values only, at the displacement (dx, dy, dz) from the shell's
-// atom; returns the number of components written to v.
-__device__ __forceinline__ int shell_values(int info, double zeta, double dx, double dy, double dz, double v[5]) {
+// atom, r2 = dx^2 + dy^2 + dz^2; returns the number of components written to v.
+__device__ __forceinline__ int shell_values(int info, double zeta, double dx, double dy, double dz, double r2,
+                                            double v[5]) {
   const int l = shell_l(info);
-  const double r2 = dx * dx + dy * dy + dz * dz;
   const double g = radial_factor(shell_rad(info), zeta, r2);
   if (l == 0) {
     v[0] = g;
@@ -230,26 +232,117 @@ __device__ __forceinline__ int shell_values(int info, double zeta, double dx, do
   v[0] = dx * dy * g;
   v[1] = dy * dz * g;
   v[2] = dz * dx * g;
-  v[3] = (dx * dx - dy * dy) * g;
+  v[3] = __dadd_rn(__dmul_rn(dx, dx), -__dmul_rn(dy, dy)) * g;
   v[4] = (3.0 * dz * dz - r2) * g;
   return 5;
 }
+// r^2 as the orbitals round it (written out so that every caller gets the same bits)
+__device__ __forceinline__ double square_of(double dx, double dy, double dz) {
+  return __fma_rn(dz, dz, __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)));
+}
+__device__ __forceinline__ int shell_values(int info, double zeta, double dx, double dy, double dz, double v[5]) {
+  return shell_values(info, zeta, dx, dy, dz, square_of(dx, dy, dz), v);
+}
 
-// FP32 path: the displacement d = r - R_a of a point from the shell's atom in
-// double-word, from the point's and the atom's double-word coordinates (the
-// atom's split once on the host: geo_hi = (x, y, z, zeta) rounded to FP32,
-// geo_lo = the remainders).
-struct DwDisp {
+// A point's displacement from an atom and its square, in FP64 or (FP32 path) in
+// double-word from the double-word coordinates of both
+struct alignas(16) Disp {
+  double x, y, z, r2;
+};
+struct alignas(16) DwDisp {
   fdw x, y, z, r2;
 };
-__device__ __forceinline__ DwDisp dw_displacement(const fdw p[3], float4 geo_hi, float4 geo_lo) {
+__device__ __forceinline__ Disp displacement(const double p[3], const double R[3]) {
+  Disp d;
+  d.x = p[0] - R[0];
+  d.y = p[1] - R[1];
+  d.z = p[2] - R[2];
+  d.r2 = square_of(d.x, d.y, d.z);
+  return d;
+}
+__device__ __forceinline__ DwDisp displacement(const fdw p[3], const fdw R[3]) {
   DwDisp d;
-  d.x = dw_add(p[0], fdw{-geo_hi.x, -geo_lo.x});
-  d.y = dw_add(p[1], fdw{-geo_hi.y, -geo_lo.y});
-  d.z = dw_add(p[2], fdw{-geo_hi.z, -geo_lo.z});
+  d.x = dw_add(p[0], dw_neg(R[0]));
+  d.y = dw_add(p[1], dw_neg(R[1]));
+  d.z = dw_add(p[2], dw_neg(R[2]));
   d.r2 = dw_add(dw_add(dw_mul(d.x, d.x), dw_mul(d.y, d.y)), dw_mul(d.z, d.z));
   return d;
 }
+
+// The shells and atoms in shared memory for kernels with a warp per point and its
+// lanes over the shells, and a point's displacements from the atoms: formed once
+// per atom (an atom has several shells: eight in the 20-function recipe, whose
+// displacements and squares were a quarter of the instructions of a shell's value)
+// into the warp's table, unless shared memory has no room for one (some thousand
+// atoms): then per shell.  kDw: double-words, else FP64.
+template <bool kDw>
+struct ShellStage {
+  using Num = typename std::conditional<kDw, fdw, double>::type;
+  using D = typename std::conditional<kDw, DwDisp, Disp>::type;
+  static_assert(sizeof(Num) == 8 && sizeof(D) == 32, "two FP32 numbers or one FP64 number");
+  static constexpr int kWarps = 8;
+  D *tab;      // [atoms] of this warp, or null
+  Num *zeta;   // [shells]
+  Num *R;      // [atoms][3]
+  int *info, *atom;
+  int n_atoms;
+  static __host__ __device__ size_t bytes(const DevSystem &s, int tables) {
+    return (size_t)s.n_atoms * (32 * tables + 24) + (size_t)s.n_shells * 16;
+  }
+  // warps per CTA (eight, fewer where that leaves room for two CTAs on an SM) and tables (0 or one per warp)
+  static void plan(const DevSystem &s, int *warps, int *tables) {
+    int w = kWarps;
+    while (w > 1 && bytes(s, w) > 112 * 1024) w /= 2;
+    *tables = bytes(s, w) <= 200 * 1024 ? w : 0;
+    *warps = *tables ? w : kWarps;
+  }
+  __device__ __forceinline__ ShellStage(const DevSystem &s, void *sm, int tables) : n_atoms(s.n_atoms) {
+    D *t = static_cast<D *>(sm);
+    zeta = reinterpret_cast<Num *>(t + (size_t)tables * n_atoms);
+    R = zeta + s.n_shells;
+    info = reinterpret_cast<int *>(R + 3 * n_atoms);
+    atom = info + s.n_shells;
+    tab = tables ? t + (size_t)(threadIdx.x >> 5) * n_atoms : nullptr;
+    for (int k = threadIdx.x; k < s.n_shells; k += blockDim.x) {
+      if constexpr (kDw)
+        zeta[k] = fdw{s.shell_dw[2 * k].w, s.shell_dw[2 * k + 1].w};
+      else
+        zeta[k] = s.shell_geo[k].w;
+      info[k] = s.shell_info[k];
+      atom[k] = s.shell_atom[k];
+    }
+    for (int t3 = threadIdx.x; t3 < 3 * n_atoms; t3 += blockDim.x) {
+      if constexpr (kDw)
+        R[t3] = dw_of(s.R[t3]);
+      else
+        R[t3] = s.R[t3];
+    }
+    __syncthreads();
+  }
+  // this warp's table for the point p
+  __device__ __forceinline__ void point(const Num p[3], int lane) {
+    if (!tab) return;
+    __syncwarp();
+    for (int a = lane; a < n_atoms; a += 32) {
+      const D d = displacement(p, R + 3 * a);
+      float4 *q = reinterpret_cast<float4 *>(tab + a);
+      const float4 *v = reinterpret_cast<const float4 *>(&d);
+      q[0] = v[0];
+      q[1] = v[1];
+    }
+    __syncwarp();
+  }
+  // the point's displacement from shell k's atom
+  __device__ __forceinline__ D disp(const Num p[3], int k) const {
+    if (!tab) return displacement(p, R + 3 * atom[k]);
+    D d;
+    const float4 *q = reinterpret_cast<const float4 *>(tab + atom[k]);
+    float4 *v = reinterpret_cast<float4 *>(&d);
+    v[0] = q[0];
+    v[1] = q[1];
+    return d;
+  }
+};
 
 // the radial factor as a double-word (relative error a few units of 2^-46)
 __device__ __forceinline__ fdw radial_dw(int rad, fdw zeta, fdw r2) {

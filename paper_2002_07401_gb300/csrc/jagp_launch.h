@@ -81,8 +81,7 @@ cudaError_t launch_j3_prep(const DevSystem &s, const double *r, double *buf, int
 template <typename T>
 cudaError_t launch_mmat(const DevSystem &s, const T *ginv, const T *bt, const T *a_up, T *mbuf, int W,
                         cudaStream_t st);
-template <typename T>
-cudaError_t launch_kinetic(const DevSystem &s, const double *r, const T *mbuf, double *kin, int W,
+cudaError_t launch_kinetic(const DevSystem &s, const double *r, const double *mbuf, double *kin, int W,
                            cudaStream_t st);
 // the mixed path's two-float M vectors on the CUDA cores (small N_up): compensated
 // sums of the FP64 inverse against the two-float Bt / A_up tables

@@ -26,26 +26,17 @@ namespace jagp {
 //   sum_c M_c grad(P_c g) = g (Sg - zeta S0 d / r),
 //   sum_c M_c lap(P_c g)  = g S0 (zeta^2 - 2 zeta (l + 1) / r).
 //
-// FP64 path: FP64 throughout.  FP32 path: the displacement, r^2 and the radial
-// factor in double-word (FP32 instructions only, see dword.cuh) so that g is
-// accurate before its rounding; the polynomial contraction in FP32.
+// Bound by the FP64 pipe.  (The mixed path's: KineticM2 below.)
 // ---------------------------------------------------------------------------
-template <typename T>
 struct Kinetic {
-  static __device__ __forceinline__ void run(DevSystem s, const double *__restrict__ r, const T *__restrict__ mbuf,
-                                             double *__restrict__ kin, int W, const uint3 bid, const uint3 gdim) {
+  static __device__ __forceinline__ void run(DevSystem s, const double *__restrict__ r,
+                                             const double *__restrict__ mbuf, double *__restrict__ kin, int W,
+                                             const uint3 bid, const uint3 gdim) {
     assume_global(r, mbuf, kin);
-    constexpr bool kDw = std::is_same<T, float>::value;
     extern __shared__ double4 sh_geo[];
     int *sh_info = reinterpret_cast<int *>(sh_geo + s.n_shells);
-    float4 *sh_dw = reinterpret_cast<float4 *>(sh_geo);
     for (int k = threadIdx.x; k < s.n_shells; k += blockDim.x) {
-      if constexpr (kDw) {
-        sh_dw[2 * k] = s.shell_dw[2 * k];
-        sh_dw[2 * k + 1] = s.shell_dw[2 * k + 1];
-      } else {
-        sh_geo[k] = s.shell_geo[k];
-      }
+      sh_geo[k] = s.shell_geo[k];
       sh_info[k] = s.shell_info[k];
     }
     __syncthreads();
@@ -55,96 +46,49 @@ struct Kinetic {
     for (long pt = (long)bid.x * (blockDim.x >> 5) + (threadIdx.x >> 5); pt < total; pt += nwarps) {
       const double *rr = r + pt * 3;
       const double px = rr[0], py = rr[1], pz = rr[2];
-      fdw pd[3];
-      if constexpr (kDw) {
-        // one FP64 -> double-word conversion per lane, shared by shuffles
-        const int kc = lane < 3 ? lane : 2;
-        const fdw mine = dw_of(kc == 0 ? px : (kc == 1 ? py : pz));
-  #pragma unroll
-        for (int k = 0; k < 3; ++k)
-          pd[k] = fdw{__shfl_sync(0xffffffffu, mine.hi, k), __shfl_sync(0xffffffffu, mine.lo, k)};
-      }
-      const T *M = mbuf + pt * s.L;
-      T tx = T(0), ty = T(0), tz = T(0), tl = T(0);
+      const double *M = mbuf + pt * s.L;
+      double tx = 0.0, ty = 0.0, tz = 0.0, tl = 0.0;
       for (int k = lane; k < s.n_shells; k += 32) {
         const int info = sh_info[k];
         const int l = shell_l(info), off = shell_off(info), rad = shell_rad(info);
-        T g, dx, dy, dz, r2, zeta, rinv = T(0);
-        if constexpr (kDw) {
-          const float4 gh = sh_dw[2 * k], gl = sh_dw[2 * k + 1];
-          const DwDisp d = dw_displacement(pd, gh, gl);
-          const fdw zw{gh.w, gl.w};
-          const fdw rw = rad ? dw_sqrt(d.r2) : fdw{0.0f, 0.0f};
-          g = dw_exp_neg(dw_neg(dw_mul(zw, rad ? rw : d.r2))).hi;
-          dx = d.x.hi;
-          dy = d.y.hi;
-          dz = d.z.hi;
-          r2 = d.r2.hi;
-          zeta = gh.w;
-          if (rad) rinv = 1.0f / rw.hi;
-        } else {
-          const double4 g4 = sh_geo[k];
-          dx = px - g4.x;
-          dy = py - g4.y;
-          dz = pz - g4.z;
-          r2 = dx * dx + dy * dy + dz * dz;
-          zeta = g4.w;
-          g = radial_factor(rad, zeta, r2);
-          if (rad) rinv = 1.0 / sqrt(r2);
-        }
-        T S0, Sx, Sy, Sz;
+        const double4 g4 = sh_geo[k];
+        const double dx = px - g4.x, dy = py - g4.y, dz = pz - g4.z;
+        const double r2 = dx * dx + dy * dy + dz * dz;
+        const double zeta = g4.w;
+        const double g = radial_factor(rad, zeta, r2);
+        double rinv = 0.0;
+        if (rad) rinv = 1.0 / sqrt(r2);
+        double S0, Sx, Sy, Sz;
         if (l == 0) {
           S0 = M[off];
-          Sx = Sy = Sz = T(0);
+          Sx = Sy = Sz = 0.0;
         } else if (l == 1) {
-          const T m0 = M[off], m1 = M[off + 1], m2 = M[off + 2];
+          const double m0 = M[off], m1 = M[off + 1], m2 = M[off + 2];
           S0 = m0 * dx + m1 * dy + m2 * dz;
           Sx = m0;
           Sy = m1;
           Sz = m2;
         } else {
-          const T m0 = M[off], m1 = M[off + 1], m2 = M[off + 2], m3 = M[off + 3], m4 = M[off + 4];
-          S0 = m0 * dx * dy + m1 * dy * dz + m2 * dz * dx + m3 * (dx * dx - dy * dy) + m4 * (T(3) * dz * dz - r2);
-          Sx = m0 * dy + m2 * dz + T(2) * (m3 - m4) * dx;
-          Sy = m0 * dx + m1 * dz - T(2) * (m3 + m4) * dy;
-          Sz = m1 * dy + m2 * dx + T(4) * m4 * dz;
+          const double m0 = M[off], m1 = M[off + 1], m2 = M[off + 2], m3 = M[off + 3], m4 = M[off + 4];
+          S0 = m0 * dx * dy + m1 * dy * dz + m2 * dz * dx + m3 * (dx * dx - dy * dy) + m4 * (3.0 * dz * dz - r2);
+          Sx = m0 * dy + m2 * dz + 2.0 * (m3 - m4) * dx;
+          Sy = m0 * dx + m1 * dz - 2.0 * (m3 + m4) * dy;
+          Sz = m1 * dy + m2 * dx + 4.0 * m4 * dz;
         }
-        T f, lapfac;
+        double f, lapfac;
         if (rad) {
           f = -zeta * S0 * rinv;
-          lapfac = zeta * zeta - T(2) * zeta * static_cast<T>(l + 1) * rinv;
+          lapfac = zeta * zeta - 2.0 * zeta * static_cast<double>(l + 1) * rinv;
         } else {
-          f = T(-2) * zeta * S0;
-          lapfac = T(4) * zeta * zeta * r2 - static_cast<T>(4 * l + 6) * zeta;
+          f = -2.0 * zeta * S0;
+          lapfac = 4.0 * zeta * zeta * r2 - static_cast<double>(4 * l + 6) * zeta;
         }
         tx = fma(g, fma(f, dx, Sx), tx);
         ty = fma(g, fma(f, dy, Sy), ty);
         tz = fma(g, fma(f, dz, Sz), tz);
         tl = fma(g * S0, lapfac, tl);
       }
-      // lane partials summed in FP64, or (FP32 partials) as double-words with
-      // FP32 instructions only
-      double gx, gy, gz, lp;
-      if constexpr (kDw) {
-        fdw sx{static_cast<float>(tx), 0.0f}, sy{static_cast<float>(ty), 0.0f}, sz{static_cast<float>(tz), 0.0f},
-            sl{static_cast<float>(tl), 0.0f};
-  #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          sx = dw_add(sx, fdw{__shfl_xor_sync(0xffffffffu, sx.hi, o), __shfl_xor_sync(0xffffffffu, sx.lo, o)});
-          sy = dw_add(sy, fdw{__shfl_xor_sync(0xffffffffu, sy.hi, o), __shfl_xor_sync(0xffffffffu, sy.lo, o)});
-          sz = dw_add(sz, fdw{__shfl_xor_sync(0xffffffffu, sz.hi, o), __shfl_xor_sync(0xffffffffu, sz.lo, o)});
-          sl = dw_add(sl, fdw{__shfl_xor_sync(0xffffffffu, sl.hi, o), __shfl_xor_sync(0xffffffffu, sl.lo, o)});
-        }
-        gx = static_cast<double>(sx.hi) + sx.lo;
-        gy = static_cast<double>(sy.hi) + sy.lo;
-        gz = static_cast<double>(sz.hi) + sz.lo;
-        lp = static_cast<double>(sl.hi) + sl.lo;
-      } else {
-        gx = warp_sum(static_cast<double>(tx));
-        gy = warp_sum(static_cast<double>(ty));
-        gz = warp_sum(static_cast<double>(tz));
-        lp = warp_sum(static_cast<double>(tl));
-      }
+      const double gx = warp_sum(tx), gy = warp_sum(ty), gz = warp_sum(tz), lp = warp_sum(tl);
       if (lane == 0) {
         double *o = kin + pt * 4;
         o[0] = gx;
@@ -155,25 +99,20 @@ struct Kinetic {
     }
 }
 };
-template <typename T>
 __global__ void __launch_bounds__(256) k_kinetic(DevSystem s, const double *__restrict__ r,
-                                                 const T *__restrict__ mbuf, double *__restrict__ kin, int W) {
-  Kinetic<T>::run(s, r, mbuf, kin, W, blockIdx, gridDim);
+                                                 const double *__restrict__ mbuf, double *__restrict__ kin, int W) {
+  Kinetic::run(s, r, mbuf, kin, W, blockIdx, gridDim);
 }
 
-template <typename T>
-cudaError_t launch_kinetic(const DevSystem &s, const double *r, const T *mbuf, double *kin, int W, cudaStream_t st) {
+cudaError_t launch_kinetic(const DevSystem &s, const double *r, const double *mbuf, double *kin, int W,
+                           cudaStream_t st) {
   if (W <= 0) return cudaSuccess;
   const long total = (long)W * s.N;
   long blocks = (total + 7) / 8;
   if (blocks > 152 * 16) blocks = 152 * 16;
   const size_t smem = (size_t)s.n_shells * (sizeof(double4) + sizeof(int));
-  return launch_or_record<Kinetic<T>, 256>(k_kinetic<T>, dim3((int)blocks), dim3(256), smem, st, s, r, mbuf, kin, W);
+  return launch_or_record<Kinetic, 256>(k_kinetic, dim3((int)blocks), dim3(256), smem, st, s, r, mbuf, kin, W);
 }
-template cudaError_t launch_kinetic<double>(const DevSystem &, const double *, const double *, double *, int,
-                                            cudaStream_t);
-template cudaError_t launch_kinetic<float>(const DevSystem &, const double *, const float *, double *, int,
-                                           cudaStream_t);
 
 // ---------------------------------------------------------------------------
 // The mixed path's contraction with two-float M vectors (M + M_lo: exact
@@ -187,17 +126,10 @@ template cudaError_t launch_kinetic<float>(const DevSystem &, const double *, co
 struct KineticM2 {
   static __device__ __forceinline__ void run(DevSystem s, const double *__restrict__ r,
                                              const float *__restrict__ mbuf, const float *__restrict__ mlo,
-                                             double *__restrict__ kin, int W, const uint3 bid, const uint3 gdim) {
+                                             double *__restrict__ kin, int W, int tables, const uint3 bid, const uint3 gdim) {
     assume_global(r, mbuf, mlo, kin);
-    extern __shared__ double4 sh_geo[];
-    int *sh_info = reinterpret_cast<int *>(sh_geo + s.n_shells);
-    float4 *sh_dw = reinterpret_cast<float4 *>(sh_geo);
-    for (int k = threadIdx.x; k < s.n_shells; k += blockDim.x) {
-      sh_dw[2 * k] = s.shell_dw[2 * k];
-      sh_dw[2 * k + 1] = s.shell_dw[2 * k + 1];
-      sh_info[k] = s.shell_info[k];
-    }
-    __syncthreads();
+    extern __shared__ float4 sh_stage[];
+    ShellStage<true> stage(s, sh_stage, tables);
     const int lane = threadIdx.x & 31;
     const long nwarps = (long)gdim.x * (blockDim.x >> 5);
     const long total = (long)W * s.N;
@@ -212,14 +144,14 @@ struct KineticM2 {
         for (int k = 0; k < 3; ++k)
           pd[k] = fdw{__shfl_sync(0xffffffffu, mine.hi, k), __shfl_sync(0xffffffffu, mine.lo, k)};
       }
+      stage.point(pd, lane);
       const float *M = mbuf + pt * s.L, *Ml = mlo + pt * s.L;
       fdw tx = zero, ty = zero, tz = zero, tl = zero;
       for (int k = lane; k < s.n_shells; k += 32) {
-        const int info = sh_info[k];
+        const int info = stage.info[k];
         const int l = shell_l(info), off = shell_off(info), rad = shell_rad(info);
-        const float4 gh = sh_dw[2 * k], gl = sh_dw[2 * k + 1];
-        const DwDisp d = dw_displacement(pd, gh, gl);
-        const fdw zw{gh.w, gl.w};
+        const DwDisp d = stage.disp(pd, k);
+        const fdw zw = stage.zeta[k];
         fdw g, rinv = zero;
         if (rad) {
           const fdw rw = dw_sqrt(d.r2);
@@ -246,9 +178,9 @@ struct KineticM2 {
                       dw_add(dw_mul(m2, dw_mul(d.z, d.x)), dw_mul(m3, dw_add(xx, dw_neg(yy)))));
           S0 = dw_add(S0, dw_mul(m4, dw_add(dw_mul_f(zz, 3.0f), dw_neg(d.r2))));
           const fdw d34 = dw_add(m3, dw_neg(m4)), s34 = dw_add(m3, m4);
-          Sx = dw_add(dw_add(dw_mul(m0, d.y), dw_mul(m2, d.z)), dw_mul_f(dw_mul(d34, d.x), 2.0f));
-          Sy = dw_add(dw_add(dw_mul(m0, d.x), dw_mul(m1, d.z)), dw_neg(dw_mul_f(dw_mul(s34, d.y), 2.0f)));
-          Sz = dw_add(dw_add(dw_mul(m1, d.y), dw_mul(m2, d.x)), dw_mul_f(dw_mul(m4, d.z), 4.0f));
+          Sx = dw_add(dw_add(dw_mul(m0, d.y), dw_mul(m2, d.z)), dw_scale(dw_mul(d34, d.x), 2.0f));
+          Sy = dw_add(dw_add(dw_mul(m0, d.x), dw_mul(m1, d.z)), dw_neg(dw_scale(dw_mul(s34, d.y), 2.0f)));
+          Sz = dw_add(dw_add(dw_mul(m1, d.y), dw_mul(m2, d.x)), dw_scale(dw_mul(m4, d.z), 4.0f));
         }
         fdw f, lapfac;
         const fdw zz2 = dw_mul(zw, zw);
@@ -256,12 +188,18 @@ struct KineticM2 {
           f = dw_neg(dw_mul(dw_mul(zw, S0), rinv));
           lapfac = dw_add(zz2, dw_neg(dw_mul_f(dw_mul(zw, rinv), static_cast<float>(2 * (l + 1)))));
         } else {
-          f = dw_neg(dw_mul_f(dw_mul(zw, S0), 2.0f));
-          lapfac = dw_add(dw_mul_f(dw_mul(zz2, d.r2), 4.0f), dw_neg(dw_mul_f(zw, static_cast<float>(4 * l + 6))));
+          f = dw_neg(dw_scale(dw_mul(zw, S0), 2.0f));
+          lapfac = dw_add(dw_scale(dw_mul(zz2, d.r2), 4.0f), dw_neg(dw_mul_f(zw, static_cast<float>(4 * l + 6))));
         }
-        tx = dw_add(tx, dw_mul(g, dw_add(Sx, dw_mul(f, d.x))));
-        ty = dw_add(ty, dw_mul(g, dw_add(Sy, dw_mul(f, d.y))));
-        tz = dw_add(tz, dw_mul(g, dw_add(Sz, dw_mul(f, d.z))));
+        fdw vx = dw_mul(f, d.x), vy = dw_mul(f, d.y), vz = dw_mul(f, d.z);
+        if (l > 0) {  // (s: grad P = 0)
+          vx = dw_add(Sx, vx);
+          vy = dw_add(Sy, vy);
+          vz = dw_add(Sz, vz);
+        }
+        tx = dw_add(tx, dw_mul(g, vx));
+        ty = dw_add(ty, dw_mul(g, vy));
+        tz = dw_add(tz, dw_mul(g, vz));
         tl = dw_add(tl, dw_mul(dw_mul(g, S0), lapfac));
       }
   #pragma unroll
@@ -283,19 +221,20 @@ struct KineticM2 {
 };
 __global__ void __launch_bounds__(256) k_kinetic_m2(DevSystem s, const double *__restrict__ r,
                                                     const float *__restrict__ mbuf, const float *__restrict__ mlo,
-                                                    double *__restrict__ kin, int W) {
-  KineticM2::run(s, r, mbuf, mlo, kin, W, blockIdx, gridDim);
+                                                    double *__restrict__ kin, int W, int tables) {
+  KineticM2::run(s, r, mbuf, mlo, kin, W, tables, blockIdx, gridDim);
 }
 
 cudaError_t launch_kinetic_m2(const DevSystem &s, const double *r, const float *mbuf, const float *mlo, double *kin,
                               int W, cudaStream_t st) {
   if (W <= 0) return cudaSuccess;
+  int warps, tables;
+  ShellStage<true>::plan(s, &warps, &tables);
   const long total = (long)W * s.N;
-  long blocks = (total + 7) / 8;
+  long blocks = (total + warps - 1) / warps;
   if (blocks > 152 * 16) blocks = 152 * 16;
-  const size_t smem = (size_t)s.n_shells * (sizeof(double4) + sizeof(int));
-  return launch_or_record<KineticM2, 256>(k_kinetic_m2, dim3((int)blocks), dim3(256), smem, st, s, r, mbuf, mlo, kin,
-                                          W);
+  return launch_or_record<KineticM2, 256>(k_kinetic_m2, dim3((int)blocks), dim3(warps * 32),
+                                          ShellStage<true>::bytes(s, tables), st, s, r, mbuf, mlo, kin, W, tables);
 }
 
 // ---------------------------------------------------------------------------

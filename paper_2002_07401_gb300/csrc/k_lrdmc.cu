@@ -224,7 +224,8 @@ __global__ void __launch_bounds__(kRatioThreads) k_lrdmc_ratios(DevSystem s, con
       const float4 gh = s.shell_dw[2 * sh], gl = s.shell_dw[2 * sh + 1];
       const int info = s.shell_info[sh], off = shell_off(info), l = shell_l(info), rad = shell_rad(info);
       const fdw zeta{gh.w, gl.w};
-      const DwDisp d = dw_displacement(od, gh, gl);
+      const fdw at[3] = {{gh.x, gl.x}, {gh.y, gl.y}, {gh.z, gl.z}};
+      const DwDisp d = displacement(od, at);
       // every hop's value is 0 in FP32 (e^-104) where even the nearest one is that far
       const float far = fmaxf(fmaxf(fabsf(d.x.hi), fabsf(d.y.hi)), fabsf(d.z.hi));
       const float near2 = fmaxf(d.r2.hi + a2.hi - 2.0f * ah.hi * far, 0.0f);

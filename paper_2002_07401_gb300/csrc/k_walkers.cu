@@ -46,24 +46,13 @@ struct BasisPoints {
   static __device__ __forceinline__ void run(DevSystem s, const double *__restrict__ r, int W, int e0, int npts,
                                              T *__restrict__ out, float *__restrict__ out_lo,
                                              double *__restrict__ rprop, uint32_t walker0, uint32_t sweep,
-                                             const uint32_t *__restrict__ sweep_dev, const uint3 bid,
+                                             const uint32_t *__restrict__ sweep_dev, int tables, const uint3 bid,
                                              const uint3 gdim) {
     assume_global(r, out);
     constexpr bool kDw = std::is_same<T, float>::value;
     if (PROPOSE && sweep_dev) sweep += *sweep_dev;  // graph replays read the sweep index from the device
-    extern __shared__ double4 sh_geo[];
-    int *sh_info = reinterpret_cast<int *>(sh_geo + s.n_shells);
-    float4 *sh_dw = reinterpret_cast<float4 *>(sh_geo);  // FP32 path: two float4 per shell in place of the double4
-    for (int k = threadIdx.x; k < s.n_shells; k += blockDim.x) {
-      if constexpr (kDw) {
-        sh_dw[2 * k] = s.shell_dw[2 * k];
-        sh_dw[2 * k + 1] = s.shell_dw[2 * k + 1];
-      } else {
-        sh_geo[k] = s.shell_geo[k];
-      }
-      sh_info[k] = s.shell_info[k];
-    }
-    __syncthreads();
+    extern __shared__ float4 sh_stage[];
+    ShellStage<kDw> stage(s, sh_stage, tables);
     const int lane = threadIdx.x & 31;
     const long nwarps = (long)gdim.x * (blockDim.x >> 5);
     const long total = (long)W * npts;
@@ -110,12 +99,11 @@ struct BasisPoints {
         for (int k = 0; k < 3; ++k)
           pd[k] = fdw{__shfl_sync(0xffffffffu, mine.hi, k), __shfl_sync(0xffffffffu, mine.lo, k)};
         float *ol = out_lo ? out_lo + ((size_t)w * s.n_up + i) * s.L : nullptr;
+        stage.point(pd, lane);
         for (int k = lane; k < s.n_shells; k += 32) {
-          const float4 gh = sh_dw[2 * k], gl = sh_dw[2 * k + 1];
-          const int info = sh_info[k];
-          const DwDisp d = dw_displacement(pd, gh, gl);
+          const int info = stage.info[k];
           float v[5], vl[5];
-          const int nc = shell_values_dw(info, fdw{gh.w, gl.w}, d, v, vl);
+          const int nc = shell_values_dw(info, stage.zeta[k], stage.disp(pd, k), v, vl);
           const int off = shell_off(info);
   #pragma unroll
           for (int c = 0; c < 5; ++c)
@@ -125,11 +113,12 @@ struct BasisPoints {
             }
         }
       } else {
+        stage.point(p, lane);
         for (int k = lane; k < s.n_shells; k += 32) {
-          const double4 g = sh_geo[k];
-          const int info = sh_info[k];
+          const int info = stage.info[k];
+          const Disp d = stage.disp(p, k);
           double v[5];
-          const int nc = shell_values(info, g.w, p[0] - g.x, p[1] - g.y, p[2] - g.z, v);
+          const int nc = shell_values(info, stage.zeta[k], d.x, d.y, d.z, d.r2, v);
           const int off = shell_off(info);
   #pragma unroll
           for (int c = 0; c < 5; ++c)
@@ -143,8 +132,9 @@ template <bool PROPOSE, typename T>
 __global__ void __launch_bounds__(256) k_basis_points(DevSystem s, const double *__restrict__ r, int W, int e0,
                                                       int npts, T *__restrict__ out, float *__restrict__ out_lo,
                                                       double *__restrict__ rprop, uint32_t walker0, uint32_t sweep,
-                                                      const uint32_t *__restrict__ sweep_dev) {
-  BasisPoints<PROPOSE, T>::run(s, r, W, e0, npts, out, out_lo, rprop, walker0, sweep, sweep_dev, blockIdx, gridDim);
+                                                      const uint32_t *__restrict__ sweep_dev, int tables) {
+  BasisPoints<PROPOSE, T>::run(s, r, W, e0, npts, out, out_lo, rprop, walker0, sweep, sweep_dev, tables, blockIdx,
+                               gridDim);
 }
 
 template <typename T>
@@ -153,16 +143,18 @@ cudaError_t launch_basis_points(const DevSystem &s, bool propose, const double *
                                 cudaStream_t st, const uint32_t *sweep_dev) {
   if (W <= 0 || npts <= 0) return cudaSuccess;
   const long total = (long)W * npts;
-  const int warps = 8;
+  using Stage = ShellStage<std::is_same<T, float>::value>;
+  int warps, tables;
+  Stage::plan(s, &warps, &tables);
   long blocks = (total + warps - 1) / warps;
   if (blocks > 152 * 16) blocks = 152 * 16;
-  const size_t smem = (size_t)s.n_shells * (sizeof(double4) + sizeof(int));
+  const size_t smem = Stage::bytes(s, tables);
   if (propose)
     return launch_or_record<BasisPoints<true, T>, 256>(k_basis_points<true, T>, dim3((int)blocks), dim3(warps * 32), smem, st, s, r, W, e0,
-                                                       npts, out, out_lo, rprop, walker0, sweep, sweep_dev);
+                                                       npts, out, out_lo, rprop, walker0, sweep, sweep_dev, tables);
   return launch_or_record<BasisPoints<false, T>, 256>(k_basis_points<false, T>, dim3((int)blocks), dim3(warps * 32), smem, st, s, r, W, e0,
                                                       npts, out, out_lo, rprop, walker0, sweep,
-                                                      (const uint32_t *)nullptr);
+                                                      (const uint32_t *)nullptr, tables);
 }
 template cudaError_t launch_basis_points<double>(const DevSystem &, bool, const double *, int, int, int, double *,
                                                  float *, double *, uint32_t, uint32_t, cudaStream_t,
