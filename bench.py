@@ -91,6 +91,18 @@ def tensor_roofline(kernel, achieved, issued, launches, prof_ms, ms, work):
             "share_of_step": prof_ms / ms if ms > 0 else None}
 
 
+def live_k(lam):
+    """Share of K that the products read: the rows of lambda between the first and the last non-zero one, per 16 columns
+    (a banded lambda's other rows are skipped)."""
+    import numpy as np
+    L = lam.shape[0]
+    live = 0
+    for c in range(0, L, 16):
+        rows = np.flatnonzero((lam[:, c:c + 16] != 0.0).any(axis=1))
+        live += (rows[-1] + 1 - rows[0]) * min(16, L - c) if rows.size else 0
+    return live / (L * L)
+
+
 def fixed_pairs(sysm):
     return (PAIRS_UP * sysm.n_up + PAIRS_DN * sysm.n_dn) / sysm.N
 PROFILE_TRAFFIC = os.path.join(ROOT, "profiles", "k_lambda_rows_C2_traffic.txt")
@@ -429,7 +441,7 @@ def forces_bench(pg, torch, dist, args, dev, rank, ws, local, fp64_tc=False, ste
         kp = (L + 63) // 64 * 64
         nsl = 7 if L <= 512 else 8
         issued = achieved * (nsl * (nsl + 1) // 2) * kp / L if achieved else None
-        roof = tensor_roofline("k_umma_gemm (tcgen05, FP64-equivalent adjoint lambda products, %d slices)" % nsl,
+        roof = tensor_roofline("k_umma_tri (tcgen05, FP64-equivalent adjoint lambda products, %d slices)" % nsl,
                                achieved, issued, lam_n, lam_ms, ms,
                                "2 L^2 FP64-equivalent flop per orbital row of the two adjoint lambda products")
     else:
@@ -596,7 +608,7 @@ def batch_bench(pg, torch, dist, args, dev, rank, ws, precision=None, sweeps=Non
         m.close()
     achieved = flops / (lam_ms / 1e3) / 1e12 if lam_ms > 0 else None
     if mixed:
-        roof = tensor_roofline("k_umma_gemm (tcgen05, BF16 fixed-point slices), all member systems", achieved,
+        roof = tensor_roofline("k_umma_tri (tcgen05, BF16 fixed-point slices), all member systems", achieved,
                                achieved * PAIRS_UP if achieved else None, lam_n, lam_ms, 0.0,
                                "2 L^2 flop per accepted orbital row, summed over the systems of one sweep; issued: "
                                "%d BF16 slice-pair products per flop (before padding K to 64)" % PAIRS_UP)
@@ -655,7 +667,8 @@ def large_bench(pg, torch, dist, args, dev, rank, ws, local):
     N, L = sysm.N, sysm.L
     kp = (L + 63) // 64 * 64
     secs = rr["prof_ms"] / 1e3
-    issued = fixed_pairs(sysm) * 2.0 * kp * L * rr["accepted"]
+    issued = fixed_pairs(sysm) * 2.0 * kp * L * rr["accepted"] * live_k(sysm.lam)
+    nnz = float(np.count_nonzero(sysm.lam))
     tc = issued / secs / 1e12 if secs > 0 else None
     return {"metric": "walker-electron moves/s", "value": W * N * args.large_steps * ws / (rr["ms_max"] / 1e3),
             "unit": "walker-electron moves/s", "ms_per_sweep": rr["ms_max"] / args.large_steps,
@@ -663,11 +676,12 @@ def large_bench(pg, torch, dist, args, dev, rank, ws, local):
             "acceptance": rr["accepted"] / (W * N * args.large_steps), "status_bits": rr["bits"],
             "gpu_launches": rr["launches"], "dtype": "f32+bf16 (f64 refresh)", "workload": LARGE_WORKLOAD,
             "clocks": rr["clocks"], "tuning": rr["tuning"],
-            "roofline": tensor_roofline("k_umma_gemm (tcgen05, BF16 fixed-point slices)",
-                                        2.0 * L * L * rr["accepted"] / secs / 1e12 if secs > 0 else None, tc,
+            "roofline": tensor_roofline("k_umma_tri (tcgen05, BF16 fixed-point slices)",
+                                        2.0 * nnz * rr["accepted"] / secs / 1e12 if secs > 0 else None, tc,
                                         rr["prof_n"], rr["prof_ms"], rr["ms"],
-                                        "2 L^2 flop per accepted orbital row (the lambda product); issued: %d BF16 "
-                                        "slice-pair products per flop" % PAIRS_UP),
+                                        "2 flop per non-zero of lambda and accepted orbital row (the lambda product); "
+                                        "issued: %d BF16 slice-pair products per flop of the non-zero row ranges"
+                                        % PAIRS_UP),
             "forces": forces}
 
 
@@ -1128,7 +1142,7 @@ def run_gpu(args):
             kp = (L + 63) // 64 * 64
             issued = fixed_pairs(sysm) * 2.0 * kp * L * rr["accepted"]  # BF16 slice-pair products per row
             tc = issued / secs / 1e12 if secs > 0 else None
-            d["roofline"] = tensor_roofline("k_umma_gemm (tcgen05, BF16 fixed-point slices)", achieved, tc,
+            d["roofline"] = tensor_roofline("k_umma_tri (tcgen05, BF16 fixed-point slices)", achieved, tc,
                                             rr["prof_n"], rr["prof_ms"], rr["ms"],
                                             "2 L^2 flop per accepted orbital row (the lambda product); issued: "
                                             "%d BF16 slice-pair products per flop on K padded to 64" % PAIRS_UP)
@@ -1172,7 +1186,7 @@ def run_gpu(args):
         issued = nsl * (nsl + 1) / 2 * 2.0 * kp * L * tc64["accepted"]
         tc = issued / secs / 1e12 if secs > 0 else None
         o["roofline"] = tensor_roofline(
-            "k_umma_gemm (tcgen05, FP64-equivalent: %d BF16 slices, FP64 epilogue)" % nsl,
+            "k_umma_tri (tcgen05, FP64-equivalent: %d BF16 slices, FP64 epilogue)" % nsl,
             2.0 * L * L * tc64["accepted"] / secs / 1e12 if secs > 0 else None, tc, tc64["prof_n"], tc64["prof_ms"],
             tc64["ms"], "2 L^2 FP64-equivalent flop per accepted orbital row; issued: %d BF16 slice-pair products "
             "per flop on K padded to 64" % (nsl * (nsl + 1) // 2))

@@ -411,7 +411,7 @@ jagp_status_t jagp_autotune(jagp_handle_t h, void *d_state, int W, jagp_tuning_t
  * heuristics), 0, 32 or 64, and 16 for tile_refresh in the mixed path with
  * N_up <= 16.  umma_*: 0 without tensor-core lambda products (FP64 without
  * fp64_tensor_cores); else bn 0 (heuristic) or a multiple of 16 up to 64 (six
- * or more tensor-memory accumulators), and stages -1, -2, -3 (chunk-major with
+ * or more tensor-memory accumulators), and stages -1, -2, -3 (stages with
  * K chunks of 64, 32, 16, only where two such stages fit in shared memory), 0
  * or 2..6.
  * Every choice changes the tiling only, so results stay as without tuning.
