@@ -309,7 +309,7 @@ struct Metropolis {
     // per-thread (at most 256) terms of the ratio and of dJ: T, or FP64 with a
     // three-body Jastrow
     __shared__ double part[512];
-    __shared__ int s_acc, s_base;
+    __shared__ int s_acc, s_n, s_base;
     __shared__ short moves[256];  // accepted (at most n <= bs)
     int nmv = 0;
     __shared__ double s_R;
@@ -477,13 +477,14 @@ struct Metropolis {
     // the accepted moves: one entry each in the list of changed rows, and (up) the
     // proposed orbitals to the table.  After the loop, because the atomic's and the
     // copies' latency there held up every accepted move of the chain.
+    // (s_n, not s_acc: a warp may still be about to read that for the last move.)
     if (tid == 0) {
-      s_acc = nmv;
+      s_n = nmv;
       s_base = nmv ? atomicAdd(count, nmv) : 0;
       if (total && nmv) atomicAdd(total, nmv);
     }
     __syncthreads();
-    const int na = s_acc;
+    const int na = s_n;
     for (int t = tid; t < na; t += bs) list[s_base + t] = w * n + moves[t];
     if (UP)
       for (int q = tid >> 5; q < na; q += bs >> 5) {
@@ -552,7 +553,7 @@ struct MetropolisBig {
     float *xf = reinterpret_cast<float *>(moves + n);  // mixed path: N * 3 positions rounded to FP32
     constexpr bool kF32 = std::is_same<T, float>::value;
     __shared__ T part[2 * 512];  // per-thread terms of the ratio and of dJ
-    __shared__ int s_acc, s_base;
+    __shared__ int s_acc, s_n, s_base;
     int nmv = 0;
     __shared__ double s_R;
     for (int t = tid; t < rs * n; t += bs) Gs[t] = gw[t];
@@ -705,13 +706,14 @@ struct MetropolisBig {
     // the accepted moves: one entry each in the list of changed rows, and (up) the
     // proposed orbitals to the table.  After the loop, because the atomic's and the
     // copies' latency there held up every accepted move of the chain.
+    // (s_n, not s_acc: a warp may still be about to read that for the last move.)
     if (tid == 0) {
-      s_acc = nmv;
+      s_n = nmv;
       s_base = nmv ? atomicAdd(count, nmv) : 0;
       if (total && nmv) atomicAdd(total, nmv);
     }
     __syncthreads();
-    const int na = s_acc;
+    const int na = s_n;
     for (int t = tid; t < na; t += bs) list[s_base + t] = w * n + moves[t];
     if (UP)
       for (int q = tid >> 5; q < na; q += bs >> 5) {
