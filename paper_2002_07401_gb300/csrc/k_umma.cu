@@ -343,16 +343,18 @@ __global__ void __launch_bounds__(128) k_umma_gemm(const __grid_constant__ CUten
 //
 // Persistent CTAs (one per SM: warp 0 TMA, warp 1 MMA, eight epilogue warps)
 // walk the tiles, so that the next tile's operands load during the epilogue.
-// Two CTAs of a cluster take neighbouring column tiles of one row tile and
-// each multicasts half of the A slices to both, which lowers the L2 reads per
-// tile from NS (128 + bn) to NS (64 + bn) rows per K.  Only the K chunks in
-// which the B tile has a non-zero element are visited (krange: [first, last)
-// per 16 rows of B, found when lambda is sliced): zeros change no exact sum, so
-// a banded pairing matrix costs its band, and the padding of K costs nothing.
+// Only the K chunks in which the B tile has a non-zero element are visited
+// (krange: [first, last) per 16 rows of B, found when lambda is sliced): zeros
+// change no exact sum, so a banded pairing matrix costs its band, and the
+// padding of K costs nothing.
+// Every CTA loads its own slices, from L2: pairs of CTAs that shared a row tile's A
+// slices were no faster (sweeps of 4096 walkers of 16 He 2.58 ms either way) and
+// slower where column tiles are few (509 walkers of 43 + 40 electrons 5.12 against
+// 4.61 ms: a pair waits for both epilogues, and an odd tile count leaves a CTA idle).
 //
 // TMEM: NS accumulators of bn <= 512 / NS columns.  The CTA asks for more than
-// half of the SM's shared memory, so that two CTAs (of clusters that each hold one
-// SM of a pair) never wait for each other's tensor memory.
+// half of the SM's shared memory, so that two CTAs never wait for each other's
+// tensor memory.
 //
 // Measured against one MMA per pair in CTA-per-tile launches: the six-slice
 // lambda products of the accepted rows of 4096 walkers (about 30 thousand rows,
@@ -369,7 +371,6 @@ struct TriArgs {
   int n, bn, tiles_n;    // output columns, columns per CTA, column tiles
   int kp, klive;         // K per slice (row pitch of a slice), elements that may be non-zero
   int cw, stages;        // K chunk width in elements (64, 32, 16), chunks in flight
-  int cl;                // CTAs per cluster (1, 2)
   const int2 *krange;    // non-zero K range per 16 rows of B, or null (= [0, klive))
   int slice_bits;
   int batch_rows, tiles_per_batch, b_batch_rows;  // batched mode (batch_rows > 0): block b of A against block b of B
@@ -383,22 +384,6 @@ struct TriArgs {
   int add;               // out64 += (scalar stores)
   int *err;
 };
-
-__device__ __forceinline__ void tma_load_2d_mc(uint32_t dst, const CUtensorMap *map, int x, int y, uint32_t bar,
-                                               uint16_t mask) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1, "
-      "{%2, %3}], [%4], %5;" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar), "h"(mask)
-      : "memory");
-}
-
-__device__ __forceinline__ void umma_commit_mc(uint32_t bar, uint16_t mask) {
-  asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
-      "h"(mask)
-      : "memory");
-}
 
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
@@ -446,12 +431,10 @@ struct UmmaTri {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int M = g.m_dev ? *g.m_dev : g.m_max;
-    const int cl = g.cl, rank = cl == 2 ? static_cast<int>(bid.x & 1u) : 0;
     const int tiles_m = g.batch_rows ? (g.m_max / g.batch_rows) * g.tiles_per_batch : (M + 127) / 128;
-    const int ctiles = (g.tiles_n + cl - 1) / cl;  // column tiles in steps of the cluster
-    const int total = tiles_m * ctiles;
-    const int first = static_cast<int>(bid.x) / cl, step = static_cast<int>(gdim.x) / cl;
-    if (first >= total) return;  // both CTAs of a cluster, before any barrier or tensor-memory use
+    const int total = tiles_m * g.tiles_n;
+    const int first = static_cast<int>(bid.x), step = static_cast<int>(gdim.x);
+    if (first >= total) return;  // before any barrier or tensor-memory use
     const uint32_t row_bytes = static_cast<uint32_t>(g.cw) * 2u;
     const uint32_t a_bytes = 128u * row_bytes, b_bytes = static_cast<uint32_t>(g.bn) * row_bytes;
     const uint32_t stage_bytes = NS * (a_bytes + b_bytes);
@@ -463,7 +446,7 @@ struct UmmaTri {
     if (threadIdx.x == 0) {
       for (int s = 0; s < g.stages; ++s) {
         mbar_init(full0 + 8u * s, 1);
-        mbar_init(empty0 + 8u * s, static_cast<uint32_t>(cl));
+        mbar_init(empty0 + 8u * s, 1);
       }
       mbar_init(tfull, 1);
       mbar_init(tempty, kTriEpiWarps);
@@ -477,30 +460,26 @@ struct UmmaTri {
     }
     tc_fence_before();
     __syncthreads();
-    if (cl == 2) {  // the peer's barriers exist before anything arrives there
-      asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-      asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    }
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     const uint32_t tiles = smem_u32(smem);
 
-    // tile t of this cluster: row tile, first column of the cluster's column tiles
+    // tile t: row tile, column tile
     auto place = [&](int t, int &ty, int &cx) {
       // kGroupM row tiles of one column step before the next, so that a wave
       // shares operand tiles in L2
-      const int span = kGroupM * ctiles, q = t / span, r = t - q * span;
+      const int span = kGroupM * g.tiles_n, q = t / span, r = t - q * span;
       const int gsize = tiles_m - q * kGroupM < kGroupM ? tiles_m - q * kGroupM : kGroupM;
       ty = q * kGroupM + r % gsize;
       cx = r / gsize;
     };
-    // K chunks [c0, c1) of the cluster's column tiles (the same in both CTAs)
+    // K chunks [c0, c1) of a column tile
     auto chunks = [&](int cx, int &c0, int &c1) {
       int lo = 0, hi = g.klive;
       if (g.krange) {
         lo = g.kp;
         hi = 0;
-        const int b0 = cx * cl * g.bn / 16, b1 = b0 + cl * g.bn / 16, nb = (g.n + 15) / 16;
+        const int b0 = cx * g.bn / 16, b1 = b0 + g.bn / 16, nb = (g.n + 15) / 16;
         for (int b = b0; b < b1 && b < nb; ++b) {
           const int2 r = g.krange[b];
           lo = r.x < lo ? r.x : lo;
@@ -522,8 +501,7 @@ struct UmmaTri {
 
     if (warp == 0) {
       if (lane == 0) {
-        // producer: every slice of A (its share of them, to both CTAs of a
-        // cluster) and of its own B tile for one K chunk per stage
+        // producer: every slice of A and of B for one K chunk per stage
         tensormap_acquire(&tmA, &tmB);
         int it = 0;
         bool ok = true;
@@ -532,7 +510,7 @@ struct UmmaTri {
           place(t, ty, cx);
           chunks(cx, c0, c1);
           rows_of(ty, bb, bt0, m0);
-          const int brow = bb * g.b_batch_rows + (cx * cl + rank) * g.bn;
+          const int brow = bb * g.b_batch_rows + cx * g.bn;
           for (int c = c0; c < c1; ++c, ++it) {
             const int s = it % g.stages;
             if (it >= g.stages && !mbar_wait(empty0 + 8u * s, ((it / g.stages) & 1u) ^ 1u)) {
@@ -543,18 +521,12 @@ struct UmmaTri {
             const uint32_t full = full0 + 8u * s, base = tiles + s * stage_bytes, bbase = base + NS * a_bytes;
             mbar_expect_tx(full, stage_bytes);
   #pragma unroll
-            for (int a = 0; a < NS; ++a) {
-              if (cl == 1)
-                tma_load_2d(base + a * a_bytes, &tmA, a * g.kp + c * g.cw, m0, full);
-              else if ((a & 1) == rank)
-                tma_load_2d_mc(base + a * a_bytes, &tmA, a * g.kp + c * g.cw, m0, full, 3);
-            }
+            for (int a = 0; a < NS; ++a) tma_load_2d(base + a * a_bytes, &tmA, a * g.kp + c * g.cw, m0, full);
   #pragma unroll
             for (int b = 0; b < NS; ++b) tma_load_2d(bbase + b * b_bytes, &tmB, b * g.kp + c * g.cw, brow, full);
           }
         }
-        // the last uses of every stage: their consumers' arrivals (of both CTAs)
-        // land, and no load is in flight, before this CTA ends
+        // the last uses of every stage: no load is in flight when this CTA ends
         for (int u = it > g.stages ? it - g.stages : 0; u < it; ++u)
           if (!mbar_wait(empty0 + 8u * (u % g.stages), (u / g.stages) & 1u)) {
             atomicExch(g.err, 1);
@@ -604,10 +576,7 @@ struct UmmaTri {
                             idesc0 | (static_cast<uint32_t>((cols - 256) >> 3) << 17), acc);
               }
             }
-            if (cl == 2)
-              umma_commit_mc(empty0 + 8u * s, 3);
-            else
-              umma_commit(empty0 + 8u * s);
+            umma_commit(empty0 + 8u * s);
           }
           if (ok) umma_commit(tfull);
         }
@@ -622,7 +591,7 @@ struct UmmaTri {
         int ty, cx, bb, bt0, m0;
         place(t, ty, cx);
         rows_of(ty, bb, bt0, m0);
-        const int n0 = (cx * cl + rank) * g.bn;
+        const int n0 = cx * g.bn;
         const int r = quarter * 32 + lane, row = m0 + r;
         const bool live = row < M && (!g.batch_rows || bt0 + r < g.batch_rows);
         const long long dst = live ? (g.out_rows ? g.out_rows[row] : row) : 0;
@@ -750,10 +719,6 @@ struct UmmaTri {
     __syncwarp();
     tc_fence_before();
     __syncthreads();
-    if (cl == 2) {
-      asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-      asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    }
     if (warp == 1) {
       tc_fence_after();
       asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
@@ -870,57 +835,38 @@ void tri_stages(int ns, int bn, int pinned, int *cw, int *stages) {
   *stages = static_cast<int>(s > 8 ? 8 : s);
 }
 
-// Columns per CTA (multiple of 16, at most limit) and CTAs per cluster: the pair
-// with the least estimated time of one CTA's share.  Clocks per K = 16 step: the
-// tensor pipe (bn / 2 per slice pair) or the operand reads (128 bytes a clock),
-// whichever is more; fixed clocks per tile for the epilogue and the pipeline's
-// fill; alone, a CTA reads twice the A slices from L2.
-void tri_tile(int ns, int n, int tiles_m, int klive, int limit, bool clusters, int *bn, int *cl) {
+// Columns per CTA (multiple of 16, at most limit): the width with the least
+// estimated time of one CTA's share.  Clocks per K = 16 step: the tensor pipe
+// (bn / 2 per slice pair), the operand reads from shared memory (128 bytes a
+// clock) or the loads from L2 (about 32 bytes a clock and SM), whichever is
+// most; fixed clocks per tile for the epilogue and the pipeline's fill.
+int tri_tile(int ns, int n, int tiles_m, int klive, int limit) {
   const int sms = sm_count();
   double best = 0.0;
-  *bn = 16;
-  *cl = 1;
-  for (int w = 16; w <= limit; w += 16)
-    for (int c = 1; c <= (clusters ? 2 : 1); ++c) {
-      const int tn = (n + w - 1) / w, padded = (tn + c - 1) / c * c;
-      int reads = 0;  // A slice reads per step
-      for (int a = 0; a < ns; ++a) reads += (ns - a) * w > 256 ? 2 : 1;
-      const double pairs = 0.5 * ns * (ns + 1), math = pairs * w / 2, smem = (reads * 4096.0 + pairs * w * 32) / 128;
-      const double l2 = ns * 32.0 * (128.0 / c + w) / 32;  // about 32 bytes a clock and SM
-      double t = math > smem ? math : smem;
-      if (l2 > t) t = l2;
-      const long long tiles = (long long)tiles_m * padded;
-      const double share = static_cast<double>((tiles + sms - 1) / sms);
-      const double cost = share * (t * ((klive + 15) / 16) + 1500.0 + 40.0 * w);
-      if (best == 0.0 || cost < best) {
-        best = cost;
-        *bn = w;
-        *cl = c;
-      }
+  int bn = 16;
+  for (int w = 16; w <= limit; w += 16) {
+    int reads = 0;  // A slice reads per step
+    for (int a = 0; a < ns; ++a) reads += (ns - a) * w > 256 ? 2 : 1;
+    const double pairs = 0.5 * ns * (ns + 1), math = pairs * w / 2, smem = (reads * 4096.0 + pairs * w * 32) / 128;
+    const double l2 = ns * 32.0 * (128.0 + w) / 32;
+    double t = math > smem ? math : smem;
+    if (l2 > t) t = l2;
+    const long long tiles = (long long)tiles_m * ((n + w - 1) / w);
+    const double share = static_cast<double>((tiles + sms - 1) / sms);
+    const double cost = share * (t * ((klive + 15) / 16) + 1500.0 + 40.0 * w);
+    if (best == 0.0 || cost < best) {
+      best = cost;
+      bn = w;
     }
+  }
+  return bn;
 }
 
 template <int NS, bool F64>
 cudaError_t launch_tri(const CUtensorMap &ta, const CUtensorMap &tb, const TriArgs &g, int grid, size_t smem,
                        cudaStream_t st) {
-  if (g.cl == 1)
-    return launch_or_record<UmmaTri<NS, F64>, kTriThreads>(k_umma_tri<NS, F64>, dim3(grid), dim3(kTriThreads), smem,
-                                                           st, ta, tb, g);
-  static std::atomic<unsigned char> raised[64];
-  cudaError_t e = group_raise_smem(reinterpret_cast<const void *>(k_umma_tri<NS, F64>), raised);
-  if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = static_cast<unsigned>(g.cl);
-  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(kTriThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_umma_tri<NS, F64>, ta, tb, g);
+  return launch_or_record<UmmaTri<NS, F64>, kTriThreads>(k_umma_tri<NS, F64>, dim3(grid), dim3(kTriThreads), smem, st,
+                                                         ta, tb, g);
 }
 }  // namespace
 
@@ -959,8 +905,7 @@ cudaError_t launch_umma_gemm(const uint16_t *A, int m_max, const int *m_dev, int
     // as many columns as NS accumulators leave room for in 512 (80 of six, 64
     // of seven or eight), or the pinned width (64 stands for the widest)
     const int widest = a_terms == 6 ? 80 : 64;
-    tri_tile(a_terms, n, tiles_m, g.klive, bn_max > 0 && bn_max < 64 ? bn_max : widest, group_recorder() == nullptr,
-             &g.bn, &g.cl);
+    g.bn = tri_tile(a_terms, n, tiles_m, g.klive, bn_max > 0 && bn_max < 64 ? bn_max : widest);
     tri_stages(a_terms, g.bn, stages_max < 0 ? chunk_width(stages_max) : 0, &g.cw, &g.stages);
     g.tiles_n = (n + g.bn - 1) / g.bn;
     g.krange = krange;
@@ -990,8 +935,8 @@ cudaError_t launch_umma_gemm(const uint16_t *A, int m_max, const int *m_dev, int
       return cudaErrorInvalidValue;
     size_t smem = 1024 + static_cast<size_t>(g.stages) * a_terms * (128 + g.bn) * g.cw * 2 + 8 * (2 * g.stages + 2) + 16;
     if (smem < 120 * 1024) smem = 120 * 1024;  // one CTA per SM (see the kernel)
-    const long long tiles = (long long)tiles_m * ((g.tiles_n + g.cl - 1) / g.cl) * g.cl;
-    const int sms = sm_count() / g.cl * g.cl;
+    const long long tiles = (long long)tiles_m * g.tiles_n;
+    const int sms = sm_count();
     const int grid = static_cast<int>(tiles < sms ? tiles : sms);
     if (!out64) return launch_tri<6, false>(ta, tb, g, grid, smem, st);
     if (a_terms == 6) return launch_tri<6, true>(ta, tb, g, grid, smem, st);
