@@ -605,7 +605,7 @@ GradLayout grad_layout(const jagp_ctx *h, int W) {
   g.rbar_at = take(w * na * 3 * 8);
   g.jpar = take(w * 3 * 8);
   g.eL = take(w * 8);
-  g.lam_part = take((size_t)g.nz * L * L * 8);
+  g.lam_part = take((size_t)adj_lambda_most_splits(W, h->ds.n_up, h->ds.n_dn, h->ds.L) * L * L * 8);
   g.tc_lam = h->tc_lambda && h->ds.n_dn == h->ds.n_up && n > 0;
   g.seg_w = g.tc_lam ? (int)std::max<size_t>(1, 2048 / n) : 0;
   g.nseg = g.tc_lam ? 2 * ((W + g.seg_w - 1) / g.seg_w) : 0;

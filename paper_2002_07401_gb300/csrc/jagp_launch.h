@@ -187,12 +187,15 @@ cudaError_t launch_adj_jastrow(const DevSystem &s, const double *r, const double
 cudaError_t launch_walker_sum(const double *in, int W, int n, double *out, cudaStream_t st);
 cudaError_t launch_adj_reduce(const double *part, int nparts, int n_atoms, double *rbar_at, const double *jpar,
                               int W, double *dR, double *djas, cudaStream_t st);
-// ranges of rows (at most 64) for launch_adj_lambda: those whose fullest SM has the
-// least FP64 work (rows, and about 8 rows' worth per tile for its start and its sums),
-// among those that leave more than three CTAs per SM to cover one another's barriers
-// (as many as there are, of at least 64 rows, if none does).
-// 32000 rows at L = 320: 30 ranges, 750 tiles, five on the fullest SM, 5.4 ms; one
-// range per 1024 rows gave 775, six on the fullest SM (6.0 ms)
+// Ranges of rows for launch_adj_lambda: those whose fullest SM has the least FP64
+// work (rows, and about 8 rows' worth per tile for its start and its sums), among
+// those that leave more than three CTAs per SM to cover one another's barriers (the
+// most, if none does).  32000 rows at L = 320: 30 ranges, 750 tiles, five on the
+// fullest SM, 5.4 ms; one range per 1024 rows gave 775, six on the fullest SM (6.0 ms).
+// At most (and reserved in the workspace, which so never shrinks as W grows): one per
+// 1024 rows, or per 64 rows while they make no more than eight tiles per SM; more
+// would take off at most 4 % of that work.
+int adj_lambda_most_splits(int W, int n, int nd, int L);
 int adj_lambda_splits(int W, int n, int nd, int L);
 cudaError_t launch_adj_lambda(const double *btbar, const double *dnphi, const double *phi_up, const double *abar,
                               int W, int n, int nd, int L, double *part, int nz, double *dlam, cudaStream_t st);

@@ -19,6 +19,8 @@
 // gradients, Hessians and gradients of the Laplacian.
 #include <math.h>
 
+#include <algorithm>
+
 #include "jagp_launch.h"
 
 namespace jagp {
@@ -800,9 +802,15 @@ cudaError_t launch_adj_reduce(const double *part, int nparts, int n_atoms, doubl
 
 static int adj_lambda_rows_per_z(long rows, int nz) { return (int)(((rows + nz - 1) / nz + 15) / 16 * 16); }
 
+int adj_lambda_most_splits(int W, int n, int nd, int L) {
+  const long rows = (long)W * (n + nd), tiles = (long)((L + 63) / 64) * ((L + 63) / 64);
+  const long few = std::min(rows / 64, (8 * 152 + tiles - 1) / tiles);
+  return (int)std::max(1l, std::min(64l, std::max(rows / 1024, few)));
+}
+
 int adj_lambda_splits(int W, int n, int nd, int L) {
   const long rows = (long)W * (n + nd), tiles = (long)((L + 63) / 64) * ((L + 63) / 64);
-  const int most = (int)(rows < 128 ? 1 : (rows / 64 < 64 ? rows / 64 : 64));
+  const int most = adj_lambda_most_splits(W, n, nd, L);
   int best = most;
   long least = 0;
   for (int nz = most; nz >= 1 && (nz == most || tiles * nz > 3 * 152); --nz) {
