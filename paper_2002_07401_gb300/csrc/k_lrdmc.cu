@@ -16,7 +16,7 @@
 // Hamiltonian the continuous local energy).
 //
 // A projection runs in rounds: every walker with time left takes one hop
-// (or ends) per round, one thread deciding for each walker; then the moved
+// (or ends) per round, a warp deciding for each walker; then the moved
 // electrons' orbital rows and their lambda products, and, on a compact copy
 // of the moved walkers' state, a refresh of G~^{-1} and the local energy of
 // the new configurations (jagp_api.cu) prepare the next round.  Decisions read the Philox4x32-10 stream (walker, generation, hop, 2).
@@ -141,17 +141,39 @@ __device__ __forceinline__ fdw warp_sum_dw(fdw v) {
   return v;
 }
 
-// squared distances r'^2 of the six hops from the displacement d of the electron
-// from a centre: r^2 + a^2 +- 2 a d_q
+// Squared distances r'^2 of the six hops from a centre at displacement d of the
+// electron, r^2 + a^2 +- 2 a d_q.  This cancels where a hop lands near the centre
+// (near: r'^2 below a quarter of r^2 + a^2): such centres are left to hop_from.
 struct HopDist {
   fdw base;     // r^2 + a^2
   fdw step[3];  // 2 a d_q
   __device__ __forceinline__ fdw r2(int k) const {
     return dw_add(base, (k & 1) ? dw_neg(step[k >> 1]) : step[k >> 1]);
   }
+  // the smallest r'^2, to FP32
+  __device__ __forceinline__ float least() const {
+    return base.hi - fmaxf(fmaxf(fabsf(step[0].hi), fabsf(step[1].hi)), fabsf(step[2].hi));
+  }
+  __device__ __forceinline__ bool near() const { return least() < 0.25f * base.hi; }
+  // near a shell's atom the distance itself (a Slater shell), the exponents of a quotient of
+  // Gaussians (an error of zeta (r^2 + a^2) units) and, closer, the polynomials lose bits
+  __device__ __forceinline__ bool near_shell(int rad, float zeta) const {
+    const float l = least();
+    return l < 0.015625f * base.hi || (l < 0.25f * base.hi && (rad || zeta * base.hi > 4.0f));
+  }
 };
 __device__ __forceinline__ HopDist hop_dist(const DwDisp &d, fdw two_a, fdw a2) {
   return {dw_add(d.r2, a2), {dw_mul(two_a, d.x), dw_mul(two_a, d.y), dw_mul(two_a, d.z)}};
+}
+// the displacement after hop k, its square a sum of three squares
+__device__ __forceinline__ DwDisp hop_from(const DwDisp &d, fdw a, int k) {
+  const fdw s = (k & 1) ? dw_neg(a) : a;
+  DwDisp h = d;
+  if (k < 2) h.x = dw_add(d.x, s);
+  else if (k < 4) h.y = dw_add(d.y, s);
+  else h.z = dw_add(d.z, s);
+  h.r2 = dw_add(dw_add(dw_mul(h.x, h.x), dw_mul(h.y, h.y)), dw_mul(h.z, h.z));
+  return h;
 }
 __device__ __forceinline__ DwDisp dw_between(const fdw *p, const fdw *q) {
   DwDisp d;
@@ -183,13 +205,16 @@ __device__ __forceinline__ fdw j2_term_dw(fdw b, float kinv, fdw r) {
 // +-a along q changes r^2 by a^2 +- 2 a d_q, so a Gaussian's six radial factors are
 // e^{-zeta (r^2 + a^2)} times or over e^{-2 zeta a d_q} (four exponentials, not
 // six), and sum_c M_c P_c, a polynomial of degree two at most, follows from its
-// value, gradient and second derivatives at the electron.  Conversions are done with integer
-// instructions.  A generation of 1024 walkers of 16 He, 26 rounds: 22.0 -> 10.2 ms
-// against six separate evaluations.
-__global__ void __launch_bounds__(kRatioThreads) k_lrdmc_ratios(DevSystem s, const double *__restrict__ r,
-                                                                 const double *__restrict__ mbuf,
-                                                                 const int *__restrict__ active, double a,
-                                                                 double *__restrict__ rho) {
+// value, gradient and second derivatives at the electron.  Where a hop lands near a
+// centre these cancel: the few shells, atoms and electrons it concerns are passed by
+// and taken afterwards, hop by hop from the hop's own displacement (in the same
+// loops that code took the kernel from 72 to 96 registers, and a generation from 36.4 to
+// 39.5 ms).  Conversions are done with integer instructions.  A generation of 1024
+// walkers of 16 He, 26 rounds: 22.0 -> 10.2 ms against six separate evaluations.
+__global__ void __launch_bounds__(kRatioThreads, 7) k_lrdmc_ratios(DevSystem s, const double *__restrict__ r,
+                                                                    const double *__restrict__ mbuf,
+                                                                    const int *__restrict__ active, double a,
+                                                                    double *__restrict__ rho) {
   extern __shared__ fdw xd[];         // the walker's positions [N][3], then per atom R, c, -c^3
   __shared__ float2 tab[64];
   const int w = blockIdx.x, N = s.N, L = s.L, na = s.n_atoms;
@@ -220,6 +245,7 @@ __global__ void __launch_bounds__(kRatioThreads) k_lrdmc_ratios(DevSystem s, con
 #pragma unroll
     for (int k = 0; k < 6; ++k) dot[k] = dj[k] = fdw{0.0f, 0.0f};
     const double *Mi = mbuf + ((size_t)w * N + i) * L;
+    unsigned later = 0;  // what has a hop near: bit 0 a shell, 1 an atom, 2 an electron
     for (int sh = lane; sh < s.n_shells; sh += 32) {
       const float4 gh = s.shell_dw[2 * sh], gl = s.shell_dw[2 * sh + 1];
       const int info = s.shell_info[sh], off = shell_off(info), l = shell_l(info), rad = shell_rad(info);
@@ -230,6 +256,11 @@ __global__ void __launch_bounds__(kRatioThreads) k_lrdmc_ratios(DevSystem s, con
       const float far = fmaxf(fmaxf(fabsf(d.x.hi), fabsf(d.y.hi)), fabsf(d.z.hi));
       const float near2 = fmaxf(d.r2.hi + a2.hi - 2.0f * ah.hi * far, 0.0f);
       if (gh.w * (rad ? sqrtf(near2) : near2) > 105.0f) continue;
+      const HopDist h = hop_dist(d, two_a, a2);
+      if (h.near_shell(rad, gh.w)) {
+        later |= 1u;
+        continue;
+      }
       // S = sum_c M_c P_c at the electron, its gradient and half its second derivatives
       const fdw m0 = dw_of_bits(Mi[off]);
       fdw S0, Sq[3] = {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}}, Cq[3] = {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}};
@@ -254,7 +285,6 @@ __global__ void __launch_bounds__(kRatioThreads) k_lrdmc_ratios(DevSystem s, con
         const fdw t = dw_add(dw_add(dw_mul(Sq[0], d.x), dw_mul(Sq[1], d.y)), dw_mul(Sq[2], d.z));
         S0 = fdw{0.5f * t.hi, 0.5f * t.lo};
       }
-      const HopDist h = hop_dist(d, two_a, a2);
       // the six hops' S: S0 +- a S_q + a^2 C_q
       fdw S[6];
 #pragma unroll
@@ -290,6 +320,10 @@ __global__ void __launch_bounds__(kRatioThreads) k_lrdmc_ratios(DevSystem s, con
         const fdw *R = ad + 5 * at, cd = R[3], mc3 = R[4];
         const DwDisp d = dw_between(od, R);
         const HopDist h = hop_dist(d, two_a, a2);
+        if (h.near()) {
+          later |= 2u;
+          continue;
+        }
         const fdw f0 = j1_term_dw(cd, mc3, bea, inv2b, b0, dw_sqrt(d.r2), tab);
 #pragma unroll
         for (int k = 0; k < 6; ++k)
@@ -305,20 +339,87 @@ __global__ void __launch_bounds__(kRatioThreads) k_lrdmc_ratios(DevSystem s, con
         const float kinv = o ? kinv2[1] : kinv2[0];
         const DwDisp d = dw_between(od, xd + 3 * q);
         const HopDist h = hop_dist(d, two_a, a2);
+        if (h.near()) {
+          later |= 4u;
+          continue;
+        }
         const fdw f0 = j2_term_dw(b, kinv, dw_sqrt(d.r2));
 #pragma unroll
         for (int k = 0; k < 6; ++k)
           dj[k] = dw_add(dj[k], dw_add(j2_term_dw(b, kinv, dw_sqrt(h.r2(k))), dw_neg(f0)));
       }
     }
+    // lane k < 6 has hop k's sums
+    fdw hd{0.0f, 0.0f}, hj{0.0f, 0.0f};
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
       const fdw dk = warp_sum_dw(dot[k]), jk = warp_sum_dw(dj[k]);
-      if (lane == k)
-        rho[(size_t)w * 6 * N + 6 * i + k] =
-            (static_cast<double>(dk.hi) + static_cast<double>(dk.lo)) *
-            exp(static_cast<double>(jk.hi) + static_cast<double>(jk.lo));
+      if (lane == k) {
+        hd = dk;
+        hj = jk;
+      }
     }
+    later = __reduce_or_sync(0xffffffffu, later);
+    if (later & 1u)
+      for (int t0 = 0; t0 < s.n_shells; t0 += 32) {
+        auto from = [&](int sh) {
+          const float4 gh = s.shell_dw[2 * sh], gl = s.shell_dw[2 * sh + 1];
+          const fdw at[3] = {{gh.x, gl.x}, {gh.y, gl.y}, {gh.z, gl.z}};
+          return displacement(od, at);
+        };
+        const int mine = t0 + lane;
+        unsigned left = __ballot_sync(
+            0xffffffffu, mine < s.n_shells && hop_dist(from(mine), two_a, a2)
+                                                  .near_shell(shell_rad(s.shell_info[mine]), s.shell_dw[2 * mine].w));
+        for (; left; left &= left - 1u) {
+          const int sh = t0 + __ffs(left) - 1, info = s.shell_info[sh];
+          const double *Ms = Mi + shell_off(info);
+          const int l = shell_l(info), rad = shell_rad(info);
+          const DwDisp h = hop_from(from(sh), ah, lane);
+          fdw S = dw_of_bits(Ms[0]);
+          if (l > 0) {
+            S = dw_mul(S, l == 1 ? h.x : dw_mul(h.x, h.y));
+            S = dw_add(S, dw_mul(dw_of_bits(Ms[1]), l == 1 ? h.y : dw_mul(h.y, h.z)));
+            S = dw_add(S, dw_mul(dw_of_bits(Ms[2]), l == 1 ? h.z : dw_mul(h.z, h.x)));
+          }
+          if (l > 1) {
+            S = dw_add(S, dw_mul(dw_of_bits(Ms[3]), dw_add(dw_mul(h.x, h.x), dw_neg(dw_mul(h.y, h.y)))));
+            S = dw_add(S, dw_mul(dw_of_bits(Ms[4]), dw_add(dw_mul_f(dw_mul(h.z, h.z), 3.0f), dw_neg(h.r2))));
+          }
+          const fdw x = dw_mul(fdw{s.shell_dw[2 * sh].w, s.shell_dw[2 * sh + 1].w}, rad ? dw_sqrt(h.r2) : h.r2);
+          hd = dw_add(hd, dw_mul(S, dw_exp_tab(dw_neg(x), tab)));
+        }
+      }
+    if (later & 2u)
+      for (int t0 = 0; t0 < na; t0 += 32) {
+        const int mine = t0 + lane;
+        unsigned left = __ballot_sync(
+            0xffffffffu, mine < na && hop_dist(dw_between(od, ad + 5 * mine), two_a, a2).near());
+        for (; left; left &= left - 1u) {
+          const fdw *R = ad + 5 * (t0 + __ffs(left) - 1);
+          const DwDisp d = dw_between(od, R);
+          const fdw f0 = j1_term_dw(R[3], R[4], bea, inv2b, b0, dw_sqrt(d.r2), tab);
+          hj = dw_add(hj, dw_add(j1_term_dw(R[3], R[4], bea, inv2b, b0, dw_sqrt(hop_from(d, ah, lane).r2), tab),
+                                 dw_neg(f0)));
+        }
+      }
+    if (later & 4u)
+      for (int t0 = 0; t0 < N; t0 += 32) {
+        const int mine = t0 + lane;
+        unsigned left = __ballot_sync(0xffffffffu, mine < N && mine != i &&
+                                                       hop_dist(dw_between(od, xd + 3 * mine), two_a, a2).near());
+        for (; left; left &= left - 1u) {
+          const int q = t0 + __ffs(left) - 1, o = (q < s.n_up) == (i < s.n_up) ? 0 : 1;
+          const fdw b = o ? b2[1] : b2[0];
+          const float kinv = o ? kinv2[1] : kinv2[0];
+          const DwDisp d = dw_between(od, xd + 3 * q);
+          hj = dw_add(hj, dw_add(j2_term_dw(b, kinv, dw_sqrt(hop_from(d, ah, lane).r2)),
+                                 dw_neg(j2_term_dw(b, kinv, dw_sqrt(d.r2)))));
+        }
+      }
+    if (lane < 6)
+      rho[(size_t)w * 6 * N + 6 * i + lane] = (static_cast<double>(hd.hi) + static_cast<double>(hd.lo)) *
+                                              exp(static_cast<double>(hj.hi) + static_cast<double>(hj.lo));
   }
 }
 
