@@ -2170,9 +2170,8 @@ static jagp_status_t jagp_lrdmc_project_impl(jagp_handle_t h, double *d_r, void 
     jagp_set_detail("lattice-regularised DMC runs on FP64 handles without the three-body Jastrow");
     return JAGP_ERR_UNSUPPORTED;
   }
-  if ((size_t)h->ds.N * 3 * 16 > 48 * 1024) {
-    jagp_set_detail("N = %d: the hop-ratio kernel keeps a walker's positions (FP64 and double-word) in 48 KB of "
-                    "shared memory (N <= 1024)", h->ds.N);
+  if (h->ds.N > 1024) {
+    jagp_set_detail("N = %d: the hop-ratio kernel keeps a walker's positions in shared memory (N <= 1024)", h->ds.N);
     return JAGP_ERR_UNSUPPORTED;
   }
   return lrdmc_project(h, d_r, d_state, W, walker0, generation, a, gamma, tau, e_ref, max_hops, d_weight, d_eL,

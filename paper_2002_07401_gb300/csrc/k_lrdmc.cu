@@ -211,6 +211,8 @@ __device__ __forceinline__ fdw j2_term_dw(fdw b, float kinv, fdw r) {
 // loops that code took the kernel from 72 to 96 registers, and a generation from 36.4 to
 // 39.5 ms).  Conversions are done with integer instructions.  A generation of 1024
 // walkers of 16 He, 26 rounds: 22.0 -> 10.2 ms against six separate evaluations.
+// ATOMS: the atoms' double-words in shared memory too (some five thousand do not fit).
+template <bool ATOMS>
 __global__ void __launch_bounds__(kRatioThreads, 7) k_lrdmc_ratios(DevSystem s, const double *__restrict__ r,
                                                                     const double *__restrict__ mbuf,
                                                                     const int *__restrict__ active, double a,
@@ -221,12 +223,21 @@ __global__ void __launch_bounds__(kRatioThreads, 7) k_lrdmc_ratios(DevSystem s, 
   fdw *const ad = xd + 3 * N;
   if (!active[w]) return;
   for (int t = threadIdx.x; t < 3 * N; t += kRatioThreads) xd[t] = dw_of_bits(r[(size_t)w * N * 3 + t]);
-  for (int t = threadIdx.x; t < na; t += kRatioThreads) {
-    for (int q = 0; q < 3; ++q) ad[5 * t + q] = dw_of_bits(s.R[3 * t + q]);
+  // atom t: R, c, -c^3
+  auto split_atom = [&](int t, fdw *q) {
+    for (int k = 0; k < 3; ++k) q[k] = dw_of_bits(s.R[3 * t + k]);
     const double c = s.c1[t];
-    ad[5 * t + 3] = dw_of_bits(c);
-    ad[5 * t + 4] = dw_of_bits(-c * c * c);
-  }
+    q[3] = dw_of_bits(c);
+    q[4] = dw_of_bits(-c * c * c);
+  };
+  if constexpr (ATOMS)
+    for (int t = threadIdx.x; t < na; t += kRatioThreads) split_atom(t, ad + 5 * t);
+  // atom t's five numbers, in shared memory or in q
+  auto atom = [&](int t, fdw *q) -> const fdw * {
+    if constexpr (ATOMS) return ad + 5 * t;
+    split_atom(t, q);
+    return q;
+  };
   for (int t = threadIdx.x; t < 64; t += kRatioThreads) tab[t] = kExpTab[t];
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -317,7 +328,8 @@ __global__ void __launch_bounds__(kRatioThreads, 7) k_lrdmc_ratios(DevSystem s, 
     }
     if (s.use_j1) {
       for (int at = lane; at < na; at += 32) {
-        const fdw *R = ad + 5 * at, cd = R[3], mc3 = R[4];
+        fdw buf[5];
+        const fdw *R = atom(at, buf), cd = R[3], mc3 = R[4];
         const DwDisp d = dw_between(od, R);
         const HopDist h = hop_dist(d, two_a, a2);
         if (h.near()) {
@@ -392,11 +404,12 @@ __global__ void __launch_bounds__(kRatioThreads, 7) k_lrdmc_ratios(DevSystem s, 
       }
     if (later & 2u)
       for (int t0 = 0; t0 < na; t0 += 32) {
+        fdw buf[5];
         const int mine = t0 + lane;
         unsigned left = __ballot_sync(
-            0xffffffffu, mine < na && hop_dist(dw_between(od, ad + 5 * mine), two_a, a2).near());
+            0xffffffffu, mine < na && hop_dist(dw_between(od, atom(mine, buf)), two_a, a2).near());
         for (; left; left &= left - 1u) {
-          const fdw *R = ad + 5 * (t0 + __ffs(left) - 1);
+          const fdw *R = atom(t0 + __ffs(left) - 1, buf);
           const DwDisp d = dw_between(od, R);
           const fdw f0 = j1_term_dw(R[3], R[4], bea, inv2b, b0, dw_sqrt(d.r2), tab);
           hj = dw_add(hj, dw_add(j1_term_dw(R[3], R[4], bea, inv2b, b0, dw_sqrt(hop_from(d, ah, lane).r2), tab),
@@ -705,13 +718,17 @@ __global__ void k_lrdmc_energy(const double *__restrict__ wbar, const double *__
 cudaError_t launch_lrdmc_ratios(const DevSystem &s, const double *r, const double *mbuf, const int *active, double a,
                                 double *rho, int W, cudaStream_t st) {
   if (W <= 0) return cudaSuccess;
-  const size_t smem = ((size_t)s.N * 3 + (size_t)s.n_atoms * 5) * sizeof(fdw);
-  if (smem > 48 * 1024) {
+  const size_t pos = (size_t)s.N * 3 * sizeof(fdw), smem = pos + (size_t)s.n_atoms * 5 * sizeof(fdw);
+  if (smem > 200 * 1024) {
+    k_lrdmc_ratios<false><<<W, kRatioThreads, pos, st>>>(s, r, mbuf, active, a, rho);  // (N <= 1024: 24 KB)
+    return cudaGetLastError();
+  }
+  if (smem > kRaiseSmem) {  // (static shared memory comes on top)
     static std::atomic<unsigned char> raised[64];
-    const cudaError_t e = group_raise_smem(reinterpret_cast<const void *>(k_lrdmc_ratios), raised);
+    const cudaError_t e = group_raise_smem(reinterpret_cast<const void *>(k_lrdmc_ratios<true>), raised);
     if (e != cudaSuccess) return e;
   }
-  k_lrdmc_ratios<<<W, kRatioThreads, smem, st>>>(s, r, mbuf, active, a, rho);
+  k_lrdmc_ratios<true><<<W, kRatioThreads, smem, st>>>(s, r, mbuf, active, a, rho);
   return cudaGetLastError();
 }
 
