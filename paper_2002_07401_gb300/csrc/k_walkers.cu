@@ -261,15 +261,16 @@ __device__ __forceinline__ void copy_row(T *__restrict__ dst, const T *__restric
 }
 
 // pitch of G~^{-1} in shared memory: odd, so that a column's entries (the ratio of
-// an up move, the rows summed by a down move's threads) lie in different banks
+// an up move, the rows summed by a down move's threads) lie in different banks.
+// (With a three-body Jastrow, which has no other kernel, n where only that fits.)
 __host__ __device__ inline int metro_pitch(int n) { return n | 1; }
 
 template <typename T>
-__host__ __device__ inline size_t metro_smem_per_walker(int n, int N) {
+__host__ __device__ inline size_t metro_smem_per_walker(int n, int N, int pitch) {
   // positions (FP64), G~^{-1}, three n-vectors, and in the mixed path the FP32
   // mirror of the positions
   const size_t mirror = std::is_same<T, float>::value ? (size_t)N * 3 * sizeof(float) : 0;
-  return ((size_t)N * 3 * sizeof(double) + (size_t)(n * metro_pitch(n) + 3 * n) * sizeof(T) + mirror + 15) & ~size_t(15);
+  return ((size_t)N * 3 * sizeof(double) + (size_t)(n * pitch + 3 * n) * sizeof(T) + mirror + 15) & ~size_t(15);
 }
 
 template <bool UP, typename T>
@@ -283,11 +284,10 @@ struct Metropolis {
                                              int *__restrict__ list, int *__restrict__ count,
                                              const float *__restrict__ pprop_lo, float *__restrict__ phi_lo,
                                              int m_begin, int m_end, int *__restrict__ total,
-                                             double *__restrict__ j3buf, const uint3 bid, const uint3 gdim) {
+                                             double *__restrict__ j3buf, int np, const uint3 bid, const uint3 gdim) {
     assume_global(r, rprop, gprop, ginv, scal, status, pprop, phi_up, list, count);
     extern __shared__ double sm[];
     const int n = s.n_up, N = s.N, tid = threadIdx.x, bs = blockDim.x;
-    const int np = metro_pitch(n);
     const int w = bid.x;
     T *gw = ginv + (size_t)w * n * n;
     double *xs = sm;                                  // N * 3 positions (FP64)
@@ -302,7 +302,7 @@ struct Metropolis {
     // proposed position, chi change, after the per-walker block
     const bool j3 = s.use_j3 && j3buf;
     const int LJ = s.LJ;
-    double *j3v = reinterpret_cast<double *>(reinterpret_cast<char *>(sm) + metro_smem_per_walker<T>(n, N));
+    double *j3v = reinterpret_cast<double *>(reinterpret_cast<char *>(sm) + metro_smem_per_walker<T>(n, N, np));
     double *chi_o = j3v + 6 * LJ, *chi_n = chi_o + LJ, *dchi = chi_n + LJ;
     if (j3)
       for (int t = tid; t < 6 * LJ; t += bs) j3v[t] = j3buf[(size_t)w * 6 * LJ + t];
@@ -512,9 +512,9 @@ __global__ void __launch_bounds__(256, (Metropolis<UP, T>::kMinBlocks)) k_metrop
                                                     T *__restrict__ phi_up, int *__restrict__ list,
                                                     int *__restrict__ count, const float *__restrict__ pprop_lo,
                                                     float *__restrict__ phi_lo, int m_begin, int m_end,
-                                                    int *__restrict__ total, double *__restrict__ j3buf) {
+                                                    int *__restrict__ total, double *__restrict__ j3buf, int np) {
   Metropolis<UP, T>::run(s, r, rprop, gprop, ginv, scal, status, pprop, phi_up, list, count, pprop_lo, phi_lo,
-                         m_begin, m_end, total, j3buf, blockIdx, gridDim);
+                         m_begin, m_end, total, j3buf, np, blockIdx, gridDim);
 }
 
 // ---------------------------------------------------------------------------
@@ -1020,7 +1020,7 @@ struct MetropolisWarp {
     const int n = s.n_up, N = s.N, np = metro_pitch(n), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int w = bid.x * kMetroWarps + warp;
     if (w >= W) return;  // warp-uniform; the kernel has no block-wide barrier
-    double *xs = reinterpret_cast<double *>(reinterpret_cast<char *>(sm) + warp * metro_smem_per_walker<T>(n, N));
+    double *xs = reinterpret_cast<double *>(reinterpret_cast<char *>(sm) + warp * metro_smem_per_walker<T>(n, N, np));
     T *Gi = reinterpret_cast<T *>(xs + N * 3);
     T *gp = Gi + n * np;
     T *vv = gp + n;
@@ -1185,22 +1185,23 @@ cudaError_t launch_metropolis(const DevSystem &s, bool up, double *r, const doub
   if (m_begin >= m_end) return cudaSuccess;
   const int n = s.n_up;
   // one CTA per walker (threads per CTA, shared memory)
-  auto cta = [&](int threads, size_t smem, double *j3) -> cudaError_t {
+  auto cta = [&](int threads, size_t smem, double *j3, int np) -> cudaError_t {
     if (up)
       return launch_or_record<Metropolis<true, T>, 256>(k_metropolis<true, T>, dim3(W), dim3(threads), smem, st, s, r,
                                                         rprop, gprop, ginv, scal, status, pprop, phi_up, list, count,
-                                                        pprop_lo, phi_lo, m_begin, m_end, total, j3);
+                                                        pprop_lo, phi_lo, m_begin, m_end, total, j3, np);
     return launch_or_record<Metropolis<false, T>, 256>(k_metropolis<false, T>, dim3(W), dim3(threads), smem, st, s, r,
                                                        rprop, gprop, ginv, scal, status, pprop, phi_up, list, count,
-                                                       pprop_lo, phi_lo, m_begin, m_end, total, j3);
+                                                       pprop_lo, phi_lo, m_begin, m_end, total, j3, np);
   };
   if (s.use_j3) {
     // the three-body Jastrow's change is formed in the CTA-per-walker kernel
-    const size_t per3 = metro_smem_per_walker<T>(n, s.N) + (size_t)9 * s.LJ * sizeof(double);
-    if (!j3buf || per3 > kMetroSmemMax) return cudaErrorInvalidValue;
-    return cta(n <= 64 ? 128 : 256, per3, j3buf);
+    auto bytes = [&](int np) { return metro_smem_per_walker<T>(n, s.N, np) + (size_t)9 * s.LJ * sizeof(double); };
+    const int np = bytes(metro_pitch(n)) <= kMetroSmemMax ? metro_pitch(n) : n;
+    if (!j3buf || bytes(np) > kMetroSmemMax) return cudaErrorInvalidValue;
+    return cta(n <= 64 ? 128 : 256, bytes(np), j3buf, np);
   }
-  const size_t per = metro_smem_per_walker<T>(n, s.N);
+  const size_t per = metro_smem_per_walker<T>(n, s.N, metro_pitch(n));
   if (n <= 32) {
     const int blocks = (W + kMetroWarps - 1) / kMetroWarps;
     if (up)
@@ -1211,7 +1212,7 @@ cudaError_t launch_metropolis(const DevSystem &s, bool up, double *r, const doub
         dim3(blocks), dim3(kMetroWarps * 32), per * kMetroWarps, st, s, r, rprop, gprop, ginv, scal, status, pprop,
         phi_up, list, count, W, pprop_lo, phi_lo, m_begin, m_end, total);
   }
-  if (per <= kMetroSmemMax) return cta(n <= 64 ? 128 : 256, per, nullptr);
+  if (per <= kMetroSmemMax) return cta(n <= 64 ? 128 : 256, per, nullptr, metro_pitch(n));
   // as many rows of G~^{-1} in shared memory as fit beside the rest
   const size_t rest = (size_t)s.N * 3 * sizeof(double) + (size_t)n * (3 * sizeof(T) + sizeof(int)) +
                       (std::is_same<T, float>::value ? (size_t)s.N * 3 * sizeof(float) : 0);
