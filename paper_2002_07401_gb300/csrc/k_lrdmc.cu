@@ -654,7 +654,8 @@ __global__ void __launch_bounds__(kSelectThreads) k_lrdmc_select(int W, uint32_t
     Se += we[q];
     last = max(last, wl[q]);
   }
-  double acc = base + (incl - sum);
+  const double before = __shfl_up_sync(0xffffffffu, incl, 1);
+  double acc = lane ? base + before : base;
   for (int b = b0; b < b1; ++b) {
     acc += weight[b];
     run[b] = acc;
@@ -673,9 +674,13 @@ __global__ void __launch_bounds__(kSelectThreads) k_lrdmc_select(int W, uint32_t
       else
         lo = mid + 1;
     }
+    // (where two threads' walkers meet, the running sum is within rounding only: a
+    // walker without weight gives way to the next one that has some)
+    while (lo < W && !(weight[lo] > 0.0)) ++lo;
     parent[j] = lo < W ? lo : last;
-    weight[j] = 1.0;
   }
+  __syncthreads();  // (every weight has been read)
+  for (int j = tid; j < W; j += kSelectThreads) weight[j] = 1.0;
   if (tid == 0) {
     stats[0] = S / W;
     stats[1] = Se / S;
