@@ -381,10 +381,11 @@ jagp_status_t jagp_walker_status(jagp_handle_t h, const void *d_state, int W, in
                                  void *stream);
 
 /* Tile autotuner (no counterpart in the paper: a property of this GPU code).
- * Times the candidate tilings of the per-walker products (proposed rows and
- * columns: one output per thread, 32x32 or 64x64 register-blocked tiles; the
- * refresh product G~ = Phi_up Bt^T likewise) and, with tensor-core lambda
- * products, their output-tile width and K chunk width, on
+ * Times the candidate tilings of the FP64 path's per-walker products (proposed
+ * rows and columns: one output per thread, 32x32 or 64x64 register-blocked tiles;
+ * the refresh product G~ = Phi_up Bt^T likewise) and, with tensor-core lambda
+ * products, their output-tile width and K chunk width (the mixed path's per-walker
+ * products have one kernel per size: they are timed, and the tile is 0), on
  * this handle's operands and the caller's state buffer of W walkers; keeps the
  * fastest in the handle for every later call.  The choices change only the
  * tiling of outputs, never the order of a sum: results are identical with or
@@ -392,8 +393,8 @@ jagp_status_t jagp_walker_status(jagp_handle_t h, const void *d_state, int W, in
  * the next sweep.  Synchronises `stream`.  out (host) receives the choices and
  * the best times (ms per call: proposals, refresh, A_up rows, Bt rows). */
 typedef struct {
-  int tile_proposals;  /* 0: one output per thread; 32 / 64: blocked tiles; 16 (refresh, mixed,
-                          N_up <= 16): four walkers per CTA, 2x2 outputs per thread */
+  int tile_proposals;  /* FP64: 0: one output per thread; 32 / 64: blocked tiles.  Mixed: no effect
+                          (but for jagp_guiding_weights' G~ above 32 rows, which takes 32 or 64) */
   int tile_refresh;
   int umma_bn_left;    /* tensor-core tile width at most, A_up = phi^T lambda (0 in plain FP64; 64: as
                           wide as tensor memory holds the accumulators of, by the shape) */
@@ -409,7 +410,7 @@ jagp_status_t jagp_autotune(jagp_handle_t h, void *d_state, int W, jagp_tuning_t
  * jagp_autotune returned for the same system and walker count).  Host-only, no
  * CUDA call; ms is ignored.  tile_proposals / tile_refresh: -1 (the shape
  * heuristics), 0, 32 or 64, and 16 for tile_refresh in the mixed path with
- * N_up <= 16.  umma_*: 0 without tensor-core lambda products (FP64 without
+ * N_up <= 16 (accepted; the same kernel runs).  umma_*: 0 without tensor-core lambda products (FP64 without
  * fp64_tensor_cores); else bn 0 (heuristic) or a multiple of 16 up to 64 (six
  * or more tensor-memory accumulators), and stages -1, -2, -3 (stages with
  * K chunks of 64, 32, 16, only where two such stages fit in shared memory), 0

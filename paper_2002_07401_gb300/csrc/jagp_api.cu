@@ -387,7 +387,23 @@ jagp_status_t run_local_energy(jagp_ctx *h, const double *r, void *state, int W,
   return JAGP_OK;
 }
 
-// G~ = Phi_up Bt^T, its inverse (FP64 elimination), log|det| and (optionally) J
+// G~ = Phi_up Bt^T of a refresh.  Mixed, N_up >= 32: (Phi_up + lo)(Bt + lo)^T per walker
+// on the tensor cores from the tables' six fixed-point slices (twenty-one pairs, FP64
+// epilogue)
+template <typename T>
+cudaError_t refresh_product(jagp_ctx *h, const Layout &L, void *state, int W, int tile, cudaStream_t st) {
+  const int n = h->ds.n_up, Lb = h->ds.L;
+  double *gm = refresh_g(L, state);
+  if (tc_refresh(h))
+    return launch_umma_gemm(at<uint16_t>(state, L.gpack_a), W * n, nullptr, kFixedSlices, at<uint16_t>(state, L.gpack_b),
+                            n, kFixedSlices, h->kp, kFixedPairs, kPairA, kPairB, nullptr, n, nullptr, h->d_err, st,
+                            at<int>(state, L.gexp_a), at<int>(state, L.gexp_b), nullptr, 0, gm, 8, n, W, 0, 0, 0, 0, 0,
+                            nullptr, Lb);
+  return refresh_geminal(at<T>(state, L.phi_up), lo_table(h, state, L.phi_lo), (size_t)n * Lb, at<T>(state, L.bt),
+                         lo_table(h, state, L.bt_lo), (size_t)n * Lb, n, Lb, gm, W, st, tile);
+}
+
+// G~, its inverse (FP64 elimination), log|det| and (optionally) J
 // (cut_tables: the tables are new as a whole, so that their slices are all cut here;
 // in a sweep lambda_products has kept them current)
 template <typename T>
@@ -398,8 +414,6 @@ jagp_status_t run_refresh(jagp_ctx *h, const double *r, void *state, int W, int 
   double *gm = refresh_g(L, state);
   group_subkey(0);  // grouped sweeps: packing, then the G~ product, then the elimination
   if (tc_refresh(h)) {
-    // G~ = (Phi_up + lo)(Bt + lo)^T per walker on the tensor cores: both tables
-    // cut into six fixed-point slices, twenty-one pairs, FP64 epilogue
     uint16_t *pa = at<uint16_t>(state, L.gpack_a), *pb = at<uint16_t>(state, L.gpack_b);
     int *ea = at<int>(state, L.gexp_a), *eb = at<int>(state, L.gexp_b);
     if (cut_tables) {
@@ -410,17 +424,9 @@ jagp_status_t run_refresh(jagp_ctx *h, const double *r, void *state, int W, int 
              launch_pack_fixed(at<float>(state, L.bt), lo_table(h, state, L.bt_lo), nullptr, nullptr, W * n, 1, 1, Lb,
                                h->kp, nullptr, nullptr, nullptr, W * n, st, pb, eb));
     }
-    group_subkey(1);
-    LAUNCH(JAGP_KERNEL_GEMM_ROWS, 1,
-           launch_umma_gemm(pa, W * n, nullptr, kFixedSlices, pb, n, kFixedSlices, h->kp, kFixedPairs, kPairA, kPairB,
-                            nullptr, n, nullptr, h->d_err, st, ea, eb, nullptr, 0, gm, 8, n, W, 0, 0, 0, 0, 0,
-                            nullptr, Lb));
-  } else {
-    group_subkey(1);
-    LAUNCH(JAGP_KERNEL_GEMM_ROWS, 1,
-           refresh_geminal(at<T>(state, L.phi_up), lo_table(h, state, L.phi_lo), (size_t)n * Lb, at<T>(state, L.bt),
-                           lo_table(h, state, L.bt_lo), (size_t)n * Lb, n, Lb, gm, W, st, h->tune_tile_refresh));
   }
+  group_subkey(1);
+  LAUNCH(JAGP_KERNEL_GEMM_ROWS, 1, refresh_product<T>(h, L, state, W, h->tune_tile_refresh, st));
   // the mixed path keeps an FP64 copy of the inverse for the local energy
   double *gi64 = h->precision == JAGP_PREC_MIXED ? at<double>(state, L.ginv64) : nullptr;
   group_subkey(2);
@@ -1155,10 +1161,10 @@ jagp_status_t tune_products(jagp_ctx *h, void *state, int W, cudaStream_t st, ja
   const int n = d.n_up, Lb = d.L;
   JAGP_CU(cudaMemsetAsync(state, 0, L.total, st));
   T *pprop = at<T>(state, L.pprop), *bt = at<T>(state, L.bt), *gprop = at<T>(state, L.gprop);
-  T *phi = at<T>(state, L.phi_up);
-  const int tiles[3] = {0, 32, 64};
+  // (the mixed path's products have one kernel per size, whatever the tile: timed once)
+  const int tiles[3] = {0, 32, 64}, ntiles = std::is_same<T, float>::value ? 1 : 3;
   float best = 0.0f;
-  for (int c = 0; c < 3; ++c) {
+  for (int c = 0; c < ntiles; ++c) {
     float ms = 0.0f;
     JAGP_CU(time_calls([&] { return launch_gemm_rows<T>(pprop, (size_t)n * Lb, bt, (size_t)n * Lb, n, n, Lb, gprop,
                                                         (size_t)n * n, n, W, st, tiles[c]); },
@@ -1170,18 +1176,12 @@ jagp_status_t tune_products(jagp_ctx *h, void *state, int W, cudaStream_t st, ja
   }
   out->tile_proposals = h->tune_tile_prop;
   out->ms[0] = best;
-  double *gm = refresh_g(L, state);
-  const int rtiles[4] = {0, 32, 64, 16};  // 16: the four-walkers-per-CTA compensated kernel (FP32, N_up <= 16)
-  const int nref = (std::is_same<T, float>::value && n <= 16) ? 4 : 3;
-  for (int c = 0; c < nref; ++c) {
+  for (int c = 0; c < ntiles; ++c) {
     float ms = 0.0f;
-    JAGP_CU(time_calls([&] { return refresh_geminal(phi, lo_table(h, state, L.phi_lo), (size_t)n * Lb, bt,
-                                                    lo_table(h, state, L.bt_lo), (size_t)n * Lb, n, Lb, gm, W, st,
-                                                    rtiles[c]); },
-                       st, &ms));
+    JAGP_CU(time_calls([&] { return refresh_product<T>(h, L, state, W, tiles[c], st); }, st, &ms));
     if (c == 0 || ms < best) {
       best = ms;
-      h->tune_tile_refresh = rtiles[c];
+      h->tune_tile_refresh = tiles[c];
     }
   }
   out->tile_refresh = h->tune_tile_refresh;
@@ -1285,6 +1285,7 @@ static jagp_status_t jagp_set_tuning_impl(jagp_handle_t h, const jagp_tuning_t *
       if (bn[side] < 0 || bn[side] % 16 || bn[side] > limit) return JAGP_ERR_INVALID_ARG;
       if (stg[side] < -3 || stg[side] == 1 || stg[side] > 6) return JAGP_ERR_INVALID_ARG;
       const int npairs = mixed ? kFixedPairs : np64;
+      // (two stages of a pinned K chunk have to fit at the width asked for, in equal tiles)
       const int actual = umma_pick_bn(h->ds.L, bn[side] ? bn[side] : limit);
       if (stg[side] < 0 && !umma_chunk_fits(npairs, mixed ? kPairA : pa64, mixed ? kPairB : pb64, actual, stg[side]))
         return JAGP_ERR_INVALID_ARG;
