@@ -100,11 +100,17 @@ typedef struct jagp_options {
   int refresh_moves;          /* 0: refresh G~^{-1} from the tables once per sweep (FP64) or
                                  after each spin half-sweep (MIXED); k > 0: also after every
                                  k moves within a spin half-sweep (e.g. 16); < 0: INVALID_ARG */
-  int fp64_tensor_cores;      /* FP64 only.  0: lambda products with FP64 instructions.  1: the
-                                 same products FP64-equivalent on the BF16 tensor cores: FP64
-                                 rows cut into 7 exact 8-bit slices (8 slices of 7 bits when
-                                 L > 512), every slice pair of weight >= 2^-56 summed exactly in
-                                 its own accumulator, combined in FP64 (Ozaki-style splitting) */
+  int fp64_tensor_cores;      /* FP64 only.  0: products with FP64 instructions.  1: FP64-equivalent
+                                 on the BF16 tensor cores: operand rows cut into 7 exact 8-bit
+                                 slices (8 slices of 7 bits when K > 512), every slice pair of
+                                 weight >= 2^-56 summed exactly in its own accumulator, combined
+                                 in FP64 (Ozaki-style splitting).  These are the lambda products
+                                 and lambda's gradient; from N_up = 32 on also the kinetic vectors
+                                 (products with G~^{-1}) and jagp_grad's products of per-walker
+                                 rows.  An operand keeps 55 (56) bits of its row's largest entry,
+                                 with electrons of very different magnitudes balanced first:
+                                 sums are as good as FP64's relative to their largest terms, while
+                                 entries far below a row's largest keep fewer than 53 bits */
 } jagp_options_t;
 
 typedef struct jagp_ctx *jagp_handle_t;

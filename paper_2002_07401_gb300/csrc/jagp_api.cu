@@ -319,25 +319,31 @@ jagp_status_t run_kinetic_mixed(jagp_ctx *h, const double *r, void *state, int W
 //   out_w[y][c] (+)= sum_{k < K} X_w[k][c] Y_w(k, y),  c < L, y < ny,
 // X_w = X + w xw of row pitch L, out_w = out + w ow of row pitch L; Y_w = Y + w
 // N_up^2 of row pitch N_up, Y_w(k, y) = Y_w[y][k] (y_rows; K = N_up) or Y_w[k][y].
-// The columns of X and the rows or columns of Y are cut into exact slices.
+// The columns of X and the rows or columns of Y are cut into exact slices, the terms k
+// balanced first (launch_balance_terms).
 jagp_status_t cols_product64(jagp_ctx *h, void *state, int W, const double *X, size_t xw, int K, const double *Y,
                              bool y_rows, int ny, double *out, size_t ow, bool add, cudaStream_t st) {
   const Layout L = layout_of(h, W);
   const int n = h->ds.n_up, Lb = h->ds.L, kpn = (n + 63) / 64 * 64, nsl = cols_slices(h), bits = cols_bits(h),
             chunk = cols_chunk(h, W);
   uint16_t *pa = at<uint16_t>(state, L.mpack_a), *pb = at<uint16_t>(state, L.mpack_b);
-  int *ea = at<int>(state, L.mexp_a), *eb = at<int>(state, L.mexp_b), *mr = at<int>(state, L.mrows);
+  int *ea = at<int>(state, L.mexp_a), *eb = at<int>(state, L.mexp_b), *mr = at<int>(state, L.mrows),
+      *sc = at<int>(state, L.mscale);
   int qa[kMaxPairs], qb[kMaxPairs];
   const int np = slice_pairs(nsl, qa, qb);
   for (int w0 = 0; w0 < W; w0 += chunk) {
     const int wc = std::min(chunk, W - w0);
     const double *Yc = Y + (size_t)w0 * n * n;
-    LAUNCH(0, 1, launch_pack_cols(X + w0 * xw, nullptr, nullptr, xw, K, Lb, kpn, wc, pb, eb, nullptr, 0, 0, st, nsl, bits));
+    LAUNCH(0, 1, launch_balance_terms(Yc, n, K, ny, y_rows, wc, sc, st));
+    LAUNCH(0, 1, launch_pack_cols(X + w0 * xw, nullptr, nullptr, xw, K, Lb, kpn, wc, pb, eb, nullptr, 0, 0, st, nsl, bits, sc, 1));
     if (y_rows)
-      LAUNCH(0, 1, launch_pack_fixed64(Yc, nullptr, nullptr, wc * ny, ny, n, n, kpn, nsl, bits, pa, mr, ea, wc * ny, st));
+      LAUNCH(0, 1,
+             launch_pack_fixed64(Yc, nullptr, nullptr, wc * ny, ny, n, n, kpn, nsl, bits, pa, mr, ea, wc * ny, st, 0, 0,
+                                 sc));
     else
       LAUNCH(0, 1,
-             launch_pack_cols(Yc, nullptr, nullptr, (size_t)n * n, K, n, kpn, wc, pa, ea, nullptr, 0, 0, st, nsl, bits));
+             launch_pack_cols(Yc, nullptr, nullptr, (size_t)n * n, K, n, kpn, wc, pa, ea, nullptr, 0, 0, st, nsl, bits, sc,
+                              -1));
     LAUNCH(JAGP_KERNEL_ENERGY, 1,
            launch_umma_gemm(pb, wc * Lb, nullptr, nsl, pa, ny, nsl, kpn, np, qa, qb, nullptr, 0, nullptr, h->d_err, st,
                             eb, ea, nullptr, 0, out + w0 * ow, bits, Lb, wc, 0, y_rows ? ny : n, (long long)ow, 1, Lb,

@@ -104,6 +104,7 @@ struct Layout {
   size_t mexp_a;   // int    [W n_up]        their exponents
   size_t mexp_b;   // int    [W L]
   size_t mrows;    // int    [W n_up]        destination rows of the M product
+  size_t mscale;   // int    [tc_w n_up]     FP64-equivalent: powers of two that balance a product's terms
   size_t j3buf;    // double [W][6][LJ]      three-body Jastrow: U_up, U_dn (spin sums of chi), M_p U_up,
                    //                        M_p U_dn, M_a U_up, M_a U_dn
   size_t total;
@@ -158,6 +159,7 @@ inline Layout make_layout(size_t W, size_t nu, size_t N, size_t L, size_t esz = 
   l.mexp_a = take(mw * nu * 4);
   l.mexp_b = take(mw * L * 4);
   l.mrows = take(mw * nu * 4);
+  l.mscale = take(mx ? 0 : mw * nu * 4);
   l.j3buf = take(W * 6 * lj * 8);
   l.total = o;
   return l;

@@ -144,15 +144,23 @@ bool umma_chunk_fits(int npairs, const int *pair_a, const int *pair_b, int bn, i
 // rows_out[m] = the source row, or (dst_stride > 0) (m / nsub) dst_stride + dst_off + m % nsub
 cudaError_t launch_pack_fixed64(const double *P, const int *list, const int *count, int nrows, int nsub, int stride,
                                 int L, int kp, int nsl, int bits, uint16_t *A, int *rows_out, int *exps,
-                                int max_rows, cudaStream_t st, long dst_stride = 0, long dst_off = 0);
+                                int max_rows, cudaStream_t st, long dst_stride = 0, long dst_off = 0,
+                                const int *scale = nullptr);
+// (scale [nrows / nsub][L]: element k of a row of walker w is taken times 2^-scale[w L + k])
+// Exponents s [W][K] that balance sum_k X[k] Y(k, y) of FP64-equivalent products, Y_w = Y + w
+// n^2 of pitch n, Y(k, y) = Y[y][k] (y_rows) or Y[k][y], y < ny: Y is to be taken times
+// 2^-s, X times 2^s (the scale of the two packings)
+cudaError_t launch_balance_terms(const double *Y, int n, int K, int ny, bool y_rows, int W, int *s, cudaStream_t st);
 // columns c < C of the per-walker matrices X_w ([R][C], X_w = X + w xw; FP64 X64,
 // or two-float X32 + Xlo) -> operand rows w C + c of nsl exact slices of
 // `bits` bits (8, or 7 for FP64 X; nsl <= 8) over the R rows (K padded to kp),
-// exponents exps[w C + c], and rows_out[w C + c] = w dst_stride + dst_off + c
+// exponents exps[w C + c], and rows_out[w C + c] = w dst_stride + dst_off + c;
+// row r of X_w (FP64) is taken times 2^(sign scale[w R + r])
 // (when given)
 cudaError_t launch_pack_cols(const double *X64, const float *X32, const float *Xlo, size_t xw, int R, int C, int kp,
                              int W, uint16_t *A, int *exps, int *rows_out, long dst_stride, long dst_off,
-                             cudaStream_t st, int nsl = kFixedSlices, int bits = 8);
+                             cudaStream_t st, int nsl = kFixedSlices, int bits = 8, const int *scale = nullptr,
+                             int sign = 1);
 // FP32 rows (two-float rows P + P_lo when P_lo is given) -> kFixedSlices exact
 // 8-bit slices per element (BF16) plus a row exponent, compacted into A / rows_out /
 // exps (unless A is null) and, when given, at each row's own place in A_at / exps_at

@@ -1124,6 +1124,70 @@ __device__ __forceinline__ int exponent_of(unsigned hi) {
   const int ef = static_cast<int>(hi >> 20);
   return ef == 0x7ff || hi == 0u ? 0 : (ef ? ef : 1) - 1022;
 }
+// the same of one value times 2^d, for a maximum over several: kNoExponent for 0,
+// kNotFinite where it is not finite; then the maximum's
+constexpr int kNoExponent = -0x7fffffff, kNotFinite = 0x7fffffff;
+__device__ __forceinline__ int element_exponent(double v, int d) {
+  const unsigned hi = abs_hi(v), lo = static_cast<unsigned>(__double2loint(v));
+  return hi >= 0x7ff00000u ? kNotFinite : ((hi | lo) == 0u ? kNoExponent : exponent_of(hi | 1u) + d);
+}
+__device__ __forceinline__ int exponent_of_max(int e) { return e == kNotFinite || e == kNoExponent ? 0 : e; }
+
+// ---------------------------------------------------------------------------
+// Powers of two that balance a product sum_k X[k][c] Y(k, y) of exact slices.  The cut
+// keeps 55 bits of a column's largest entry over k, which is what the sum needs only
+// while no k is weak in X and strong in Y: an electron far from all atoms has a row of
+// G~ of 1e-12, say, and entries of G~^{-1} of 1e12, beside which the others' would lose
+// all their bits (local energies of 34 + 33 electrons, two of them so, were off by 19 %;
+// with this 1e-12, as with FP64 instructions).  s_k <= 0: Y(k, .) is taken times 2^-s_k,
+// X[k][.] times 2^s_k, so that the largest |Y(k, .)| of every k has the same exponent.
+// A CTA per walker; bound by one read of Y, far below the product's operands (gradients
+// of 256 walkers of 64 He: 27.7 ms with and without).
+// ---------------------------------------------------------------------------
+struct BalanceTerms {
+  static __device__ __forceinline__ void run(const double *__restrict__ Y, int n, int K, int ny, int y_rows,
+                                             int *__restrict__ s, const uint3 bid, const uint3 gdim) {
+    assume_global(Y, s);
+    extern __shared__ int ek[];  // [K] exponent of the largest |Y(k, .)|
+    __shared__ int top[8];
+    const int w = bid.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const double *Yw = Y + (size_t)w * n * n;
+    if (y_rows) {
+      for (int k = tid; k < K; k += 256) {
+        int e = kNoExponent;
+#pragma unroll 4
+        for (int y = 0; y < ny; ++y) e = max(e, element_exponent(Yw[(size_t)y * n + k], 0));
+        ek[k] = e;
+      }
+    } else {
+      for (int k = warp; k < K; k += 8) {
+        int e = kNoExponent;
+        for (int y = lane; y < ny; y += 32) e = max(e, element_exponent(Yw[(size_t)k * n + y], 0));
+        e = __reduce_max_sync(0xffffffffu, e);
+        if (lane == 0) ek[k] = e;
+      }
+    }
+    __syncthreads();
+    int m = kNoExponent;
+    for (int k = tid; k < K; k += 256)
+      if (ek[k] != kNotFinite) m = max(m, ek[k]);
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (lane == 0) top[warp] = m;
+    __syncthreads();
+    for (int q = 0; q < 8; ++q) m = max(m, top[q]);
+    for (int k = tid; k < K; k += 256)
+      s[(size_t)w * K + k] = ek[k] == kNotFinite || ek[k] == kNoExponent ? 0 : ek[k] - m;
+  }
+};
+__global__ void __launch_bounds__(256) k_balance_terms(const double *__restrict__ Y, int n, int K, int ny, int y_rows,
+                                                       int *__restrict__ s) {
+  BalanceTerms::run(Y, n, K, ny, y_rows, s, blockIdx, gridDim);
+}
+cudaError_t launch_balance_terms(const double *Y, int n, int K, int ny, bool y_rows, int W, int *s, cudaStream_t st) {
+  if (W <= 0 || K <= 0) return cudaSuccess;
+  return launch_or_record<BalanceTerms, 256>(k_balance_terms, dim3(W), dim3(256), (size_t)K * sizeof(int), st, Y, n, K,
+                                             ny, y_rows ? 1 : 0, s);
+}
 
 // FP64 rows -> NSL exact slices of BITS bits per element relative to 2^e, e = 1 +
 // the binary exponent of the row's largest magnitude.  A warp per row, two
@@ -1134,7 +1198,8 @@ struct PackFixed64 {
   static __device__ __forceinline__ void run(const double *__restrict__ P, const int *__restrict__ list,
                                              const int *__restrict__ count, int nrows, int nsub, int stride, int L,
                                              int kp, uint16_t *__restrict__ A, int *__restrict__ rows_out,
-                                             int *__restrict__ exps, long dst_stride, long dst_off, const uint3 bid,
+                                             int *__restrict__ exps, long dst_stride, long dst_off,
+                                             const int *__restrict__ scale, const uint3 bid,
                                              const uint3 gdim) {
     assume_global(P, A, rows_out, exps);
     const int rows = count ? *count : nrows;
@@ -1143,13 +1208,10 @@ struct PackFixed64 {
     for (long m = (long)bid.x * (blockDim.x >> 5) + (threadIdx.x >> 5); m < rows; m += nw) {
       const long phys = list ? (long)list[m] : (m / nsub) * stride + (m % nsub);
       const double *src = P + phys * L;
-      unsigned mx = 0;
-      for (int k = lane; k < L; k += 32) {
-        const unsigned h = abs_hi(src[k]) | (src[k] != 0.0 ? 1u : 0u);  // (a subnormal's leading word may be 0)
-        mx = h > mx ? h : mx;
-      }
-      mx = __reduce_max_sync(0xffffffffu, mx);
-      const int e = exponent_of(mx);
+      const int *sc = scale ? scale + (m / nsub) * L : nullptr;  // element k is taken times 2^-sc[k]
+      int mx = kNoExponent;
+      for (int k = lane; k < L; k += 32) mx = max(mx, element_exponent(src[k], sc ? -sc[k] : 0));
+      const int e = exponent_of_max(__reduce_max_sync(0xffffffffu, mx));
       if (lane == 0) {
         // the row of the result: the source row, or (m / nsub) * dst_stride + dst_off + m % nsub
         rows_out[m] = dst_stride > 0 ? (int)((m / nsub) * dst_stride + dst_off + m % nsub) : (int)phys;
@@ -1158,8 +1220,8 @@ struct PackFixed64 {
       uint16_t *dst = A + m * NSL * (long)kp;
       for (int k = 2 * lane; k < kp; k += 64) {
         uint16_t t0[NSL], t1[NSL];
-        cut_slices<NSL, BITS>(k < L ? src[k] : 0.0, e, t0);
-        cut_slices<NSL, BITS>(k + 1 < L ? src[k + 1] : 0.0, e, t1);
+        cut_slices<NSL, BITS>(k < L ? src[k] : 0.0, sc && k < L ? e + sc[k] : e, t0);
+        cut_slices<NSL, BITS>(k + 1 < L ? src[k + 1] : 0.0, sc && k + 1 < L ? e + sc[k + 1] : e, t1);
   #pragma unroll
         for (int t = 0; t < NSL; ++t)
           *reinterpret_cast<uint32_t *>(dst + t * kp + k) = t0[t] | (static_cast<uint32_t>(t1[t]) << 16);
@@ -1172,33 +1234,39 @@ __global__ void __launch_bounds__(256) k_pack_fixed64(const double *__restrict__
                                                       const int *__restrict__ count, int nrows, int nsub, int stride,
                                                       int L, int kp, uint16_t *__restrict__ A,
                                                       int *__restrict__ rows_out, int *__restrict__ exps,
-                                                      long dst_stride, long dst_off) {
+                                                      long dst_stride, long dst_off,
+                                                      const int *__restrict__ scale) {
   PackFixed64<NSL, BITS>::run(P, list, count, nrows, nsub, stride, L, kp, A, rows_out, exps, dst_stride, dst_off,
-                              blockIdx, gridDim);
+                              scale, blockIdx, gridDim);
 }
 
 template <int NSL, int BITS>
 static cudaError_t pack_fixed64(const double *P, const int *list, const int *count, int nrows, int nsub, int stride,
                                 int L, int kp, uint16_t *A, int *rows_out, int *exps, int blocks, cudaStream_t st,
-                                long dst_stride, long dst_off) {
+                                long dst_stride, long dst_off, const int *scale) {
   return launch_or_record<PackFixed64<NSL, BITS>, 256>(k_pack_fixed64<NSL, BITS>, dim3(blocks), dim3(256), 0, st, P,
                                                        list, count, nrows, nsub > 0 ? nsub : 1, stride, L, kp, A,
-                                                       rows_out, exps, dst_stride, dst_off);
+                                                       rows_out, exps, dst_stride, dst_off, scale);
 }
 
 cudaError_t launch_pack_fixed64(const double *P, const int *list, const int *count, int nrows, int nsub, int stride,
                                 int L, int kp, int nsl, int bits, uint16_t *A, int *rows_out, int *exps,
-                                int max_rows, cudaStream_t st, long dst_stride, long dst_off) {
+                                int max_rows, cudaStream_t st, long dst_stride, long dst_off,
+                                const int *scale) {
   if (max_rows <= 0) return cudaSuccess;
+  if (scale && (list || nsub <= 0)) return cudaErrorInvalidValue;
   long blocks = (max_rows + 7) / 8;
   if (blocks > 152 * 16) blocks = 152 * 16;
   const int nb = (int)blocks;
   if (nsl == 6 && bits == 8)
-    return pack_fixed64<6, 8>(P, list, count, nrows, nsub, stride, L, kp, A, rows_out, exps, nb, st, dst_stride, dst_off);
+    return pack_fixed64<6, 8>(P, list, count, nrows, nsub, stride, L, kp, A, rows_out, exps, nb, st, dst_stride, dst_off,
+                              scale);
   if (nsl == 7 && bits == 8)
-    return pack_fixed64<7, 8>(P, list, count, nrows, nsub, stride, L, kp, A, rows_out, exps, nb, st, dst_stride, dst_off);
+    return pack_fixed64<7, 8>(P, list, count, nrows, nsub, stride, L, kp, A, rows_out, exps, nb, st, dst_stride, dst_off,
+                              scale);
   if (nsl == 8 && bits == 7)
-    return pack_fixed64<8, 7>(P, list, count, nrows, nsub, stride, L, kp, A, rows_out, exps, nb, st, dst_stride, dst_off);
+    return pack_fixed64<8, 7>(P, list, count, nrows, nsub, stride, L, kp, A, rows_out, exps, nb, st, dst_stride, dst_off,
+                              scale);
   return cudaErrorInvalidValue;
 }
 
@@ -1223,28 +1291,28 @@ struct PackCols {
                                              const float *__restrict__ Xlo, size_t xw, int R, int C, int kp,
                                              uint16_t *__restrict__ A, int *__restrict__ exps,
                                              int *__restrict__ rows_out, long dst_stride, long dst_off,
-                                             const uint3 bid, const uint3 gdim) {
+                                             const int *__restrict__ scale, int sign, const uint3 bid, const uint3 gdim) {
     assume_global(A, exps);
     if constexpr (kF64) assume_global(X64); else assume_global(X32);
     __shared__ double t64[kF64 ? 64 : 1][33];
     __shared__ float th[kF64 ? 1 : 64][33], tl[kF64 ? 1 : 64][33];
-    __shared__ unsigned cmax[8][32];
+    __shared__ int cmax[8][32];
     __shared__ int cexp[32];
     const int tid = threadIdx.x, cl = tid & 31, jr = tid >> 5;
     const int w = bid.y, c0 = bid.x * 32;
     const int c = c0 + cl;
     const size_t base = (size_t)w * xw;
-    // the columns' largest magnitudes, as integer bits (FP64: the leading words)
-    unsigned mx = 0;
+    // row j is taken times 2^(sign scale[j]) (FP64)
+    const int *sc = kF64 && scale ? scale + (size_t)w * R : nullptr;
+    // the columns' largest magnitudes, as integer bits (FP64: their exponents)
+    int mx = kF64 ? kNoExponent : 0;
     if (c < C)
       for (int j = jr; j < R; j += 8) {
-        unsigned h;
-        if constexpr (kF64) {
-          const double v = X64[base + (size_t)j * C + c];
-          h = abs_hi(v) | (v != 0.0 ? 1u : 0u);
-        } else {
-          h = __float_as_uint(fmaxf(0.0f, fabsf(X32[base + (size_t)j * C + c])));  // (NaN: 0)
-        }
+        int h;
+        if constexpr (kF64)
+          h = element_exponent(X64[base + (size_t)j * C + c], sc ? sign * sc[j] : 0);
+        else
+          h = __float_as_int(fmaxf(0.0f, fabsf(X32[base + (size_t)j * C + c])));  // (NaN: 0)
         mx = h > mx ? h : mx;
       }
     cmax[jr][cl] = mx;
@@ -1253,9 +1321,9 @@ struct PackCols {
       for (int q = 1; q < 8; ++q) mx = cmax[q][cl] > mx ? cmax[q][cl] : mx;
       int e;
       if constexpr (kF64) {
-        e = exponent_of(mx);
+        e = exponent_of_max(mx);
       } else {
-        const float m = __uint_as_float(mx);
+        const float m = __int_as_float(mx);
         e = m > 0.0f ? ilogbf(m) + 1 : 0;
       }
       cexp[cl] = e;
@@ -1290,7 +1358,7 @@ struct PackCols {
         for (int h = 0; h < 2; ++h) {
           const int jj = 2 * (tid & 31) + h;
           if constexpr (kF64) {
-            cut_slices<NSL, BITS>(t64[jj][col], e, sl[h]);
+            cut_slices<NSL, BITS>(t64[jj][col], sc && j0 + jj < R ? e - sign * sc[j0 + jj] : e, sl[h]);
           } else {
             float x = ldexpf(th[jj][col], 7 - e), xl = ldexpf(tl[jj][col], 7 - e);
   #pragma unroll
@@ -1316,33 +1384,38 @@ template <bool kF64, int NSL, int BITS>
 __global__ void __launch_bounds__(256) k_pack_cols(const double *__restrict__ X64, const float *__restrict__ X32,
                                                    const float *__restrict__ Xlo, size_t xw, int R, int C, int kp,
                                                    uint16_t *__restrict__ A, int *__restrict__ exps,
-                                                   int *__restrict__ rows_out, long dst_stride, long dst_off) {
-  PackCols<kF64, NSL, BITS>::run(X64, X32, Xlo, xw, R, C, kp, A, exps, rows_out, dst_stride, dst_off, blockIdx,
-                                 gridDim);
+                                                   int *__restrict__ rows_out, long dst_stride, long dst_off,
+                                                   const int *__restrict__ scale, int sign) {
+  PackCols<kF64, NSL, BITS>::run(X64, X32, Xlo, xw, R, C, kp, A, exps, rows_out, dst_stride, dst_off, scale, sign,
+                                 blockIdx, gridDim);
 }
 
 template <bool kF64, int NSL, int BITS>
 static cudaError_t pack_cols(const double *X64, const float *X32, const float *Xlo, size_t xw, int R, int C, int kp,
                              int W, uint16_t *A, int *exps, int *rows_out, long dst_stride, long dst_off,
-                             cudaStream_t st) {
+                             cudaStream_t st, const int *scale, int sign) {
   return launch_or_record<PackCols<kF64, NSL, BITS>, 256>(k_pack_cols<kF64, NSL, BITS>, dim3((C + 31) / 32, W),
                                                           dim3(256), 0, st, X64, X32, Xlo, xw, R, C, kp, A, exps,
-                                                          rows_out, dst_stride, dst_off);
+                                                          rows_out, dst_stride, dst_off, scale, sign);
 }
 
 cudaError_t launch_pack_cols(const double *X64, const float *X32, const float *Xlo, size_t xw, int R, int C, int kp,
                              int W, uint16_t *A, int *exps, int *rows_out, long dst_stride, long dst_off,
-                             cudaStream_t st, int nsl, int bits) {
+                             cudaStream_t st, int nsl, int bits, const int *scale, int sign) {
   if (W <= 0 || C <= 0) return cudaSuccess;
-  if (kp % 64 != 0 || kp < R || (X64 == nullptr) == (X32 == nullptr)) return cudaErrorInvalidValue;
+  if (kp % 64 != 0 || kp < R || (X64 == nullptr) == (X32 == nullptr) || (scale && !X64)) return cudaErrorInvalidValue;
   if (X32 && nsl == 6 && bits == 8)
-    return pack_cols<false, 6, 8>(X64, X32, Xlo, xw, R, C, kp, W, A, exps, rows_out, dst_stride, dst_off, st);
+    return pack_cols<false, 6, 8>(X64, X32, Xlo, xw, R, C, kp, W, A, exps, rows_out, dst_stride, dst_off, st, scale,
+                               sign);
   if (X64 && nsl == 6 && bits == 8)
-    return pack_cols<true, 6, 8>(X64, X32, Xlo, xw, R, C, kp, W, A, exps, rows_out, dst_stride, dst_off, st);
+    return pack_cols<true, 6, 8>(X64, X32, Xlo, xw, R, C, kp, W, A, exps, rows_out, dst_stride, dst_off, st, scale,
+                               sign);
   if (X64 && nsl == 7 && bits == 8)
-    return pack_cols<true, 7, 8>(X64, X32, Xlo, xw, R, C, kp, W, A, exps, rows_out, dst_stride, dst_off, st);
+    return pack_cols<true, 7, 8>(X64, X32, Xlo, xw, R, C, kp, W, A, exps, rows_out, dst_stride, dst_off, st, scale,
+                               sign);
   if (X64 && nsl == 8 && bits == 7)
-    return pack_cols<true, 8, 7>(X64, X32, Xlo, xw, R, C, kp, W, A, exps, rows_out, dst_stride, dst_off, st);
+    return pack_cols<true, 8, 7>(X64, X32, Xlo, xw, R, C, kp, W, A, exps, rows_out, dst_stride, dst_off, st, scale,
+                               sign);
   return cudaErrorInvalidValue;
 }
 
