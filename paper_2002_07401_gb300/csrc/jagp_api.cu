@@ -358,7 +358,7 @@ jagp_status_t run_mmat64(jagp_ctx *h, void *state, int W, cudaStream_t st) {
   const double *gi = at<double>(state, L.ginv), *bt = at<double>(state, L.bt), *a_up = at<double>(state, L.a_up);
   double *m = at<double>(state, L.mbuf);
   if (!tc_products(h)) {
-    LAUNCH(JAGP_KERNEL_ENERGY, 1, launch_mmat<double>(h->ds, gi, bt, a_up, m, W, st));
+    LAUNCH(JAGP_KERNEL_ENERGY, 1, launch_mmat(h->ds, gi, bt, a_up, m, W, st));
     return JAGP_OK;
   }
   const int n = h->ds.n_up, nd = h->ds.n_dn;

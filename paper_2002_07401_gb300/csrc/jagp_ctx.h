@@ -21,11 +21,12 @@ struct jagp_ctx {
   long long launches = 0;
   int prof_kernel = 0;
   std::vector<std::pair<cudaEvent_t, cudaEvent_t>> prof_events;
-  // mixed path: lambda as fixed-point slices (kFixedSlices exact 8-bit integer
-  // terms per element, BF16) with one exponent per output column, for the tensor cores
+  // lambda as fixed-point slices (mixed path: kFixedSlices exact 8-bit integer terms per
+  // element, FP64-equivalent: tc_slices of tc_bits, BF16) with one exponent per output
+  // column, for the tensor cores
   int kp = 0;                            // L padded to a multiple of 64
-  const uint16_t *split_lamT = nullptr;  // [L][5 kp]: row n slices lambda[:, n]  (A_up = phi^T lambda)
-  const uint16_t *split_lam = nullptr;   // [L][5 kp]: row n slices lambda[n, :]  (Bt = lambda phi)
+  const uint16_t *split_lamT = nullptr;  // [L][slices kp]: row n slices lambda[:, n]  (A_up = phi^T lambda)
+  const uint16_t *split_lam = nullptr;   // [L][slices kp]: row n slices lambda[n, :]  (Bt = lambda phi)
   const int *exp_lamT = nullptr;         // [L] exponents of those rows
   const int *exp_lam = nullptr;          // [L]
   // non-zero K range [x, y) per 16 rows of the sliced lambda^T and lambda
@@ -33,7 +34,7 @@ struct jagp_ctx {
   int *d_err = nullptr;                  // tensor-core pipeline timeout flag
   // tile choices of jagp_autotune (0 / -1: the shape heuristics)
   int tune_bn_left = 0, tune_bn_right = 0;  // tensor-core tile width of the lambda products
-  int tune_st_left = 0, tune_st_right = 0;  // and pipeline depth (0: as many stages as fit)
+  int tune_st_left = 0, tune_st_right = 0;  // and K chunk (-1, -2, -3: 64, 32, 16; else by the shape)
   int tune_tile_prop = -1;                  // per-walker proposal products (gemm_rows tile)
   int tune_tile_refresh = -1;               // per-walker refresh product G~ = Phi_up Bt^T
   // guided sampling (jagp_set_guiding): eps > 0 samples Psi_G instead of Psi_T

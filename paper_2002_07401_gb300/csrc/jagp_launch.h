@@ -78,8 +78,7 @@ cudaError_t launch_j3_prep(const DevSystem &s, const double *r, double *buf, int
 
 // M vectors of the kinetic energy (see k_linalg.cu), then the orbital
 // derivative contractions and the final per-walker local energy.
-template <typename T>
-cudaError_t launch_mmat(const DevSystem &s, const T *ginv, const T *bt, const T *a_up, T *mbuf, int W,
+cudaError_t launch_mmat(const DevSystem &s, const double *ginv, const double *bt, const double *a_up, double *mbuf, int W,
                         cudaStream_t st);
 cudaError_t launch_kinetic(const DevSystem &s, const double *r, const double *mbuf, double *kin, int W,
                            cudaStream_t st);
@@ -228,7 +227,7 @@ cudaError_t launch_sr_jastrow(const DevSystem &s, const double *r, double *O, lo
                               cudaStream_t st);
 // workspace of the SR solve (offsets in doubles)
 struct SrLayout {
-  size_t obar, diag, dinv, x, r, z, p, q, u, part, ec, t, sc, dots, total;
+  size_t obar, diag, dinv, x, r, z, p, q, part, ec, t, sc, dots, total;
 };
 SrLayout sr_layout(int M, int P);
 // Obar, diag S and f = -(2/M) sum_i (e_i - ebar)(O_i - Obar) from the samples

@@ -1514,31 +1514,29 @@ template cudaError_t launch_refresh_inverse<float>(double *, float *, double *, 
 //   down: M[n_up + j] = sum_i Ginv[j][i] A_up[i]   (A_up[i] = phi(r_i^up)^T lambda)
 // and the same M with the Laplacians.  One CTA per (walker, 64 columns).
 // ---------------------------------------------------------------------------
-template <typename T>
 struct Mmat {
-  static __device__ __forceinline__ void run(DevSystem s, const T *__restrict__ ginv, const T *__restrict__ bt,
-                                             const T *__restrict__ a_up, T *__restrict__ mbuf, const uint3 bid,
+  static __device__ __forceinline__ void run(DevSystem s, const double *__restrict__ ginv, const double *__restrict__ bt,
+                                             const double *__restrict__ a_up, double *__restrict__ mbuf, const uint3 bid,
                                              const uint3 gdim) {
     assume_global(ginv, bt, a_up, mbuf);
-    extern __shared__ double smd[];
-    T *sm = reinterpret_cast<T *>(smd);
+    extern __shared__ double sm[];
     const int n = s.n_up, nd = s.n_dn, N = s.N, L = s.L;
     const int w = bid.y, c0 = bid.x * 64, tid = threadIdx.x;
-    T *Gs = sm;              // n*n
-    T *Bs = Gs + n * n;      // n*64
-    T *As = Bs + n * 64;     // n*64
+    double *Gs = sm;              // n*n
+    double *Bs = Gs + n * n;      // n*64
+    double *As = Bs + n * 64;     // n*64
     for (int t = tid; t < n * n; t += 256) Gs[t] = ginv[(size_t)w * n * n + t];
     for (int t = tid; t < n * 64; t += 256) {
       const int j = t >> 6, c = t & 63;
       const bool in = c0 + c < L;
-      Bs[t] = in ? bt[((size_t)w * n + j) * L + c0 + c] : T(0);
-      As[t] = in ? a_up[((size_t)w * n + j) * L + c0 + c] : T(0);
+      Bs[t] = in ? bt[((size_t)w * n + j) * L + c0 + c] : 0.0;
+      As[t] = in ? a_up[((size_t)w * n + j) * L + c0 + c] : 0.0;
     }
     __syncthreads();
     for (int idx = tid; idx < N * 64; idx += 256) {
       const int e = idx >> 6, c = idx & 63;
       if (c0 + c >= L) continue;
-      T acc = T(0);
+      double acc = 0.0;
       if (e < n) {
         for (int j = 0; j < n; ++j) acc = fma(Gs[j * n + e], Bs[j * 64 + c], acc);
       } else {
@@ -1550,44 +1548,42 @@ struct Mmat {
     }
 }
 };
-template <typename T>
-__global__ void __launch_bounds__(256) k_mmat(DevSystem s, const T *__restrict__ ginv, const T *__restrict__ bt,
-                                              const T *__restrict__ a_up, T *__restrict__ mbuf) {
-  Mmat<T>::run(s, ginv, bt, a_up, mbuf, blockIdx, gridDim);
+__global__ void __launch_bounds__(256) k_mmat(DevSystem s, const double *__restrict__ ginv, const double *__restrict__ bt,
+                                              const double *__restrict__ a_up, double *__restrict__ mbuf) {
+  Mmat::run(s, ginv, bt, a_up, mbuf, blockIdx, gridDim);
 }
 
 // The same contraction for N_up too large to stage G~^{-1} whole: 64 x 64
 // output tiles (electrons x basis functions), 4 x 4 per thread, the sum over
 // j (or i) in chunks of 16 in the same order as above.  Up tiles come first in
 // blockIdx.y, then down tiles, so that no tile mixes the two formulas.
-template <typename T>
 struct MmatTiled {
-  static __device__ __forceinline__ void run(DevSystem s, const T *__restrict__ ginv, const T *__restrict__ bt,
-                                             const T *__restrict__ a_up, T *__restrict__ mbuf, const uint3 bid,
+  static __device__ __forceinline__ void run(DevSystem s, const double *__restrict__ ginv, const double *__restrict__ bt,
+                                             const double *__restrict__ a_up, double *__restrict__ mbuf, const uint3 bid,
                                              const uint3 gdim) {
     assume_global(ginv, bt, a_up, mbuf);
-    __shared__ T Xs[16][64];  // Xs[k][e]: G~^{-1}[k][e] (up) or G~^{-1}[e][k] (down)
-    __shared__ T Ys[16][64];  // Ys[k][c]: Bt[k][c] (up) or A_up[k][c] (down)
+    __shared__ double Xs[16][64];  // Xs[k][e]: G~^{-1}[k][e] (up) or G~^{-1}[e][k] (down)
+    __shared__ double Ys[16][64];  // Ys[k][c]: Bt[k][c] (up) or A_up[k][c] (down)
     const int n = s.n_up, N = s.N, L = s.L;
     const int w = bid.z, c0 = bid.x * 64, tid = threadIdx.x;
     const int up_tiles = (n + 63) / 64;
     const bool up = (int)bid.y < up_tiles;
     const int e0 = up ? bid.y * 64 : (bid.y - up_tiles) * 64;  // within the species
     const int ne = up ? n : s.n_dn;
-    const T *G = ginv + (size_t)w * n * n;
-    const T *Y = (up ? bt : a_up) + (size_t)w * n * L;
+    const double *G = ginv + (size_t)w * n * n;
+    const double *Y = (up ? bt : a_up) + (size_t)w * n * L;
     const int tx = tid & 15, ty = tid >> 4;
-    T acc[4][4];
+    double acc[4][4];
   #pragma unroll
     for (int a = 0; a < 4; ++a)
   #pragma unroll
-      for (int b = 0; b < 4; ++b) acc[a][b] = T(0);
+      for (int b = 0; b < 4; ++b) acc[a][b] = 0.0;
     for (int k0 = 0; k0 < n; k0 += 16) {
   #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int idx = tid + q * 256;
         const int kk = idx >> 6, col = idx & 63, k = k0 + kk;
-        T xv = T(0), yv = T(0);
+        double xv = 0.0, yv = 0.0;
         if (k < n) {
           const int e = e0 + col;
           if (e < ne) xv = up ? G[(size_t)k * n + e] : G[(size_t)e * n + k];
@@ -1599,7 +1595,7 @@ struct MmatTiled {
       __syncthreads();
   #pragma unroll
       for (int kk = 0; kk < 16; ++kk) {
-        T xa[4], yb[4];
+        double xa[4], yb[4];
   #pragma unroll
         for (int a = 0; a < 4; ++a) xa[a] = Xs[kk][ty * 4 + a];
   #pragma unroll
@@ -1616,7 +1612,7 @@ struct MmatTiled {
     for (int a = 0; a < 4; ++a) {
       const int e = e0 + ty * 4 + a;
       if (e >= ne) continue;
-      T *o = mbuf + ((size_t)w * N + ebase + e) * L;
+      double *o = mbuf + ((size_t)w * N + ebase + e) * L;
   #pragma unroll
       for (int b = 0; b < 4; ++b) {
         const int c = c0 + tx * 4 + b;
@@ -1625,10 +1621,9 @@ struct MmatTiled {
     }
 }
 };
-template <typename T>
-__global__ void __launch_bounds__(256) k_mmat_tiled(DevSystem s, const T *__restrict__ ginv, const T *__restrict__ bt,
-                                                    const T *__restrict__ a_up, T *__restrict__ mbuf) {
-  MmatTiled<T>::run(s, ginv, bt, a_up, mbuf, blockIdx, gridDim);
+__global__ void __launch_bounds__(256) k_mmat_tiled(DevSystem s, const double *__restrict__ ginv, const double *__restrict__ bt,
+                                                    const double *__restrict__ a_up, double *__restrict__ mbuf) {
+  MmatTiled::run(s, ginv, bt, a_up, mbuf, blockIdx, gridDim);
 }
 
 // The mixed path's M vectors for small N_up on the CUDA cores: the sums of
@@ -1728,23 +1723,18 @@ cudaError_t launch_mmat_dw(const DevSystem &s, const double *ginv64, const float
                                        mlo);
 }
 
-template <typename T>
-cudaError_t launch_mmat(const DevSystem &s, const T *ginv, const T *bt, const T *a_up, T *mbuf, int W,
+cudaError_t launch_mmat(const DevSystem &s, const double *ginv, const double *bt, const double *a_up, double *mbuf, int W,
                         cudaStream_t st) {
   if (W <= 0) return cudaSuccess;
   const int n = s.n_up;
-  const size_t smem = (size_t)(n * n + 2 * n * 64) * sizeof(T);
+  const size_t smem = (size_t)(n * n + 2 * n * 64) * sizeof(double);
   if (smem > kMmatSmemMax) {
     dim3 grid((s.L + 63) / 64, (n + 63) / 64 + (s.n_dn + 63) / 64, W);
-    return launch_or_record<MmatTiled<T>, 256>(k_mmat_tiled<T>, grid, dim3(256), 0, st, s, ginv, bt, a_up, mbuf);
+    return launch_or_record<MmatTiled, 256>(k_mmat_tiled, grid, dim3(256), 0, st, s, ginv, bt, a_up, mbuf);
   }
   dim3 grid((s.L + 63) / 64, W);
-  return launch_or_record<Mmat<T>, 256>(k_mmat<T>, grid, dim3(256), smem, st, s, ginv, bt, a_up, mbuf);
+  return launch_or_record<Mmat, 256>(k_mmat, grid, dim3(256), smem, st, s, ginv, bt, a_up, mbuf);
 }
-template cudaError_t launch_mmat<double>(const DevSystem &, const double *, const double *, const double *, double *,
-                                         int, cudaStream_t);
-template cudaError_t launch_mmat<float>(const DevSystem &, const float *, const float *, const float *, float *, int,
-                                        cudaStream_t);
 
 // the kernels of this file raise their shared-memory limit when first
 // launched (launch_or_record)

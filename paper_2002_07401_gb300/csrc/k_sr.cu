@@ -418,7 +418,6 @@ SrLayout sr_layout(int M, int P) {
   l.z = take(P);
   l.p = take(P);
   l.q = take(P);
-  l.u = take(P);
   l.part = take((size_t)kRowChunks * P);
   l.ec = take(M);
   l.t = take(M);
