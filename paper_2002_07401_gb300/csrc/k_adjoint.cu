@@ -447,7 +447,7 @@ __global__ void __launch_bounds__(kJasWarps * 32) k_adj_jastrow(DevSystem s, con
         for (int q = 0; q < 3; ++q) re[q] = z3 * d[q];
         if (s.use_j1) {
           double f1, f2, f3, fb, hv[3], gl;
-          j1_d3(c1, s.b_ea, r2 * ri, &f1, &f2, &f3, &fb);
+          j1_d3(c1, s.b_ea, r2 == 0.0 ? 0.0 : r2 * ri, &f1, &f2, &f3, &fb);  // (dJ/db is finite at the nucleus)
           radial_adj(f1, f2, f3, d, ri, gJb + 3 * e, hv, &gl);
           gl *= lJb;
 #pragma unroll
@@ -498,7 +498,7 @@ __global__ void __launch_bounds__(kJasWarps * 32) k_adj_jastrow(DevSystem s, con
         const bool same = eup == (k < s.n_up);
         double kk, bb, v1, v2, v3, hv[3], gl;
         j2_params(s, same, &kk, &bb);
-        const double ik = kk == 4.0 ? 0.25 : 0.5, rr = r2 * ri, iq = 1.0 / (1.0 + bb * rr);
+        const double ik = kk == 4.0 ? 0.25 : 0.5, rr = r2 == 0.0 ? 0.0 : r2 * ri, iq = 1.0 / (1.0 + bb * rr);
         j2_d3(ik, bb, iq, &v1, &v2, &v3);
         const double dg[3] = {gJb[3 * e] - gJb[3 * k], gJb[3 * e + 1] - gJb[3 * k + 1], gJb[3 * e + 2] - gJb[3 * k + 2]};
         radial_adj(v1, v2, v3, d, ri, dg, hv, &gl);
