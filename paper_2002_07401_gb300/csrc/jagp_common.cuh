@@ -276,7 +276,8 @@ __device__ __forceinline__ DwDisp displacement(const fdw p[3], const fdw R[3]) {
 // per atom (an atom has several shells: eight in the 20-function recipe, whose
 // displacements and squares were a quarter of the instructions of a shell's value)
 // into the warp's table, unless shared memory has no room for one (some thousand
-// atoms): then per shell.  kDw: double-words, else FP64.
+// atoms): then per shell, from the atoms in shared memory or (tables < 0: more than
+// eight thousand) in global memory.  kDw: double-words, else FP64.
 template <bool kDw>
 struct ShellStage {
   using Num = typename std::conditional<kDw, fdw, double>::type;
@@ -285,26 +286,28 @@ struct ShellStage {
   static constexpr int kWarps = 8;
   D *tab;      // [atoms] of this warp, or null
   Num *zeta;   // [shells]
-  Num *R;      // [atoms][3]
+  Num *R;      // [atoms][3], or null
   int *info, *atom;
+  const double *R_sys;
   int n_atoms;
   static __host__ __device__ size_t bytes(const DevSystem &s, int tables) {
-    return (size_t)s.n_atoms * (32 * tables + 24) + (size_t)s.n_shells * 16;
+    return (tables >= 0 ? (size_t)s.n_atoms * (32 * tables + 24) : 0) + (size_t)s.n_shells * 16;
   }
-  // warps per CTA (eight, fewer where that leaves room for two CTAs on an SM) and tables (0 or one per warp)
+  // warps per CTA (eight, fewer where that leaves room for two CTAs on an SM) and tables
+  // (one per warp, 0, or -1 where the atoms do not fit either)
   static void plan(const DevSystem &s, int *warps, int *tables) {
     int w = kWarps;
     while (w > 1 && bytes(s, w) > 112 * 1024) w /= 2;
-    *tables = bytes(s, w) <= 200 * 1024 ? w : 0;
-    *warps = *tables ? w : kWarps;
+    *tables = bytes(s, w) <= 200 * 1024 ? w : (bytes(s, 0) <= 200 * 1024 ? 0 : -1);
+    *warps = *tables > 0 ? w : kWarps;
   }
-  __device__ __forceinline__ ShellStage(const DevSystem &s, void *sm, int tables) : n_atoms(s.n_atoms) {
+  __device__ __forceinline__ ShellStage(const DevSystem &s, void *sm, int tables) : R_sys(s.R), n_atoms(s.n_atoms) {
     D *t = static_cast<D *>(sm);
-    zeta = reinterpret_cast<Num *>(t + (size_t)tables * n_atoms);
-    R = zeta + s.n_shells;
-    info = reinterpret_cast<int *>(R + 3 * n_atoms);
+    zeta = reinterpret_cast<Num *>(t + (tables > 0 ? (size_t)tables * n_atoms : 0));
+    R = tables >= 0 ? zeta + s.n_shells : nullptr;
+    info = reinterpret_cast<int *>(zeta + s.n_shells + (tables >= 0 ? 3 * n_atoms : 0));
     atom = info + s.n_shells;
-    tab = tables ? t + (size_t)(threadIdx.x >> 5) * n_atoms : nullptr;
+    tab = tables > 0 ? t + (size_t)(threadIdx.x >> 5) * n_atoms : nullptr;
     for (int k = threadIdx.x; k < s.n_shells; k += blockDim.x) {
       if constexpr (kDw)
         zeta[k] = fdw{s.shell_dw[2 * k].w, s.shell_dw[2 * k + 1].w};
@@ -313,13 +316,15 @@ struct ShellStage {
       info[k] = s.shell_info[k];
       atom[k] = s.shell_atom[k];
     }
-    for (int t3 = threadIdx.x; t3 < 3 * n_atoms; t3 += blockDim.x) {
-      if constexpr (kDw)
-        R[t3] = dw_of(s.R[t3]);
-      else
-        R[t3] = s.R[t3];
-    }
+    if (R)
+      for (int t3 = threadIdx.x; t3 < 3 * n_atoms; t3 += blockDim.x) R[t3] = coord(t3);
     __syncthreads();
+  }
+  __device__ __forceinline__ Num coord(int t3) const {
+    if constexpr (kDw)
+      return dw_of(R_sys[t3]);
+    else
+      return R_sys[t3];
   }
   // this warp's table for the point p
   __device__ __forceinline__ void point(const Num p[3], int lane) {
@@ -336,7 +341,12 @@ struct ShellStage {
   }
   // the point's displacement from shell k's atom
   __device__ __forceinline__ D disp(const Num p[3], int k) const {
-    if (!tab) return displacement(p, R + 3 * atom[k]);
+    if (!tab) {
+      const int a = 3 * atom[k];
+      if (R) return displacement(p, R + a);
+      const Num q[3] = {coord(a), coord(a + 1), coord(a + 2)};
+      return displacement(p, q);
+    }
     D d;
     const float4 *q = reinterpret_cast<const float4 *>(tab + atom[k]);
     float4 *v = reinterpret_cast<float4 *>(&d);
