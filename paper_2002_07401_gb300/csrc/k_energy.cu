@@ -374,12 +374,15 @@ __global__ void __launch_bounds__(128) k_elocal(DevSystem s, const double *__res
 // and reduced four sums per electron (sweeps of 4096 walkers of 16 He 2.94 ms, of 64
 // walkers of 256 He 26.9; 2.70 and 25.5 with this kernel, before in 345 us and 2.2 ms).
 // ---------------------------------------------------------------------------
+// ATOMS: the atoms' constants in shared memory; else (some four thousand atoms, which do
+// not fit) formed where they are used.
 constexpr int kElocalDwThreads = 512;  // at most
+template <bool ATOMS>
 struct ElocalDw {
   static __host__ __device__ int splits(int N, int threads) { return threads >= 2 * N ? threads / N : 1; }
   // floats: coordinates, atoms' constants, sums of the electrons per split
   static size_t smem(const DevSystem &s, int threads) {
-    return sizeof(float) * (((size_t)(s.N + s.n_atoms) * 6 + (size_t)s.n_atoms * 8 + 3) / 4 * 4 +
+    return sizeof(float) * (((size_t)s.N * 6 + (ATOMS ? (size_t)s.n_atoms * 14 : 0) + 3) / 4 * 4 +
                             (size_t)splits(s.N, threads) * s.N * 8);
   }
   static __device__ __forceinline__ void run(DevSystem s, const double *__restrict__ r,
@@ -387,16 +390,16 @@ struct ElocalDw {
                                              double *__restrict__ parts, double *__restrict__ scal,
                                              const double *__restrict__ j3buf, const uint3 bid, const uint3 gdim) {
     assume_global(r, kin, eL);
-    const int w = bid.x, N = s.N, tid = threadIdx.x, bs = blockDim.x, na = s.n_atoms;
+    const int w = bid.x, N = s.N, tid = threadIdx.x, bs = blockDim.x, na = s.n_atoms, ns = ATOMS ? na : 0;
     const int lane = tid & 31, warp = tid >> 5, nw = bs >> 5;
     extern __shared__ float4 sf4[];
     float *xh = reinterpret_cast<float *>(sf4), *xl = xh + 3 * N;  // electron coordinates as double-words
-    float *ah = xl + 3 * N, *al = ah + 3 * na;                     // atom coordinates
+    float *ah = xl + 3 * N, *al = ah + 3 * ns;                     // atom coordinates
     // per atom, as double-words: -Z, and for J1 -c^4/2, c^3/(2b), -b c
-    float *ac = al + 3 * na;
+    float *ac = al + 3 * ns;
     // grad J (x, y) and (z), lap J of electron e in split k: jg[k N + e], jl[k N + e]
     const int R = splits(N, bs);
-    float4 *jg = sf4 + (6 * (N + na) + 8 * na + 3) / 4, *jl = jg + R * N;
+    float4 *jg = sf4 + (6 * N + 14 * ns + 3) / 4, *jl = jg + R * N;
     // two-body Jastrow constants [same spin, opposite spin]: b k (dw), k, -2 b (dw)
     __shared__ float j2c[2][5];
     for (int t = tid; t < N * 3; t += bs) {
@@ -404,16 +407,15 @@ struct ElocalDw {
       xh[t] = v.hi;
       xl[t] = v.lo;
     }
-    for (int t = tid; t < na * 3; t += bs) {
+    for (int t = tid; t < ns * 3; t += bs) {
       const fdw v = dw_of(s.R[t]);
       ah[t] = v.hi;
       al[t] = v.lo;
     }
-    for (int a = tid; a < na; a += bs) {
+    auto atom_constants = [&](int a, float *q) {
       const double c = s.c1[a], b = s.b_ea;
       const fdw z = dw_of(-s.Z[a]), c4 = dw_of(-0.5 * c * c * c * c);
       const fdw c3 = dw_of(b == 0.0 ? 0.0 : c * c * c / (2.0 * b)), bc = dw_of(-b * c);
-      float *q = ac + 8 * a;
       q[0] = z.hi;
       q[1] = z.lo;
       q[2] = c4.hi;
@@ -422,7 +424,8 @@ struct ElocalDw {
       q[5] = c3.lo;
       q[6] = bc.hi;
       q[7] = bc.lo;
-    }
+    };
+    for (int a = tid; a < ns; a += bs) atom_constants(a, ac + 8 * a);
     if (tid < 2) {
       double kk, bb;
       j2_params(s, tid == 0, &kk, &bb);
@@ -435,7 +438,7 @@ struct ElocalDw {
     }
     for (int t = tid; t < R * N; t += bs) jg[t] = jl[t] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     __syncthreads();
-    // every constant comes from shared memory, so the loops are FP32 only
+    // every constant comes from shared memory (ATOMS), so the loops are FP32 only
     const fdw zero{0.0f, 0.0f};
     fdw tkin = zero, vee = zero, vei = zero, jv = zero;
     const int half = N / 2;
@@ -447,10 +450,22 @@ struct ElocalDw {
 #pragma unroll
         for (int k = 0; k < 3; ++k) pe[k] = fdw{xh[3 * e + k], xl[3 * e + k]};
         for (int a = split; a < na; a += R) {
-          const float *q = ac + 8 * a;
-          const fdw dx = dw_add(pe[0], fdw{-ah[3 * a], -al[3 * a]});
-          const fdw dy = dw_add(pe[1], fdw{-ah[3 * a + 1], -al[3 * a + 1]});
-          const fdw dz = dw_add(pe[2], fdw{-ah[3 * a + 2], -al[3 * a + 2]});
+          const float *q = ac + 8 * a, *qh = ah + 3 * a, *ql = al + 3 * a;
+          float own[14];
+          if constexpr (!ATOMS) {
+            atom_constants(a, own);
+            for (int k = 0; k < 3; ++k) {
+              const fdw v = dw_of(s.R[3 * a + k]);
+              own[8 + k] = v.hi;
+              own[11 + k] = v.lo;
+            }
+            q = own;
+            qh = own + 8;
+            ql = own + 11;
+          }
+          const fdw dx = dw_add(pe[0], fdw{-qh[0], -ql[0]});
+          const fdw dy = dw_add(pe[1], fdw{-qh[1], -ql[1]});
+          const fdw dz = dw_add(pe[2], fdw{-qh[2], -ql[2]});
           const fdw r2 = dw_add(dw_add(dw_mul(dx, dx), dw_mul(dy, dy)), dw_mul(dz, dz));
           const fdw rr = dw_sqrt(r2), rinv = dw_recip(rr);
           vei = dw_add(vei, dw_mul(rinv, fdw{q[0], q[1]}));
@@ -581,10 +596,11 @@ struct ElocalDw {
     }
 }
 };
+template <bool ATOMS>
 __global__ void __launch_bounds__(kElocalDwThreads)
     k_elocal_dw(DevSystem s, const double *__restrict__ r, const double *__restrict__ kin, double *__restrict__ eL,
                 double *__restrict__ parts, double *__restrict__ scal, const double *__restrict__ j3buf) {
-  ElocalDw::run(s, r, kin, eL, parts, scal, j3buf, blockIdx, gridDim);
+  ElocalDw<ATOMS>::run(s, r, kin, eL, parts, scal, j3buf, blockIdx, gridDim);
 }
 
 cudaError_t launch_elocal_dw(const DevSystem &s, const double *r, const double *kin, double *eL, double *parts, int W,
@@ -598,9 +614,14 @@ cudaError_t launch_elocal_dw(const DevSystem &s, const double *r, const double *
   while (threads < kElocalDwThreads && (long)W * threads < 152L * 1024) threads *= 2;
   if (threads == 128 && (s.N <= 128 ? 128 / s.N * s.N : 64) < 96) threads = 256;
   if (group_recorder()) threads = 256;
-  const size_t smem = ElocalDw::smem(s, threads);
-  return launch_or_record<ElocalDw, kElocalDwThreads>(k_elocal_dw, dim3(W), dim3(threads), smem, st, s, r, kin, eL,
-                                                      parts, scal, j3buf);
+  // (216 KB: static shared memory and the arguments of a grouped launch come on top)
+  const size_t smem = ElocalDw<true>::smem(s, threads);
+  if (smem > 216 * 1024)
+    return launch_or_record<ElocalDw<false>, kElocalDwThreads>(k_elocal_dw<false>, dim3(W), dim3(threads),
+                                                               ElocalDw<false>::smem(s, threads), st, s, r, kin, eL,
+                                                               parts, scal, j3buf);
+  return launch_or_record<ElocalDw<true>, kElocalDwThreads>(k_elocal_dw<true>, dim3(W), dim3(threads), smem, st, s, r,
+                                                            kin, eL, parts, scal, j3buf);
 }
 
 cudaError_t launch_elocal(const DevSystem &s, const double *r, const double *kin, double *eL, double *parts, int W,

@@ -42,3 +42,18 @@ def test_orbitals(prec):
     assert np.all(np.abs(la.cpu().numpy() - la_ref) <= tol * np.maximum(1.0, np.abs(la_ref)))
     assert np.array_equal(sg.cpu().numpy(), sg_ref)
     h.close()
+
+
+# mixed precision: about as many atoms as shared memory holds the constants of (4100 and three walkers of four electrons
+# are beside it with the electrons' sums), and far more
+@pytest.mark.parametrize("prec,na", [("fp64", 9800), ("mixed", 3700), ("mixed", 4100), ("mixed", 9800)])
+def test_local_energy(prec, na):
+    sysm, x = _case(na)
+    e_ref = oracle.Oracle(sysm).local_energy_batch(x)
+    h = _handle(sysm, prec, len(x))
+    r = h.positions(x)
+    h.eval(r)
+    e = h.local_energy(r).cpu().numpy()
+    tol = 1e-5 if prec == "mixed" else 1e-10
+    assert np.all(np.abs(e - e_ref) <= tol * np.maximum(1.0, np.abs(e_ref)))
+    h.close()
