@@ -4,6 +4,7 @@
 //   e_L = -1/2 sum_i lap_i Psi/Psi - sum_{i,a} Z_a/r_ia + sum_{i<j} 1/r_ij + sum_{a<b} Z_a Z_b/R_ab.
 #include <math.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "j3.cuh"
@@ -365,8 +366,8 @@ __global__ void __launch_bounds__(128) k_elocal(DevSystem s, const double *__res
 // combined in FP64 at the end.
 //
 // Bound by FP32 issue (about 650 instructions per electron-atom pair, 450 per
-// electron pair), so that lanes are kept busy and a pair is formed once: R =
-// threads / N threads per electron share its atoms and its distances o to a
+// electron pair), so that lanes are kept busy and a pair is formed once: R
+// threads per electron share its atoms and its distances o to a
 // partner (e + o) mod N, o = 1 .. N/2.  An electron's sums stay in its thread's
 // registers; a partner's go to shared memory, which is free of conflicts because
 // the partners of one o differ (a barrier between two o).  A warp per electron
@@ -379,16 +380,16 @@ __global__ void __launch_bounds__(128) k_elocal(DevSystem s, const double *__res
 constexpr int kElocalDwThreads = 512;  // at most
 template <bool ATOMS>
 struct ElocalDw {
-  static __host__ __device__ int splits(int N, int threads) { return threads >= 2 * N ? threads / N : 1; }
   // floats: coordinates, atoms' constants, sums of the electrons per split
-  static size_t smem(const DevSystem &s, int threads) {
+  static size_t smem(const DevSystem &s, int R) {
     return sizeof(float) * (((size_t)s.N * 6 + (ATOMS ? (size_t)s.n_atoms * 14 : 0) + 3) / 4 * 4 +
-                            (size_t)splits(s.N, threads) * s.N * 8);
+                            (size_t)R * s.N * 8);
   }
   static __device__ __forceinline__ void run(DevSystem s, const double *__restrict__ r,
                                              const double *__restrict__ kin, double *__restrict__ eL,
                                              double *__restrict__ parts, double *__restrict__ scal,
-                                             const double *__restrict__ j3buf, const uint3 bid, const uint3 gdim) {
+                                             const double *__restrict__ j3buf, int R, const uint3 bid,
+                                             const uint3 gdim) {
     assume_global(r, kin, eL);
     const int w = bid.x, N = s.N, tid = threadIdx.x, bs = blockDim.x, na = s.n_atoms, ns = ATOMS ? na : 0;
     const int lane = tid & 31, warp = tid >> 5, nw = bs >> 5;
@@ -398,7 +399,6 @@ struct ElocalDw {
     // per atom, as double-words: -Z, and for J1 -c^4/2, c^3/(2b), -b c
     float *ac = al + 3 * ns;
     // grad J (x, y) and (z), lap J of electron e in split k: jg[k N + e], jl[k N + e]
-    const int R = splits(N, bs);
     float4 *jg = sf4 + (6 * N + 14 * ns + 3) / 4, *jl = jg + R * N;
     // two-body Jastrow constants [same spin, opposite spin]: b k (dw), k, -2 b (dw)
     __shared__ float j2c[2][5];
@@ -599,29 +599,38 @@ struct ElocalDw {
 template <bool ATOMS>
 __global__ void __launch_bounds__(kElocalDwThreads)
     k_elocal_dw(DevSystem s, const double *__restrict__ r, const double *__restrict__ kin, double *__restrict__ eL,
-                double *__restrict__ parts, double *__restrict__ scal, const double *__restrict__ j3buf) {
-  ElocalDw<ATOMS>::run(s, r, kin, eL, parts, scal, j3buf, blockIdx, gridDim);
+                double *__restrict__ parts, double *__restrict__ scal, const double *__restrict__ j3buf, int R) {
+  ElocalDw<ATOMS>::run(s, r, kin, eL, parts, scal, j3buf, R, blockIdx, gridDim);
 }
 
 cudaError_t launch_elocal_dw(const DevSystem &s, const double *r, const double *kin, double *eL, double *parts, int W,
                              cudaStream_t st, double *scal, const double *j3buf) {
   if (W <= 0) return cudaSuccess;
   if (s.use_j3 && !j3buf) return cudaErrorInvalidValue;
-  // threads: 128 where the walkers fill the SMs (32 warps each), more where they do
-  // not; 256 also where a whole number of threads per electron leaves over a
-  // quarter of 128 idle (N = 85: a third).  Grouped launches: 256, one kernel for all.
-  int threads = 128;
-  while (threads < kElocalDwThreads && (long)W * threads < 152L * 1024) threads *= 2;
-  if (threads == 128 && (s.N <= 128 ? 128 / s.N * s.N : 64) < 96) threads = 256;
-  if (group_recorder()) threads = 256;
+  // R threads per electron, in all about 128 up to N = 32, 256 up to 128, 512 above, but
+  // no more than pay for the sum over them (80 instructions each, not shared: R^2 of the
+  // order of an electron's pairs).  By the system alone, so that the sums' order, and with
+  // it the last bits of e_L, does not depend on how many walkers there are; chosen from
+  // 128, 192, 256, 384 and 512 threads and caps of 20, 80 and 300 over 1 to 4096
+  // walkers: 4096 of N = 32 132 us (178 with 256 threads), 16 walkers 14; 509 of N = 83
+  // 102 (122 with 512).  Up to 512 threads by the walkers' number, all shared out, took 95
+  // us for 512 walkers of two electrons, now 10.
+  const int target = s.N <= 32 ? 128 : (s.N <= 128 ? 256 : kElocalDwThreads);
+  const int most = static_cast<int>(ceil(sqrt((650.0 * s.n_atoms + 225.0 * s.N) / 300.0)));
+  int R = std::max(1, std::min(target / s.N, most));
+  int threads = std::min(kElocalDwThreads, (R * s.N + 31) / 32 * 32);
+  if (group_recorder()) {  // one launch for all systems
+    threads = 256;
+    if (R * s.N > threads) R = 1;
+  }
   // (216 KB: static shared memory and the arguments of a grouped launch come on top)
-  const size_t smem = ElocalDw<true>::smem(s, threads);
+  const size_t smem = ElocalDw<true>::smem(s, R);
   if (smem > 216 * 1024)
     return launch_or_record<ElocalDw<false>, kElocalDwThreads>(k_elocal_dw<false>, dim3(W), dim3(threads),
-                                                               ElocalDw<false>::smem(s, threads), st, s, r, kin, eL,
-                                                               parts, scal, j3buf);
+                                                               ElocalDw<false>::smem(s, R), st, s, r, kin, eL,
+                                                               parts, scal, j3buf, R);
   return launch_or_record<ElocalDw<true>, kElocalDwThreads>(k_elocal_dw<true>, dim3(W), dim3(threads), smem, st, s, r,
-                                                            kin, eL, parts, scal, j3buf);
+                                                            kin, eL, parts, scal, j3buf, R);
 }
 
 cudaError_t launch_elocal(const DevSystem &s, const double *r, const double *kin, double *eL, double *parts, int W,
