@@ -91,7 +91,9 @@ bool tc_refresh(const jagp_ctx *h) { return h->precision == JAGP_PREC_MIXED && h
 // rows take the tensor cores as the lambda products do, from N_up = 32 on: below,
 // the slices of a column padded to 64 terms cost as much to write as the FP64
 // product itself (N_up = 16, L = 320, 2048 walkers: 275 us either way); at N_up = 64, L = 1536 a
-// product of 256 walkers takes 0.3 ms instead of 2.7.
+// product of 256 walkers takes 0.3 ms instead of 2.7.  Few walkers near N_up = 32 pay for the
+// eight launches (e_L of 16 walkers, L = 320: 0.21 ms, 0.18 with FP64 instructions; of 256 0.52
+// against 0.63); the walkers' number does not choose, so that e_L does not depend on it.
 bool tc_products(const jagp_ctx *h) {
   return h->precision == JAGP_PREC_FP64 && h->tc_lambda && h->ds.n_up >= kTcProductsMinUp;
 }
