@@ -136,7 +136,7 @@ cudaError_t launch_umma_gemm(const uint16_t *A, int m_max, const int *m_dev, int
                              int batches = 0, int stages_max = 0, int b_batch_rows = 0, long long o_bstride = 0,
                              long long o_rstride = 0, long long o_cstride = 0, const int2 *krange = nullptr,
                              int klive = 0, bool add = false);
-// whether two chunk-major stages (stages_max = -1, -2, -3: K chunks of 64, 32,
+// whether two stages of every slice (stages_max = -1, -2, -3: K chunks of 64, 32,
 // 16) of these pairs fit at tile width bn
 bool umma_chunk_fits(int npairs, const int *pair_a, const int *pair_b, int bn, int stages_max);
 // FP64 rows -> nsl exact slices of `bits` bits per element plus a row exponent;

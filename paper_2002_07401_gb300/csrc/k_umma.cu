@@ -782,7 +782,7 @@ int g_smem_optin = 220 * 1024;  // the kernel's dynamic shared-memory limit, set
 uint32_t chunk_stage_bytes(int na, int nb, int bn, int cw) {
   return (static_cast<uint32_t>(na) * 128u + static_cast<uint32_t>(nb * bn)) * static_cast<uint32_t>(cw) * 2u;
 }
-// chunk width of the chunk-major modes: stages_max -1, -2, -3 -> 64, 32, 16
+// K chunk width: stages_max -1, -2, -3 -> 64, 32, 16
 int chunk_width(int stages_max) { return stages_max == -1 ? 64 : (stages_max == -2 ? 32 : 16); }
 // room for the stages: the limit less the 1 KB alignment slack and the barriers
 uint32_t chunk_budget() { return static_cast<uint32_t>(g_smem_optin - 1024 - 64); }
@@ -1421,7 +1421,7 @@ cudaError_t launch_pack_cols(const double *X64, const float *X32, const float *X
 
 cudaError_t setup_umma_attributes() {
   // the largest opt-in shared memory per block (227 KB on this part), so that
-  // two or more chunk-major stages of six slices fit (with K chunks of 32 or 16)
+  // two or more stages of every slice fit (with K chunks of 32 or 16)
   int dev = 0, optin = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
