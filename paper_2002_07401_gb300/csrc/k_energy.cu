@@ -619,6 +619,7 @@ cudaError_t launch_elocal_dw(const DevSystem &s, const double *r, const double *
   const int most = static_cast<int>(ceil(sqrt((650.0 * s.n_atoms + 225.0 * s.N) / 300.0)));
   int R = std::max(1, std::min(target / s.N, most));
   int threads = std::min(kElocalDwThreads, (R * s.N + 31) / 32 * 32);
+  R = std::max(R, std::min(threads / s.N, (4 * R + 2) / 3));  // (a last warp's idle lanes; R = 7 of N = 16: 8)
   if (group_recorder()) {  // one launch for all systems
     threads = 256;
     if (R * s.N > threads) R = 1;
